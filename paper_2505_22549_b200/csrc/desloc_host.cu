@@ -20,12 +20,11 @@
 namespace desloc {
 
 const void *lookup_step_kernel(int opt, bool post, bool bf16, int mt, int mask, bool diag) {
-    // A local step (mask 0) is the same code for either ordering and lives in the pre-average
-    // units.  Up to MAX_MT workers it uses the all-workers-per-chunk instantiation (more bytes
-    // per block and per pointer set-up); beyond that, and for M = 1, workers are separate work
-    // items of the local kernel.
+    // A local step (mask 0) has nothing to do with the other workers: it takes the one-replica
+    // kernel, whose blocks move 2-3 % more bytes per second than tiles of all replicas.  It lives
+    // in the pre-average units and is the same code for either ordering.
     const bool pre = !post || mask == 0;
-    const int m = (mask == 0 && !(mt >= 2 && mt <= MAX_MT)) ? 1 : mt;
+    const int m = mask == 0 ? 1 : mt;
     if (opt == OPT_ADAM) {
         if (diag) return pre ? lookup_adam_pre_diag(bf16, m, mask) : lookup_adam_post_diag(bf16, m, mask);
         return pre ? lookup_adam_pre(bf16, m, mask) : lookup_adam_post(bf16, m, mask);
@@ -69,6 +68,7 @@ struct HostGroup {
 struct WorkerRes {
     desloc::Chunk *d_chunks = nullptr;   // tiles of the step kernels
     int64_t nchunks = 0;
+    int64_t chunk_elems = 0;             // longest chunk of the plan
     long long *d_tstart = nullptr;       // [num_tensors + 1] first tile of every tensor
     std::vector<HostGroup> groups;
     void **d_tables = nullptr;  // [3][nptr] x, u, v
@@ -133,6 +133,7 @@ cudaError_t make_worker_res(WorkerRes &r, int M, const int64_t *numel, int num_t
         }
     }
     r.nchunks = nchunks;
+    r.chunk_elems = chunk_elems;
     cudaError_t e0 = cudaMalloc(&r.d_chunks, chunks.size() * sizeof(desloc::Chunk));
     if (e0 == cudaSuccess)
         e0 = cudaMemcpy(r.d_chunks, chunks.data(), chunks.size() * sizeof(desloc::Chunk), cudaMemcpyHostToDevice);
@@ -314,7 +315,7 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
             d_gscale = ctx->res.d_norms + c.M;
         }
 
-        const desloc::LaunchPlan plan = desloc::plan_launch(c, mask, ctx->res.nchunks, diag);
+        const desloc::LaunchPlan plan = desloc::plan_launch(c, mask, ctx->res.nchunks, ctx->res.chunk_elems, diag);
         if (!plan.fn) {
             rc = DESLOC_E_INVALID;
             break;
@@ -335,6 +336,8 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
         desloc::fill_hyper(a, c, lr_t, clip_bound_t);
         a.err = ctx->d_err;
         a.wait_limit = ctx->wait_limit;
+        a.parts = plan.parts;
+        a.part_elems = plan.part_elems;
         a.direct = ctx->staging_mode < 0 ? (plan.direct ? 1 : 0) : ctx->staging_mode;
 
         void *params[] = {&a};
@@ -353,7 +356,7 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
         }
         if (!host_grads) {
             e = cudaLaunchKernel(plan.fn, dim3(capped(plan)),
-                                 dim3(desloc::BLOCK_THREADS), params, plan.smem, stream);
+                                 dim3(static_cast<unsigned>(plan.threads)), params, plan.smem, stream);
             if (e == cudaSuccess) ctx->launches += 1;
         } else {
             // The device gradient buffers may still be read by earlier work on `stream`.
@@ -389,9 +392,11 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
                 a.chunks = ctx->res.d_chunks + grp.c0;
                 a.nchunks = grp.c1 - grp.c0;
                 a.diag_chunk0 = grp.c0;
-                const desloc::LaunchPlan gp = desloc::plan_launch(c, mask, a.nchunks, diag);
+                const desloc::LaunchPlan gp = desloc::plan_launch(c, mask, a.nchunks, ctx->res.chunk_elems, diag);
+                a.parts = gp.parts;
+                a.part_elems = gp.part_elems;
                 e = cudaLaunchKernel(gp.fn, dim3(capped(gp)),
-                                     dim3(desloc::BLOCK_THREADS), params, gp.smem, stream);
+                                     dim3(static_cast<unsigned>(gp.threads)), params, gp.smem, stream);
                 if (e == cudaSuccess) ctx->launches += 1;
             }
         }

@@ -13,28 +13,26 @@ const void *kernel_ptr() {
     return reinterpret_cast<const void *>(&desloc_step_kernel<OPT, MASK, MT, GT, POST, DIAG>);
 }
 
-// Masks FIRST..LAST for every MT in 2..MAX_MT.  LAST = 7 for Adam / ADOPT, 3 for SGDM (no
-// second state).  FIRST = 0 for the pre-average units (mask 0, the local step, is the same
-// code for either ordering) and 1 for the post-average ones.
-template <int OPT, bool POST, bool DIAG, typename GT, int FIRST, int NMASK, int... I>
+// Masks 1..NMASK for every MT in 2..MAX_MT.  NMASK = 7 for Adam / ADOPT, 3 for SGDM (no second
+// state).  Mask 0, the local step, is the one-replica kernel whatever the worker count.
+template <int OPT, bool POST, bool DIAG, typename GT, int NMASK, int... I>
 const void *pick_sync(int mt, int mask, std::integer_sequence<int, I...>) {
     static const void *const tbl[] = {
-        kernel_ptr<OPT, POST, DIAG, GT, 2 + I / NMASK, FIRST + I % NMASK>()...};
-    if (mt < 2 || mt > MAX_MT || mask < FIRST || mask >= FIRST + NMASK) return nullptr;
-    return tbl[(mt - 2) * NMASK + (mask - FIRST)];
+        kernel_ptr<OPT, POST, DIAG, GT, 2 + I / NMASK, 1 + I % NMASK>()...};
+    if (mt < 2 || mt > MAX_MT || mask < 1 || mask > NMASK) return nullptr;
+    return tbl[(mt - 2) * NMASK + (mask - 1)];
 }
 
 template <int OPT, bool POST, bool DIAG>
 const void *lookup_sync(bool bf16, int mt, int mask) {
-    constexpr int FIRST = POST ? 1 : 0;
-    constexpr int NMASK = ((OPT == OPT_SGDM) ? 3 : 7) + 1 - FIRST;
+    constexpr int NMASK = (OPT == OPT_SGDM) ? 3 : 7;
     using Seq = std::make_integer_sequence<int, (MAX_MT - 1) * NMASK>;
-    return bf16 ? pick_sync<OPT, POST, DIAG, bf16_t, FIRST, NMASK>(mt, mask, Seq{})
-                : pick_sync<OPT, POST, DIAG, float, FIRST, NMASK>(mt, mask, Seq{});
+    return bf16 ? pick_sync<OPT, POST, DIAG, bf16_t, NMASK>(mt, mask, Seq{})
+                : pick_sync<OPT, POST, DIAG, float, NMASK>(mt, mask, Seq{});
 }
 
-// One unit per (optimizer, ordering, diagnostics).  mt = 1 is the one-replica-per-tile kernel
-// (a single worker, or the local steps of more than MAX_MT workers); it lives in the pre units.
+// One unit per (optimizer, ordering, diagnostics).  mt = 1 is the one-replica-per-tile kernel (a
+// single worker, or a local step: the same code for either ordering); it lives in the pre units.
 template <int OPT, bool POST, bool DIAG>
 const void *lookup_unit(bool bf16, int mt, int mask) {
     if (mt == 1) {

@@ -83,7 +83,7 @@ inline uint32_t mask_at(const desloc_config *c, int64_t t) {
 // many as amortise the per-chunk pointer look-up on a large problem (max_tiles_per_chunk), fewer
 // on a small one, so that it still spreads over about four blocks per SM of a B200.
 inline int64_t chunk_elems_for(int32_t M, const int64_t *numel, int32_t num_tensors) {
-    const int64_t T = M <= MAX_MT ? tile_elems(M) : GENERIC_CHUNK_ELEMS;
+    const int64_t T = M <= MAX_MT ? plan_tile_elems(M) : GENERIC_CHUNK_ELEMS;
     const int64_t most = M <= MAX_MT ? max_tiles_per_chunk(M) : 8;
     int64_t tiles = 0;
     for (int32_t k = 0; k < num_tensors; ++k) tiles += (numel[k] + T - 1) / T;
@@ -127,11 +127,18 @@ inline int64_t count_chunks(const int64_t *numel, int32_t num_tensors, int64_t c
     return n;
 }
 
-// One thread block per chunk (per worker and chunk where workers are separate work items): does
-// the grid of a context with M workers fit, whatever the first chunks are cut to?
+// The one-replica kernel cuts a chunk into equal parts of at most this many of its tiles.
+inline int64_t parts_for(int64_t chunk_elems, int tiles) {
+    const int64_t most = static_cast<int64_t>(tiles) * tile_elems(1);
+    return (chunk_elems + most - 1) / most;
+}
+
+// One thread block per part of a chunk and worker on a local step, one per chunk on the others: does
+// the largest grid of a context with M workers fit, whatever the first chunks are cut to?
 inline bool grid_fits(int32_t M, const int64_t *numel, int32_t num_tensors) {
     const int64_t nchunks = count_chunks(numel, num_tensors, chunk_elems_for(M, numel, num_tensors)) + num_tensors;
-    const int64_t per_chunk = (M == 1 || M > MAX_MT) ? M : 1;
+    const int64_t chunk_elems = chunk_elems_for(M, numel, num_tensors);
+    const int64_t per_chunk = M * parts_for(chunk_elems, 3);
     return nchunks <= 0x7fffffffLL / per_chunk;
 }
 
@@ -176,6 +183,8 @@ inline void fill_hyper(StepArgs &a, const desloc_config &c, float lr_t, float cl
     a.wait_limit = DEFAULT_WAIT_LIMIT;
     a.err = nullptr;
     a.direct = 0;
+    a.parts = 1;
+    a.part_elems = 0;
 }
 
 // Which kernel a step of this configuration runs, and over how many blocks.
@@ -184,6 +193,8 @@ struct LaunchPlan {
     long long grid = 0;
     bool strides = true;  // a smaller grid may stride over the work items (not the runtime-M kernel)
     int smem = 0;         // dynamic shared memory of the launch
+    int threads = BLOCK_THREADS;
+    int parts = 1, part_elems = 0;   // one-replica kernel: parts of a chunk
     bool direct = false;  // too small to gain from staging: update straight from global memory
 };
 
@@ -191,6 +202,9 @@ struct LaunchPlan {
 // skip the staging.  Measured on the 4096-parameter, two-worker workload: 3.08 us per step in a
 // CUDA graph of 16 steps against 3.34 us staged.
 constexpr long long DIRECT_GRID = 2 * 148;
+// One-replica kernel: blocks resident at once (seven per SM).  A problem this small takes
+// one tile per block, straight from global memory.
+constexpr long long LOCAL_WAVE = 7 * 148;
 
 // The tile kernels use more than the 48 KB of shared memory a kernel gets by default: raise the
 // function's limit to what the launch asks for.  Not an allocation.
@@ -199,22 +213,35 @@ inline cudaError_t prepare_launch(const LaunchPlan &p) {
     return cudaFuncSetAttribute(p.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
 }
 
-inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, long long nchunks, bool diag) {
+inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, long long nchunks, int64_t chunk_elems,
+                              bool diag) {
     LaunchPlan p;
     // The mean of one replica is the replica: M = 1 always runs the local kernel.
     const uint32_t kmask = (c.M == 1) ? 0u : mask;
     const bool post = (c.flags & DESLOC_FLAG_POST_AVERAGE) != 0;
     const bool bf16 = c.grad_dtype == DESLOC_BF16;
-    const bool per_worker_items = (c.M == 1) || (kmask == 0 && c.M > MAX_MT);
-    const bool generic = kmask != 0 && c.M > MAX_MT;
+    const bool local = kmask == 0;
+    const bool generic = !local && c.M > MAX_MT;
     p.fn = generic ? lookup_generic_kernel(c.opt, post, bf16, static_cast<int>(kmask), diag)
                    : lookup_step_kernel(c.opt, post, bf16, c.M, static_cast<int>(kmask), diag);
     p.strides = !generic;
-    p.smem = generic ? 0 : step_smem_bytes(c.opt, per_worker_items ? 1 : c.M, bf16);
-    p.grid = per_worker_items ? nchunks * c.M : nchunks;
-    const int mt = per_worker_items ? 1 : c.M;
-    p.direct = p.grid <= DIRECT_GRID && mt <= MAX_MT &&
-               chunk_elems_for(c.M, c.numel, c.num_tensors) == tile_elems(mt);
+    const int mt = local ? 1 : c.M;
+    p.smem = generic ? 0 : step_smem_bytes(c.opt, mt, bf16);
+    if (!generic) p.threads = step_threads(mt);
+    p.grid = nchunks;
+    if (local) {
+        // (the diagnostics write one partial sum per chunk: their blocks take whole chunks)
+        const int64_t tile = tile_elems(1), tiles = chunk_elems / tile;
+        int64_t parts = diag ? 1 : parts_for(chunk_elems, local_tiles(c.opt, bf16));
+        // a problem that fits in one wave of blocks is pure latency: one tile per block
+        if (!diag && nchunks * tiles * c.M <= LOCAL_WAVE) parts = tiles;
+        p.parts = static_cast<int>(parts);
+        p.part_elems = static_cast<int>((tiles + parts - 1) / parts * tile);
+        p.grid = nchunks * parts * c.M;
+        p.direct = p.grid <= LOCAL_WAVE && p.part_elems <= tile;
+    } else if (!generic) {
+        p.direct = p.grid <= DIRECT_GRID && chunk_elems <= plan_tile_elems(c.M);
+    }
     return p;
 }
 

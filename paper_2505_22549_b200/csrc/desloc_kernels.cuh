@@ -44,7 +44,7 @@ namespace desloc {
 
 constexpr int OPT_ADAM = 0, OPT_ADOPT = 1, OPT_SGDM = 2;
 constexpr int SYNC_X = 1, SYNC_U = 2, SYNC_V = 4;
-constexpr int BLOCK_THREADS = 256;
+constexpr int BLOCK_THREADS = 256; // of every kernel but the one-replica step kernel
 constexpr int MAX_MT = 8;          // largest worker count with a kernel instantiated for it
 constexpr int DIAG_G = 0, DIAG_X = 1, DIAG_D = 2, DIAG_KINDS = 3;
 constexpr int REDUCE_CHUNK_ELEMS = BLOCK_THREADS * 16;  // chunks of the reduction kernels (4096)
@@ -53,11 +53,22 @@ constexpr int DRAIN_WAIT_LIMIT = 1 << 22;               // bound on the wait for
 
 // Elements per tile and worker for a kernel that holds mt replicas per tile: bulk copies of
 // 2-4 KB per state array (copies of 1 KB and 512 B, with 256-element tiles, were 5 % slower on
-// eight workers), 28-57 KB of shared memory per buffer.
-__host__ __device__ constexpr int tile_elems(int mt) { return mt <= 2 ? 1024 : 512; }
+// eight workers), 7-57 KB of shared memory per buffer.
+__host__ __device__ constexpr int tile_elems(int mt) { return mt == 2 ? 1024 : 512; }
+// The unit in which a context's chunk table is cut (chunks are whole multiples of it).
+__host__ __device__ constexpr int plan_tile_elems(int m) { return m <= 2 ? 1024 : 512; }
 // Tiles per chunk on large problems (one pointer look-up and one pipeline fill serve them all):
 // 8 measured best (4: sync steps 2 % slower; 16: 0.5-1 % slower; 32: 2 % slower).
 __host__ __device__ constexpr int max_tiles_per_chunk(int) { return 8; }
+
+// The one-replica kernel (local steps, a single worker) takes at most this many tiles of a chunk
+// per block: four, one for each of its buffers, or three where a tile is 8 KB (fp32 gradients and
+// two states).  Measured on B200 (Adam, eight workers, 50 GB moved): bf16 gradients 6.99 TB/s, against
+// 6.92 with six tiles per block in the same buffers, 6.85 with eight tiles of 1024 elements in
+// three buffers, and 6.78 for the kernel that holds all eight replicas per tile; fp32 gradients 6.99
+// with three, 6.87 with four -- blocks that request everything they will ever need at once
+// and leave keep the memory system busiest.
+__host__ __device__ constexpr int local_tiles(int opt, bool bf16) { return !bf16 && opt != OPT_SGDM ? 3 : 4; }
 
 struct __align__(16) Chunk {
     int32_t tensor;  // index into the tensor list
@@ -82,6 +93,8 @@ struct StepArgs {
     int *err;             // set to 1 when a bounded wait ran out (may be nullptr)
     int wait_limit;       // iterations a block polls for its tile before it gives up
     int direct;           // non-zero: no staging, every chunk straight from global memory (tiny launches)
+    int parts;            // one-replica kernel: a chunk is this many work items ...
+    int part_elems;       // ... of this many elements (a multiple of the tile; the last ones may be empty)
     int nt;
     int M;
     float b1, omb1;   // beta1, 1 - beta1
@@ -340,7 +353,7 @@ struct GlobalAcc4 {
 // all tiles of a chunk.  At the end of the chunk a warp reduces each of them (shuffle tree) into
 // its slot of shared memory and the block total is the eight warp slots added in order:
 // deterministic, and a few dozen shuffles per thread and chunk.
-template <bool DIAG, int MT>
+template <bool DIAG, int MT, int THREADS = BLOCK_THREADS>
 struct ThreadNorms {
     float acc[DIAG ? DIAG_KINDS * MT : 1];
     __device__ __forceinline__ void clear() {
@@ -350,7 +363,7 @@ struct ThreadNorms {
     __device__ __forceinline__ void add(int kind, int m, float v) {
         if constexpr (DIAG) acc[kind * MT + m] += v;
     }
-    // all threads of the block call; slots: [DIAG_KINDS * MT][BLOCK_THREADS / 32]
+    // all threads of the block call; slots: [DIAG_KINDS * MT][THREADS / 32]
     __device__ __forceinline__ void reduce_into(float *slots) const {
         if constexpr (DIAG) {
 #pragma unroll
@@ -358,7 +371,7 @@ struct ThreadNorms {
                 float v = acc[j];
 #pragma unroll
                 for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-                if ((threadIdx.x & 31) == 0) slots[j * (BLOCK_THREADS / 32) + (threadIdx.x >> 5)] = v;
+                if ((threadIdx.x & 31) == 0) slots[j * (THREADS / 32) + (threadIdx.x >> 5)] = v;
             }
         }
     }
@@ -386,9 +399,9 @@ __device__ __forceinline__ FV<VEC> mean_over_workers(const Acc &acc, int arr, in
 // Post-average (Algorithms 4-5): every worker updates its states, the ones to be averaged are
 // replaced by their means, the parameter step uses those, and a synced x is averaged last.
 // A thread re-reads values it stored itself (never another thread's), so no barrier is needed.
-template <int OPT, int MASK, int MT, bool POST, bool DIAG, bool PLAIN = false, typename Acc>
+template <int OPT, int MASK, int MT, bool POST, bool DIAG, bool PLAIN = false, typename Acc, typename Norms>
 __device__ __forceinline__ void update_position(const StepArgs &a, const Acc &acc, const float *sscale,
-                                                int q, ThreadNorms<DIAG, MT> &wn) {
+                                                int q, Norms &wn) {
     constexpr bool active = true;
     constexpr int VEC = Acc::VEC;
     constexpr bool SX = MASK & SYNC_X, SU = MASK & SYNC_U;
@@ -531,19 +544,27 @@ __device__ __forceinline__ bool bar_wait(uint64_t *bar, uint32_t parity, int lim
     return false;
 }
 
-constexpr int STAGES = 2;         // tile buffers per block (three stages at two blocks per SM: 0.84)
-// Resident blocks per SM: what the two buffers leave room for (three up to four workers, two
-// beyond).
-__host__ __device__ constexpr int step_min_blocks(int mt) { return mt <= 4 ? 3 : 2; }
+// Threads, tile buffers and resident blocks per SM.  All replicas of a tile: two buffers of
+// 28-57 KB and 256 threads, as many blocks as the buffers leave room for (three up to four
+// workers, two beyond; three buffers at two blocks per SM: 0.84 of the copy bandwidth).  One
+// replica: four buffers of 7 KB (bf16 gradients; 5 KB without v) and 128 threads, one float4 of
+// each array per thread and tile, six to ten blocks (three buffers and three tiles: 0.4 % slower;
+// five or six buffers: 3-8 % slower, too few blocks).
+__host__ __device__ constexpr int step_threads(int mt) { return mt == 1 ? 128 : BLOCK_THREADS; }
+__host__ __device__ constexpr int step_stages(int opt, int mt, bool bf16) {
+    return mt == 1 ? local_tiles(opt, bf16) : 2;
+}
+__host__ __device__ constexpr int step_min_blocks(int mt) { return mt == 1 ? 8 : mt <= 4 ? 3 : 2; }
 
 // A chunk is a run of consecutive tiles of one tensor.  The block looks its pointers up
-// once, then streams the tiles through a ring of STAGES buffers: while tile k is updated in
-// place, tile k + 1 is already landing; when tile k's copy back has left its buffer, tile
-// k + STAGES is requested into it.
+// once, then streams the tiles through a ring of S buffers: while tile k is updated in
+// place, tiles k + 1 .. k + S - 1 are already landing; when tile k's copy back has left its
+// buffer, tile k + S is requested into it.
 template <int OPT, int MASK, int MT, typename GT, bool POST, bool DIAG>
-__global__ void __launch_bounds__(BLOCK_THREADS, step_min_blocks(MT))
+__global__ void __launch_bounds__(step_threads(MT), step_min_blocks(MT))
 desloc_step_kernel(const __grid_constant__ StepArgs a) {
-    constexpr int T = tile_elems(MT), VEC = T / BLOCK_THREADS, S = STAGES;
+    constexpr int THREADS = step_threads(MT);
+    constexpr int T = tile_elems(MT), VEC = T / THREADS, S = step_stages(OPT, MT, sizeof(GT) == 2);
     constexpr int ALIGN_ELEMS = 16 / static_cast<int>(sizeof(GT));   // bulk copies move multiples of 16 bytes
     constexpr bool HAS_V = OPT != OPT_SGDM;
     using L = TileLayout<OPT, MT, GT, T>;
@@ -552,7 +573,7 @@ desloc_step_kernel(const __grid_constant__ StepArgs a) {
     __shared__ char *sp[4][MT];
     __shared__ float sscale[MT];
     __shared__ __align__(8) uint64_t bar[S];
-    ThreadNorms<DIAG, MT> wn;
+    ThreadNorms<DIAG, MT, THREADS> wn;
     const int tid = threadIdx.x;
     if (tid < S) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&bar[tid])) : "memory");
@@ -568,28 +589,39 @@ desloc_step_kernel(const __grid_constant__ StepArgs a) {
     // inner loop without them (three instructions of about forty per coordinate: with eight
     // workers at sustained clocks 0.4-0.7 % of the step).  The fallback paths keep the one form.
     const bool plain = a.gscale == nullptr && a.rho > 3.4028235e38f;   // rho = +inf: clip off
-    // Work items: chunks of all MT replicas; with MT = 1, (worker, chunk) pairs -- the single
-    // replica and the local steps of more than MAX_MT workers.  One item per block as launched;
-    // a smaller grid strides over the rest.
-    const long long nitems = MT == 1 ? a.nchunks * a.M : a.nchunks;
+    // Work items: chunks of all MT replicas; with MT = 1 (a single worker, local steps) parts of a
+    // chunk of one replica, worker by worker.  One item per block as launched (fewer than 2^31); a
+    // smaller grid strides over the rest.
+    const long long nitems = MT == 1 ? a.nchunks * a.parts * a.M : a.nchunks;
     for (long long item = blockIdx.x; item < nitems; item += gridDim.x) {
-        const long long c = MT == 1 ? item % a.nchunks : item;
-        const int m0 = MT == 1 ? static_cast<int>(item / a.nchunks) : 0;
+        long long c = item;
+        int m0 = 0, sub0 = 0;
+        if constexpr (MT == 1) {
+            const unsigned it = static_cast<unsigned>(item), nc = static_cast<unsigned>(a.nchunks);
+            const unsigned q = it / static_cast<unsigned>(a.parts);   // (worker, chunk)
+            sub0 = static_cast<int>(it - q * a.parts) * a.part_elems;
+            m0 = static_cast<int>(q / nc);
+            c = q - m0 * nc;
+        }
+        // (asked for before the chunk and pointer look-ups, not behind them)
+        const float my_scale = tid < MT && a.gscale ? a.gscale[m0 + tid] : 1.f;
         const Chunk ch = a.chunks[c];   // the same 16 bytes for every thread
-        const int count = ch.count;
+        const int count = MT == 1 ? min(ch.count - sub0, a.part_elems) : ch.count;
+        const long long start = ch.start + sub0;
+        if (MT == 1 && count <= 0) continue;   // a short chunk has fewer parts
         __syncthreads();  // the previous item is done with the shared state; the barriers exist
         char *p = nullptr;
         if (owner) {
             const long long idx = static_cast<long long>(m0 + m) * a.nt + ch.tensor;
-            if (arr == 0) p = reinterpret_cast<char *>(a.x[idx]) + ch.start * 4;
-            if (arr == 1) p = reinterpret_cast<char *>(a.u[idx]) + ch.start * 4;
-            if (arr == 2) p = reinterpret_cast<char *>(a.v[idx]) + ch.start * 4;
+            if (arr == 0) p = reinterpret_cast<char *>(a.x[idx]) + start * 4;
+            if (arr == 1) p = reinterpret_cast<char *>(a.u[idx]) + start * 4;
+            if (arr == 2) p = reinterpret_cast<char *>(a.v[idx]) + start * 4;
             if (arr == 3)
                 p = const_cast<char *>(reinterpret_cast<const char *>(grad_ptr(a, idx))) +
-                    ch.start * static_cast<long long>(sizeof(GT));
+                    start * static_cast<long long>(sizeof(GT));
             sp[arr][m] = p;
         }
-        if (tid < MT) sscale[tid] = a.gscale ? a.gscale[m0 + tid] : 1.f;
+        if (tid < MT) sscale[tid] = my_scale;
         wn.clear();
         // bulk copies need 16-byte aligned addresses; a tile of the chunk also a byte count that
         // is a multiple of 16 (only the chunk's last tile can miss that: it is then updated
@@ -657,12 +689,12 @@ desloc_step_kernel(const __grid_constant__ StepArgs a) {
             if (wide_ok) {
                 const GlobalAcc4<MT, GT> acc4{sp};
                 const int p1 = count >> 2;
-                for (int q = (e0 >> 2) + tid; q < p1; q += BLOCK_THREADS)
+                for (int q = (e0 >> 2) + tid; q < p1; q += THREADS)
                     update_position<OPT, MASK, MT, POST, DIAG>(a, acc4, sscale, q, wn);
                 e0 = p1 << 2;
             }
             const GlobalAcc<MT, GT> acc{sp};
-            for (int e = e0 + tid; e < count; e += BLOCK_THREADS)
+            for (int e = e0 + tid; e < count; e += THREADS)
                 update_position<OPT, MASK, MT, POST, DIAG>(a, acc, sscale, e, wn);
         }
         // the copies back must have left shared memory before the buffers are reused or freed
@@ -676,7 +708,7 @@ desloc_step_kernel(const __grid_constant__ StepArgs a) {
             if (tid < DIAG_KINDS * MT) {
                 float total = 0.f;
 #pragma unroll
-                for (int w = 0; w < BLOCK_THREADS / 32; ++w) total += slots[tid * (BLOCK_THREADS / 32) + w];
+                for (int w = 0; w < THREADS / 32; ++w) total += slots[tid * (THREADS / 32) + w];
                 const int kind = tid / MT, mm = tid - kind * MT;
                 a.diag[(static_cast<long long>(kind) * a.M + m0 + mm) * a.diag_stride + a.diag_chunk0 + c] = total;
             }
@@ -687,11 +719,11 @@ desloc_step_kernel(const __grid_constant__ StepArgs a) {
 
 // Dynamic shared memory a launch of desloc_step_kernel<opt, ., mt, grad type, ., .> needs.
 __host__ __device__ constexpr int step_smem_bytes(int opt, int mt, bool bf16) {
-    return STAGES * mt * tile_elems(mt) * ((bf16 ? 2 : 4) + 4 * (opt == OPT_SGDM ? 2 : 3));
+    return step_stages(opt, mt, bf16) * mt * tile_elems(mt) * ((bf16 ? 2 : 4) + 4 * (opt == OPT_SGDM ? 2 : 3));
 }
 
 // Lookup of an instantiation: opt, post-average?, bf16 gradients?, MT in 1..MAX_MT, mask,
-// with or without the norm diagnostics (MT = 1 exists for mask 0 only).
+// with or without the norm diagnostics (MT = 1 exists for mask 0 only, and mask 0 for MT = 1).
 // Returns nullptr for combinations that do not exist (sync masks with M > MAX_MT).
 const void *lookup_step_kernel(int opt, bool post, bool bf16, int mt, int mask, bool diag);
 

@@ -98,7 +98,7 @@ extern "C" DESLOC_API int desloc_step_static(const desloc_config *cfg, float *co
     const int64_t nchunks = desloc::count_chunks(cfg->numel, cfg->num_tensors, chunk_elems, g_heads);
     if (nchunks > kMaxChunks) return DESLOC_E_TOO_LARGE;
     const uint32_t mask = desloc::mask_at(cfg, t);
-    const desloc::LaunchPlan plan = desloc::plan_launch(*cfg, mask, nchunks, false);
+    const desloc::LaunchPlan plan = desloc::plan_launch(*cfg, mask, nchunks, chunk_elems, false);
     if (!plan.fn) return DESLOC_E_INVALID;
 
     int dev_before = -1;
@@ -178,11 +178,13 @@ extern "C" DESLOC_API int desloc_step_static(const desloc_config *cfg, float *co
         a.diag = nullptr;
         desloc::fill_hyper(a, *cfg, lr_t, clip_bound_t);
         a.direct = plan.direct ? 1 : 0;
+        a.parts = plan.parts;
+        a.part_elems = plan.part_elems;
         void *params[] = {&a};
         e = desloc::prepare_launch(plan);
         if (e == cudaSuccess)
             e = cudaLaunchKernel(plan.fn, dim3(static_cast<unsigned>(plan.grid)),
-                                 dim3(desloc::BLOCK_THREADS), params, plan.smem, st);
+                                 dim3(static_cast<unsigned>(plan.threads)), params, plan.smem, st);
         if (e != cudaSuccess) { rc = DESLOC_E_CUDA; break; }
     } while (false);
     if (rc == DESLOC_E_CUDA) (void)cudaGetLastError();

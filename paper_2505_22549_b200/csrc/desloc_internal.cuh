@@ -127,10 +127,9 @@ inline int64_t count_chunks(const int64_t *numel, int32_t num_tensors, int64_t c
     return n;
 }
 
-// The one-replica kernel cuts a chunk into equal parts of at most this many of its tiles.
-inline int64_t parts_for(int64_t chunk_elems, int tiles) {
-    const int64_t most = static_cast<int64_t>(tiles) * tile_elems(1);
-    return (chunk_elems + most - 1) / most;
+// Blocks that share a chunk of all mt replicas (of one, for mt = 1).
+inline int64_t parts_for(int64_t chunk_elems, int mt) {
+    return (chunk_elems + most_part_elems(mt) - 1) / most_part_elems(mt);
 }
 
 // One thread block per part of a chunk and worker on a local step, one per chunk on the others: does
@@ -138,7 +137,7 @@ inline int64_t parts_for(int64_t chunk_elems, int tiles) {
 inline bool grid_fits(int32_t M, const int64_t *numel, int32_t num_tensors) {
     const int64_t nchunks = count_chunks(numel, num_tensors, chunk_elems_for(M, numel, num_tensors)) + num_tensors;
     const int64_t chunk_elems = chunk_elems_for(M, numel, num_tensors);
-    const int64_t per_chunk = M * parts_for(chunk_elems, 3);
+    const int64_t per_chunk = M * parts_for(chunk_elems, 1);
     return nchunks <= 0x7fffffffLL / per_chunk;
 }
 
@@ -193,8 +192,9 @@ struct LaunchPlan {
     long long grid = 0;
     bool strides = true;  // a smaller grid may stride over the work items (not the runtime-M kernel)
     int smem = 0;         // dynamic shared memory of the launch
+    int smem_limit = 0;   // of any launch of this kernel
     int threads = BLOCK_THREADS;
-    int parts = 1, part_elems = 0;   // one-replica kernel: parts of a chunk
+    int parts = 1, part_elems = 0;   // blocks that share a chunk, and elements of it for each
     bool direct = false;  // too small to gain from staging: update straight from global memory
 };
 
@@ -202,15 +202,16 @@ struct LaunchPlan {
 // skip the staging.  Measured on the 4096-parameter, two-worker workload: 3.08 us per step in a
 // CUDA graph of 16 steps against 3.34 us staged.
 constexpr long long DIRECT_GRID = 2 * 148;
-// One-replica kernel: blocks resident at once (seven per SM).  A problem this small takes
-// one tile per block, straight from global memory.
+// One-replica kernel: a problem of at most seven blocks per SM takes one tile per block, straight
+// from global memory.
 constexpr long long LOCAL_WAVE = 7 * 148;
 
 // The tile kernels use more than the 48 KB of shared memory a kernel gets by default: raise the
-// function's limit to what the launch asks for.  Not an allocation.
+// function's limit to the most that any launch of it asks for (launches of other contexts, with
+// more tiles per block, share it).  Not an allocation.
 inline cudaError_t prepare_launch(const LaunchPlan &p) {
-    if (p.smem <= 32 * 1024) return cudaSuccess;   // with the kernel's static part still under 48 KB
-    return cudaFuncSetAttribute(p.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
+    if (p.smem_limit <= 32 * 1024) return cudaSuccess;   // with the kernel's static part still under 48 KB
+    return cudaFuncSetAttribute(p.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem_limit);
 }
 
 inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, long long nchunks, int64_t chunk_elems,
@@ -226,21 +227,21 @@ inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, long long n
                    : lookup_step_kernel(c.opt, post, bf16, c.M, static_cast<int>(kmask), diag);
     p.strides = !generic;
     const int mt = local ? 1 : c.M;
-    p.smem = generic ? 0 : step_smem_bytes(c.opt, mt, bf16);
-    if (!generic) p.threads = step_threads(mt);
     p.grid = nchunks;
-    if (local) {
+    if (!generic) {
+        const int64_t tile = tile_elems(c.opt, mt, bf16), tiles = chunk_elems / tile;
+        const int64_t replicas = local ? c.M : 1;
         // (the diagnostics write one partial sum per chunk: their blocks take whole chunks)
-        const int64_t tile = tile_elems(1), tiles = chunk_elems / tile;
-        int64_t parts = diag ? 1 : parts_for(chunk_elems, local_tiles(c.opt, bf16));
-        // a problem that fits in one wave of blocks is pure latency: one tile per block
-        if (!diag && nchunks * tiles * c.M <= LOCAL_WAVE) parts = tiles;
+        int64_t parts = diag ? 1 : parts_for(chunk_elems, mt);
+        // a step that fits in one wave of blocks is pure latency: one tile per block
+        if (!diag && nchunks * tiles * replicas <= (local ? LOCAL_WAVE : DIRECT_GRID)) parts = tiles;
         p.parts = static_cast<int>(parts);
         p.part_elems = static_cast<int>((tiles + parts - 1) / parts * tile);
-        p.grid = nchunks * parts * c.M;
-        p.direct = p.grid <= LOCAL_WAVE && p.part_elems <= tile;
-    } else if (!generic) {
-        p.direct = p.grid <= DIRECT_GRID && chunk_elems <= plan_tile_elems(c.M);
+        p.threads = step_threads(mt);
+        p.smem = step_smem_bytes(c.opt, mt, bf16, p.part_elems);
+        p.smem_limit = step_smem_bytes(c.opt, mt, bf16, most_part_elems(mt));
+        p.grid = nchunks * parts * replicas;
+        p.direct = p.grid <= (local ? LOCAL_WAVE : DIRECT_GRID) && p.part_elems <= (local ? tile : plan_tile_elems(mt));
     }
     return p;
 }

@@ -2,12 +2,12 @@
 // worker replicas (Algorithm 1 with the Adam, ADOPT and SGDM rules of Algorithms 2-3).
 //
 // Work decomposition.  The tensor list is cut into chunks of one tensor (table built once on the
-// host); a chunk is a run of up to 8 tiles of tile_elems(M) elements.  A thread block takes
-// one chunk of ALL M replicas (for M = 1, and on local steps of more than eight workers, of
-// one replica) and streams its tiles through two shared-memory buffers:
+// host); a chunk is a run of up to 8 or 16 tiles.  A thread block takes a chunk (or a part of one) of
+// ALL M replicas -- on local steps, and for M = 1, of one replica -- and streams its tiles
+// through two shared-memory buffers (one replica: as many as it has tiles):
 //   1. the first 4*M threads look up the chunk's pointers once; each owns one (array, worker)
 //      and issues ONE 1-D bulk asynchronous copy per tile (cp.async.bulk, the TMA engine; no
-//      multicast, this GPU's own memory) of its 1-4 KB slice into the tile's buffer, all
+//      multicast, this GPU's own memory) of its 1-2 KB slice into the tile's buffer, all
 //      signalling the buffer's mbarrier;
 //   2. the block waits for the mbarrier (bounded; see bar_wait), then every thread updates its
 //      coordinates in place in shared memory: the arrays whose period divides t are averaged
@@ -16,7 +16,7 @@
 //   3. the owners of x, u, v each issue one bulk copy of the updated slice back, and, once
 //      that copy has read the buffer, request the tile after next into it.
 // While tile k is updated, tile k + 1 is landing and tile k - 1 is on its way back.  Two to
-// three blocks are resident per SM.  A chunk whose pointers are not 16-byte aligned, and a
+// seven blocks are resident per SM (one replica: ten).  A chunk whose pointers are not 16-byte aligned, and a
 // ragged last tile whose byte counts are not multiples of 16, take the same arithmetic straight
 // from and to global memory: four coordinates per thread with 128-bit accesses where the fp32
 // arrays are 16-byte and the gradients at least 8-byte aligned, else one coordinate per thread.
@@ -51,24 +51,29 @@ constexpr int REDUCE_CHUNK_ELEMS = BLOCK_THREADS * 16;  // chunks of the reducti
 constexpr int GENERIC_CHUNK_ELEMS = 1024;               // chunks of contexts with M > MAX_MT
 constexpr int DRAIN_WAIT_LIMIT = 1 << 22;               // bound on the wait for copies in flight
 
-// Elements per tile and worker for a kernel that holds mt replicas per tile: bulk copies of
-// 2-4 KB per state array (copies of 1 KB and 512 B, with 256-element tiles, were 5 % slower on
-// eight workers), 7-57 KB of shared memory per buffer.
-__host__ __device__ constexpr int tile_elems(int mt) { return mt == 2 ? 1024 : 512; }
+// Elements per tile and worker for a kernel that holds mt replicas per tile: bulk copies of 2 KB per
+// state array, 7-57 KB of shared memory per buffer (with bf16 gradients copies of 1 KB and 512 B,
+// with 256-element tiles, were 5 % slower on eight workers).  Eight replicas with fp32 gradients and
+// two states would need 64 KB per buffer, which leaves room for one block per SM: 256-element
+// tiles and three blocks move 6.64 TB/s there instead of 5.5 (all-sync steps of 14 GB).
+__host__ __device__ constexpr int tile_elems(int opt, int mt, bool bf16) {
+    return mt == 8 && !bf16 && opt != OPT_SGDM ? 256 : 512;
+}
 // The unit in which a context's chunk table is cut (chunks are whole multiples of it).
 __host__ __device__ constexpr int plan_tile_elems(int m) { return m <= 2 ? 1024 : 512; }
 // Tiles per chunk on large problems (one pointer look-up and one pipeline fill serve them all):
 // 8 measured best (4: sync steps 2 % slower; 16: 0.5-1 % slower; 32: 2 % slower).
 __host__ __device__ constexpr int max_tiles_per_chunk(int) { return 8; }
 
-// The one-replica kernel (local steps, a single worker) takes at most this many tiles of a chunk
-// per block: four, one for each of its buffers, or three where a tile is 8 KB (fp32 gradients and
-// two states).  Measured on B200 (Adam, eight workers, 50 GB moved): bf16 gradients 6.99 TB/s, against
-// 6.92 with six tiles per block in the same buffers, 6.85 with eight tiles of 1024 elements in
-// three buffers, and 6.78 for the kernel that holds all eight replicas per tile; fp32 gradients 6.99
-// with three, 6.87 with four -- blocks that request everything they will ever need at once
-// and leave keep the memory system busiest.
-__host__ __device__ constexpr int local_tiles(int opt, bool bf16) { return !bf16 && opt != OPT_SGDM ? 3 : 4; }
+// Elements of a chunk that one block takes.  One replica (local steps, a single worker): three
+// tiles, one for each of its buffers.  Blocks that request everything they will ever need at once
+// and leave keep the memory system busiest, the more of them the better: measured on B200 (Adam,
+// bf16 gradients, 14 GB per step, a third of a second into the board's power cap) 6.92 TB/s with three
+// tiles and ten blocks per SM, 6.86 with four and seven, 6.84-6.91 with two and ten to fifteen,
+// 6.24-6.49 with tiles twice or four times as long, 6.79 for tiles of all replicas.  Two replicas: four tiles
+// through two buffers, 6.85 against 6.78 with eight tiles of 1024 elements.  More: whole chunks
+// (four tiles instead of eight cost eight workers 2 %, four workers nothing).
+__host__ __device__ constexpr int most_part_elems(int mt) { return mt == 1 ? 3 * 512 : mt == 2 ? 4 * 512 : 8 * 512; }
 
 struct __align__(16) Chunk {
     int32_t tensor;  // index into the tensor list
@@ -93,7 +98,7 @@ struct StepArgs {
     int *err;             // set to 1 when a bounded wait ran out (may be nullptr)
     int wait_limit;       // iterations a block polls for its tile before it gives up
     int direct;           // non-zero: no staging, every chunk straight from global memory (tiny launches)
-    int parts;            // one-replica kernel: a chunk is this many work items ...
+    int parts;            // a chunk is this many work items (per replica, for the one-replica kernel) ...
     int part_elems;       // ... of this many elements (a multiple of the tile; the last ones may be empty)
     int nt;
     int M;
@@ -544,27 +549,26 @@ __device__ __forceinline__ bool bar_wait(uint64_t *bar, uint32_t parity, int lim
     return false;
 }
 
-// Threads, tile buffers and resident blocks per SM.  All replicas of a tile: two buffers of
-// 28-57 KB and 256 threads, as many blocks as the buffers leave room for (three up to four
+// Threads, tile buffers and resident blocks per SM.  Three and more replicas of a tile: two buffers
+// of 21-57 KB and 256 threads, as many blocks as the buffers leave room for (three up to four
 // workers, two beyond; three buffers at two blocks per SM: 0.84 of the copy bandwidth).  One
-// replica: four buffers of 7 KB (bf16 gradients; 5 KB without v) and 128 threads, one float4 of
-// each array per thread and tile, six to ten blocks (three buffers and three tiles: 0.4 % slower;
-// five or six buffers: 3-8 % slower, too few blocks).
-__host__ __device__ constexpr int step_threads(int mt) { return mt == 1 ? 128 : BLOCK_THREADS; }
-__host__ __device__ constexpr int step_stages(int opt, int mt, bool bf16) {
-    return mt == 1 ? local_tiles(opt, bf16) : 2;
+// replica: up to three buffers of 7 KB (bf16 gradients; 5 KB without v) and 128 threads, one float4 of
+// each array per thread and tile, ten blocks.
+__host__ __device__ constexpr int step_threads(int mt) { return mt <= 2 ? 128 : BLOCK_THREADS; }
+__host__ __device__ constexpr int step_stages(int mt) { return mt == 1 ? 3 : 2; }
+__host__ __device__ constexpr int step_min_blocks(int opt, int mt, bool bf16) {
+    return mt == 1 ? 10 : mt == 2 ? 7 : mt <= 4 || tile_elems(opt, mt, bf16) < 512 ? 3 : 2;
 }
-__host__ __device__ constexpr int step_min_blocks(int mt) { return mt == 1 ? 8 : mt <= 4 ? 3 : 2; }
 
 // A chunk is a run of consecutive tiles of one tensor.  The block looks its pointers up
 // once, then streams the tiles through a ring of S buffers: while tile k is updated in
 // place, tiles k + 1 .. k + S - 1 are already landing; when tile k's copy back has left its
 // buffer, tile k + S is requested into it.
 template <int OPT, int MASK, int MT, typename GT, bool POST, bool DIAG>
-__global__ void __launch_bounds__(step_threads(MT), step_min_blocks(MT))
+__global__ void __launch_bounds__(step_threads(MT), step_min_blocks(OPT, MT, sizeof(GT) == 2))
 desloc_step_kernel(const __grid_constant__ StepArgs a) {
     constexpr int THREADS = step_threads(MT);
-    constexpr int T = tile_elems(MT), VEC = T / THREADS, S = step_stages(OPT, MT, sizeof(GT) == 2);
+    constexpr int T = tile_elems(OPT, MT, sizeof(GT) == 2), VEC = T / THREADS, S = step_stages(MT);
     constexpr int ALIGN_ELEMS = 16 / static_cast<int>(sizeof(GT));   // bulk copies move multiples of 16 bytes
     constexpr bool HAS_V = OPT != OPT_SGDM;
     using L = TileLayout<OPT, MT, GT, T>;
@@ -589,26 +593,22 @@ desloc_step_kernel(const __grid_constant__ StepArgs a) {
     // inner loop without them (three instructions of about forty per coordinate: with eight
     // workers at sustained clocks 0.4-0.7 % of the step).  The fallback paths keep the one form.
     const bool plain = a.gscale == nullptr && a.rho > 3.4028235e38f;   // rho = +inf: clip off
-    // Work items: chunks of all MT replicas; with MT = 1 (a single worker, local steps) parts of a
-    // chunk of one replica, worker by worker.  One item per block as launched (fewer than 2^31); a
-    // smaller grid strides over the rest.
-    const long long nitems = MT == 1 ? a.nchunks * a.parts * a.M : a.nchunks;
+    // Work items: parts of a chunk, of all MT replicas or (MT = 1: a single worker, local steps) of
+    // one replica, worker by worker.  One item per block as launched (fewer than 2^31); a smaller
+    // grid strides over the rest.
+    const long long nitems = a.nchunks * a.parts * (MT == 1 ? a.M : 1);
     for (long long item = blockIdx.x; item < nitems; item += gridDim.x) {
-        long long c = item;
-        int m0 = 0, sub0 = 0;
-        if constexpr (MT == 1) {
-            const unsigned it = static_cast<unsigned>(item), nc = static_cast<unsigned>(a.nchunks);
-            const unsigned q = it / static_cast<unsigned>(a.parts);   // (worker, chunk)
-            sub0 = static_cast<int>(it - q * a.parts) * a.part_elems;
-            m0 = static_cast<int>(q / nc);
-            c = q - m0 * nc;
-        }
+        const unsigned it = static_cast<unsigned>(item), nc = static_cast<unsigned>(a.nchunks);
+        const unsigned q = it / static_cast<unsigned>(a.parts);   // (worker, chunk)
+        const int part0 = static_cast<int>(it - q * a.parts) * a.part_elems;
+        const int m0 = MT == 1 ? static_cast<int>(q / nc) : 0;
+        const long long c = q - m0 * nc;
         // (asked for before the chunk and pointer look-ups, not behind them)
         const float my_scale = tid < MT && a.gscale ? a.gscale[m0 + tid] : 1.f;
         const Chunk ch = a.chunks[c];   // the same 16 bytes for every thread
-        const int count = MT == 1 ? min(ch.count - sub0, a.part_elems) : ch.count;
-        const long long start = ch.start + sub0;
-        if (MT == 1 && count <= 0) continue;   // a short chunk has fewer parts
+        const int count = min(ch.count - part0, a.part_elems);
+        const long long start = ch.start + part0;
+        if (count <= 0) continue;   // a short chunk has fewer parts
         __syncthreads();  // the previous item is done with the shared state; the barriers exist
         char *p = nullptr;
         if (owner) {
@@ -717,9 +717,11 @@ desloc_step_kernel(const __grid_constant__ StepArgs a) {
     }
 }
 
-// Dynamic shared memory a launch of desloc_step_kernel<opt, ., mt, grad type, ., .> needs.
-__host__ __device__ constexpr int step_smem_bytes(int opt, int mt, bool bf16) {
-    return step_stages(opt, mt, bf16) * mt * tile_elems(mt) * ((bf16 ? 2 : 4) + 4 * (opt == OPT_SGDM ? 2 : 3));
+// Dynamic shared memory a launch of desloc_step_kernel<opt, ., mt, grad type, ., .> needs whose
+// blocks take up to part_elems elements: a buffer per tile, at most step_stages(mt) of them.
+__host__ __device__ constexpr int step_smem_bytes(int opt, int mt, bool bf16, int part_elems) {
+    const int t = tile_elems(opt, mt, bf16), tiles = (part_elems + t - 1) / t;
+    return (tiles < step_stages(mt) ? tiles : step_stages(mt)) * mt * t * ((bf16 ? 2 : 4) + 4 * (opt == OPT_SGDM ? 2 : 3));
 }
 
 // Lookup of an instantiation: opt, post-average?, bf16 gradients?, MT in 1..MAX_MT, mask,

@@ -24,3 +24,16 @@ def test_local_steps_at_part_and_wave_edges(opt, gd, M, numel):
     w = di.Workload("parts", opt, M, numel, gd, "normal1" if sum(numel) < 100_000 else "student_t3", lr=1e-2, weight_decay=0.05,
                     clip_rho=1.5, K=(0, 0, 0), adopt_norm_clip=(opt == "adopt"), eps=1e-3, seed=M)
     check(run_both(w, 2, align=4, v_init=0.25))
+
+
+@pytest.mark.parametrize("opt,gd", [("adam", "bf16"), ("adopt", "f32"), ("sgdm", "f32")])
+@pytest.mark.parametrize("M,numel", [
+    (2, (2 * LARGE + 1024 * 7 + 3, 8191, 2047, 2049)),               # two replicas: a chunk in four parts
+    (2, (296 * 512 - 8, 8)), (2, (298 * 512,)),                      # one tile per block, and just beyond a wave
+    (8, (LARGE + 255, 257, 4097, 3)),                                # eight replicas: 256-element tiles with fp32 gradients
+])
+def test_averaging_steps_at_part_and_tile_edges(opt, gd, M, numel):
+    w = di.Workload("parts", opt, M, numel, gd, "normal1" if sum(numel) < 400_000 else "student_t3", lr=1e-2, weight_decay=0.05,
+                    clip_rho=1.5, adopt_norm_clip=(opt == "adopt"), eps=1e-3, seed=M)
+    top = 3 if opt == "sgdm" else 7
+    check(run_both(w, 2, align=4, v_init=0.25, forced_masks=[top, 1]))

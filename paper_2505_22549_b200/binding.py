@@ -255,9 +255,9 @@ def desloc_get_diag_norms(ctx: int, M: int, num_tensors: int, stream: int = 0):
     rc = _lib.desloc_get_diag_norms(ctx, per, tot, stream or None)
     if rc != DESLOC_OK:
         raise DeslocError(rc, "desloc_get_diag_norms", _lib.desloc_last_cuda_error(ctx))
-    per_l = [[[per[(k * M + m) * num_tensors + j] for j in range(num_tensors)] for m in range(M)]
-             for k in range(3)]
-    tot_l = [[tot[k * M + m] for m in range(M)] for k in range(3)]
+    row = lambda r: per[r * num_tensors:(r + 1) * num_tensors]      # a slice is a list, made natively
+    per_l = [[row(k * M + m) for m in range(M)] for k in range(3)]
+    tot_l = [tot[k * M:(k + 1) * M] for k in range(3)]
     return per_l, tot_l
 
 

@@ -2,7 +2,8 @@
 
     python -m paper_2505_22549_b200.build [--force] [--verbose]
 
-Translation units compile in parallel; the result is paper_2505_22549_b200/lib/libdesloc.so.
+Translation units compile in parallel; the results are paper_2505_22549_b200/lib/libdesloc.so and, built with g++
+against torch's headers, the CPython module paper_2505_22549_b200/_native.so that module.py calls the library through.
 """
 from __future__ import annotations
 
@@ -18,6 +19,8 @@ CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "build")
 LIBDIR = os.path.join(HERE, "lib")
 LIB = os.path.join(LIBDIR, "libdesloc.so")
+NATIVE_SRC = os.path.join(CSRC, "desloc_py.cpp")
+NATIVE = os.path.join(HERE, "_native.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 
 NVCC_FLAGS = [
@@ -47,6 +50,31 @@ def _fingerprint(src: str) -> str:
         h.update(open(f, "rb").read())
     h.update(" ".join(NVCC_FLAGS).encode())
     return h.hexdigest()
+
+
+def _build_native(force: bool) -> None:
+    """The CPython module (host code only)."""
+    import sysconfig
+    import torch
+    from torch.utils import cpp_extension as ce
+    libs = os.path.join(os.path.dirname(torch.__file__), "lib")
+    dirs = ce.include_paths() + [sysconfig.get_paths()["include"], os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include")]
+    tmp, stamp = NATIVE + f".tmp{os.getpid()}", os.path.join(OBJ, "_native.stamp")
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}"]
+    cmd += [a for d in dirs for a in ("-isystem", d)] + [NATIVE_SRC, "-L", libs]
+    cmd += ["-ltorch_python", "-ltorch_cpu", "-ltorch", "-lc10_cuda", "-lc10"]
+    h = hashlib.sha256(" ".join(cmd + [torch.__version__, sys.version]).encode())
+    for f in [NATIVE_SRC] + sorted(glob.glob(os.path.join(INCLUDE, "*.h"))):
+        h.update(open(f, "rb").read())
+    if not force and os.path.exists(NATIVE) and os.path.exists(stamp) and open(stamp).read() == h.hexdigest():
+        return
+    r = subprocess.run(cmd + ["-o", tmp], capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"g++ failed on {NATIVE_SRC}:\n{r.stdout}\n{r.stderr}")
+    os.replace(tmp, NATIVE)
+    with open(stamp, "w") as f:
+        f.write(h.hexdigest())
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -79,7 +107,9 @@ def _build(force: bool, verbose: bool, extra_flags) -> str:
         return obj, True
 
     with cf.ThreadPoolExecutor(max_workers=min(8, os.cpu_count() or 2)) as ex:
+        native = ex.submit(_build_native, force)
         results = list(ex.map(compile_one, _sources()))
+        native.result()
     objs = [o for o, _ in results]
     if not any(changed for _, changed in results) and os.path.exists(LIB):
         return LIB

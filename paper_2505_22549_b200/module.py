@@ -1,11 +1,26 @@
 """``DesLoc``: owns nothing but a context handle; holds references to the caller's tensors."""
 from __future__ import annotations
 
-from typing import List, Optional, Sequence
+import ctypes
+from typing import Optional, Sequence
 
 import torch
 
 from . import binding as B
+
+try:
+    from . import _native
+except ImportError as e:
+    raise ImportError(f"the native part of this module is missing ({e}): build it with "
+                      "`python -m paper_2505_22549_b200.build`") from e
+
+_entry = lambda f: ctypes.cast(f, ctypes.c_void_p).value
+_native.bind(*(_entry(getattr(B.raw_lib(), "desloc_" + n))
+               for n in ("step", "step_masked", "step_normclip", "step_diag", "rel_change")))
+
+_GRAD_MISFIT = "gradient tensor of wrong dtype, size or layout"
+_SNAP_MISFIT = "snapshot tensor of wrong dtype, size or layout"
+_HOST_MISFIT = "host gradient tensor of wrong dtype, size, layout or device"
 
 
 class BoundGrads:
@@ -13,6 +28,7 @@ class BoundGrads:
 
     def __init__(self, array, keep):
         self.array, self._keep = array, keep
+        self.address = ctypes.addressof(array)
 
 
 class DesLoc:
@@ -45,52 +61,61 @@ class DesLoc:
         self.cfg = B.make_config(M, numel, opt, grad_dtype, beta1, beta2, eps, weight_decay,
                                  clip_rho, K[0], K[1], K[2], flags)
         flat = lambda a: [t.data_ptr() for lst in a for t in lst]
+        self._index = dev.index if dev.index is not None else torch.cuda.current_device()
         self.ctx: Optional[int] = B.desloc_create(
-            self.cfg, flat(x), flat(u), flat(v) if v is not None else None,
-            dev.index if dev.index is not None else torch.cuda.current_device())
-        self._gkey = None
-        self._garr = None
+            self.cfg, flat(x), flat(u), flat(v) if v is not None else None, self._index)
+        self._tables()
+
+    def _tables(self) -> None:
+        # one buffer of pointers per kind of argument, written anew at every call
+        self._table = _native.Table(self.numel, self.M)
+        self._table2 = _native.Table(self.numel, self.M)
 
     def bind_grads(self, grads: Sequence[Sequence[torch.Tensor]]):
         """Check a set of gradient tensors once and return a handle every step method accepts in
         place of the nested lists: a loop that reuses its gradient buffers then pays no
         per-step marshalling.  The handle keeps the tensors alive."""
-        return BoundGrads(self._grad_array(grads), grads)
+        n = self.M * len(self.numel)
+        array = (ctypes.c_void_p * n).from_buffer_copy((ctypes.c_void_p * n).from_address(self._grad_address(grads)))
+        return BoundGrads(array, grads)
 
-    def _grad_array(self, grads):
-        if isinstance(grads, BoundGrads):
-            return grads.array
-        want = torch.bfloat16 if self.grad_dtype == B.DESLOC_BF16 else torch.float32
-        ptrs: List[int] = []
-        for lst in grads:
-            for t, n in zip(lst, self.numel):
-                if t.dtype != want or t.numel() != n or not t.is_contiguous():
-                    raise ValueError("gradient tensor of wrong dtype, size or layout")
-                ptrs.append(t.data_ptr())
-        if len(ptrs) != self.M * len(self.numel):
-            raise ValueError("need one gradient list per worker")
-        key = tuple(ptrs)
-        if key != self._gkey:
-            self._gkey, self._garr = key, B.ptr_array(ptrs)
-        return self._garr
+    def _grad_address(self, grads) -> int:
+        """Address of the array of gradient pointers, good until the next call of this method."""
+        if type(grads) is BoundGrads:
+            return grads.address
+        return self._fill(self._table, grads, self.grad_dtype, 0, _GRAD_MISFIT)
+
+    def _fill(self, table, nested, kind: int, where: int, misfit: str) -> int:
+        """Checks and marshals nested lists of tensors into the buffer of `table`; its address."""
+        address = table.fill(nested, kind, where, misfit)
+        if address is None:
+            raise ValueError(misfit + " (not a torch.Tensor)")
+        return address
+
+    def _raise(self, status: int, where: str):
+        raise B.DeslocError(status, where, B.desloc_last_cuda_error(self.ctx))
 
     def step(self, t: int, lr: float, grads, clip_bound: float = 0.0) -> int:
         """Step t on torch's current stream; returns the sync mask."""
-        stream = torch.cuda.current_stream(self.device).cuda_stream
-        return B.desloc_step(self.ctx, t, lr, clip_bound, self._grad_array(grads), stream)
+        r = _native.step(self.ctx, t, lr, clip_bound, 0.0, self._grad_address(grads), self._index, 0)
+        if r < 0:
+            self._raise(r, "desloc_step")
+        return r
 
     def step_normclip(self, t: int, lr: float, grads, max_norm: float, clip_bound: float = 0.0) -> int:
         """Step t with norm-based gradient clipping (per worker, over the whole tensor list)."""
-        stream = torch.cuda.current_stream(self.device).cuda_stream
-        return B.desloc_step_normclip(self.ctx, t, lr, clip_bound, max_norm,
-                                      self._grad_array(grads), stream)
+        r = _native.step(self.ctx, t, lr, clip_bound, max_norm, self._grad_address(grads), self._index, 1)
+        if r < 0:
+            self._raise(r, "desloc_step_normclip")
+        return r
 
     def step_diag(self, t: int, lr: float, grads, max_norm: float = 0.0, clip_bound: float = 0.0) -> int:
         """Step t that also accumulates the gradient, parameter and update norms (read them with
         diag_norms()); max_norm > 0 adds norm-based clipping in front."""
-        stream = torch.cuda.current_stream(self.device).cuda_stream
-        return B.desloc_step_diag(self.ctx, t, lr, clip_bound, max_norm, self._grad_array(grads),
-                                  stream)
+        r = _native.step(self.ctx, t, lr, clip_bound, max_norm, self._grad_address(grads), self._index, 2)
+        if r < 0:
+            self._raise(r, "desloc_step_diag")
+        return r
 
     def diag_norms(self):
         """(per_tensor [3][M][num_tensors], total [3][M]) of the latest step_diag; kind 0 =
@@ -105,14 +130,11 @@ class DesLoc:
 
     def rel_change(self, array: int, then: Sequence[Sequence[torch.Tensor]]):
         """Per-worker ||s - then|| / ||then|| against a snapshot (lists like x); synchronises."""
-        ptrs = []
-        for lst in then:
-            for t, n in zip(lst, self.numel):
-                if t.dtype != torch.float32 or t.numel() != n or not t.is_contiguous():
-                    raise ValueError("snapshot tensor of wrong dtype, size or layout")
-                ptrs.append(t.data_ptr())
-        stream = torch.cuda.current_stream(self.device).cuda_stream
-        return B.desloc_rel_change(self.ctx, array, ptrs, self.M, stream)
+        r = _native.rel_change(self.ctx, array, self._fill(self._table2, then, B.DESLOC_F32, 0, _SNAP_MISFIT),
+                               self._index, self.M)
+        if not isinstance(r, list):
+            self._raise(r, "desloc_rel_change")
+        return r
 
     def set_workers(self, x, u, v, first_new: int) -> None:
         """New worker set (lists like the constructor's); workers first_new.. start from the mean
@@ -127,24 +149,20 @@ class DesLoc:
                              flat(v) if v is not None else None, stream)
         self._keep = (x, u, v)
         self.M = M
-        self._gkey = self._garr = None
+        self._tables()
 
     def step_host(self, t: int, lr: float, host_grads, dev_grads, clip_bound: float = 0.0) -> int:
         """Step t with gradients in (pinned) host tensors; dev_grads are device staging tensors."""
-        want = torch.bfloat16 if self.grad_dtype == B.DESLOC_BF16 else torch.float32
-        hp = []
-        for lst in host_grads:
-            for t_, n in zip(lst, self.numel):
-                if t_.dtype != want or t_.numel() != n or not t_.is_contiguous() or t_.is_cuda:
-                    raise ValueError("host gradient tensor of wrong dtype, size, layout or device")
-                hp.append(t_.data_ptr())
+        hp = self._fill(self._table2, host_grads, self.grad_dtype, 1, _HOST_MISFIT)
+        n = self.M * len(self.numel)
+        at = lambda address: (ctypes.c_void_p * n).from_address(address)
         stream = torch.cuda.current_stream(self.device).cuda_stream
-        return B.desloc_step_host(self.ctx, t, lr, clip_bound, hp, self._grad_array(dev_grads),
-                                  stream)
+        return B.desloc_step_host(self.ctx, t, lr, clip_bound, at(hp), at(self._grad_address(dev_grads)), stream)
 
     def step_masked(self, mask: int, lr: float, grads, clip_bound: float = 0.0) -> None:
-        stream = torch.cuda.current_stream(self.device).cuda_stream
-        B.desloc_step_masked(self.ctx, mask, lr, clip_bound, self._grad_array(grads), stream)
+        r = _native.step_masked(self.ctx, mask, lr, clip_bound, self._grad_address(grads), self._index)
+        if r < 0:
+            self._raise(r, "desloc_step_masked")
 
     def counters(self):
         return B.desloc_get_counters(self.ctx)

@@ -349,6 +349,8 @@ desloc_step_generic_kernel(const __grid_constant__ StepArgs a) {
     // exactly one chunk per block (this kernel does not stride: with a chunk loop around the
     // same body the compiler needs spill slots)
     const long long c = blockIdx.x;
+    begin_and_let_next_begin();
+    wait_for_earlier_kernels();
     if (c < a.nchunks) {
         const Chunk ch = a.chunks[c];
         int mis = 0;

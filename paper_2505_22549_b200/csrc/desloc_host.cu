@@ -54,7 +54,9 @@ struct Slot {
     void **host = nullptr;  // pinned
     void **dev = nullptr;
     cudaEvent_t done = nullptr;
-    bool in_flight = false;
+    bool in_flight = false;     // `done` has been recorded behind a kernel that reads the table
+    bool used_since = false;    // ... and other kernels on `stream` have read it since
+    cudaStream_t stream = nullptr;
 };
 
 // desloc_step_host: tensor groups whose copies and kernels are pipelined
@@ -186,6 +188,7 @@ struct desloc_ctx {
     int wait_limit = desloc::DEFAULT_WAIT_LIMIT;
     WorkerRes res;
     int next_slot = 0;
+    bool many_streams = false;   // steps have been called on more than one stream
     int cur_slot = -1;           // slot holding the table equal to last_grads
     std::vector<const void *> last_grads;
     cudaStream_t last_stream = nullptr;
@@ -232,14 +235,19 @@ int stage_grads(desloc_ctx *ctx, const void *const *grads, cudaStream_t stream, 
     Slot &s = ctx->res.slots[ctx->next_slot];
     if (s.in_flight) {
         // Re-use of a slot whose kernel was enqueued kSlots table changes ago: wait for it.
-        cudaError_t e = cudaEventSynchronize(s.done);
+        // (Kernels that read it without an event are in front of the copy below if they are on
+        // this stream; on another one -- the context has changed streams for the first time since --
+        // that stream may be gone by now, so wait for the device.)
+        cudaError_t e = s.used_since && s.stream != stream ? cudaDeviceSynchronize() : cudaEventSynchronize(s.done);
         if (e != cudaSuccess) return cuda_fail(ctx, e);
         s.in_flight = false;
+        s.used_since = false;
     }
     std::memcpy(s.host, grads, bytes);
     cudaError_t e = cudaMemcpyAsync(s.dev, s.host, bytes, cudaMemcpyHostToDevice, stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e);
     std::memcpy(ctx->last_grads.data(), grads, bytes);
+    if (ctx->cur_slot >= 0 && stream != ctx->last_stream) ctx->many_streams = true;
     ctx->cur_slot = ctx->next_slot;
     ctx->next_slot = (ctx->next_slot + 1) % kSlots;
     ctx->last_stream = stream;
@@ -355,8 +363,7 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
             if (ctx->prepared.size() < ctx->prepared.capacity()) ctx->prepared.push_back(plan.fn);
         }
         if (!host_grads) {
-            e = cudaLaunchKernel(plan.fn, dim3(capped(plan)),
-                                 dim3(static_cast<unsigned>(plan.threads)), params, plan.smem, stream);
+            e = desloc::launch_kernel(plan.fn, capped(plan), plan.threads, plan.smem, stream, params, true);
             if (e == cudaSuccess) ctx->launches += 1;
         } else {
             // The device gradient buffers may still be read by earlier work on `stream`.
@@ -395,8 +402,8 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
                 const desloc::LaunchPlan gp = desloc::plan_launch(c, mask, a.nchunks, ctx->res.chunk_elems, diag);
                 a.parts = gp.parts;
                 a.part_elems = gp.part_elems;
-                e = cudaLaunchKernel(gp.fn, dim3(capped(gp)),
-                                     dim3(static_cast<unsigned>(gp.threads)), params, gp.smem, stream);
+                // (no overlap: this kernel also depends on the other stream's copies)
+                e = desloc::launch_kernel(gp.fn, capped(gp), gp.threads, gp.smem, stream, params, false);
                 if (e == cudaSuccess) ctx->launches += 1;
             }
         }
@@ -405,13 +412,20 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
             break;
         }
         if (!capturing) {
+            // An event behind the first kernel that reads a table; a loop on one stream with the same
+            // gradient buffers needs no more (0.5 us of host time a step), see stage_grads().
             Slot &s = ctx->res.slots[ctx->cur_slot];
-            e = cudaEventRecord(s.done, stream);
-            if (e != cudaSuccess) {
-                rc = cuda_fail(ctx, e);
-                break;
+            if (s.in_flight && !ctx->many_streams) {
+                s.used_since = true;
+            } else {
+                e = cudaEventRecord(s.done, stream);
+                if (e != cudaSuccess) {
+                    rc = cuda_fail(ctx, e);
+                    break;
+                }
+                s.in_flight = true;
+                s.stream = stream;
             }
-            s.in_flight = true;
         }
         if (diag) ctx->diag_valid = true;
         ctx->counters[0] += 1;

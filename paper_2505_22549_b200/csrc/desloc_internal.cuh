@@ -214,6 +214,25 @@ inline cudaError_t prepare_launch(const LaunchPlan &p) {
     return cudaFuncSetAttribute(p.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem_limit);
 }
 
+// Launches `fn`.  overlap: the kernel may begin while the one in front of it in the stream still runs
+// (see begin_and_let_next_begin); also under capture, where it becomes an edge of the graph.  Measured
+// on B200: a graph window of 16 dependent steps on 4096 parameters 28.0 us instead of 43.0, a 5 M-parameter
+// step of four workers 82.0 us instead of 85.7, 135 M parameters 2044 us instead of 2050.
+inline cudaError_t launch_kernel(const void *fn, unsigned grid, unsigned threads, size_t smem, cudaStream_t stream,
+                                 void **params, bool overlap) {
+    cudaLaunchConfig_t lc{};
+    lc.gridDim = dim3(grid);
+    lc.blockDim = dim3(threads);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = stream;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = &at;
+    lc.numAttrs = overlap ? 1 : 0;
+    return cudaLaunchKernelExC(&lc, fn, params);
+}
+
 inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, long long nchunks, int64_t chunk_elems,
                               bool diag) {
     LaunchPlan p;

@@ -81,6 +81,15 @@ struct __align__(16) Chunk {
     int64_t start;   // first element within the tensor
 };
 
+// Programmatic dependent launch.  Every kernel here is launched so that it may begin while the kernel in
+// front of it in the stream is still running: each block tells the next kernel at once that it may come
+// (its blocks move in as the last ones of this kernel leave), does what depends on no earlier kernel --
+// barriers, look-ups in tables that only copies write -- and then waits until everything in front
+// of it is complete and visible.  No state, gradient, scale factor or partial sum is touched
+// before that.  The wait is the launch's own dependency, resolved by the hardware, not a poll.
+__device__ __forceinline__ void begin_and_let_next_begin() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_earlier_kernels() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 constexpr int INLINE_PTRS = 32;  // gradient pointers that fit in the kernel parameters
 
 struct StepArgs {
@@ -579,6 +588,7 @@ desloc_step_kernel(const __grid_constant__ StepArgs a) {
     __shared__ __align__(8) uint64_t bar[S];
     ThreadNorms<DIAG, MT, THREADS> wn;
     const int tid = threadIdx.x;
+    begin_and_let_next_begin();
     if (tid < S) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&bar[tid])) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -603,8 +613,6 @@ desloc_step_kernel(const __grid_constant__ StepArgs a) {
         const int part0 = static_cast<int>(it - q * a.parts) * a.part_elems;
         const int m0 = MT == 1 ? static_cast<int>(q / nc) : 0;
         const long long c = q - m0 * nc;
-        // (asked for before the chunk and pointer look-ups, not behind them)
-        const float my_scale = tid < MT && a.gscale ? a.gscale[m0 + tid] : 1.f;
         const Chunk ch = a.chunks[c];   // the same 16 bytes for every thread
         const int count = min(ch.count - part0, a.part_elems);
         const long long start = ch.start + part0;
@@ -621,7 +629,6 @@ desloc_step_kernel(const __grid_constant__ StepArgs a) {
                     start * static_cast<long long>(sizeof(GT));
             sp[arr][m] = p;
         }
-        if (tid < MT) sscale[tid] = my_scale;
         wn.clear();
         // bulk copies need 16-byte aligned addresses; a tile of the chunk also a byte count that
         // is a multiple of 16 (only the chunk's last tile can miss that: it is then updated
@@ -646,9 +653,13 @@ desloc_step_kernel(const __grid_constant__ StepArgs a) {
                                 "r"(static_cast<uint32_t>(MT * cnt * (static_cast<int>(sizeof(GT)) + 4 * L::NS)))
                              : "memory");
         };
+        wait_for_earlier_kernels();
 #pragma unroll
         for (int k = 0; k < S; ++k)
             if (k < staged) request(k);
+        // (behind the requests: its latency hides in theirs; a block barrier follows before it is used)
+        if (tid < MT) sscale[tid] = a.gscale ? a.gscale[m0 + tid] : 1.f;
+        if (staged == 0) __syncthreads();
 #pragma unroll 1
         for (int k = 0; k < staged; ++k) {
             const int st = k % S;

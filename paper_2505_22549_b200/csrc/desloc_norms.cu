@@ -85,6 +85,8 @@ template <typename GT>
 __global__ void __launch_bounds__(BLOCK_THREADS, 3)
 sumsq_kernel(const Chunk *chunks, long long nchunks, const void *const *g, int nt, int M,
              float *partial) {
+    begin_and_let_next_begin();
+    wait_for_earlier_kernels();
     __shared__ float warp_sums[BLOCK_THREADS / 32];
     const long long ngroups = (nchunks + SUMSQ_GROUP - 1) / SUMSQ_GROUP;
     const long long nitems = ngroups * M;
@@ -159,6 +161,8 @@ sumsq_kernel(const Chunk *chunks, long long nchunks, const void *const *g, int n
 __global__ void __launch_bounds__(BLOCK_THREADS, 3)
 sumsq_bulk_kernel(const Chunk *chunks, long long nchunks, const void *const *g, int nt, int M,
                   float *partial, int *err, int wait_limit) {
+    begin_and_let_next_begin();
+    wait_for_earlier_kernels();
     using GT = bf16_t;
     constexpr int CHUNK_BYTES = REDUCE_CHUNK_ELEMS * static_cast<int>(sizeof(GT));
     constexpr int LPC = 2, CB = 8 / LPC;   // as in sumsq_kernel
@@ -240,6 +244,8 @@ sumsq_bulk_kernel(const Chunk *chunks, long long nchunks, const void *const *g, 
 __global__ void __launch_bounds__(BLOCK_THREADS, 6)
 relchange_kernel(const Chunk *chunks, long long nchunks, const float *const *now,
                  const float *const *then, int nt, int M, float *partial) {
+    begin_and_let_next_begin();
+    wait_for_earlier_kernels();
     __shared__ float warp_sums[BLOCK_THREADS / 32];
     const long long nitems = nchunks * M;
     const int tid = threadIdx.x;
@@ -307,6 +313,8 @@ __device__ __forceinline__ double row_sum_f64(const T *row, long long n, double 
 __global__ void __launch_bounds__(BLOCK_THREADS)
 norm_finalize_kernel(const float *partial, long long nchunks, float max_norm, float *norms,
                      float *scales) {
+    begin_and_let_next_begin();
+    wait_for_earlier_kernels();
     __shared__ double sh[BLOCK_THREADS];
     const int m = blockIdx.x;
     const double ss = row_sum_f64(partial + static_cast<long long>(m) * nchunks, nchunks, sh);
@@ -321,6 +329,8 @@ norm_finalize_kernel(const float *partial, long long nchunks, float max_norm, fl
 
 __global__ void __launch_bounds__(BLOCK_THREADS)
 relchange_finalize_kernel(const float *partial, long long nchunks, int M, float *out) {
+    begin_and_let_next_begin();
+    wait_for_earlier_kernels();
     __shared__ double sh[BLOCK_THREADS];
     const int m = blockIdx.x;
     const double num = row_sum_f64(partial + static_cast<long long>(m) * nchunks, nchunks, sh);
@@ -333,6 +343,8 @@ relchange_finalize_kernel(const float *partial, long long nchunks, int M, float 
 __global__ void __launch_bounds__(BLOCK_THREADS, 4)
 mean_fill_kernel(const Chunk *chunks, long long nchunks, const float *const *src, int m_src,
                  float *const *dst, int m_dst, int nt) {
+    begin_and_let_next_begin();
+    wait_for_earlier_kernels();
     for (long long c = blockIdx.x; c < nchunks; c += gridDim.x) {
         const Chunk ch = chunks[c];
         for (int e = threadIdx.x; e < ch.count; e += BLOCK_THREADS) {
@@ -352,6 +364,8 @@ mean_fill_kernel(const Chunk *chunks, long long nchunks, const float *const *src
 __global__ void __launch_bounds__(BLOCK_THREADS)
 diag_tensor_kernel(const float *partial, long long stride, const long long *tstart, int nt, int M,
                    double *sums, float *norms) {
+    begin_and_let_next_begin();
+    wait_for_earlier_kernels();
     __shared__ double sh[BLOCK_THREADS];
     const int k = blockIdx.x, m = blockIdx.y, kind = blockIdx.z;
     const long long row = static_cast<long long>(kind) * M + m;
@@ -365,10 +379,28 @@ diag_tensor_kernel(const float *partial, long long stride, const long long *tsta
 // One block per (kind, worker): the whole-model norm from the per-tensor sums of squares.
 __global__ void __launch_bounds__(BLOCK_THREADS)
 diag_total_kernel(const double *sums, int nt, float *totals) {
+    begin_and_let_next_begin();
+    wait_for_earlier_kernels();
     __shared__ double sh[BLOCK_THREADS];
     const long long row = blockIdx.x;
     const double ss = row_sum_f64(sums + row * nt, nt, sh);
     if (threadIdx.x == 0) totals[row] = static_cast<float>(sqrt(ss));
+}
+
+// All launches of this file may begin while the kernel in front of them still runs.
+template <typename... P, typename... A>
+cudaError_t launch(void (*kernel)(P...), dim3 grid, size_t smem, cudaStream_t stream, A... args) {
+    cudaLaunchConfig_t lc{};
+    lc.gridDim = grid;
+    lc.blockDim = dim3(BLOCK_THREADS);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = stream;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = &at;
+    lc.numAttrs = 1;
+    return cudaLaunchKernelEx(&lc, kernel, static_cast<P>(args)...);
 }
 
 unsigned grid_for(long long nitems) {
@@ -382,47 +414,38 @@ cudaError_t launch_grad_norms(const Chunk *chunks, long long nchunks, const void
                               float *scales, int *err, int wait_limit, cudaStream_t stream) {
     const long long ngroups = (nchunks + SUMSQ_GROUP - 1) / SUMSQ_GROUP;
     const unsigned grid = grid_for(ngroups * M);
+    cudaError_t e;
     if (bf16) {
         constexpr int smem = SUMSQ_GROUP * REDUCE_CHUNK_ELEMS * 2;
-        cudaError_t e0 = cudaFuncSetAttribute(sumsq_bulk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e0 != cudaSuccess) return e0;
-        sumsq_bulk_kernel<<<grid, BLOCK_THREADS, smem, stream>>>(chunks, nchunks, g, nt, M, partial, err,
-                                                                 wait_limit);
+        e = cudaFuncSetAttribute(sumsq_bulk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        e = launch(sumsq_bulk_kernel, grid, smem, stream, chunks, nchunks, g, nt, M, partial, err, wait_limit);
     } else
-        sumsq_kernel<float><<<grid, BLOCK_THREADS, 0, stream>>>(chunks, nchunks, g, nt, M, partial);
-    cudaError_t e = cudaGetLastError();
+        e = launch(sumsq_kernel<float>, grid, 0, stream, chunks, nchunks, g, nt, M, partial);
     if (e != cudaSuccess) return e;
-    norm_finalize_kernel<<<M, BLOCK_THREADS, 0, stream>>>(partial, ngroups, max_norm, norms, scales);
-    return cudaGetLastError();
+    return launch(norm_finalize_kernel, M, 0, stream, partial, ngroups, max_norm, norms, scales);
 }
 
 cudaError_t launch_rel_change(const Chunk *chunks, long long nchunks, const float *const *now,
                               const float *const *then, int nt, int M, float *partial, float *out,
                               cudaStream_t stream) {
-    relchange_kernel<<<grid_for(nchunks * M), BLOCK_THREADS, 0, stream>>>(chunks, nchunks, now, then,
-                                                                          nt, M, partial);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch(relchange_kernel, grid_for(nchunks * M), 0, stream, chunks, nchunks, now, then, nt, M, partial);
     if (e != cudaSuccess) return e;
-    relchange_finalize_kernel<<<M, BLOCK_THREADS, 0, stream>>>(partial, nchunks, M, out);
-    return cudaGetLastError();
+    return launch(relchange_finalize_kernel, M, 0, stream, partial, nchunks, M, out);
 }
 
 cudaError_t launch_diag_norms(const float *partial, long long stride, const long long *tstart,
                               int nt, int M, double *sums, float *per_tensor, float *totals,
                               cudaStream_t stream) {
-    diag_tensor_kernel<<<dim3(nt, M, DIAG_KINDS), BLOCK_THREADS, 0, stream>>>(partial, stride, tstart,
-                                                                            nt, M, sums, per_tensor);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch(diag_tensor_kernel, dim3(nt, M, DIAG_KINDS), 0, stream, partial, stride, tstart, nt, M, sums,
+                           per_tensor);
     if (e != cudaSuccess) return e;
-    diag_total_kernel<<<DIAG_KINDS * M, BLOCK_THREADS, 0, stream>>>(sums, nt, totals);
-    return cudaGetLastError();
+    return launch(diag_total_kernel, DIAG_KINDS * M, 0, stream, sums, nt, totals);
 }
 
 cudaError_t launch_mean_fill(const Chunk *chunks, long long nchunks, const float *const *src,
                              int m_src, float *const *dst, int m_dst, int nt, cudaStream_t stream) {
-    mean_fill_kernel<<<grid_for(nchunks), BLOCK_THREADS, 0, stream>>>(chunks, nchunks, src, m_src,
-                                                                      dst, m_dst, nt);
-    return cudaGetLastError();
+    return launch(mean_fill_kernel, grid_for(nchunks), 0, stream, chunks, nchunks, src, m_src, dst, m_dst, nt);
 }
 
 }  // namespace desloc

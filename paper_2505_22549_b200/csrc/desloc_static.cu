@@ -183,8 +183,7 @@ extern "C" DESLOC_API int desloc_step_static(const desloc_config *cfg, float *co
         void *params[] = {&a};
         e = desloc::prepare_launch(plan);
         if (e == cudaSuccess)
-            e = cudaLaunchKernel(plan.fn, dim3(static_cast<unsigned>(plan.grid)),
-                                 dim3(static_cast<unsigned>(plan.threads)), params, plan.smem, st);
+            e = desloc::launch_kernel(plan.fn, static_cast<unsigned>(plan.grid), plan.threads, plan.smem, st, params, true);
         if (e != cudaSuccess) { rc = DESLOC_E_CUDA; break; }
     } while (false);
     if (rc == DESLOC_E_CUDA) (void)cudaGetLastError();

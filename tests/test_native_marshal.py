@@ -1,0 +1,43 @@
+"""The native marshalling of nested tensor lists: addresses in worker-major order, and the refusals of module.py."""
+import ctypes
+
+import pytest
+import torch
+
+
+@pytest.fixture(scope="module")
+def native():
+    import paper_2505_22549_b200.module as m
+    return m._native
+
+
+@pytest.mark.parametrize("kind,dtype", [(0, torch.float32), (1, torch.bfloat16)])
+def test_addresses_are_those_of_the_tensors(native, kind, dtype):
+    shapes, M = [(4,), (2, 3), (1,)], 3
+    lists = [[torch.zeros(s, dtype=dtype) for s in shapes] for _ in range(M)]
+    lists[1][1] = torch.nn.Parameter(lists[1][1])
+    table = native.Table([4, 6, 1], M)
+    for nested in (lists, tuple(tuple(r) for r in lists)):
+        at = table.fill(nested, kind, 1, "misfit")
+        got = list((ctypes.c_void_p * 9).from_address(at))
+        assert got == [t.data_ptr() for row in lists for t in row]
+
+
+@pytest.mark.parametrize("spoil", ["dtype", "size", "layout", "workers", "short"])
+def test_misfits_are_refused(native, spoil):
+    good = lambda: [[torch.zeros(4), torch.zeros(6)] for _ in range(2)]
+    table, lists = native.Table([4, 6], 2), good()
+    if spoil == "dtype":
+        lists[1][0] = torch.zeros(4, dtype=torch.bfloat16)
+    elif spoil == "size":
+        lists[0][1] = torch.zeros(5)
+    elif spoil == "layout":
+        lists[0][1] = torch.zeros(12)[::2]
+    elif spoil == "workers":
+        lists = lists[:1]
+    else:
+        lists[1] = lists[1][:1]
+    with pytest.raises(ValueError):
+        table.fill(lists, 0, 0, "misfit")
+    assert table.fill(good(), 0, 0, "misfit")
+    assert table.fill([[1, 2], [3, 4]], 0, 0, "misfit") is None      # not tensors: the caller says so

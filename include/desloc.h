@@ -217,8 +217,8 @@ DESLOC_API int desloc_step_diag(desloc_ctx *ctx, int64_t t, float lr_t, float cl
  *   total_out      : host, [3][M] floats, the norm over the whole tensor list, or NULL.
  * Per-chunk partials are fp32; they are added per tensor, and the tensors per worker, in fp64
  * in a fixed order (no atomics: the same buffers and inputs give the same bits; where the chunks
- * of a tensor begin follows the alignment of worker 0's x, see desloc_plan_chunks_at()).  Two small launches on `stream`, then the
- * copies; the call waits for `stream`.  DESLOC_E_INVALID if no diagnostics step has run since
+ * of a tensor begin follows the alignment of worker 0's x, see desloc_plan_chunks_at()).  One small launch on `stream`; the
+ * call waits for `stream`.  DESLOC_E_INVALID if no diagnostics step has run since
  * the context was created or its workers were changed.
  */
 DESLOC_API int desloc_get_diag_norms(desloc_ctx *ctx, float *per_tensor_out, float *total_out,

@@ -51,7 +51,7 @@ constexpr int kSlots = 8;  // staging slots for per-step gradient pointer tables
 constexpr int kHostGroups = 8;  // pipeline depth of desloc_step_host
 
 struct Slot {
-    void **host = nullptr;  // pinned
+    void **host = nullptr;
     void **dev = nullptr;
     cudaEvent_t done = nullptr;
     bool in_flight = false;     // `done` has been recorded behind a kernel that reads the table
@@ -75,22 +75,26 @@ struct WorkerRes {
     std::vector<HostGroup> groups;
     void **d_tables = nullptr;  // [3][nptr] x, u, v
     Slot slots[kSlots];
-    float *d_partial = nullptr;  // reductions: partial sums [2][M][nrchunks]
-    float *d_norms = nullptr;    // [3][M]: gradient norms, clip factors, relative change
+    void **h_slots = nullptr;   // the slots' tables, pinned, and
+    void **d_slots = nullptr;   // on the device
+    float *d_partial = nullptr;  // reductions: partial sums [2][M][reduce_row(nrchunks)]
+    float *d_norms = nullptr;    // [2][M]: gradient norms, clip factors
     void **h_snap = nullptr;     // pinned pointer table for desloc_rel_change
     void **d_snap = nullptr;
     float *d_diag = nullptr;     // diagnostics step: [3][M][nchunks] per-chunk sums of squares
-    double *d_diag_sums = nullptr;  // [3][M][num_tensors]
-    float *d_diag_out = nullptr;    // [3][M][num_tensors] per-tensor norms, then [3][M] totals
+    // Results the host waits for go to its memory straight from the kernels, without a copy:
+    // [3][M][num_tensors] per-tensor norms, [3][M] totals, [M] relative changes.
+    float *h_out = nullptr;      // mapped pinned memory, and
+    float *d_out = nullptr;      // the same as the kernels address it
 };
 
 void free_worker_res(WorkerRes &r) {
     for (Slot &s : r.slots) {
         if (s.done) cudaEventDestroy(s.done);
-        if (s.host) cudaFreeHost(s.host);
-        if (s.dev) cudaFree(s.dev);
         s = Slot();
     }
+    if (r.h_slots) cudaFreeHost(r.h_slots);
+    if (r.d_slots) cudaFree(r.d_slots);
     if (r.d_chunks) cudaFree(r.d_chunks);
     if (r.d_tstart) cudaFree(r.d_tstart);
     if (r.d_tables) cudaFree(r.d_tables);
@@ -99,8 +103,7 @@ void free_worker_res(WorkerRes &r) {
     if (r.h_snap) cudaFreeHost(r.h_snap);
     if (r.d_snap) cudaFree(r.d_snap);
     if (r.d_diag) cudaFree(r.d_diag);
-    if (r.d_diag_sums) cudaFree(r.d_diag_sums);
-    if (r.d_diag_out) cudaFree(r.d_diag_out);
+    if (r.h_out) cudaFreeHost(r.h_out);
     r = WorkerRes();
 }
 
@@ -154,21 +157,26 @@ cudaError_t make_worker_res(WorkerRes &r, int M, const int64_t *numel, int num_t
     cudaError_t e = cudaMalloc(&r.d_tables, tables.size() * sizeof(void *));
     if (e == cudaSuccess)
         e = cudaMemcpy(r.d_tables, tables.data(), tables.size() * sizeof(void *), cudaMemcpyHostToDevice);
-    const size_t npart = static_cast<size_t>(2) * M * static_cast<size_t>(nrchunks);
+    const size_t npart = static_cast<size_t>(2) * M * static_cast<size_t>(desloc::reduce_row(nrchunks));
     if (e == cudaSuccess) e = cudaMalloc(&r.d_partial, npart * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&r.d_norms, static_cast<size_t>(3) * M * sizeof(float));
-    if (e == cudaSuccess) e = cudaMemset(r.d_norms, 0, static_cast<size_t>(3) * M * sizeof(float));
+    if (e == cudaSuccess) e = cudaMalloc(&r.d_norms, static_cast<size_t>(2) * M * sizeof(float));
+    if (e == cudaSuccess) e = cudaMemset(r.d_norms, 0, static_cast<size_t>(2) * M * sizeof(float));
     if (e == cudaSuccess) e = cudaMallocHost(&r.h_snap, static_cast<size_t>(nptr) * sizeof(void *));
     if (e == cudaSuccess) e = cudaMalloc(&r.d_snap, static_cast<size_t>(nptr) * sizeof(void *));
     const size_t ndiag = static_cast<size_t>(desloc::DIAG_KINDS) * M;
     if (e == cudaSuccess) e = cudaMalloc(&r.d_diag, ndiag * static_cast<size_t>(nchunks) * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&r.d_diag_sums, ndiag * num_tensors * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&r.d_diag_out, ndiag * (num_tensors + 1) * sizeof(float));
+    if (e == cudaSuccess)
+        e = cudaHostAlloc(reinterpret_cast<void **>(&r.h_out), (ndiag * (num_tensors + 1) + M) * sizeof(float),
+                          cudaHostAllocMapped);
+    if (e == cudaSuccess) e = cudaHostGetDevicePointer(reinterpret_cast<void **>(&r.d_out), r.h_out, 0);
+    const size_t room = static_cast<size_t>(nptr + 15) & ~size_t{15};   // tables on 128-byte boundaries
+    if (e == cudaSuccess) e = cudaMallocHost(&r.h_slots, kSlots * room * sizeof(void *));
+    if (e == cudaSuccess) e = cudaMalloc(&r.d_slots, kSlots * room * sizeof(void *));
     for (int i = 0; i < kSlots && e == cudaSuccess; ++i) {
         Slot &s = r.slots[i];
-        e = cudaMallocHost(&s.host, static_cast<size_t>(nptr) * sizeof(void *));
-        if (e == cudaSuccess) e = cudaMalloc(&s.dev, static_cast<size_t>(nptr) * sizeof(void *));
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s.done, cudaEventDisableTiming);
+        s.host = r.h_slots + i * room;
+        s.dev = r.d_slots + i * room;
+        e = cudaEventCreateWithFlags(&s.done, cudaEventDisableTiming);
     }
     return e;
 }
@@ -597,18 +605,15 @@ int desloc_get_diag_norms(desloc_ctx *ctx, float *per_tensor_out, float *total_o
     if (e == cudaSuccess && dev_before != ctx->device) e = cudaSetDevice(ctx->device);
     if (e != cudaSuccess) return cuda_fail(ctx, e);
     const size_t rows = static_cast<size_t>(desloc::DIAG_KINDS) * c.M;
-    float *d_per = ctx->res.d_diag_out, *d_tot = ctx->res.d_diag_out + rows * c.num_tensors;
+    const size_t per = rows * c.num_tensors;
     e = desloc::launch_diag_norms(ctx->res.d_diag, ctx->res.nchunks, ctx->res.d_tstart, c.num_tensors, c.M,
-                                  ctx->res.d_diag_sums, d_per, d_tot, st);
-    if (e == cudaSuccess) {
-        ctx->launches += 2;
-        if (per_tensor_out)
-            e = cudaMemcpyAsync(per_tensor_out, d_per, rows * c.num_tensors * sizeof(float),
-                                cudaMemcpyDeviceToHost, st);
-    }
-    if (e == cudaSuccess && total_out)
-        e = cudaMemcpyAsync(total_out, d_tot, rows * sizeof(float), cudaMemcpyDeviceToHost, st);
+                                  ctx->res.d_out, ctx->res.d_out + per, st);
+    if (e == cudaSuccess) ctx->launches += 1;
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e == cudaSuccess) {
+        if (per_tensor_out) std::memcpy(per_tensor_out, ctx->res.h_out, per * sizeof(float));
+        if (total_out) std::memcpy(total_out, ctx->res.h_out + per, rows * sizeof(float));
+    }
     if (dev_before != ctx->device) cudaSetDevice(dev_before);
     return e == cudaSuccess ? DESLOC_OK : cuda_fail(ctx, e);
 }
@@ -682,19 +687,20 @@ int desloc_rel_change(desloc_ctx *ctx, int32_t array, const float *const *then, 
     // The call ends with a stream synchronisation, so the pinned table is free again on return.
     std::memcpy(ctx->res.h_snap, then, tbytes);
     e = cudaMemcpyAsync(ctx->res.d_snap, ctx->res.h_snap, tbytes, cudaMemcpyHostToDevice, st);
-    float *d_out = ctx->res.d_norms + 2 * ctx->cfg.M;
+    const size_t at = static_cast<size_t>(desloc::DIAG_KINDS) * ctx->cfg.M * (ctx->cfg.num_tensors + 1);
     if (e == cudaSuccess)
         e = desloc::launch_rel_change(
             ctx->d_rchunks, ctx->nrchunks,
             reinterpret_cast<const float *const *>(ctx->res.d_tables + array * ctx->nptr),
             reinterpret_cast<const float *const *>(ctx->res.d_snap), ctx->cfg.num_tensors, ctx->cfg.M,
-            ctx->res.d_partial, d_out, st);
-    if (e == cudaSuccess) {
-        ctx->launches += 2;
-        e = cudaMemcpyAsync(out, d_out, static_cast<size_t>(ctx->cfg.M) * sizeof(float),
-                            cudaMemcpyDeviceToHost, st);
-    }
+            ctx->res.d_partial, ctx->res.d_out + at, ctx->d_err, ctx->wait_limit, st);
+    if (e == cudaSuccess) ctx->launches += 2;
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e == cudaSuccess && *static_cast<volatile int *>(ctx->h_err) != 0) {
+        if (dev_before != ctx->device) cudaSetDevice(dev_before);
+        return DESLOC_E_DEVICE_WAIT;
+    }
+    if (e == cudaSuccess) std::memcpy(out, ctx->res.h_out + at, static_cast<size_t>(ctx->cfg.M) * sizeof(float));
     if (dev_before != ctx->device) cudaSetDevice(dev_before);
     return e == cudaSuccess ? DESLOC_OK : cuda_fail(ctx, e);
 }

@@ -3,321 +3,206 @@
 // ||s_now - s_then||_2 / ||s_then||_2 (Section 5.1, "Metrics"), and the finalisation of the
 // per-tensor gradient / parameter / update norms a diagnostics step accumulated.
 //
-// Both are two-stage and deterministic: stage 1 writes one fp32 partial per (worker, chunk)
-// -- per-thread sums of up to 16 squares, a shuffle tree, then the eight warp sums in order;
-// stage 2 adds the partials of a worker in fp64 in a fixed pattern.  No atomics.
+// All are two-stage and deterministic: stage 1 writes one fp32 partial per work item -- per-thread
+// sums of up to 128 squares, a shuffle tree, then the warp sums in order; stage 2 adds the
+// partials of a row in fp64 in a fixed pattern.  No atomics.
 #include "desloc_norms.cuh"
+
+#include <type_traits>
 
 namespace desloc {
 
 namespace {
 
-__device__ __forceinline__ float block_sum(float v, float *warp_sums) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    __syncthreads();  // warp_sums may still be read from the previous use
-    if (lane == 0) warp_sums[warp] = v;
-    __syncthreads();
-    float t = 0.f;
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int w = 0; w < BLOCK_THREADS / 32; ++w) t += warp_sums[w];
-    }
-    return t;  // valid in thread 0
+// ---- stage 1: sums of squares over 32 KB of one worker's array(s) ------------------------------
+// Bound: HBM reads.  A block requests all it will read -- 32 KB, as bulk copies into shared memory --
+// at once, sums it and leaves; six blocks per SM keep 192 KB in flight.  (Before: 64 KB per block and
+// three blocks for bf16 gradients, register loads for fp32 gradients and for the rate of change.)
+// Measured on 135 M parameters x 4 workers: rate of change (4.3 GB) 620 us instead of 740, the whole call;
+// 20 M x 8 workers 200 us instead of 245; the norm-clipped step 2210 us instead of 2259 with bf16 gradients,
+// 2494 instead of 2533 with tightly packed fp32 gradients.
+constexpr int RED_THREADS = 128;
+constexpr int RED_BYTES = 32 * 1024;
+
+// MODE 0, 1: g of fp32, bf16 -- one sum of g^2.  MODE 2: a state and its snapshot -- sums of
+// (now - then)^2 and of then^2.
+constexpr int RED_F32 = 0, RED_BF16 = 1, RED_CHANGE = 2;
+__host__ __device__ constexpr int red_chunks(int mode) {   // reduction chunks (4096 elements) per work item
+    return RED_BYTES / (REDUCE_CHUNK_ELEMS * (mode == RED_BF16 ? 2 : mode == RED_F32 ? 4 : 8));
 }
 
-// partial[m * ngroups + q] = sum of g^m squared over chunk group q (SUMSQ_GROUP consecutive
-// chunks).  Work item = (worker, group): a block streams up to 64 KB of one worker's gradient
-// with eight independent loads per thread in flight, and reduces once.
-constexpr int SUMSQ_GROUP = 8;
-
-template <typename GT>
-__device__ __forceinline__ float chunk_sumsq(const Chunk &ch, const void *const *g, int nt, int m,
-                                             float acc) {
-    const int tid = threadIdx.x;
-    const char *base = reinterpret_cast<const char *>(g[static_cast<long long>(m) * nt + ch.tensor]) +
-                       ch.start * static_cast<long long>(sizeof(GT));
-    const bool aligned = (reinterpret_cast<uintptr_t>(base) & (sizeof(GT) == 2 ? 7u : 15u)) == 0;
-    if (aligned) {
-        const int n4 = ch.count >> 2;
-        FV<4> v[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int p = tid + j * BLOCK_THREADS;
-            if (p < n4) v[j] = ld_grad<4, GT>(base, static_cast<long long>(p) * 4);
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int p = tid + j * BLOCK_THREADS;
-            if (p < n4) {
-#pragma unroll
-                for (int k = 0; k < 4; ++k) acc = fmaf(v[j].a[k], v[j].a[k], acc);
-            }
-        }
-        const int rem = ch.count & 3;
-        if (tid < rem) {
-            const float t = ld_grad<1, GT>(base, (n4 << 2) + tid).a[0];
-            acc = fmaf(t, t, acc);
-        }
-    } else {
-        for (int e = tid; e < ch.count; e += BLOCK_THREADS) {
-            const float t = ld_grad<1, GT>(base, e).a[0];
-            acc = fmaf(t, t, acc);
-        }
-    }
-    return acc;
-}
-
-// Eight bf16 values in one 128-bit load.
-__device__ __forceinline__ float sumsq8_bf16(const uint4 &t, float acc) {
-    const unsigned w[4] = {t.x, t.y, t.z, t.w};
+template <int MODE>
+__device__ __forceinline__ void add_squares(const uint4 &p, const uint4 &q, float (&acc)[2]) {
+    const unsigned w[4] = {p.x, p.y, p.z, p.w}, z[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const float lo = __uint_as_float(w[k] << 16), hi = __uint_as_float(w[k] & 0xffff0000u);
-        acc = fmaf(lo, lo, acc);
-        acc = fmaf(hi, hi, acc);
-    }
-    return acc;
-}
-
-template <typename GT>
-__global__ void __launch_bounds__(BLOCK_THREADS, 3)
-sumsq_kernel(const Chunk *chunks, long long nchunks, const void *const *g, int nt, int M,
-             float *partial) {
-    begin_and_let_next_begin();
-    wait_for_earlier_kernels();
-    __shared__ float warp_sums[BLOCK_THREADS / 32];
-    const long long ngroups = (nchunks + SUMSQ_GROUP - 1) / SUMSQ_GROUP;
-    const long long nitems = ngroups * M;
-    const int tid = threadIdx.x;
-    for (long long item = blockIdx.x; item < nitems; item += gridDim.x) {
-        const long long q = item % ngroups;
-        const int m = static_cast<int>(item / ngroups);
-        const long long c0 = q * SUMSQ_GROUP;
-        float acc0 = 0.f, acc1 = 0.f;
-        {
-            // All chunk descriptors and gradient pointers of the group first (one dependent-load
-            // chain for the whole item), then the data: full, 16-byte aligned chunks take 128-bit
-            // loads, eight of them in flight per thread (four bf16 chunks or two fp32 chunks).
-            constexpr int LPC = sizeof(GT) == 2 ? 2 : 4;  // 128-bit loads per thread and chunk
-            constexpr int CB = 8 / LPC;                   // chunks per batch
-            const uint4 *wide[SUMSQ_GROUP];
-#pragma unroll
-            for (int j = 0; j < SUMSQ_GROUP; ++j) {
-                wide[j] = nullptr;
-                if (c0 + j < nchunks) {
-                    const Chunk ch = chunks[c0 + j];
-                    const char *base =
-                        reinterpret_cast<const char *>(g[static_cast<long long>(m) * nt + ch.tensor]) +
-                        ch.start * static_cast<long long>(sizeof(GT));
-                    if (ch.count == REDUCE_CHUNK_ELEMS && (reinterpret_cast<uintptr_t>(base) & 15u) == 0)
-                        wide[j] = reinterpret_cast<const uint4 *>(base);
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < SUMSQ_GROUP; k += CB) {
-                uint4 r[CB][LPC];
-#pragma unroll
-                for (int j = 0; j < CB; ++j) {
-                    if (wide[k + j]) {
-#pragma unroll
-                        for (int l = 0; l < LPC; ++l)
-                            r[j][l] = *(wide[k + j] + tid + l * BLOCK_THREADS);
-                    }
-                }
-#pragma unroll
-                for (int j = 0; j < CB; ++j) {
-                    if (wide[k + j]) {
-#pragma unroll
-                        for (int l = 0; l < LPC; ++l) {
-                            float &acc = (l & 1) ? acc1 : acc0;
-                            if constexpr (sizeof(GT) == 2) {
-                                acc = sumsq8_bf16(r[j][l], acc);
-                            } else {
-                                const float f[4] = {__uint_as_float(r[j][l].x), __uint_as_float(r[j][l].y),
-                                                    __uint_as_float(r[j][l].z), __uint_as_float(r[j][l].w)};
-#pragma unroll
-                                for (int q4 = 0; q4 < 4; ++q4) acc = fmaf(f[q4], f[q4], acc);
-                            }
-                        }
-                    } else if (c0 + k + j < nchunks) {
-                        acc0 = chunk_sumsq<GT>(chunks[c0 + k + j], g, nt, m, acc0);
-                    }
-                }
-            }
+        if constexpr (MODE == RED_BF16) {
+            const float lo = __uint_as_float(w[k] << 16), hi = __uint_as_float(w[k] & 0xffff0000u);
+            acc[0] = fmaf(lo, lo, acc[0]);
+            acc[1] = fmaf(hi, hi, acc[1]);
+        } else if constexpr (MODE == RED_F32) {
+            const float f = __uint_as_float(w[k]);
+            acc[k & 1] = fmaf(f, f, acc[k & 1]);
+        } else {
+            const float b = __uint_as_float(z[k]), d = __uint_as_float(w[k]) - b;
+            acc[0] = fmaf(d, d, acc[0]);
+            acc[1] = fmaf(b, b, acc[1]);
         }
-        const float total = block_sum(acc0 + acc1, warp_sums);
-        if (tid == 0) partial[static_cast<long long>(m) * ngroups + q] = total;
     }
 }
 
-// The same reduction for bf16 gradients with the group's full, 16-byte aligned chunks brought
-// into shared memory by bulk asynchronous copies (8 KB each, all requested at once, three blocks
-// per SM: up to 192 KB in flight per SM) and summed from there in the order sumsq_kernel uses,
-// so that both kernels give the same bits.  Chunks that cannot be staged are read directly.
-// On the 1.7 G-parameter workload (13.7 GB of gradients) the norm-clipped step takes 28.25 ms
-// with this pass against 28.45 ms with sumsq_kernel (2.0 ms against 2.2 ms for the pass).
-__global__ void __launch_bounds__(BLOCK_THREADS, 3)
-sumsq_bulk_kernel(const Chunk *chunks, long long nchunks, const void *const *g, int nt, int M,
-                  float *partial, int *err, int wait_limit) {
-    begin_and_let_next_begin();
-    wait_for_earlier_kernels();
-    using GT = bf16_t;
+// partial[m * stride + q]: item q of worker m (MODE 2: the squares of `then` at (M + m) * stride + q).
+// One work item per block: red_chunks(MODE) consecutive reduction chunks of one worker.
+template <int MODE>
+__global__ void __launch_bounds__(RED_THREADS, 6)
+sumsq_kernel(const Chunk *chunks, long long nchunks, const void *const *now, const void *const *then, int nt, int M,
+             float *partial, long long stride, int *err, int wait_limit) {
+    using GT = std::conditional_t<MODE == RED_BF16, bf16_t, float>;
+    constexpr int NC = red_chunks(MODE), NA = MODE == RED_CHANGE ? 2 : 1;
     constexpr int CHUNK_BYTES = REDUCE_CHUNK_ELEMS * static_cast<int>(sizeof(GT));
-    constexpr int LPC = 2, CB = 8 / LPC;   // as in sumsq_kernel
-    extern __shared__ __align__(128) char stage[];   // SUMSQ_GROUP chunks
-    __shared__ float warp_sums[BLOCK_THREADS / 32];
-    __shared__ int s_staged[SUMSQ_GROUP];
+    extern __shared__ __align__(128) char stage[];   // [chunk][array][CHUNK_BYTES]
+    __shared__ const char *s_base[NC][2];
+    __shared__ int s_count[NC], s_head[NC], s_staged[NC];   // elements, how many in front of the staged ones
+    __shared__ float warp_sums[2][RED_THREADS / 32];
     __shared__ __align__(8) uint64_t bar;
-    const long long ngroups = (nchunks + SUMSQ_GROUP - 1) / SUMSQ_GROUP;
-    const long long nitems = ngroups * M;
     const int tid = threadIdx.x;
+    begin_and_let_next_begin();
+    const unsigned ngroups = static_cast<unsigned>((nchunks + NC - 1) / NC);
+    const int m = static_cast<int>(blockIdx.x / ngroups);
+    const long long q = blockIdx.x - m * ngroups;
     if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(smem_u32(&bar)), "r"(SUMSQ_GROUP) : "memory");
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(smem_u32(&bar)), "r"(NC) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    uint32_t phase = 0;
-    for (long long item = blockIdx.x; item < nitems; item += gridDim.x) {
-        const long long q = item % ngroups;
-        const int m = static_cast<int>(item / ngroups);
-        const long long c0 = q * SUMSQ_GROUP;
-        __syncthreads();   // the previous item is done with the stage; the barrier exists
-        if (tid < SUMSQ_GROUP) {
-            // one thread per chunk of the group: request it, or leave it to the direct path
-            uint32_t bytes = 0;
-            if (c0 + tid < nchunks) {
-                const Chunk ch = chunks[c0 + tid];
-                const char *base =
-                    reinterpret_cast<const char *>(g[static_cast<long long>(m) * nt + ch.tensor]) +
-                    ch.start * static_cast<long long>(sizeof(GT));
-                if (ch.count == REDUCE_CHUNK_ELEMS && (reinterpret_cast<uintptr_t>(base) & 15u) == 0) {
-                    bytes = CHUNK_BYTES;
-                    bulk_load(stage + tid * CHUNK_BYTES, base, bytes, &bar);
-                }
-            }
-            s_staged[tid] = bytes != 0;
-            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
-                         :: "r"(smem_u32(&bar)), "r"(bytes) : "memory");
-        }
-        __syncthreads();
-        const bool landed = bar_wait(&bar, phase, wait_limit);
-        if (__syncthreads_or(!landed)) {
-            // give up: say so, let the copies land (bounded as well), leave
-            if (tid == 0 && err) *reinterpret_cast<volatile int *>(err) = 1;
-            bar_wait(&bar, phase, DRAIN_WAIT_LIMIT);
-            __syncthreads();
-            return;
-        }
-        phase ^= 1u;
-        float acc0 = 0.f, acc1 = 0.f;
-#pragma unroll
-        for (int k = 0; k < SUMSQ_GROUP; k += CB) {
-            uint4 r[CB][LPC];
-#pragma unroll
-            for (int j = 0; j < CB; ++j) {
-                if (s_staged[k + j]) {
-                    const uint4 *src = reinterpret_cast<const uint4 *>(stage + (k + j) * CHUNK_BYTES);
-#pragma unroll
-                    for (int l = 0; l < LPC; ++l) r[j][l] = src[tid + l * BLOCK_THREADS];
-                }
-            }
-#pragma unroll
-            for (int j = 0; j < CB; ++j) {
-                if (s_staged[k + j]) {
-#pragma unroll
-                    for (int l = 0; l < LPC; ++l) {
-                        float &acc = (l & 1) ? acc1 : acc0;
-                        acc = sumsq8_bf16(r[j][l], acc);
-                    }
-                } else if (c0 + k + j < nchunks) {
-                    acc0 = chunk_sumsq<GT>(chunks[c0 + k + j], g, nt, m, acc0);
-                }
-            }
-        }
-        const float total = block_sum(acc0 + acc1, warp_sums);
-        if (tid == 0) partial[static_cast<long long>(m) * ngroups + q] = total;
+    // one thread per chunk of the item
+    const char *p0 = nullptr, *p1 = nullptr;
+    int count = 0;
+    if (tid < NC && q * NC + tid < nchunks) {
+        const Chunk ch = chunks[q * NC + tid];
+        const long long idx = static_cast<long long>(m) * nt + ch.tensor, off = ch.start * static_cast<long long>(sizeof(GT));
+        p0 = reinterpret_cast<const char *>(now[idx]) + off;
+        if constexpr (MODE == RED_CHANGE) p1 = reinterpret_cast<const char *>(then[idx]) + off;
+        count = ch.count;
     }
-}
-
-// partial[(0|1) * M * nchunks + m * nchunks + c]: sum of (now - then)^2 and of then^2.
-__global__ void __launch_bounds__(BLOCK_THREADS, 6)
-relchange_kernel(const Chunk *chunks, long long nchunks, const float *const *now,
-                 const float *const *then, int nt, int M, float *partial) {
-    begin_and_let_next_begin();
+    __syncthreads();   // the barrier exists
     wait_for_earlier_kernels();
-    __shared__ float warp_sums[BLOCK_THREADS / 32];
-    const long long nitems = nchunks * M;
-    const int tid = threadIdx.x;
-    for (long long item = blockIdx.x; item < nitems; item += gridDim.x) {
-        const long long c = item % nchunks;
-        const int m = static_cast<int>(item / nchunks);
-        const Chunk ch = chunks[c];
-        const long long idx = static_cast<long long>(m) * nt + ch.tensor;
-        const char *pa = reinterpret_cast<const char *>(now[idx]) + ch.start * 4;
-        const char *pb = reinterpret_cast<const char *>(then[idx]) + ch.start * 4;
-        const bool aligned = ((reinterpret_cast<uintptr_t>(pa) | reinterpret_cast<uintptr_t>(pb)) & 15u) == 0;
-        float num = 0.f, den = 0.f;
-        if (aligned) {
-            const int n4 = ch.count >> 2;
-            for (int p = tid; p < n4; p += BLOCK_THREADS) {
-                const FV<4> a = ld_f32<4>(pa, static_cast<long long>(p) * 4);
-                const FV<4> b = ld_f32<4>(pb, static_cast<long long>(p) * 4);
+    if (tid < NC) {
+        // Staged is what lies behind the first 128-byte boundary, in whole 16-byte pieces; the elements in
+        // front of it and the last ones are read directly (all of them where the two arrays lie
+        // differently).  Copies that start off a 128-byte line fetch every line twice: 4.2 TB/s instead of 6.9
+        // on a tightly packed fp32 buffer.
+        constexpr int ESZ = static_cast<int>(sizeof(GT)), PIECE = 16 / ESZ;
+        const uintptr_t a0 = reinterpret_cast<uintptr_t>(p0), a1 = MODE == RED_CHANGE ? reinterpret_cast<uintptr_t>(p1) : a0;
+        const bool can = a0 % ESZ == 0 && ((a0 ^ a1) & 15u) == 0;
+        const int head = can ? min(count, static_cast<int>((0 - a0) & 127u) / ESZ) : 0;
+        const int staged = can ? (count - head) & ~(PIECE - 1) : 0;
+        const uint32_t bytes = staged * static_cast<uint32_t>(ESZ);
+        if (bytes) {
+            bulk_load(stage + tid * NA * CHUNK_BYTES, p0 + head * ESZ, bytes, &bar);
+            if constexpr (MODE == RED_CHANGE) bulk_load(stage + (tid * NA + 1) * CHUNK_BYTES, p1 + head * ESZ, bytes, &bar);
+        }
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
+                     :: "r"(smem_u32(&bar)), "r"(NA * bytes) : "memory");
+        s_base[tid][0] = p0; s_base[tid][1] = p1;
+        s_count[tid] = count; s_head[tid] = head; s_staged[tid] = staged;
+    }
+    __syncthreads();
+    float acc[2] = {0.f, 0.f};
+    // what is not staged
+#pragma unroll 1
+    for (int k = 0; k < NC; ++k) {
+        for (int r = tid; r < s_count[k] - s_staged[k]; r += RED_THREADS) {
+            const int e = r < s_head[k] ? r : r + s_staged[k];
+            const float a = ld_grad<1, GT>(s_base[k][0], e).a[0];
+            if constexpr (MODE == RED_CHANGE) {
+                const float b = ld_f32<1>(s_base[k][1], e).a[0], d = a - b;
+                acc[0] = fmaf(d, d, acc[0]);
+                acc[1] = fmaf(b, b, acc[1]);
+            } else {
+                acc[0] = fmaf(a, a, acc[0]);
+            }
+        }
+    }
+    const bool landed = bar_wait(&bar, 0, wait_limit);
+    if (__syncthreads_or(!landed)) {
+        // give up: say so, let the copies land (bounded as well), leave
+        if (tid == 0 && err) *reinterpret_cast<volatile int *>(err) = 1;
+        bar_wait(&bar, 0, DRAIN_WAIT_LIMIT);
+        __syncthreads();
+        return;
+    }
+#pragma unroll 1
+    for (int k = 0; k < NC; ++k) {
+        const uint4 *a = reinterpret_cast<const uint4 *>(stage + k * NA * CHUNK_BYTES);
+        const uint4 *b = a + (NA - 1) * (CHUNK_BYTES / 16);
+        const int n = s_staged[k] * static_cast<int>(sizeof(GT)) / 16;
+#pragma unroll 4
+        for (int v = tid; v < n; v += RED_THREADS) add_squares<MODE>(a[v], b[v], acc);
+    }
+    if constexpr (MODE != RED_CHANGE) acc[0] += acc[1];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const float d = a.a[k] - b.a[k];
-                    num = fmaf(d, d, num);
-                    den = fmaf(b.a[k], b.a[k], den);
-                }
-            }
-            const int rem = ch.count & 3;
-            if (tid < rem) {
-                const float a = ld_f32<1>(pa, (n4 << 2) + tid).a[0], b = ld_f32<1>(pb, (n4 << 2) + tid).a[0];
-                num = fmaf(a - b, a - b, num);
-                den = fmaf(b, b, den);
-            }
-        } else {
-            for (int e = tid; e < ch.count; e += BLOCK_THREADS) {
-                const float a = ld_f32<1>(pa, e).a[0], b = ld_f32<1>(pb, e).a[0];
-                num = fmaf(a - b, a - b, num);
-                den = fmaf(b, b, den);
-            }
-        }
-        const float tn = block_sum(num, warp_sums);
-        const float td = block_sum(den, warp_sums);
-        if (tid == 0) {
-            partial[static_cast<long long>(m) * nchunks + c] = tn;
-            partial[(static_cast<long long>(M) + m) * nchunks + c] = td;
-        }
+    for (int j = 0; j < NA; ++j) {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) acc[j] += __shfl_down_sync(0xffffffffu, acc[j], off);
+        if ((tid & 31) == 0) warp_sums[j][tid >> 5] = acc[j];
+    }
+    __syncthreads();
+    if (tid < NA) {
+        float t = 0.f;
+#pragma unroll
+        for (int w = 0; w < RED_THREADS / 32; ++w) t += warp_sums[tid][w];
+        partial[(static_cast<long long>(tid) * M + m) * stride + q] = t;
     }
 }
 
-// One block per row: out_sum[row] = sum of partial[row * n .. +n) in fp64, fixed pattern
-// (thread i adds entries i, i+256, ... in order; then a shared-memory tree).
-template <typename T>
-__device__ __forceinline__ double row_sum_f64(const T *row, long long n, double *sh) {
+// ---- stage 2 -------------------------------------------------------------------------------------
+// Sum of row[0 .. n) in fp64 in a fixed pattern (each thread its groups of four, in order; then a
+// shuffle tree and the warps in order), the same in every thread.  All loads of a thread are independent:
+// a row of 16 K partials takes 2-3 us instead of 10 with one serial load per thread and 256 entries.
+// `row` is 16-byte aligned and n a multiple of four where WIDE.
+template <bool WIDE>
+__device__ __forceinline__ double row_sum_f64(const float *row, long long n, double *sh) {
     double acc = 0.0;
-    for (long long i = threadIdx.x; i < n; i += BLOCK_THREADS) acc += static_cast<double>(row[i]);
-    sh[threadIdx.x] = acc;
-    __syncthreads();
-    for (int s = BLOCK_THREADS / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
-        __syncthreads();
+    const int threads = blockDim.x;
+    if constexpr (WIDE) {
+        const float4 *r4 = reinterpret_cast<const float4 *>(row);
+#pragma unroll 8
+        for (long long i = threadIdx.x; i < n / 4; i += threads) {
+            const float4 v = r4[i];
+            acc += (static_cast<double>(v.x) + v.y) + (static_cast<double>(v.z) + v.w);
+        }
+    } else {
+#pragma unroll 8
+        for (long long i = threadIdx.x; i < n; i += threads) acc += static_cast<double>(row[i]);
     }
-    const double r = sh[0];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
+    __syncthreads();   // sh may still be read from the previous use
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
     __syncthreads();
+    double r = 0.0;
+    for (int w = 0; w < threads / 32; ++w) r += sh[w];
     return r;
 }
 
+// Rows of partials are padded to a multiple of four entries: block m adds zeros there.
+__device__ __forceinline__ void pad_row(float *row, long long n, long long stride) {
+    if (threadIdx.x < stride - n) row[n + threadIdx.x] = 0.f;
+    __syncthreads();
+}
+
+constexpr int FINAL_THREADS = 512;
+
 // norms[m] = ||g^m||_2, scales[m] = min(1, max_norm / norms[m]) (1 when max_norm <= 0).
-__global__ void __launch_bounds__(BLOCK_THREADS)
-norm_finalize_kernel(const float *partial, long long nchunks, float max_norm, float *norms,
-                     float *scales) {
+__global__ void __launch_bounds__(FINAL_THREADS)
+norm_finalize_kernel(float *partial, long long n, long long stride, float max_norm, float *norms, float *scales) {
+    __shared__ double sh[FINAL_THREADS / 32];
     begin_and_let_next_begin();
     wait_for_earlier_kernels();
-    __shared__ double sh[BLOCK_THREADS];
     const int m = blockIdx.x;
-    const double ss = row_sum_f64(partial + static_cast<long long>(m) * nchunks, nchunks, sh);
+    float *row = partial + m * stride;
+    pad_row(row, n, stride);
+    const double ss = row_sum_f64<true>(row, stride, sh);
     if (threadIdx.x == 0) {
         const double nrm = sqrt(ss);
         norms[m] = static_cast<float>(nrm);
@@ -327,14 +212,17 @@ norm_finalize_kernel(const float *partial, long long nchunks, float max_norm, fl
     }
 }
 
-__global__ void __launch_bounds__(BLOCK_THREADS)
-relchange_finalize_kernel(const float *partial, long long nchunks, int M, float *out) {
+__global__ void __launch_bounds__(FINAL_THREADS)
+relchange_finalize_kernel(float *partial, long long n, long long stride, int M, float *out) {
+    __shared__ double sh[FINAL_THREADS / 32];
     begin_and_let_next_begin();
     wait_for_earlier_kernels();
-    __shared__ double sh[BLOCK_THREADS];
     const int m = blockIdx.x;
-    const double num = row_sum_f64(partial + static_cast<long long>(m) * nchunks, nchunks, sh);
-    const double den = row_sum_f64(partial + (static_cast<long long>(M) + m) * nchunks, nchunks, sh);
+    float *row = partial + m * stride, *row2 = partial + (static_cast<long long>(M) + m) * stride;
+    pad_row(row, n, stride);
+    pad_row(row2, n, stride);
+    const double num = row_sum_f64<true>(row, stride, sh);
+    const double den = row_sum_f64<true>(row2, stride, sh);
     if (threadIdx.x == 0) out[m] = static_cast<float>(sqrt(num) / sqrt(den));
 }
 
@@ -358,41 +246,45 @@ mean_fill_kernel(const Chunk *chunks, long long nchunks, const float *const *src
     }
 }
 
-// Norm diagnostics of a DIAG step.  partial[(kind * M + m) * stride + c] holds the sum of
-// squares of chunk c; tstart[k] .. tstart[k + 1] are the chunks of tensor k.  One block per
-// (tensor, worker, kind): fp64 sum of the tensor's chunks, its root as the per-tensor norm.
-__global__ void __launch_bounds__(BLOCK_THREADS)
-diag_tensor_kernel(const float *partial, long long stride, const long long *tstart, int nt, int M,
-                   double *sums, float *norms) {
-    begin_and_let_next_begin();
-    wait_for_earlier_kernels();
-    __shared__ double sh[BLOCK_THREADS];
-    const int k = blockIdx.x, m = blockIdx.y, kind = blockIdx.z;
-    const long long row = static_cast<long long>(kind) * M + m;
-    const double ss = row_sum_f64(partial + row * stride + tstart[k], tstart[k + 1] - tstart[k], sh);
-    if (threadIdx.x == 0) {
-        sums[row * nt + k] = ss;
-        norms[row * nt + k] = static_cast<float>(sqrt(ss));
-    }
-}
+// Norm diagnostics of a DIAG step.  partial[row * stride + c], row = kind * M + m, holds the sum of
+// squares of chunk c; tstart[k] .. tstart[k + 1] are the chunks of tensor k.  A warp per (row,
+// tensor): fp64 sum of the tensor's chunks, its root as the per-tensor norm.  The first `rows` blocks
+// take a whole row each: the norm over the tensor list.  One launch, and both results go
+// straight to the host's memory: the read-out after a 135 M-parameter step (272 tensors, 4 workers)
+// takes 30-55 us, the whole call, as two launches and two copies did; 5 M parameters 23-27 us instead of 39.
+constexpr int DIAG_WARPS = 8;
 
-// One block per (kind, worker): the whole-model norm from the per-tensor sums of squares.
-__global__ void __launch_bounds__(BLOCK_THREADS)
-diag_total_kernel(const double *sums, int nt, float *totals) {
+__global__ void __launch_bounds__(DIAG_WARPS * 32)
+diag_norms_kernel(const float *partial, long long stride, const long long *tstart, int nt, int rows, float *norms,
+                  float *totals) {
+    __shared__ double sh[DIAG_WARPS];
     begin_and_let_next_begin();
     wait_for_earlier_kernels();
-    __shared__ double sh[BLOCK_THREADS];
-    const long long row = blockIdx.x;
-    const double ss = row_sum_f64(sums + row * nt, nt, sh);
-    if (threadIdx.x == 0) totals[row] = static_cast<float>(sqrt(ss));
+    if (blockIdx.x < rows) {
+        const double ss = row_sum_f64<false>(partial + blockIdx.x * stride, stride, sh);
+        if (threadIdx.x == 0) totals[blockIdx.x] = static_cast<float>(sqrt(ss));
+        return;
+    }
+    const long long item = static_cast<long long>(blockIdx.x - rows) * DIAG_WARPS + (threadIdx.x >> 5);
+    if (item >= static_cast<long long>(rows) * nt) return;
+    const long long row = item / nt;
+    const int k = static_cast<int>(item - row * nt);
+    const float *src = partial + row * stride;
+    const long long c1 = tstart[k + 1];
+    double acc = 0.0;
+#pragma unroll 8
+    for (long long c = tstart[k] + (threadIdx.x & 31); c < c1; c += 32) acc += static_cast<double>(src[c]);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
+    if ((threadIdx.x & 31) == 0) norms[item] = static_cast<float>(sqrt(acc));
 }
 
 // All launches of this file may begin while the kernel in front of them still runs.
 template <typename... P, typename... A>
-cudaError_t launch(void (*kernel)(P...), dim3 grid, size_t smem, cudaStream_t stream, A... args) {
+cudaError_t launch(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, A... args) {
     cudaLaunchConfig_t lc{};
     lc.gridDim = grid;
-    lc.blockDim = dim3(BLOCK_THREADS);
+    lc.blockDim = dim3(threads);
     lc.dynamicSmemBytes = smem;
     lc.stream = stream;
     cudaLaunchAttribute at{};
@@ -409,43 +301,49 @@ unsigned grid_for(long long nitems) {
 
 }  // namespace
 
+template <int MODE>
+static cudaError_t launch_sumsq(const Chunk *chunks, long long nchunks, const void *const *now, const void *const *then,
+                                int nt, int M, float *partial, long long *items, long long *stride, int *err,
+                                int wait_limit, cudaStream_t stream) {
+    *items = (nchunks + red_chunks(MODE) - 1) / red_chunks(MODE);
+    *stride = reduce_row(*items);
+    return launch(sumsq_kernel<MODE>, grid_for(*items * M), RED_THREADS, RED_BYTES, stream, chunks, nchunks, now, then, nt,
+                  M, partial, *stride, err, wait_limit);
+}
+
 cudaError_t launch_grad_norms(const Chunk *chunks, long long nchunks, const void *const *g, int nt,
                               int M, bool bf16, float max_norm, float *partial, float *norms,
                               float *scales, int *err, int wait_limit, cudaStream_t stream) {
-    const long long ngroups = (nchunks + SUMSQ_GROUP - 1) / SUMSQ_GROUP;
-    const unsigned grid = grid_for(ngroups * M);
-    cudaError_t e;
-    if (bf16) {
-        constexpr int smem = SUMSQ_GROUP * REDUCE_CHUNK_ELEMS * 2;
-        e = cudaFuncSetAttribute(sumsq_bulk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        e = launch(sumsq_bulk_kernel, grid, smem, stream, chunks, nchunks, g, nt, M, partial, err, wait_limit);
-    } else
-        e = launch(sumsq_kernel<float>, grid, 0, stream, chunks, nchunks, g, nt, M, partial);
+    long long items, stride;
+    const cudaError_t e =
+        bf16 ? launch_sumsq<RED_BF16>(chunks, nchunks, g, nullptr, nt, M, partial, &items, &stride, err, wait_limit, stream)
+             : launch_sumsq<RED_F32>(chunks, nchunks, g, nullptr, nt, M, partial, &items, &stride, err, wait_limit, stream);
     if (e != cudaSuccess) return e;
-    return launch(norm_finalize_kernel, M, 0, stream, partial, ngroups, max_norm, norms, scales);
+    return launch(norm_finalize_kernel, M, FINAL_THREADS, 0, stream, partial, items, stride, max_norm, norms, scales);
 }
 
 cudaError_t launch_rel_change(const Chunk *chunks, long long nchunks, const float *const *now,
                               const float *const *then, int nt, int M, float *partial, float *out,
-                              cudaStream_t stream) {
-    cudaError_t e = launch(relchange_kernel, grid_for(nchunks * M), 0, stream, chunks, nchunks, now, then, nt, M, partial);
+                              int *err, int wait_limit, cudaStream_t stream) {
+    long long items, stride;
+    const cudaError_t e = launch_sumsq<RED_CHANGE>(
+        chunks, nchunks, reinterpret_cast<const void *const *>(now), reinterpret_cast<const void *const *>(then), nt, M,
+        partial, &items, &stride, err, wait_limit, stream);
     if (e != cudaSuccess) return e;
-    return launch(relchange_finalize_kernel, M, 0, stream, partial, nchunks, M, out);
+    return launch(relchange_finalize_kernel, M, FINAL_THREADS, 0, stream, partial, items, stride, M, out);
 }
 
 cudaError_t launch_diag_norms(const float *partial, long long stride, const long long *tstart,
-                              int nt, int M, double *sums, float *per_tensor, float *totals,
-                              cudaStream_t stream) {
-    cudaError_t e = launch(diag_tensor_kernel, dim3(nt, M, DIAG_KINDS), 0, stream, partial, stride, tstart, nt, M, sums,
-                           per_tensor);
-    if (e != cudaSuccess) return e;
-    return launch(diag_total_kernel, DIAG_KINDS * M, 0, stream, sums, nt, totals);
+                              int nt, int M, float *per_tensor, float *totals, cudaStream_t stream) {
+    const int rows = DIAG_KINDS * M;
+    const long long blocks = rows + (static_cast<long long>(rows) * nt + DIAG_WARPS - 1) / DIAG_WARPS;
+    return launch(diag_norms_kernel, grid_for(blocks), DIAG_WARPS * 32, 0, stream, partial, stride, tstart, nt, rows,
+                  per_tensor, totals);
 }
 
 cudaError_t launch_mean_fill(const Chunk *chunks, long long nchunks, const float *const *src,
                              int m_src, float *const *dst, int m_dst, int nt, cudaStream_t stream) {
-    return launch(mean_fill_kernel, grid_for(nchunks), 0, stream, chunks, nchunks, src, m_src, dst, m_dst, nt);
+    return launch(mean_fill_kernel, grid_for(nchunks), BLOCK_THREADS, 0, stream, chunks, nchunks, src, m_src, dst, m_dst, nt);
 }
 
 }  // namespace desloc

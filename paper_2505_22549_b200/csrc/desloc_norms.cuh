@@ -4,7 +4,10 @@
 
 namespace desloc {
 
-// partial: scratch of at least M * nchunks floats; norms, scales: [M] floats, all on the device.
+// Entries of a row of partials: the rows are padded to whole 16-byte pieces.
+inline long long reduce_row(long long items) { return (items + 3) & ~3LL; }
+
+// partial: scratch of at least M * reduce_row(nchunks) floats; norms, scales: [M] floats, all on the device.
 // scales[m] = min(1, max_norm / ||g^m||_2), or 1 when max_norm <= 0.  Two launches.
 // err, wait_limit: the flag a block sets when its bounded wait for a bulk copy runs out, and the
 // bound (as for the step kernels).
@@ -12,17 +15,17 @@ cudaError_t launch_grad_norms(const Chunk *chunks, long long nchunks, const void
                               int M, bool bf16, float max_norm, float *partial, float *norms,
                               float *scales, int *err, int wait_limit, cudaStream_t stream);
 
-// partial: scratch of at least 2 * M * nchunks floats; out[m] = ||now - then|| / ||then||.
+// partial: scratch of at least 2 * M * reduce_row(nchunks) floats; out[m] = ||now - then|| / ||then||
+// (out may be host memory that the device can write to).  Two launches.
 cudaError_t launch_rel_change(const Chunk *chunks, long long nchunks, const float *const *now,
                               const float *const *then, int nt, int M, float *partial, float *out,
-                              cudaStream_t stream);
+                              int *err, int wait_limit, cudaStream_t stream);
 
 // Norms of a diagnostics step: partial [DIAG_KINDS][M][stride] per-chunk sums of squares,
-// tstart [nt + 1] first chunk of every tensor; writes sums [DIAG_KINDS][M][nt] (fp64 scratch),
-// per_tensor [DIAG_KINDS][M][nt] and totals [DIAG_KINDS][M] (floats), all on the device.
+// tstart [nt + 1] first chunk of every tensor; writes per_tensor [DIAG_KINDS][M][nt] and totals
+// [DIAG_KINDS][M] (floats; may be host memory that the device can write to).  One launch.
 cudaError_t launch_diag_norms(const float *partial, long long stride, const long long *tstart,
-                              int nt, int M, double *sums, float *per_tensor, float *totals,
-                              cudaStream_t stream);
+                              int nt, int M, float *per_tensor, float *totals, cudaStream_t stream);
 
 // Every element of the m_dst destination replicas := mean over the m_src source replicas.
 // src / dst are device tables indexed [m * nt + tensor].

@@ -60,15 +60,13 @@ struct WorkerSum {
         }
     }
     __device__ __forceinline__ FV<VEC> mean(int M) const {
-        const float mf = static_cast<float>(M);
+        const float mf = static_cast<float>(M), inv = 1.f / mf;
         FV<VEC> r;
 #pragma unroll
         for (int c = 0; c < VEC; ++c) {
             const float hi = s[c] + err[c];
             const float lo = err[c] - (hi - s[c]);          // hi + lo = s + err
-            const float q = hi / mf;
-            const float rem = fmaf(-q, mf, hi) + lo;        // what q * M still misses
-            r.a[c] = q + rem / mf;
+            r.a[c] = div_by_count(hi, lo, mf, inv);
         }
         return r;
     }

@@ -198,9 +198,20 @@ __device__ __forceinline__ float tree_sum(const float (&s)[MT]) {
     }
 }
 
+// hi / n for a small whole number n: the product with the rounded reciprocal, corrected by what
+// q * n misses -- the quotient of an IEEE division without its slow path, whose branch kept the
+// compiler from interleaving the workers: all-sync steps of six, seven workers 6.14, 6.22 -> 6.49, 6.54 TB/s.  lo: a low part of the dividend.
+__device__ __forceinline__ float div_by_count(float hi, float lo, float n, float inv_n) {
+    const float q = hi * inv_n;
+    const float r = fmaf(fmaf(-q, n, hi) + lo, inv_n, q);
+    return fabsf(q) <= 3.0e38f ? r : q;   // (infinities and NaN stay what they are)
+}
+
 template <int MT>
 __device__ __forceinline__ float mean_of(const float (&s)[MT]) {
-    return tree_sum<0, MT, MT>(s) / static_cast<float>(MT);
+    const float t = tree_sum<0, MT, MT>(s);
+    if constexpr ((MT & (MT - 1)) == 0) return t * (1.f / MT);   // exact
+    else return div_by_count(t, 0.f, static_cast<float>(MT), 1.f / MT);
 }
 
 // One worker's state update from the clipped gradient: `up`, `vp` are the previous states the

@@ -1,13 +1,14 @@
-// DES-LOC step for worker counts beyond the register-resident kernels (M > MAX_MT) on steps
-// that average something.  Same update as desloc_step_kernel, runtime M, compile-time mask.
-// Worker sums run in the order m = 0..M-1 as compensated fp32 sums (see WorkerSum): exact for
-// equal replicas, and within an ulp of a sequential fp64 reference.
+// DES-LOC step for the worker counts and variants that have no tile kernel (M > 16; from nine workers on also
+// the post-average ordering and the norm diagnostics) on steps that average something.  Same update
+// as desloc_step_kernel, runtime M, compile-time mask.  Worker sums run in the order m = 0..M-1 as
+// compensated fp32 sums (see WorkerSum): exact for equal replicas, and within an ulp of a
+// sequential fp64 reference.
 //
 // A block takes one chunk and first puts the chunk-relative pointers of all M workers into
 // shared memory, so that the per-position loops read them as broadcasts instead of chasing the
 // pointer tables in global memory.  Per position (4 elements per thread):
-//   pre-average   the arrays to be averaged are summed one array at a time, eight workers'
-//                 loads in flight; then the workers are updated in batches sized to the
+//   pre-average   the arrays to be averaged are summed in one pass, two or four workers' loads in
+//                 flight; then the workers are updated in batches sized to the
 //                 register budget, loading only what was not averaged (ADOPT also its own v).
 //                 Each array is read once and written once.
 //   post-average  phase A updates the states batch by batch, sums the ones to be averaged and
@@ -35,6 +36,20 @@ constexpr int GEN_BUDGET = 24;      // registers a batch of workers may hold in 
 __host__ __device__ constexpr int gen_batch(int per_worker, int budget) {
     const int b = budget / per_worker;
     return b < 2 ? 1 : (b < 4 ? 2 : 4);
+}
+
+// Sum of N workers' values as a binary tree.
+template <int VEC, int N>
+__device__ __forceinline__ FV<VEC> sum_of(const FV<VEC> (&v)[N]) {
+    FV<VEC> t;
+#pragma unroll
+    for (int c = 0; c < VEC; ++c) {
+        float q[N];
+#pragma unroll
+        for (int j = 0; j < N; ++j) q[j] = v[j].a[c];
+        t.a[c] = tree_sum<0, N, N>(q);
+    }
+    return t;
 }
 
 // Sum over the workers of one coordinate group, in the order m = 0..M-1, as a compensated fp32
@@ -77,15 +92,7 @@ struct WorkerSum {
     __device__ __forceinline__ void add_batch(const FV<VEC> (&v)[B], int n) {
         static_assert((B & (B - 1)) == 0, "batches are powers of two");
         if (n >= B) {
-            FV<VEC> t;
-#pragma unroll
-            for (int c = 0; c < VEC; ++c) {
-                float q[B];
-#pragma unroll
-                for (int j = 0; j < B; ++j) q[j] = v[j].a[c];
-                t.a[c] = tree_sum<0, B, B>(q);
-            }
-            add(t);
+            add(sum_of<VEC, B>(v));
         } else {
 #pragma unroll
             for (int j = 0; j < B; ++j)
@@ -94,9 +101,10 @@ struct WorkerSum {
     }
 };
 
-// Worker means of the arrays selected by SX, SU, SV in one pass over the workers: the loads of
-// a batch of workers (all selected arrays) are issued together -- four workers for one array,
-// two for two or three -- and then added in worker order, one accumulator per array.
+// Worker means of the arrays selected by SX, SU, SV in one pass over the workers: trees of four
+// workers enter the compensated sums in order, the last one to three workers value by value (the order
+// of compensated_mean(), so that a step with norm diagnostics gives the bits of one without).  The
+// loads of four workers are issued together for one array, of two for two or three.
 template <int VEC, bool SX, bool SU, bool SV>
 __device__ __forceinline__ void means_of_workers(char *const (*sp)[GEN_MAX_M], int M, long long e,
                                                  bool active, FV<VEC> &xb, FV<VEC> &ub, FV<VEC> &vb) {
@@ -104,21 +112,43 @@ __device__ __forceinline__ void means_of_workers(char *const (*sp)[GEN_MAX_M], i
     constexpr int NB = NS == 1 ? 4 : 2;
     WorkerSum<VEC> ax, au, av;
     ax.clear(); au.clear(); av.clear();
+    int m0 = 0;
 #pragma unroll 1
-    for (int m0 = 0; m0 < M; m0 += NB) {
-        FV<VEC> bx[NB], bu[NB], bv[NB];
+    for (; m0 + 4 <= M; m0 += 4) {
+        FV<VEC> px[4 / NB], pu[4 / NB], pv[4 / NB];   // sums of NB workers
 #pragma unroll
-        for (int j = 0; j < NB; ++j) {
-            if (active && m0 + j < M) {
-                if constexpr (SX) bx[j] = ld_f32<VEC>(sp[0][m0 + j], e);
-                if constexpr (SU) bu[j] = ld_f32<VEC>(sp[1][m0 + j], e);
-                if constexpr (SV) bv[j] = ld_f32<VEC>(sp[2][m0 + j], e);
+        for (int h = 0; h < 4 / NB; ++h) {
+            FV<VEC> bx[NB], bu[NB], bv[NB];
+#pragma unroll
+            for (int j = 0; j < NB; ++j) {
+                if (active) {
+                    if constexpr (SX) bx[j] = ld_f32<VEC>(sp[0][m0 + h * NB + j], e);
+                    if constexpr (SU) bu[j] = ld_f32<VEC>(sp[1][m0 + h * NB + j], e);
+                    if constexpr (SV) bv[j] = ld_f32<VEC>(sp[2][m0 + h * NB + j], e);
+                }
+            }
+            if (active) {
+                if constexpr (SX) px[h] = sum_of<VEC, NB>(bx);
+                if constexpr (SU) pu[h] = sum_of<VEC, NB>(bu);
+                if constexpr (SV) pv[h] = sum_of<VEC, NB>(bv);
             }
         }
         if (active) {
-            if constexpr (SX) ax.template add_batch<NB>(bx, M - m0);
-            if constexpr (SU) au.template add_batch<NB>(bu, M - m0);
-            if constexpr (SV) av.template add_batch<NB>(bv, M - m0);
+            if constexpr (SX) ax.add(sum_of<VEC, 4 / NB>(px));
+            if constexpr (SU) au.add(sum_of<VEC, 4 / NB>(pu));
+            if constexpr (SV) av.add(sum_of<VEC, 4 / NB>(pv));
+        }
+    }
+#pragma unroll 1
+    for (; m0 < M; ++m0) {
+        if (active) {
+            FV<VEC> bx, bu, bv;
+            if constexpr (SX) bx = ld_f32<VEC>(sp[0][m0], e);
+            if constexpr (SU) bu = ld_f32<VEC>(sp[1][m0], e);
+            if constexpr (SV) bv = ld_f32<VEC>(sp[2][m0], e);
+            if constexpr (SX) ax.add(bx);
+            if constexpr (SU) au.add(bu);
+            if constexpr (SV) av.add(bv);
         }
     }
     if constexpr (SX) xb = ax.mean(M);

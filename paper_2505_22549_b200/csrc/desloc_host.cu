@@ -25,6 +25,12 @@ const void *lookup_step_kernel(int opt, bool post, bool bf16, int mt, int mask, 
     // in the pre-average units and is the same code for either ordering.
     const bool pre = !post || mask == 0;
     const int m = mask == 0 ? 1 : mt;
+    if (m > MAX_MT) {
+        if (post || diag || m > MAX_TILE_MT) return nullptr;
+        if (opt == OPT_ADAM) return m < 13 ? lookup_adam_m9(bf16, m, mask) : lookup_adam_m13(bf16, m, mask);
+        if (opt == OPT_ADOPT) return m < 13 ? lookup_adopt_m9(bf16, m, mask) : lookup_adopt_m13(bf16, m, mask);
+        return m < 13 ? lookup_sgdm_m9(bf16, m, mask) : lookup_sgdm_m13(bf16, m, mask);
+    }
     if (opt == OPT_ADAM) {
         if (diag) return pre ? lookup_adam_pre_diag(bf16, m, mask) : lookup_adam_post_diag(bf16, m, mask);
         return pre ? lookup_adam_pre(bf16, m, mask) : lookup_adam_post(bf16, m, mask);

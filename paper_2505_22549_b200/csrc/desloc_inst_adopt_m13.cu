@@ -1,0 +1,8 @@
+// desloc_step_kernel instantiations: ADOPT, pre-average ordering, 13 to 16 workers.
+#include "desloc_inst.cuh"
+
+namespace desloc {
+const void *lookup_adopt_m13(bool bf16, int mt, int mask) {
+    return lookup_sync<OPT_ADOPT, false, false, 13, 16>(bf16, mt, mask);
+}
+}  // namespace desloc

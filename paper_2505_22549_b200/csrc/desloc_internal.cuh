@@ -128,8 +128,9 @@ inline int64_t count_chunks(const int64_t *numel, int32_t num_tensors, int64_t c
 }
 
 // Blocks that share a chunk of all mt replicas (of one, for mt = 1).
-inline int64_t parts_for(int64_t chunk_elems, int mt) {
-    return (chunk_elems + most_part_elems(mt) - 1) / most_part_elems(mt);
+inline int64_t parts_for(int64_t chunk_elems, int opt, int mt, bool bf16) {
+    const int64_t most = most_part_elems(opt, mt, bf16);
+    return (chunk_elems + most - 1) / most;
 }
 
 // One thread block per part of a chunk and worker on a local step, one per chunk on the others: does
@@ -137,7 +138,7 @@ inline int64_t parts_for(int64_t chunk_elems, int mt) {
 inline bool grid_fits(int32_t M, const int64_t *numel, int32_t num_tensors) {
     const int64_t nchunks = count_chunks(numel, num_tensors, chunk_elems_for(M, numel, num_tensors)) + num_tensors;
     const int64_t chunk_elems = chunk_elems_for(M, numel, num_tensors);
-    const int64_t per_chunk = M * parts_for(chunk_elems, 1);
+    const int64_t per_chunk = M * parts_for(chunk_elems, OPT_ADAM, 1, true);
     return nchunks <= 0x7fffffffLL / per_chunk;
 }
 
@@ -241,26 +242,29 @@ inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, long long n
     const bool post = (c.flags & DESLOC_FLAG_POST_AVERAGE) != 0;
     const bool bf16 = c.grad_dtype == DESLOC_BF16;
     const bool local = kmask == 0;
-    const bool generic = !local && c.M > MAX_MT;
+    // More than eight workers: tiles of all replicas up to sixteen, the runtime-M kernel beyond, for the
+    // post-average ordering and for the norm diagnostics.  All-sync steps of sixteen workers (Adam, bf16
+    // gradients): 6.52 TB/s in tiles, 6.29 in the runtime-M kernel; nine workers 6.2 and 5.89.
+    const bool generic = !local && c.M > MAX_MT && (c.M > MAX_TILE_MT || post || diag);
     p.fn = generic ? lookup_generic_kernel(c.opt, post, bf16, static_cast<int>(kmask), diag)
                    : lookup_step_kernel(c.opt, post, bf16, c.M, static_cast<int>(kmask), diag);
     p.strides = !generic;
     const int mt = local ? 1 : c.M;
     p.grid = nchunks;
     if (!generic) {
-        const int64_t tile = tile_elems(c.opt, mt, bf16), tiles = chunk_elems / tile;
+        const int64_t tile = tile_elems(c.opt, mt, bf16), tiles = (chunk_elems + tile - 1) / tile;
         const int64_t replicas = local ? c.M : 1;
         // (the diagnostics write one partial sum per chunk: their blocks take whole chunks)
-        int64_t parts = diag ? 1 : parts_for(chunk_elems, mt);
+        int64_t parts = diag ? 1 : parts_for(chunk_elems, c.opt, mt, bf16);
         // a step that fits in one wave of blocks is pure latency: one tile per block
         if (!diag && nchunks * tiles * replicas <= (local ? LOCAL_WAVE : DIRECT_GRID)) parts = tiles;
         p.parts = static_cast<int>(parts);
         p.part_elems = static_cast<int>((tiles + parts - 1) / parts * tile);
-        p.threads = step_threads(mt);
+        p.threads = step_threads(c.opt, mt, bf16);
         p.smem = step_smem_bytes(c.opt, mt, bf16, p.part_elems);
-        p.smem_limit = step_smem_bytes(c.opt, mt, bf16, most_part_elems(mt));
+        p.smem_limit = step_smem_bytes(c.opt, mt, bf16, most_part_elems(c.opt, mt, bf16));
         p.grid = nchunks * parts * replicas;
-        p.direct = p.grid <= (local ? LOCAL_WAVE : DIRECT_GRID) && p.part_elems <= (local ? tile : plan_tile_elems(mt));
+        p.direct = p.grid <= (local ? LOCAL_WAVE : DIRECT_GRID) && p.part_elems <= (local || mt > MAX_MT ? tile : plan_tile_elems(mt));
     }
     return p;
 }

@@ -45,7 +45,8 @@ namespace desloc {
 constexpr int OPT_ADAM = 0, OPT_ADOPT = 1, OPT_SGDM = 2;
 constexpr int SYNC_X = 1, SYNC_U = 2, SYNC_V = 4;
 constexpr int BLOCK_THREADS = 256; // of every kernel but the one-replica step kernel
-constexpr int MAX_MT = 8;          // largest worker count with a kernel instantiated for it
+constexpr int MAX_MT = 8;          // largest worker count with a kernel instantiated for every step
+constexpr int MAX_TILE_MT = 16;    // ... for the pre-average sync steps without norm diagnostics
 constexpr int DIAG_G = 0, DIAG_X = 1, DIAG_D = 2, DIAG_KINDS = 3;
 constexpr int REDUCE_CHUNK_ELEMS = BLOCK_THREADS * 16;  // chunks of the reduction kernels (4096)
 constexpr int GENERIC_CHUNK_ELEMS = 1024;               // chunks of contexts with M > MAX_MT
@@ -56,7 +57,18 @@ constexpr int DRAIN_WAIT_LIMIT = 1 << 22;               // bound on the wait for
 // with 256-element tiles, were 5 % slower on eight workers).  Eight replicas with fp32 gradients and
 // two states would need 64 KB per buffer, which leaves room for one block per SM: 256-element
 // tiles and three blocks move 6.64 TB/s there instead of 5.5 (all-sync steps of 14 GB).
+//
+// Nine to sixteen replicas: as many elements, in units of a warp, as two buffers and two blocks per
+// SM leave room for -- these kernels are bound by the bytes they keep in flight (twelve replicas, all-sync, with
+// 256 elements 4.95 TB/s, with 320 6.2).
+__host__ __device__ constexpr int tile_bytes_per_elem(int opt, int mt, bool bf16) {
+    return mt * ((bf16 ? 2 : 4) + 4 * (opt == OPT_SGDM ? 2 : 3));
+}
 __host__ __device__ constexpr int tile_elems(int opt, int mt, bool bf16) {
+    if (mt > MAX_MT) {
+        const int t = 56 * 1024 / tile_bytes_per_elem(opt, mt, bf16) / 32 * 32;
+        return t < 512 ? t : 512;
+    }
     return mt == 8 && !bf16 && opt != OPT_SGDM ? 256 : 512;
 }
 // The unit in which a context's chunk table is cut (chunks are whole multiples of it).
@@ -73,7 +85,9 @@ __host__ __device__ constexpr int max_tiles_per_chunk(int) { return 8; }
 // 6.24-6.49 with tiles twice or four times as long, 6.79 for tiles of all replicas.  Two replicas: four tiles
 // through two buffers, 6.85 against 6.78 with eight tiles of 1024 elements.  More: whole chunks
 // (four tiles instead of eight cost eight workers 2 %, four workers nothing).
-__host__ __device__ constexpr int most_part_elems(int mt) { return mt == 1 ? 3 * 512 : mt == 2 ? 4 * 512 : 8 * 512; }
+__host__ __device__ constexpr int most_part_elems(int opt, int mt, bool bf16) {
+    return mt == 1 ? 3 * 512 : mt == 2 ? 4 * 512 : mt <= MAX_MT ? 8 * 512 : 8 * tile_elems(opt, mt, bf16);
+}
 
 struct __align__(16) Chunk {
     int32_t tensor;  // index into the tensor list
@@ -141,6 +155,9 @@ __device__ __forceinline__ FV<VEC> ld_f32(const char *base, long long elem) {
     if constexpr (VEC == 4) {
         const float4 t = *(reinterpret_cast<const float4 *>(base) + (elem >> 2));
         r.a[0] = t.x; r.a[1] = t.y; r.a[2] = t.z; r.a[3] = t.w;
+    } else if constexpr (VEC == 2) {
+        const float2 t = *(reinterpret_cast<const float2 *>(base) + (elem >> 1));
+        r.a[0] = t.x; r.a[1] = t.y;
     } else {
         r.a[0] = *(reinterpret_cast<const float *>(base) + elem);
     }
@@ -151,6 +168,8 @@ template <int VEC>
 __device__ __forceinline__ void st_f32(char *base, long long elem, const FV<VEC> &r) {
     if constexpr (VEC == 4) {
         *(reinterpret_cast<float4 *>(base) + (elem >> 2)) = make_float4(r.a[0], r.a[1], r.a[2], r.a[3]);
+    } else if constexpr (VEC == 2) {
+        *(reinterpret_cast<float2 *>(base) + (elem >> 1)) = make_float2(r.a[0], r.a[1]);
     } else {
         *(reinterpret_cast<float *>(base) + elem) = r.a[0];
     }
@@ -168,6 +187,10 @@ __device__ __forceinline__ FV<VEC> ld_grad(const char *base, long long elem) {
         r.a[1] = __uint_as_float(t.x & 0xffff0000u);
         r.a[2] = __uint_as_float(t.y << 16);
         r.a[3] = __uint_as_float(t.y & 0xffff0000u);
+    } else if constexpr (VEC == 2) {
+        const unsigned t = *(reinterpret_cast<const unsigned *>(base) + (elem >> 1));
+        r.a[0] = __uint_as_float(t << 16);
+        r.a[1] = __uint_as_float(t & 0xffff0000u);
     } else {
         const unsigned short t = *(reinterpret_cast<const unsigned short *>(base) + elem);
         r.a[0] = __uint_as_float(static_cast<unsigned>(t) << 16);
@@ -193,7 +216,7 @@ __device__ __forceinline__ float tree_sum(const float (&s)[MT]) {
         return s[LO];
     } else {
         constexpr int H = (N > 4) ? 4 : (N > 2 ? 2 : 1);
-        static_assert(N <= 8, "tree_sum covers up to eight workers");
+        static_assert(N <= 8, "tree_sum covers up to eight values");
         return tree_sum<LO, H, MT>(s) + tree_sum<LO + H, N - H, MT>(s);
     }
 }
@@ -207,11 +230,35 @@ __device__ __forceinline__ float div_by_count(float hi, float lo, float n, float
     return fabsf(q) <= 3.0e38f ? r : q;   // (infinities and NaN stay what they are)
 }
 
+// More than eight workers: trees of four, then a compensated sum ("two-sum") over them in order -- the
+// running sum and the exact rounding error of every addition, about 48 bits -- like the runtime-M kernel's.
+template <int MT>
+__device__ __forceinline__ float compensated_mean(const float (&s)[MT]) {
+    float sum = tree_sum<0, 4, MT>(s), err = 0.f;
+    const auto add = [&](float x) {
+        const float t = sum + x, bp = t - sum;
+        err += (sum - (t - bp)) + (x - bp);
+        sum = t;
+    };
+    add(tree_sum<4, 4, MT>(s));
+    if constexpr (MT >= 12) add(tree_sum<8, 4, MT>(s));
+    if constexpr (MT >= 16) add(tree_sum<12, 4, MT>(s));
+#pragma unroll
+    for (int m = MT / 4 * 4; m < MT; ++m) add(s[m]);
+    const float hi = sum + err, lo = err - (hi - sum);   // hi + lo = sum + err
+    return div_by_count(hi, lo, static_cast<float>(MT), 1.f / MT);
+}
+
 template <int MT>
 __device__ __forceinline__ float mean_of(const float (&s)[MT]) {
-    const float t = tree_sum<0, MT, MT>(s);
-    if constexpr ((MT & (MT - 1)) == 0) return t * (1.f / MT);   // exact
-    else return div_by_count(t, 0.f, static_cast<float>(MT), 1.f / MT);
+    if constexpr (MT > MAX_MT) {
+        static_assert(MT <= MAX_TILE_MT, "three or four trees of four, and up to three more");
+        return compensated_mean<MT>(s);
+    } else {
+        const float t = tree_sum<0, MT, MT>(s);
+        if constexpr ((MT & (MT - 1)) == 0) return t * (1.f / MT);   // exact
+        else return div_by_count(t, 0.f, static_cast<float>(MT), 1.f / MT);
+    }
 }
 
 // One worker's state update from the clipped gradient: `up`, `vp` are the previous states the
@@ -350,27 +397,18 @@ struct SmemAcc {
     }
 };
 
-// Straight from / to global memory, one coordinate per position (unaligned or ragged tiles).
-template <int MT, typename GT>
+// Straight from / to global memory, V coordinates per position with accesses that wide (bf16
+// gradients: half): one (unaligned or ragged tiles), four -- chunks whose fp32 arrays are 16-byte aligned while
+// the bf16 gradients are only 8-byte aligned, as in a flat layout padded to 16 bytes where the gradient of a
+// tensor at an odd multiple of four elements sits 8 bytes off, and the aligned part of a ragged
+// last tile -- or two, for the same chunks of more than eight workers (registers).
+template <int MT, typename GT, int V>
 struct GlobalAcc {
-    static constexpr int VEC = 1;
+    static constexpr int VEC = V;
     char *const (*sp)[MT];   // chunk-relative base pointers: 0 x, 1 u, 2 v, 3 g
-    __device__ __forceinline__ FV<1> ld(int arr, int m, int q) const { return ld_f32<1>(sp[arr][m], q); }
-    __device__ __forceinline__ void st(int arr, int m, int q, const FV<1> &r) const { st_f32<1>(sp[arr][m], q, r); }
-    __device__ __forceinline__ FV<1> ldg(int m, int q) const { return ld_grad<1, GT>(sp[3][m], q); }
-};
-
-// The same with four coordinates per position and 128-bit accesses (64-bit for bf16 gradients):
-// chunks whose fp32 arrays are 16-byte aligned while the bf16 gradients are only 8-byte aligned
-// -- a flat layout padded to 16 bytes, where the gradient of a tensor at an odd multiple of
-// four elements sits 8 bytes off -- and the aligned part of a ragged last tile.
-template <int MT, typename GT>
-struct GlobalAcc4 {
-    static constexpr int VEC = 4;
-    char *const (*sp)[MT];
-    __device__ __forceinline__ FV<4> ld(int arr, int m, int q) const { return ld_f32<4>(sp[arr][m], 4LL * q); }
-    __device__ __forceinline__ void st(int arr, int m, int q, const FV<4> &r) const { st_f32<4>(sp[arr][m], 4LL * q, r); }
-    __device__ __forceinline__ FV<4> ldg(int m, int q) const { return ld_grad<4, GT>(sp[3][m], 4LL * q); }
+    __device__ __forceinline__ FV<V> ld(int arr, int m, int q) const { return ld_f32<V>(sp[arr][m], static_cast<long long>(V) * q); }
+    __device__ __forceinline__ void st(int arr, int m, int q, const FV<V> &r) const { st_f32<V>(sp[arr][m], static_cast<long long>(V) * q, r); }
+    __device__ __forceinline__ FV<V> ldg(int m, int q) const { return ld_grad<V, GT>(sp[3][m], static_cast<long long>(V) * q); }
 };
 
 // ---- diagnostics ------------------------------------------------------------------------------
@@ -570,14 +608,18 @@ __device__ __forceinline__ bool bar_wait(uint64_t *bar, uint32_t parity, int lim
 }
 
 // Threads, tile buffers and resident blocks per SM.  Three and more replicas of a tile: two buffers
-// of 21-57 KB and 256 threads, as many blocks as the buffers leave room for (three up to four
-// workers, two beyond; three buffers at two blocks per SM: 0.84 of the copy bandwidth).  One
+// of 21-57 KB and 256 threads (one per element beyond eight replicas), as many blocks as the buffers leave room for,
+// four at most (three buffers at two blocks per SM: 0.84 of the copy bandwidth).  One
 // replica: up to three buffers of 7 KB (bf16 gradients; 5 KB without v) and 128 threads, one float4 of
 // each array per thread and tile, ten blocks.
-__host__ __device__ constexpr int step_threads(int mt) { return mt <= 2 ? 128 : BLOCK_THREADS; }
+__host__ __device__ constexpr int step_threads(int opt, int mt, bool bf16) {
+    return mt <= 2 ? 128 : mt <= MAX_MT ? BLOCK_THREADS : tile_elems(opt, mt, bf16);
+}
 __host__ __device__ constexpr int step_stages(int mt) { return mt == 1 ? 3 : 2; }
 __host__ __device__ constexpr int step_min_blocks(int opt, int mt, bool bf16) {
-    return mt == 1 ? 10 : mt == 2 ? 7 : mt <= 4 || tile_elems(opt, mt, bf16) < 512 ? 3 : 2;
+    if (mt <= 2) return mt == 1 ? 10 : 7;
+    const int room = 225 * 1024 / (2 * tile_elems(opt, mt, bf16) * tile_bytes_per_elem(opt, mt, bf16) + 1024);
+    return room < 2 ? 2 : room > 4 ? 4 : room;
 }
 
 // A chunk is a run of consecutive tiles of one tensor.  The block looks its pointers up
@@ -585,14 +627,14 @@ __host__ __device__ constexpr int step_min_blocks(int opt, int mt, bool bf16) {
 // place, tiles k + 1 .. k + S - 1 are already landing; when tile k's copy back has left its
 // buffer, tile k + S is requested into it.
 template <int OPT, int MASK, int MT, typename GT, bool POST, bool DIAG>
-__global__ void __launch_bounds__(step_threads(MT), step_min_blocks(OPT, MT, sizeof(GT) == 2))
+__global__ void __launch_bounds__(step_threads(OPT, MT, sizeof(GT) == 2), step_min_blocks(OPT, MT, sizeof(GT) == 2))
 desloc_step_kernel(const __grid_constant__ StepArgs a) {
-    constexpr int THREADS = step_threads(MT);
+    constexpr int THREADS = step_threads(OPT, MT, sizeof(GT) == 2);
     constexpr int T = tile_elems(OPT, MT, sizeof(GT) == 2), VEC = T / THREADS, S = step_stages(MT);
     constexpr int ALIGN_ELEMS = 16 / static_cast<int>(sizeof(GT));   // bulk copies move multiples of 16 bytes
     constexpr bool HAS_V = OPT != OPT_SGDM;
     using L = TileLayout<OPT, MT, GT, T>;
-    static_assert(4 * MT <= 32, "the (array, worker) owners are lanes of the first warp");
+    static_assert(4 * MT <= THREADS && T % THREADS == 0, "a thread per (array, worker); whole tiles");
     extern __shared__ __align__(128) char tile_mem[];   // S buffers of L::BYTES
     __shared__ char *sp[4][MT];
     __shared__ float sscale[MT];
@@ -709,13 +751,14 @@ desloc_step_kernel(const __grid_constant__ StepArgs a) {
             // what could not be staged: the whole chunk, or its ragged last tile
             int e0 = staged * T;
             if (wide_ok) {
-                const GlobalAcc4<MT, GT> acc4{sp};
-                const int p1 = count >> 2;
-                for (int q = (e0 >> 2) + tid; q < p1; q += THREADS)
-                    update_position<OPT, MASK, MT, POST, DIAG>(a, acc4, sscale, q, wn);
-                e0 = p1 << 2;
+                constexpr int V = MT <= MAX_MT ? 4 : 2;
+                const GlobalAcc<MT, GT, V> wide{sp};
+                const int p1 = count / V;
+                for (int q = e0 / V + tid; q < p1; q += THREADS)
+                    update_position<OPT, MASK, MT, POST, DIAG>(a, wide, sscale, q, wn);
+                e0 = p1 * V;
             }
-            const GlobalAcc<MT, GT> acc{sp};
+            const GlobalAcc<MT, GT, 1> acc{sp};
             for (int e = e0 + tid; e < count; e += THREADS)
                 update_position<OPT, MASK, MT, POST, DIAG>(a, acc, sscale, e, wn);
         }
@@ -746,12 +789,13 @@ __host__ __device__ constexpr int step_smem_bytes(int opt, int mt, bool bf16, in
     return (tiles < step_stages(mt) ? tiles : step_stages(mt)) * mt * t * ((bf16 ? 2 : 4) + 4 * (opt == OPT_SGDM ? 2 : 3));
 }
 
-// Lookup of an instantiation: opt, post-average?, bf16 gradients?, MT in 1..MAX_MT, mask,
+// Lookup of an instantiation: opt, post-average?, bf16 gradients?, MT in 1..MAX_MT (pre-average and
+// without norms: 1..MAX_TILE_MT), mask,
 // with or without the norm diagnostics (MT = 1 exists for mask 0 only, and mask 0 for MT = 1).
-// Returns nullptr for combinations that do not exist (sync masks with M > MAX_MT).
+// Returns nullptr for combinations that do not exist.
 const void *lookup_step_kernel(int opt, bool post, bool bf16, int mt, int mask, bool diag);
 
-// Runtime-M kernel for sync steps of M > MAX_MT.
+// Runtime-M kernel for the sync steps of M > MAX_MT that have no tile kernel.
 const void *lookup_generic_kernel(int opt, bool post, bool bf16, int mask, bool diag);
 
 }  // namespace desloc

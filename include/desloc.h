@@ -154,7 +154,7 @@ DESLOC_API int desloc_step(desloc_ctx *ctx, int64_t t, float lr_t, float clip_bo
  *                are to overlap with compute), same indexing and dtype as for desloc_step().
  *   dev_grads  : host array of M*num_tensors DEVICE pointers to caller-owned staging buffers
  *                of the same sizes; they receive the copies and are what the kernels read.
- * The tensor list is cut into up to 8 groups; each group's gradients are copied on a stream
+ * The tensor list is cut into up to 8 groups, of falling size; each group's gradients are copied on a stream
  * the context owns (tensors adjacent in both host and device memory go as one copy) and the
  * group's part of the step is launched on `stream` as soon as its copies have landed, so all
  * but the last group's compute hides behind the transfers.  The copies wait for work already
@@ -289,7 +289,8 @@ DESLOC_API int64_t desloc_plan_chunks(const int64_t *numel, int32_t num_tensors,
 /* Elements per chunk -- the run of tiles one thread block streams through, for all workers -- of
    a context created from cfg (M, numel and num_tensors are read).  A tile is 1024 elements for
    M <= 2, 512 for M = 3..8 (M > 8: 1024-element chunks, no tiles); a chunk is up to 8 tiles
-   on a large problem, fewer on a small one.  Negative desloc_status on bad
+   on a large problem, fewer on a small one (so many that the blocks of an averaging step come
+   in full rounds).  Negative desloc_status on bad
    input. */
 DESLOC_API int64_t desloc_chunk_elems(const desloc_config *cfg);
 

@@ -54,7 +54,8 @@ using desloc::validate_config;
 namespace {
 
 constexpr int kSlots = 8;  // staging slots for per-step gradient pointer tables
-constexpr int kHostGroups = 8;  // pipeline depth of desloc_step_host
+constexpr int kHostGroups = 8;  // most groups that desloc_step_host is pipelined in, and
+constexpr int64_t kHostSplit = 1600000;   // the fewest parameters worth splitting again
 
 struct Slot {
     void **host = nullptr;
@@ -128,18 +129,24 @@ cudaError_t make_worker_res(WorkerRes &r, int M, const int64_t *numel, int num_t
     std::vector<long long> tstart(static_cast<size_t>(num_tensors) + 1, 0);
     r.groups.clear();
     {
-        // tensor groups of about equal size for desloc_step_host
-        int64_t acc = 0, c0 = 0;
+        // Tensor groups for desloc_step_host: three quarters of what is left, each time.  A group's kernel
+        // takes a ninth of its copies' time, so it hides behind the next group's even at a quarter of the size, and
+        // the last group, whose kernel nothing hides, is small.  A copy costs 6 us beside its bytes, one per
+        // worker and group at best: below 1.6 M parameters that is more than the kernel.  (25 M parameters x
+        // 4 workers: 3817 us with eight equal groups, 3774 us with three; the copies alone 3690.)
+        int64_t left = total, acc = 0, c0 = 0;
         int32_t k0 = 0;
         for (int32_t k = 0; k < num_tensors; ++k) {
             tstart[k + 1] = tstart[k] + desloc::chunks_of(numel[k], chunk_elems, heads[k]);
             acc += numel[k];
             const int done_groups = static_cast<int>(r.groups.size());
-            const bool last = k == num_tensors - 1;
-            if (last || (done_groups < kHostGroups - 1 && acc * kHostGroups >= total * (done_groups + 1))) {
+            const bool split = done_groups < kHostGroups - 1 && (done_groups == 0 || left > kHostSplit);
+            if (k == num_tensors - 1 || (split && 4 * acc >= 3 * left)) {
                 r.groups.push_back({k0, k + 1, c0, tstart[k + 1]});
                 k0 = k + 1;
                 c0 = tstart[k + 1];
+                left -= acc;
+                acc = 0;
             }
         }
     }
@@ -416,6 +423,7 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
                 const desloc::LaunchPlan gp = desloc::plan_launch(c, mask, a.nchunks, ctx->res.chunk_elems, diag);
                 a.parts = gp.parts;
                 a.part_elems = gp.part_elems;
+                if (ctx->staging_mode < 0) a.direct = gp.direct ? 1 : 0;
                 // (no overlap: this kernel also depends on the other stream's copies)
                 e = desloc::launch_kernel(gp.fn, capped(gp), gp.threads, gp.smem, stream, params, false);
                 if (e == cudaSuccess) ctx->launches += 1;

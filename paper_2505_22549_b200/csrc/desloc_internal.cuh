@@ -79,15 +79,32 @@ inline uint32_t mask_at(const desloc_config *c, int64_t t) {
     return m;
 }
 
+constexpr int NUM_SMS = 148;   // of a B200
+
 // Chunk length of a context: a run of tiles of the kernel that serves its worker count -- as
 // many as amortise the per-chunk pointer look-up on a large problem (max_tiles_per_chunk), fewer
 // on a small one, so that it still spreads over about four blocks per SM of a B200.
+// Three to eight workers, whose averaging steps give a chunk to a block: a problem between two and
+// 8 * 8 rounds of blocks takes the run that fills its last round -- as few rounds of at most 8 tiles as
+// it needs, and the shortest run that does with these.  All-sync steps, Adam, bf16 gradients, against
+// the first rule: eight workers, 400 K parameters 16.2 us instead of 22.7, 700 K 27.3 (32.1), 2 M 72.3 (80.2), 5 M 164.8
+// (172.2); four workers, 1 M 19.5 (21.1), 2 M 36.2 (39.3).
 inline int64_t chunk_elems_for(int32_t M, const int64_t *numel, int32_t num_tensors) {
     const int64_t T = M <= MAX_MT ? plan_tile_elems(M) : GENERIC_CHUNK_ELEMS;
     const int64_t most = M <= MAX_MT ? max_tiles_per_chunk(M) : 8;
     int64_t tiles = 0;
     for (int32_t k = 0; k < num_tensors; ++k) tiles += (numel[k] + T - 1) / T;
-    int64_t per_chunk = tiles / (4 * 148);
+    int64_t per_chunk = tiles / (4 * NUM_SMS);
+    if (M > 2 && M <= MAX_MT) {
+        const int64_t slots = static_cast<int64_t>(NUM_SMS) * step_min_blocks(OPT_ADAM, M, true);
+        // chunks of t tiles, a tensor's last one half full on average
+        const auto chunks_with = [&](int64_t t) { return (tiles + num_tensors * (t - 1) / 2 + t - 1) / t; };
+        const int64_t rounds = (chunks_with(most) + slots - 1) / slots;
+        if (tiles > 2 * slots && rounds <= 8) {
+            per_chunk = 1;
+            while (per_chunk < most && chunks_with(per_chunk) > rounds * slots) ++per_chunk;
+        }
+    }
     if (per_chunk < 1) per_chunk = 1;
     if (per_chunk > most) per_chunk = most;
     return per_chunk * T;
@@ -131,6 +148,22 @@ inline int64_t count_chunks(const int64_t *numel, int32_t num_tensors, int64_t c
 inline int64_t parts_for(int64_t chunk_elems, int opt, int mt, bool bf16) {
     const int64_t most = most_part_elems(opt, mt, bf16);
     return (chunk_elems + most - 1) / most;
+}
+
+// The same where `items` chunks (times replicas, for mt = 1) make no more than four rounds of blocks: the split that
+// takes the fewest tile times, a round costing its tiles and 0.7 of one to fill and drain.  Measured, all-sync: sixteen
+// workers, 100 K parameters 11.7 us instead of 15.9, 1.5 M 107 (114); two workers, 200 K 3.5 (5.2), 2 M 18.9 (20.1).
+inline int64_t parts_for(int64_t items, int64_t chunk_elems, int opt, int mt, bool bf16) {
+    const int64_t least = parts_for(chunk_elems, opt, mt, bf16), tile = tile_elems(opt, mt, bf16);
+    const int64_t tiles = (chunk_elems + tile - 1) / tile;
+    const int64_t slots = static_cast<int64_t>(NUM_SMS) * step_min_blocks(opt, mt, bf16);
+    int64_t best = least, best_cost = INT64_MAX;
+    if (items * least > 4 * slots) return least;
+    for (int64_t p = least; p <= tiles; ++p) {
+        const int64_t cost = (items * p + slots - 1) / slots * (10 * ((tiles + p - 1) / p) + 7);
+        if (cost < best_cost) best = p, best_cost = cost;
+    }
+    return best;
 }
 
 // One thread block per part of a chunk and worker on a local step, one per chunk on the others: does
@@ -202,10 +235,9 @@ struct LaunchPlan {
 // Launches of at most this many blocks of single-tile chunks (two per SM of a B200: one wave)
 // skip the staging.  Measured on the 4096-parameter, two-worker workload: 3.08 us per step in a
 // CUDA graph of 16 steps against 3.34 us staged.
-constexpr long long DIRECT_GRID = 2 * 148;
-// One-replica kernel: a problem of at most seven blocks per SM takes one tile per block, straight
-// from global memory.
-constexpr long long LOCAL_WAVE = 7 * 148;
+constexpr long long DIRECT_GRID = 2 * NUM_SMS;
+// One-replica kernel: at most seven blocks of one tile per SM go straight to global memory.
+constexpr long long LOCAL_WAVE = 7 * NUM_SMS;
 
 // The tile kernels use more than the 48 KB of shared memory a kernel gets by default: raise the
 // function's limit to the most that any launch of it asks for (launches of other contexts, with
@@ -255,9 +287,7 @@ inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, long long n
         const int64_t tile = tile_elems(c.opt, mt, bf16), tiles = (chunk_elems + tile - 1) / tile;
         const int64_t replicas = local ? c.M : 1;
         // (the diagnostics write one partial sum per chunk: their blocks take whole chunks)
-        int64_t parts = diag ? 1 : parts_for(chunk_elems, c.opt, mt, bf16);
-        // a step that fits in one wave of blocks is pure latency: one tile per block
-        if (!diag && nchunks * tiles * replicas <= (local ? LOCAL_WAVE : DIRECT_GRID)) parts = tiles;
+        const int64_t parts = diag ? 1 : parts_for(nchunks * replicas, chunk_elems, c.opt, mt, bf16);
         p.parts = static_cast<int>(parts);
         p.part_elems = static_cast<int>((tiles + parts - 1) / parts * tile);
         p.threads = step_threads(c.opt, mt, bf16);

@@ -172,7 +172,7 @@ __device__ __forceinline__ double row_sum_f64(const float *row, long long n, dou
             acc += (static_cast<double>(v.x) + v.y) + (static_cast<double>(v.z) + v.w);
         }
     } else {
-#pragma unroll 8
+#pragma unroll 16
         for (long long i = threadIdx.x; i < n; i += threads) acc += static_cast<double>(row[i]);
     }
 #pragma unroll
@@ -247,36 +247,26 @@ mean_fill_kernel(const Chunk *chunks, long long nchunks, const float *const *src
 }
 
 // Norm diagnostics of a DIAG step.  partial[row * stride + c], row = kind * M + m, holds the sum of
-// squares of chunk c; tstart[k] .. tstart[k + 1] are the chunks of tensor k.  A warp per (row,
+// squares of chunk c; tstart[k] .. tstart[k + 1] are the chunks of tensor k.  A block per (row,
 // tensor): fp64 sum of the tensor's chunks, its root as the per-tensor norm.  The first `rows` blocks
 // take a whole row each: the norm over the tensor list.  One launch, and both results go
-// straight to the host's memory: the read-out after a 135 M-parameter step (272 tensors, 4 workers)
-// takes 30-55 us, the whole call, as two launches and two copies did; 5 M parameters 23-27 us instead of 39.
-constexpr int DIAG_WARPS = 8;
+// straight to the host's memory.  (A warp per row and tensor spent 20 us in a row on the 6912 chunks of an
+// embedding; three partial sums per chunk, for shorter blocks in the step, made the step no faster.)
+constexpr int DIAG_THREADS = 256;
 
-__global__ void __launch_bounds__(DIAG_WARPS * 32)
+__global__ void __launch_bounds__(DIAG_THREADS)
 diag_norms_kernel(const float *partial, long long stride, const long long *tstart, int nt, int rows, float *norms,
                   float *totals) {
-    __shared__ double sh[DIAG_WARPS];
+    __shared__ double sh[DIAG_THREADS / 32];
     begin_and_let_next_begin();
     wait_for_earlier_kernels();
-    if (blockIdx.x < rows) {
-        const double ss = row_sum_f64<false>(partial + blockIdx.x * stride, stride, sh);
-        if (threadIdx.x == 0) totals[blockIdx.x] = static_cast<float>(sqrt(ss));
-        return;
-    }
-    const long long item = static_cast<long long>(blockIdx.x - rows) * DIAG_WARPS + (threadIdx.x >> 5);
-    if (item >= static_cast<long long>(rows) * nt) return;
-    const long long row = item / nt;
+    const bool whole = blockIdx.x < rows;
+    const long long item = static_cast<long long>(blockIdx.x) - rows;
+    const long long row = whole ? blockIdx.x : item / nt;
     const int k = static_cast<int>(item - row * nt);
-    const float *src = partial + row * stride;
-    const long long c1 = tstart[k + 1];
-    double acc = 0.0;
-#pragma unroll 8
-    for (long long c = tstart[k] + (threadIdx.x & 31); c < c1; c += 32) acc += static_cast<double>(src[c]);
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
-    if ((threadIdx.x & 31) == 0) norms[item] = static_cast<float>(sqrt(acc));
+    const long long c0 = whole ? 0 : tstart[k], c1 = whole ? stride : tstart[k + 1];
+    const double ss = row_sum_f64<false>(partial + row * stride + c0, c1 - c0, sh);
+    if (threadIdx.x == 0) (whole ? totals + row : norms + item)[0] = static_cast<float>(sqrt(ss));
 }
 
 // All launches of this file may begin while the kernel in front of them still runs.
@@ -336,8 +326,8 @@ cudaError_t launch_rel_change(const Chunk *chunks, long long nchunks, const floa
 cudaError_t launch_diag_norms(const float *partial, long long stride, const long long *tstart,
                               int nt, int M, float *per_tensor, float *totals, cudaStream_t stream) {
     const int rows = DIAG_KINDS * M;
-    const long long blocks = rows + (static_cast<long long>(rows) * nt + DIAG_WARPS - 1) / DIAG_WARPS;
-    return launch(diag_norms_kernel, grid_for(blocks), DIAG_WARPS * 32, 0, stream, partial, stride, tstart, nt, rows,
+    const long long blocks = rows + static_cast<long long>(rows) * nt;
+    return launch(diag_norms_kernel, grid_for(blocks), DIAG_THREADS, 0, stream, partial, stride, tstart, nt, rows,
                   per_tensor, totals);
 }
 

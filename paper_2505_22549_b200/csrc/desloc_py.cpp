@@ -28,6 +28,7 @@ struct Entry {
     decltype(&desloc_step_normclip) step_normclip = nullptr;
     decltype(&desloc_step_diag) step_diag = nullptr;
     decltype(&desloc_rel_change) rel_change = nullptr;
+    decltype(&desloc_get_diag_norms) diag_norms = nullptr;
 } g_entry;
 
 struct Table {
@@ -221,6 +222,20 @@ PyObject *call_step_masked(PyObject *, PyObject *const *args, Py_ssize_t nargs) 
     return PyLong_FromLong(rc);
 }
 
+// A list of n floats.
+PyObject *float_list(const float *v, size_t n) {
+    PyObject *list = PyList_New(static_cast<Py_ssize_t>(n));
+    for (size_t i = 0; list && i < n; ++i) {
+        PyObject *f = PyFloat_FromDouble(v[i]);
+        if (!f) {
+            Py_CLEAR(list);
+            break;
+        }
+        PyList_SET_ITEM(list, static_cast<Py_ssize_t>(i), f);
+    }
+    return list;
+}
+
 // (context, array, pointer array, device, workers) -> list of floats, or a negative status
 PyObject *call_rel_change(PyObject *, PyObject *const *args, Py_ssize_t nargs) {
     void *ctx = nullptr, *ptrs = nullptr;
@@ -246,27 +261,68 @@ PyObject *call_rel_change(PyObject *, PyObject *const *args, Py_ssize_t nargs) {
         return nullptr;
     }
     if (rc != DESLOC_OK) return PyLong_FromLong(rc);
-    PyObject *list = PyList_New(static_cast<Py_ssize_t>(out.size()));
-    for (size_t m = 0; list && m < out.size(); ++m) {
-        PyObject *f = PyFloat_FromDouble(out[m]);
-        if (!f) {
-            Py_DECREF(list);
-            return nullptr;
-        }
-        PyList_SET_ITEM(list, static_cast<Py_ssize_t>(m), f);
-    }
-    return list;
+    return float_list(out.data(), out.size());
 }
 
-// bind(addresses of desloc_step, _step_masked, _step_normclip, _step_diag, _rel_change)
+// (context, workers, tensors, device) -> ([3][workers][tensors], [3][workers]) as nested lists, or a negative status
+PyObject *call_diag_norms(PyObject *, PyObject *const *args, Py_ssize_t nargs) {
+    void *ctx = nullptr;
+    int64_t workers = 0, tensors = 0, device = 0;
+    if (nargs != 4) {
+        PyErr_SetString(PyExc_TypeError, "diag_norms(ctx, workers, tensors, device)");
+        return nullptr;
+    }
+    if (!as_pointer(args[0], &ctx) || !as_int64(args[1], &workers) || !as_int64(args[2], &tensors) ||
+        !as_int64(args[3], &device))
+        return nullptr;
+    int rc = 0;
+    std::vector<float> per, tot;
+    try {
+        per.resize(static_cast<size_t>(3 * workers * tensors));
+        tot.resize(static_cast<size_t>(3 * workers));
+        void *stream = c10::cuda::getCurrentCUDAStream(static_cast<c10::DeviceIndex>(device)).stream();
+        Py_BEGIN_ALLOW_THREADS
+        rc = g_entry.diag_norms(static_cast<desloc_ctx *>(ctx), per.data(), tot.data(), stream);
+        Py_END_ALLOW_THREADS
+    } catch (const std::exception &e) {
+        PyErr_SetString(PyExc_RuntimeError, e.what());
+        return nullptr;
+    }
+    if (rc != DESLOC_OK) return PyLong_FromLong(rc);
+    PyObject *a = PyList_New(3), *b = PyList_New(3);
+    bool ok = a && b;
+    for (int k = 0; ok && k < 3; ++k) {
+        PyObject *rows = PyList_New(static_cast<Py_ssize_t>(workers)), *t = float_list(tot.data() + k * workers, workers);
+        ok = rows && t;
+        for (int64_t m = 0; ok && m < workers; ++m) {
+            PyObject *row = float_list(per.data() + (k * workers + m) * tensors, tensors);
+            ok = row != nullptr;
+            if (ok) PyList_SET_ITEM(rows, static_cast<Py_ssize_t>(m), row);
+        }
+        if (ok) {
+            PyList_SET_ITEM(a, k, rows);
+            PyList_SET_ITEM(b, k, t);
+        } else {
+            Py_XDECREF(rows);
+            Py_XDECREF(t);
+        }
+    }
+    PyObject *both = ok ? PyTuple_Pack(2, a, b) : nullptr;
+    Py_XDECREF(a);
+    Py_XDECREF(b);
+    return both;
+}
+
+// bind(addresses of desloc_step, _step_masked, _step_normclip, _step_diag, _rel_change, _get_diag_norms)
 PyObject *bind_entries(PyObject *, PyObject *args) {
-    unsigned long long a[5];
-    if (!PyArg_ParseTuple(args, "KKKKK", &a[0], &a[1], &a[2], &a[3], &a[4])) return nullptr;
+    unsigned long long a[6];
+    if (!PyArg_ParseTuple(args, "KKKKKK", &a[0], &a[1], &a[2], &a[3], &a[4], &a[5])) return nullptr;
     g_entry.step = reinterpret_cast<decltype(g_entry.step)>(a[0]);
     g_entry.step_masked = reinterpret_cast<decltype(g_entry.step_masked)>(a[1]);
     g_entry.step_normclip = reinterpret_cast<decltype(g_entry.step_normclip)>(a[2]);
     g_entry.step_diag = reinterpret_cast<decltype(g_entry.step_diag)>(a[3]);
     g_entry.rel_change = reinterpret_cast<decltype(g_entry.rel_change)>(a[4]);
+    g_entry.diag_norms = reinterpret_cast<decltype(g_entry.diag_norms)>(a[5]);
     Py_RETURN_NONE;
 }
 
@@ -278,6 +334,7 @@ PyCFunction fast(F f) {
 PyMethodDef methods[] = {{"bind", bind_entries, METH_VARARGS, nullptr},
                          {"step", fast(call_step), METH_FASTCALL, nullptr},
                          {"step_masked", fast(call_step_masked), METH_FASTCALL, nullptr},
+                         {"diag_norms", fast(call_diag_norms), METH_FASTCALL, nullptr},
                          {"rel_change", fast(call_rel_change), METH_FASTCALL, nullptr},
                          {nullptr, nullptr, 0, nullptr}};
 

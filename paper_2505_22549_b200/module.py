@@ -16,7 +16,7 @@ except ImportError as e:
 
 _entry = lambda f: ctypes.cast(f, ctypes.c_void_p).value
 _native.bind(*(_entry(getattr(B.raw_lib(), "desloc_" + n))
-               for n in ("step", "step_masked", "step_normclip", "step_diag", "rel_change")))
+               for n in ("step", "step_masked", "step_normclip", "step_diag", "rel_change", "get_diag_norms")))
 
 _GRAD_MISFIT = "gradient tensor of wrong dtype, size or layout"
 _SNAP_MISFIT = "snapshot tensor of wrong dtype, size or layout"
@@ -120,8 +120,10 @@ class DesLoc:
     def diag_norms(self):
         """(per_tensor [3][M][num_tensors], total [3][M]) of the latest step_diag; kind 0 =
         gradient as read, 1 = new parameters, 2 = update d_t.  Synchronises the current stream."""
-        stream = torch.cuda.current_stream(self.device).cuda_stream
-        return B.desloc_get_diag_norms(self.ctx, self.M, len(self.numel), stream)
+        r = _native.diag_norms(self.ctx, self.M, len(self.numel), self._index)
+        if isinstance(r, int):
+            self._raise(r, "desloc_get_diag_norms")
+        return r
 
     def grad_norms(self):
         """(norms, clip factors) of the latest step_normclip; synchronises the current stream."""

@@ -61,9 +61,7 @@ struct Slot {
     void **host = nullptr;
     void **dev = nullptr;
     cudaEvent_t done = nullptr;
-    bool in_flight = false;     // `done` has been recorded behind a kernel that reads the table
-    bool used_since = false;    // ... and other kernels on `stream` have read it since
-    cudaStream_t stream = nullptr;
+    bool in_flight = false;     // `done` has been recorded behind the first kernel that reads the table
 };
 
 // desloc_step_host: tensor groups whose copies and kernels are pipelined
@@ -209,7 +207,6 @@ struct desloc_ctx {
     int wait_limit = desloc::DEFAULT_WAIT_LIMIT;
     WorkerRes res;
     int next_slot = 0;
-    bool many_streams = false;   // steps have been called on more than one stream
     int cur_slot = -1;           // slot holding the table equal to last_grads
     std::vector<const void *> last_grads;
     cudaStream_t last_stream = nullptr;
@@ -255,20 +252,18 @@ int stage_grads(desloc_ctx *ctx, const void *const *grads, cudaStream_t stream, 
     }
     Slot &s = ctx->res.slots[ctx->next_slot];
     if (s.in_flight) {
-        // Re-use of a slot whose kernel was enqueued kSlots table changes ago: wait for it.
-        // (Kernels that read it without an event are in front of the copy below if they are on
-        // this stream; on another one -- the context has changed streams for the first time since --
-        // that stream may be gone by now, so wait for the device.)
-        cudaError_t e = s.used_since && s.stream != stream ? cudaDeviceSynchronize() : cudaEventSynchronize(s.done);
+        // Re-use of a slot whose table was staged kSlots table changes ago: wait until its copy has
+        // left the pinned buffer.  (Later kernels that read the same table need no event: every step of a
+        // context updates the same state, so whatever stream this one is on comes behind them, and the copy
+        // below with it.)
+        cudaError_t e = cudaEventSynchronize(s.done);
         if (e != cudaSuccess) return cuda_fail(ctx, e);
         s.in_flight = false;
-        s.used_since = false;
     }
     std::memcpy(s.host, grads, bytes);
     cudaError_t e = cudaMemcpyAsync(s.dev, s.host, bytes, cudaMemcpyHostToDevice, stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e);
     std::memcpy(ctx->last_grads.data(), grads, bytes);
-    if (ctx->cur_slot >= 0 && stream != ctx->last_stream) ctx->many_streams = true;
     ctx->cur_slot = ctx->next_slot;
     ctx->next_slot = (ctx->next_slot + 1) % kSlots;
     ctx->last_stream = stream;
@@ -434,19 +429,16 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
             break;
         }
         if (!capturing) {
-            // An event behind the first kernel that reads a table; a loop on one stream with the same
-            // gradient buffers needs no more (0.5 us of host time a step), see stage_grads().
+            // An event behind the first kernel that reads a table; a loop with the same gradient buffers
+            // needs no more (0.5 us of host time a step), see stage_grads().
             Slot &s = ctx->res.slots[ctx->cur_slot];
-            if (s.in_flight && !ctx->many_streams) {
-                s.used_since = true;
-            } else {
+            if (!s.in_flight) {
                 e = cudaEventRecord(s.done, stream);
                 if (e != cudaSuccess) {
                     rc = cuda_fail(ctx, e);
                     break;
                 }
                 s.in_flight = true;
-                s.stream = stream;
             }
         }
         if (diag) ctx->diag_valid = true;

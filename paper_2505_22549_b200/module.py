@@ -81,7 +81,7 @@ class DesLoc:
 
     def _grad_address(self, grads) -> int:
         """Address of the array of gradient pointers, good until the next call of this method."""
-        if type(grads) is BoundGrads:
+        if isinstance(grads, BoundGrads):
             return grads.address
         return self._fill(self._table, grads, self.grad_dtype, 0, _GRAD_MISFIT)
 

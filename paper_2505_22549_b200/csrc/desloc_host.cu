@@ -360,14 +360,13 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
         desloc::fill_hyper(a, c, lr_t, clip_bound_t);
         a.err = ctx->d_err;
         a.wait_limit = ctx->wait_limit;
-        a.parts = plan.parts;
-        a.part_elems = plan.part_elems;
-        a.direct = ctx->staging_mode < 0 ? (plan.direct ? 1 : 0) : ctx->staging_mode;
+        desloc::fill_plan(a, plan);
+        if (ctx->staging_mode >= 0) a.direct = ctx->staging_mode;
 
         void *params[] = {&a};
         const auto capped = [ctx](const desloc::LaunchPlan &lp) {
             const bool cap = lp.strides && ctx->max_blocks > 0 && lp.grid > ctx->max_blocks;
-            return static_cast<unsigned>(cap ? ctx->max_blocks : lp.grid);
+            return dim3(static_cast<unsigned>(cap ? ctx->max_blocks : lp.grid), lp.grid_y);
         };
         // (once per kernel: the attribute call costs a microsecond that a latency-bound step notices)
         if (std::find(ctx->prepared.begin(), ctx->prepared.end(), plan.fn) == ctx->prepared.end()) {
@@ -416,9 +415,8 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
                 a.nchunks = grp.c1 - grp.c0;
                 a.diag_chunk0 = grp.c0;
                 const desloc::LaunchPlan gp = desloc::plan_launch(c, mask, a.nchunks, ctx->res.chunk_elems, diag);
-                a.parts = gp.parts;
-                a.part_elems = gp.part_elems;
-                if (ctx->staging_mode < 0) a.direct = gp.direct ? 1 : 0;
+                desloc::fill_plan(a, gp);
+                if (ctx->staging_mode >= 0) a.direct = ctx->staging_mode;
                 // (no overlap: this kernel also depends on the other stream's copies)
                 e = desloc::launch_kernel(gp.fn, capped(gp), gp.threads, gp.smem, stream, params, false);
                 if (e == cudaSuccess) ctx->launches += 1;

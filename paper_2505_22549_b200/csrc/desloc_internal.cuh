@@ -217,13 +217,15 @@ inline void fill_hyper(StepArgs &a, const desloc_config &c, float lr_t, float cl
     a.err = nullptr;
     a.direct = 0;
     a.parts = 1;
+    a.parts_inv = 0;
     a.part_elems = 0;
 }
 
 // Which kernel a step of this configuration runs, and over how many blocks.
 struct LaunchPlan {
     const void *fn = nullptr;
-    long long grid = 0;
+    long long grid = 0;       // blocks in x
+    unsigned grid_y = 1;      // one-replica kernel: workers
     bool strides = true;  // a smaller grid may stride over the work items (not the runtime-M kernel)
     int smem = 0;         // dynamic shared memory of the launch
     int smem_limit = 0;   // of any launch of this kernel
@@ -251,10 +253,10 @@ inline cudaError_t prepare_launch(const LaunchPlan &p) {
 // (see begin_and_let_next_begin); also under capture, where it becomes an edge of the graph.  Measured
 // on B200: a graph window of 16 dependent steps on 4096 parameters 28.0 us instead of 43.0, a 5 M-parameter
 // step of four workers 82.0 us instead of 85.7, 135 M parameters 2044 us instead of 2050.
-inline cudaError_t launch_kernel(const void *fn, unsigned grid, unsigned threads, size_t smem, cudaStream_t stream,
+inline cudaError_t launch_kernel(const void *fn, dim3 grid, unsigned threads, size_t smem, cudaStream_t stream,
                                  void **params, bool overlap) {
     cudaLaunchConfig_t lc{};
-    lc.gridDim = dim3(grid);
+    lc.gridDim = grid;
     lc.blockDim = dim3(threads);
     lc.dynamicSmemBytes = smem;
     lc.stream = stream;
@@ -293,10 +295,19 @@ inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, long long n
         p.threads = step_threads(c.opt, mt, bf16);
         p.smem = step_smem_bytes(c.opt, mt, bf16, p.part_elems);
         p.smem_limit = step_smem_bytes(c.opt, mt, bf16, most_part_elems(c.opt, mt, bf16));
-        p.grid = nchunks * parts * replicas;
-        p.direct = p.grid <= (local ? LOCAL_WAVE : DIRECT_GRID) && p.part_elems <= (local || mt > MAX_MT ? tile : plan_tile_elems(mt));
+        p.grid = nchunks * parts;
+        if (local) p.grid_y = static_cast<unsigned>(c.M);
+        p.direct = p.grid * replicas <= (local ? LOCAL_WAVE : DIRECT_GRID) && p.part_elems <= (local || mt > MAX_MT ? tile : plan_tile_elems(mt));
     }
     return p;
+}
+
+// How a launch cuts its chunks, into the kernel arguments.
+inline void fill_plan(StepArgs &a, const LaunchPlan &p) {
+    a.parts = p.parts;
+    a.parts_inv = p.parts > 1 ? static_cast<unsigned>(((1ull << 32) + p.parts - 1) / p.parts) : 0;
+    a.part_elems = p.part_elems;
+    a.direct = p.direct ? 1 : 0;
 }
 
 }  // namespace desloc

@@ -122,6 +122,7 @@ struct StepArgs {
     int wait_limit;       // iterations a block polls for its tile before it gives up
     int direct;           // non-zero: no staging, every chunk straight from global memory (tiny launches)
     int parts;            // a chunk is this many work items (per replica, for the one-replica kernel) ...
+    unsigned parts_inv;   // ceil(2^32 / parts) for more than one part (see item_chunk)
     int part_elems;       // ... of this many elements (a multiple of the tile; the last ones may be empty)
     int nt;
     int M;
@@ -134,6 +135,12 @@ struct StepArgs {
     float rho;        // coordinate clip radius, +inf when off
     float cbound;     // ADOPT normalised-gradient bound, +inf when off
 };
+
+// item / parts by a multiplication (the division is twenty instructions of every thread): exact for
+// item < 2^32 / parts, far beyond what fits into memory.
+__device__ __forceinline__ unsigned item_chunk(const StepArgs &a, unsigned item) {
+    return a.parts == 1 ? item : __umulhi(item, a.parts_inv);
+}
 
 __device__ __forceinline__ const void *grad_ptr(const StepArgs &a, long long idx) {
     return a.g ? a.g[idx] : a.g_inline[idx];
@@ -638,6 +645,7 @@ desloc_step_kernel(const __grid_constant__ StepArgs a) {
     extern __shared__ __align__(128) char tile_mem[];   // S buffers of L::BYTES
     __shared__ char *sp[4][MT];
     __shared__ float sscale[MT];
+    __shared__ unsigned misfit;
     __shared__ __align__(8) uint64_t bar[S];
     ThreadNorms<DIAG, MT, THREADS> wn;
     const int tid = threadIdx.x;
@@ -657,20 +665,19 @@ desloc_step_kernel(const __grid_constant__ StepArgs a) {
     // workers at sustained clocks 0.4-0.7 % of the step).  The fallback paths keep the one form.
     const bool plain = a.gscale == nullptr && a.rho > 3.4028235e38f;   // rho = +inf: clip off
     // Work items: parts of a chunk, of all MT replicas or (MT = 1: a single worker, local steps) of
-    // one replica, worker by worker.  One item per block as launched (fewer than 2^31); a smaller
-    // grid strides over the rest.
-    const long long nitems = a.nchunks * a.parts * (MT == 1 ? a.M : 1);
+    // replica blockIdx.y.  One item per block as launched (fewer than 2^31); a smaller grid
+    // strides over the rest.
+    const int m0 = MT == 1 ? static_cast<int>(blockIdx.y) : 0;
+    const long long nitems = a.nchunks * a.parts;
     for (long long item = blockIdx.x; item < nitems; item += gridDim.x) {
-        const unsigned it = static_cast<unsigned>(item), nc = static_cast<unsigned>(a.nchunks);
-        const unsigned q = it / static_cast<unsigned>(a.parts);   // (worker, chunk)
-        const int part0 = static_cast<int>(it - q * a.parts) * a.part_elems;
-        const int m0 = MT == 1 ? static_cast<int>(q / nc) : 0;
-        const long long c = q - m0 * nc;
+        const unsigned c = item_chunk(a, static_cast<unsigned>(item));
+        const int part0 = static_cast<int>(static_cast<unsigned>(item) - c * a.parts) * a.part_elems;
         const Chunk ch = a.chunks[c];   // the same 16 bytes for every thread
         const int count = min(ch.count - part0, a.part_elems);
         const long long start = ch.start + part0;
         if (count <= 0) continue;   // a short chunk has fewer parts
-        __syncthreads();  // the previous item is done with the shared state; the barriers exist
+        // the previous item is done with the shared state
+        if (item != blockIdx.x) __syncthreads();
         char *p = nullptr;
         if (owner) {
             const long long idx = static_cast<long long>(m0 + m) * a.nt + ch.tensor;
@@ -683,13 +690,26 @@ desloc_step_kernel(const __grid_constant__ StepArgs a) {
             sp[arr][m] = p;
         }
         wn.clear();
-        // bulk copies need 16-byte aligned addresses; a tile of the chunk also a byte count that
-        // is a multiple of 16 (only the chunk's last tile can miss that: it is then updated
-        // straight from global memory, like every tile of a chunk whose pointers are unaligned)
-        const bool unaligned = __syncthreads_or((reinterpret_cast<uintptr_t>(p) & 15u) != 0) != 0;
-        // 128-bit accesses from global memory need less: 8 bytes for bf16 gradients
+        // Bulk copies need 16-byte aligned addresses (bit 0); 128-bit accesses from global memory less: 8
+        // bytes for bf16 gradients (bit 1).
         const uintptr_t need = (arr == 3 && sizeof(GT) == 2) ? 7u : 15u;
-        const bool wide_ok = __syncthreads_or((reinterpret_cast<uintptr_t>(p) & need) != 0) == 0;
+        unsigned off = ((reinterpret_cast<uintptr_t>(p) & 15u) != 0 ? 1u : 0u) |
+                       ((reinterpret_cast<uintptr_t>(p) & need) != 0 ? 2u : 0u);
+        if constexpr (4 * MT <= 32) {
+            // all owners are lanes of the first warp: one reduction there, one barrier for the block
+            if (tid < 32) {
+                off = __reduce_or_sync(0xffffffffu, off);
+                if (tid == 0) misfit = off;
+            }
+            __syncthreads();   // (the barriers exist, too)
+            off = misfit;
+        } else {
+            const int any1 = __syncthreads_or(off & 1u), any2 = __syncthreads_or(off & 2u);
+            off = (any1 ? 1u : 0u) | (any2 ? 2u : 0u);
+        }
+        // (a tile needs a byte count that is a multiple of 16, too: only a chunk's last tile can miss that, and
+        // is then updated straight from global memory, like every tile of a chunk whose pointers are unaligned)
+        const bool unaligned = (off & 1u) != 0, wide_ok = (off & 2u) == 0;
         const int ntiles = (count + T - 1) / T;
         // (a launch of a single wave of single-tile chunks has nothing to overlap: staging would
         // only add the copy engine's round trip to every step of a latency-bound problem)
@@ -710,14 +730,22 @@ desloc_step_kernel(const __grid_constant__ StepArgs a) {
 #pragma unroll
         for (int k = 0; k < S; ++k)
             if (k < staged) request(k);
-        // (behind the requests: its latency hides in theirs; a block barrier follows before it is used)
+        // (behind the requests: its latency hides in theirs)
         if (tid < MT) sscale[tid] = a.gscale ? a.gscale[m0 + tid] : 1.f;
-        if (staged == 0) __syncthreads();
+        if (!plain || staged < ntiles) __syncthreads();
 #pragma unroll 1
         for (int k = 0; k < staged; ++k) {
             const int st = k % S;
             const int cnt = min(T, count - k * T);
+            // Every thread waits for the tile itself and touches its own coordinates only, so one barrier
+            // per tile is enough: behind the updates, in front of the copies back.
             const bool landed = bar_wait(&bar[st], (phases >> st) & 1u, a.wait_limit);
+            const SmemAcc<OPT, MT, GT, T, VEC> acc{tile_mem + st * L::BYTES};
+            if (landed && tid * VEC < cnt) {
+                if (plain) update_position<OPT, MASK, MT, POST, DIAG, true>(a, acc, sscale, tid, wn);
+                else update_position<OPT, MASK, MT, POST, DIAG, false>(a, acc, sscale, tid, wn);
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // our writes, then the copy engine's reads
             if (__syncthreads_or(!landed)) {
                 // Give up on this step: say so, let the copies already requested land (bounded as
                 // well), store nothing more, leave.  The host reports the flag on its next call.
@@ -729,19 +757,12 @@ desloc_step_kernel(const __grid_constant__ StepArgs a) {
                 return;
             }
             phases ^= 1u << st;
-            const SmemAcc<OPT, MT, GT, T, VEC> acc{tile_mem + st * L::BYTES};
-            if (tid * VEC < cnt) {
-                if (plain) update_position<OPT, MASK, MT, POST, DIAG, true>(a, acc, sscale, tid, wn);
-                else update_position<OPT, MASK, MT, POST, DIAG, false>(a, acc, sscale, tid, wn);
-            }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // our writes, then the copy engine's reads
-            __syncthreads();
             if (owner && arr != 3) {
                 bulk_store(p + static_cast<long long>(k) * T * 4, tile_mem + st * L::BYTES + slot,
                            static_cast<uint32_t>(cnt * 4));
                 asm volatile("cp.async.bulk.commit_group;" ::: "memory");
             }
-            if (k + S < staged) {
+            if ((MT != 1 || DIAG) && k + S < staged) {   // (one replica: a buffer for every tile)
                 // the buffer is free once this thread's own copy back has read it
                 if (owner && arr != 3) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
                 request(k + S);

@@ -177,13 +177,11 @@ extern "C" DESLOC_API int desloc_step_static(const desloc_config *cfg, float *co
         a.gscale = nullptr;
         a.diag = nullptr;
         desloc::fill_hyper(a, *cfg, lr_t, clip_bound_t);
-        a.direct = plan.direct ? 1 : 0;
-        a.parts = plan.parts;
-        a.part_elems = plan.part_elems;
+        desloc::fill_plan(a, plan);
         void *params[] = {&a};
         e = desloc::prepare_launch(plan);
         if (e == cudaSuccess)
-            e = desloc::launch_kernel(plan.fn, static_cast<unsigned>(plan.grid), plan.threads, plan.smem, st, params, true);
+            e = desloc::launch_kernel(plan.fn, dim3(static_cast<unsigned>(plan.grid), plan.grid_y), plan.threads, plan.smem, st, params, true);
         if (e != cudaSuccess) { rc = DESLOC_E_CUDA; break; }
     } while (false);
     if (rc == DESLOC_E_CUDA) (void)cudaGetLastError();

@@ -215,21 +215,14 @@ __device__ __forceinline__ void generic_position(const StepArgs &a, char *const 
                     float gg = 0.f, dd = 0.f, xx = 0.f;
                     if (active) {
                         gg = sum_sq<VEC>(G[b]);
-                        const float sc = PLAIN ? 1.f : sscale[m0 + b];
-                        FV<VEC> D;
-#pragma unroll
-                        for (int c = 0; c < VEC; ++c) {
-                            const float up = SU ? ub.a[c] : U[b].a[c];
-                            const float vown = NEED_V ? V[b].a[c] : 0.f;
-                            const float vp = SV ? vb.a[c] : vown;
-                            const float xp = SX ? xb.a[c] : X[b].a[c];
-                            float un, vn;
-                            state_update<OPT, PLAIN>(a, PLAIN ? G[b].a[c] : G[b].a[c] * sc, up, vp, vown, un, vn);
-                            D.a[c] = direction<OPT>(a, un, vn);
-                            X[b].a[c] = apply_step(a, xp, D.a[c]);
-                            U[b].a[c] = un;
-                            V[b].a[c] = vn;
-                        }
+                        FV<VEC> vown{}, un, vn;
+                        if constexpr (NEED_V) vown = V[b];
+                        state_update<OPT, PLAIN, VEC, false>(a, G[b], PLAIN ? 1.f : sscale[m0 + b], SU ? ub : U[b],
+                                                      SV ? vb : vown, vown, un, vn);
+                        const FV<VEC> D = minus_direction<OPT, PLAIN, VEC, false>(a, un, vn);
+                        X[b] = apply_step<VEC, false>(a, SX ? xb : X[b], D);
+                        U[b] = un;
+                        V[b] = vn;
                         dd = sum_sq<VEC>(D);
                         xx = sum_sq<VEC>(X[b]);
                         st_f32<VEC>(sp[0][m0 + b], e, X[b]);
@@ -266,19 +259,14 @@ __device__ __forceinline__ void generic_position(const StepArgs &a, char *const 
                     float gg = 0.f, dd = 0.f, xx = 0.f;
                     if (active) {
                         gg = sum_sq<VEC>(G[b]);
-                        const float sc = PLAIN ? 1.f : sscale[m0 + b];
-                        FV<VEC> D;
-#pragma unroll
-                        for (int c = 0; c < VEC; ++c) {
-                            const float vown = OPT != OPT_SGDM ? V[b].a[c] : 0.f;
-                            float un, vn;
-                            state_update<OPT, PLAIN>(a, PLAIN ? G[b].a[c] : G[b].a[c] * sc, U[b].a[c], vown, vown, un, vn);
-                            U[b].a[c] = un;
-                            V[b].a[c] = vn;
-                            if constexpr (!P::D_NEEDS_MEAN) {
-                                D.a[c] = direction<OPT>(a, un, vn);
-                                X[b].a[c] = apply_step(a, X[b].a[c], D.a[c]);
-                            }
+                        FV<VEC> vown{}, un, vn, D;
+                        if constexpr (OPT != OPT_SGDM) vown = V[b];
+                        state_update<OPT, PLAIN, VEC, false>(a, G[b], PLAIN ? 1.f : sscale[m0 + b], U[b], vown, vown, un, vn);
+                        U[b] = un;
+                        V[b] = vn;
+                        if constexpr (!P::D_NEEDS_MEAN) {
+                            D = minus_direction<OPT, PLAIN, VEC, false>(a, un, vn);
+                            X[b] = apply_step<VEC, false>(a, X[b], D);
                         }
                         // a state that is not averaged has its final value now (phase B re-reads
                         // it where Adam needs it per worker)
@@ -325,14 +313,11 @@ __device__ __forceinline__ void generic_position(const StepArgs &a, char *const 
                     if (m0 + b < M) {
                         float dd = 0.f, xx = 0.f;
                         if (active) {
-                            FV<VEC> D;
-#pragma unroll
-                            for (int c = 0; c < VEC; ++c) {
-                                const float un = P::SU ? mu.a[c] : K[b].a[c];
-                                const float vn = P::SV ? mv.a[c] : (P::KEEP_V ? K[b].a[c] : 0.f);
-                                D.a[c] = direction<OPT>(a, un, vn);
-                                X[b].a[c] = apply_step(a, X[b].a[c], D.a[c]);
-                            }
+                            FV<VEC> vn{};
+                            if constexpr (P::SV) vn = mv;
+                            else if constexpr (P::KEEP_V) vn = K[b];
+                            const FV<VEC> D = minus_direction<OPT, PLAIN, VEC, false>(a, P::SU ? mu : K[b], vn);
+                            X[b] = apply_step<VEC, false>(a, X[b], D);
                             dd = sum_sq<VEC>(D);
                             if constexpr (!P::SX) {
                                 xx = sum_sq<VEC>(X[b]);
@@ -405,7 +390,7 @@ desloc_step_generic_kernel(const __grid_constant__ StepArgs a) {
             const int n4 = ch.count >> 2;
             // (no gradient factor and no coordinate clip, the common case: a copy of the loop
             // without them -- this kernel is bound by instruction issue)
-            if (a.gscale == nullptr && a.rho > 3.4028235e38f) {
+            if (plain_step(a)) {
                 for (int p = tid; DIAG ? (p - lane < n4) : (p < n4); p += BLOCK_THREADS)
                     generic_position<OPT, GT, POST, MASK, 4, DIAG, true>(a, sp, sscale, static_cast<long long>(p) * 4,
                                                                         p < n4, wd);

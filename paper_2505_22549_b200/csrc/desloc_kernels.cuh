@@ -136,6 +136,11 @@ struct StepArgs {
     float cbound;     // ADOPT normalised-gradient bound, +inf when off
 };
 
+// No factor on the gradient, coordinate clip off (rho = +inf), epsilon^2 a normal number.
+__device__ __forceinline__ bool plain_step(const StepArgs &a) {
+    return a.gscale == nullptr && a.rho > 3.4028235e38f && a.lam2 >= 1.17549435e-38f;
+}
+
 // item / parts by a multiplication (the division is twenty instructions of every thread): exact for
 // item < 2^32 / parts, far beyond what fits into memory.
 __device__ __forceinline__ unsigned item_chunk(const StepArgs &a, unsigned item) {
@@ -213,7 +218,74 @@ __device__ __forceinline__ float sum_sq(const FV<VEC> &r) {
     return s;
 }
 
-// ---- the arithmetic of one coordinate ------------------------------------------------------
+// ---- two coordinates at a time ------------------------------------------------------------------
+// sm_100 has two-wide fp32 add, multiply and fused multiply-add, each half rounded as the scalar
+// instruction rounds it: the same bits for half the instructions.  At the board's power cap that is speed: all-sync
+// steps of sixteen workers 0.977 -> 1.003 of copy, local steps 1.053 -> 1.056.  An odd count takes the scalar
+// forms, and so do (PACK = false) SGDM, whose averaging steps lost 0.3 % to the pairing, and the runtime-M
+// kernel, which has no registers for pairs of constants (up to 6 % slower with them).
+template <int VEC, bool PACK = true>
+__device__ __forceinline__ FV<VEC> vfma(const FV<VEC> &x, const FV<VEC> &y, const FV<VEC> &z) {
+    FV<VEC> r;
+    if constexpr (PACK && VEC % 2 == 0) {
+#pragma unroll
+        for (int c = 0; c < VEC; c += 2) {
+            const float2 t = __ffma2_rn(make_float2(x.a[c], x.a[c + 1]), make_float2(y.a[c], y.a[c + 1]),
+                                        make_float2(z.a[c], z.a[c + 1]));
+            r.a[c] = t.x; r.a[c + 1] = t.y;
+        }
+    } else {
+#pragma unroll
+        for (int c = 0; c < VEC; ++c) r.a[c] = __fmaf_rn(x.a[c], y.a[c], z.a[c]);
+    }
+    return r;
+}
+template <int VEC, bool PACK = true>
+__device__ __forceinline__ FV<VEC> vmul(const FV<VEC> &x, const FV<VEC> &y) {
+    FV<VEC> r;
+    if constexpr (PACK && VEC % 2 == 0) {
+#pragma unroll
+        for (int c = 0; c < VEC; c += 2) {
+            const float2 t = __fmul2_rn(make_float2(x.a[c], x.a[c + 1]), make_float2(y.a[c], y.a[c + 1]));
+            r.a[c] = t.x; r.a[c + 1] = t.y;
+        }
+    } else {
+#pragma unroll
+        for (int c = 0; c < VEC; ++c) r.a[c] = __fmul_rn(x.a[c], y.a[c]);
+    }
+    return r;
+}
+template <int VEC, bool PACK = true>
+__device__ __forceinline__ FV<VEC> vadd(const FV<VEC> &x, const FV<VEC> &y) {
+    FV<VEC> r;
+    if constexpr (PACK && VEC % 2 == 0) {
+#pragma unroll
+        for (int c = 0; c < VEC; c += 2) {
+            const float2 t = __fadd2_rn(make_float2(x.a[c], x.a[c + 1]), make_float2(y.a[c], y.a[c + 1]));
+            r.a[c] = t.x; r.a[c + 1] = t.y;
+        }
+    } else {
+#pragma unroll
+        for (int c = 0; c < VEC; ++c) r.a[c] = __fadd_rn(x.a[c], y.a[c]);
+    }
+    return r;
+}
+template <int VEC>
+__device__ __forceinline__ FV<VEC> splat(float v) {
+    FV<VEC> r;
+#pragma unroll
+    for (int c = 0; c < VEC; ++c) r.a[c] = v;
+    return r;
+}
+template <int VEC>
+__device__ __forceinline__ FV<VEC> clamp(const FV<VEC> &x, float bound) {
+    FV<VEC> r;
+#pragma unroll
+    for (int c = 0; c < VEC; ++c) r.a[c] = fminf(fmaxf(x.a[c], -bound), bound);
+    return r;
+}
+
+// ---- the arithmetic of a thread's coordinates ------------------------------------------------------
 // Worker sum as a fixed binary tree: the first 2^k workers (2^k the largest power of two
 // below the count) against the rest, recursively -- ((s0+s1)+(s2+s3))+((s4+s5)+(s6+s7)) for
 // eight.  Deterministic, and exact when all M values are equal and M is a power of two.
@@ -268,9 +340,6 @@ __device__ __forceinline__ float mean_of(const float (&s)[MT]) {
     }
 }
 
-// One worker's state update from the clipped gradient: `up`, `vp` are the previous states the
-// update starts from (the worker's own or the worker mean); `vown` is always the worker's own
-// previous v, which ADOPT's normaliser uses (Algorithm 3).
 // 1 / sqrt(a) to within an ulp: the hardware approximation (2 ulp) with one Newton step.  This
 // replaces IEEE sqrt followed by IEEE division (two roundings, about 20 instructions): with the
 // tiles staged by the copy engine the arithmetic sits on each block's critical path, and the
@@ -282,37 +351,59 @@ __device__ __forceinline__ float rsqrt_1ulp(float a) {
     return a > 0.f && a < 3.0e38f ? r : y;   // keep the limits (1/0 = inf, 1/inf = 0) free of NaN
 }
 
-template <int OPT, bool PLAIN = false>
-__device__ __forceinline__ void state_update(const StepArgs &a, float g, float up, float vp,
-                                             float vown, float &un, float &vn) {
-    // coordinate-wise clip: sgn(g) min(|g|, rho)  (Section 3.1); rho = +inf when off
-    const float gh = PLAIN ? g : fminf(fmaxf(g, -a.rho), a.rho);
-    if constexpr (OPT == OPT_ADAM) {
-        un = fmaf(a.b1, up, a.omb1 * gh);
-        vn = fmaf(a.b2, vp, (a.omb2 * gh) * gh);
-    } else if constexpr (OPT == OPT_ADOPT) {
-        vn = fmaf(a.b2, vp, (a.omb2 * gh) * gh);
-        float r = gh * rsqrt_1ulp(fmaxf(vown, a.eps2));  // g / max(sqrt(v), eps)
-        r = fminf(fmaxf(r, -a.cbound), a.cbound);
-        un = fmaf(a.b1, up, a.omb1 * r);
+// The same of VEC values.  PLAIN: they are known to be normal numbers or above (the smallest is
+// epsilon squared), so the approximation needs no scaling around it.
+template <bool PLAIN, int VEC, bool P>
+__device__ __forceinline__ FV<VEC> rsqrt_1ulp(const FV<VEC> &a) {
+    FV<VEC> r;
+    if constexpr (PLAIN) {
+        FV<VEC> y;
+#pragma unroll
+        for (int c = 0; c < VEC; ++c) asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y.a[c]) : "f"(a.a[c]));
+        r = vmul<VEC, P>(y, vfma<VEC, P>(vmul<VEC, P>(vmul<VEC, P>(a, splat<VEC>(-0.5f)), y), y, splat<VEC>(1.5f)));
+#pragma unroll
+        for (int c = 0; c < VEC; ++c) r.a[c] = a.a[c] < 3.0e38f ? r.a[c] : y.a[c];
     } else {
-        un = fmaf(a.b1, up, a.omb1 * gh);
-        vn = 0.f;
+#pragma unroll
+        for (int c = 0; c < VEC; ++c) r.a[c] = rsqrt_1ulp(a.a[c]);
     }
+    return r;
 }
 
-// The update d_t of Algorithms 2-3 from the new states.
-template <int OPT>
-__device__ __forceinline__ float direction(const StepArgs &a, float un, float vn) {
-    if constexpr (OPT == OPT_ADAM)
-        return (a.lr * un) * rsqrt_1ulp(vn + a.lam2);
-    else
-        return a.lr * un;
+// One worker's state update from its gradient: `up`, `vp` are the previous states the update
+// starts from (the worker's own or the worker mean); `vown` is always the worker's own previous v, which
+// ADOPT's normaliser uses (Algorithm 3).  PLAIN: no factor `sc` on the gradient, no coordinate
+// clip, and an epsilon whose square is a normal number.
+template <int OPT, bool PLAIN, int VEC, bool P = OPT != OPT_SGDM>
+__device__ __forceinline__ void state_update(const StepArgs &a, const FV<VEC> &g, float sc, const FV<VEC> &up,
+                                             const FV<VEC> &vp, const FV<VEC> &vown, FV<VEC> &un, FV<VEC> &vn) {
+    // coordinate-wise clip: sgn(g) min(|g|, rho)  (Section 3.1); rho = +inf when off
+    FV<VEC> gh = g;
+    if constexpr (!PLAIN) gh = clamp<VEC>(vmul<VEC, P>(g, splat<VEC>(sc)), a.rho);
+    FV<VEC> r = gh;
+    if constexpr (OPT == OPT_ADOPT) {
+        FV<VEC> low;
+#pragma unroll
+        for (int c = 0; c < VEC; ++c) low.a[c] = fmaxf(vown.a[c], a.eps2);
+        r = clamp<VEC>(vmul<VEC, P>(gh, rsqrt_1ulp<PLAIN, VEC, P>(low)), a.cbound);   // g / max(sqrt(v), eps)
+    }
+    un = vfma<VEC, P>(splat<VEC>(a.b1), up, vmul<VEC, P>(splat<VEC>(a.omb1), r));
+    if constexpr (OPT == OPT_SGDM) vn = splat<VEC>(0.f);
+    else vn = vfma<VEC, P>(splat<VEC>(a.b2), vp, vmul<VEC, P>(vmul<VEC, P>(splat<VEC>(a.omb2), gh), gh));
+}
+
+// -d_t: the update of Algorithms 2-3 from the new states, its sign turned.
+template <int OPT, bool PLAIN, int VEC, bool P = OPT != OPT_SGDM>
+__device__ __forceinline__ FV<VEC> minus_direction(const StepArgs &a, const FV<VEC> &un, const FV<VEC> &vn) {
+    const FV<VEC> t = vmul<VEC, P>(splat<VEC>(-a.lr), un);
+    if constexpr (OPT == OPT_ADAM) return vmul<VEC, P>(t, rsqrt_1ulp<PLAIN, VEC, P>(vadd<VEC, P>(vn, splat<VEC>(a.lam2))));
+    else return t;
 }
 
 // x* (1 - eta wd) - d, written as x* - (eta wd x* + d): one rounding at x's scale
-__device__ __forceinline__ float apply_step(const StepArgs &a, float xp, float d) {
-    return xp - fmaf(a.lrwd, xp, d);
+template <int VEC, bool P = true>
+__device__ __forceinline__ FV<VEC> apply_step(const StepArgs &a, const FV<VEC> &xp, const FV<VEC> &minus_d) {
+    return vadd<VEC, P>(xp, vfma<VEC, P>(splat<VEC>(-a.lrwd), xp, minus_d));
 }
 
 // ---- helpers of the runtime-M kernel ---------------------------------------------------------
@@ -447,20 +538,34 @@ struct ThreadNorms {
     }
 };
 
-template <int VEC, int MT, typename Acc>
+template <int LO, int N, int VEC, int MT, bool P>
+__device__ __forceinline__ FV<VEC> tree_sum_v(const FV<VEC> (&s)[MT]) {
+    if constexpr (N == 1) {
+        return s[LO];
+    } else {
+        constexpr int H = (N > 4) ? 4 : (N > 2 ? 2 : 1);   // as tree_sum
+        return vadd<VEC, P>(tree_sum_v<LO, H, VEC, MT, P>(s), tree_sum_v<LO + H, N - H, VEC, MT, P>(s));
+    }
+}
+
+template <int VEC, int MT, bool P, typename Acc>
 __device__ __forceinline__ FV<VEC> mean_over_workers(const Acc &acc, int arr, int q) {
     FV<VEC> S[MT];
 #pragma unroll
     for (int m = 0; m < MT; ++m) S[m] = acc.ld(arr, m, q);
-    FV<VEC> r;
+    if constexpr (MT <= MAX_MT && (MT & (MT - 1)) == 0) {
+        return vmul<VEC, P>(tree_sum_v<0, MT, VEC, MT, P>(S), splat<VEC>(1.f / MT));
+    } else {
+        FV<VEC> r;
 #pragma unroll
-    for (int c = 0; c < VEC; ++c) {
-        float s[MT];
+        for (int c = 0; c < VEC; ++c) {
+            float s[MT];
 #pragma unroll
-        for (int m = 0; m < MT; ++m) s[m] = S[m].a[c];
-        r.a[c] = mean_of<MT>(s);
+            for (int m = 0; m < MT; ++m) s[m] = S[m].a[c];
+            r.a[c] = mean_of<MT>(s);
+        }
+        return r;
     }
-    return r;
 }
 
 // ---- one position (VEC coordinates) of all MT workers, in place --------------------------------
@@ -472,117 +577,71 @@ __device__ __forceinline__ FV<VEC> mean_over_workers(const Acc &acc, int arr, in
 template <int OPT, int MASK, int MT, bool POST, bool DIAG, bool PLAIN = false, typename Acc, typename Norms>
 __device__ __forceinline__ void update_position(const StepArgs &a, const Acc &acc, const float *sscale,
                                                 int q, Norms &wn) {
-    constexpr bool active = true;
     constexpr int VEC = Acc::VEC;
     constexpr bool SX = MASK & SYNC_X, SU = MASK & SYNC_U;
     constexpr bool SV = (MASK & SYNC_V) && OPT != OPT_SGDM;
     constexpr bool HAS_V = OPT != OPT_SGDM;
     if constexpr (!POST) {
         FV<VEC> xb{}, ub{}, vb{};
-        if (active) {
-            if constexpr (SX) xb = mean_over_workers<VEC, MT>(acc, 0, q);
-            if constexpr (SU) ub = mean_over_workers<VEC, MT>(acc, 1, q);
-            if constexpr (SV) vb = mean_over_workers<VEC, MT>(acc, 2, q);
-        }
+        if constexpr (SX) xb = mean_over_workers<VEC, MT, OPT != OPT_SGDM>(acc, 0, q);
+        if constexpr (SU) ub = mean_over_workers<VEC, MT, OPT != OPT_SGDM>(acc, 1, q);
+        if constexpr (SV) vb = mean_over_workers<VEC, MT, OPT != OPT_SGDM>(acc, 2, q);
         constexpr bool NEED_V = HAS_V && (!SV || OPT == OPT_ADOPT);   // ADOPT: its own old v
 #pragma unroll
         for (int m = 0; m < MT; ++m) {
-            float gg = 0.f, dd = 0.f, xx = 0.f;
-            if (active) {
-                const FV<VEC> G = acc.ldg(m, q);
-                FV<VEC> X{}, U{}, V{}, D;
-                if constexpr (!SX) X = acc.ld(0, m, q);
-                if constexpr (!SU) U = acc.ld(1, m, q);
-                if constexpr (NEED_V) V = acc.ld(2, m, q);
-                const float sc = PLAIN ? 1.f : sscale[m];
-#pragma unroll
-                for (int c = 0; c < VEC; ++c) {
-                    const float up = SU ? ub.a[c] : U.a[c];
-                    const float vown = NEED_V ? V.a[c] : 0.f;
-                    const float vp = SV ? vb.a[c] : vown;
-                    const float xp = SX ? xb.a[c] : X.a[c];
-                    float un, vn;
-                    state_update<OPT, PLAIN>(a, PLAIN ? G.a[c] : G.a[c] * sc, up, vp, vown, un, vn);
-                    D.a[c] = direction<OPT>(a, un, vn);
-                    X.a[c] = apply_step(a, xp, D.a[c]);
-                    U.a[c] = un;
-                    V.a[c] = vn;
-                }
-                acc.st(0, m, q, X);
-                acc.st(1, m, q, U);
-                if constexpr (HAS_V) acc.st(2, m, q, V);
-                if constexpr (DIAG) {
-                    gg = sum_sq<VEC>(G); dd = sum_sq<VEC>(D); xx = sum_sq<VEC>(X);
-                }
+            const FV<VEC> G = acc.ldg(m, q);
+            FV<VEC> X{}, U{}, V{}, un, vn;
+            if constexpr (!SX) X = acc.ld(0, m, q);
+            if constexpr (!SU) U = acc.ld(1, m, q);
+            if constexpr (NEED_V) V = acc.ld(2, m, q);
+            state_update<OPT, PLAIN, VEC>(a, G, PLAIN ? 1.f : sscale[m], SU ? ub : U, SV ? vb : V, V, un, vn);
+            const FV<VEC> D = minus_direction<OPT, PLAIN, VEC>(a, un, vn);
+            X = apply_step<VEC, OPT != OPT_SGDM>(a, SX ? xb : X, D);
+            acc.st(0, m, q, X);
+            acc.st(1, m, q, un);
+            if constexpr (HAS_V) acc.st(2, m, q, vn);
+            if constexpr (DIAG) {
+                wn.add(DIAG_G, m, sum_sq<VEC>(G));
+                wn.add(DIAG_D, m, sum_sq<VEC>(D));
+                wn.add(DIAG_X, m, sum_sq<VEC>(X));
             }
-            wn.add(DIAG_G, m, gg);
-            wn.add(DIAG_D, m, dd);
-            wn.add(DIAG_X, m, xx);
         }
     } else {
-        using P = PostPlan<OPT, MASK>;
         // states
 #pragma unroll
         for (int m = 0; m < MT; ++m) {
-            float gg = 0.f;
-            if (active) {
-                const FV<VEC> G = acc.ldg(m, q);
-                FV<VEC> U = acc.ld(1, m, q), V{};
-                if constexpr (HAS_V) V = acc.ld(2, m, q);
-                const float sc = PLAIN ? 1.f : sscale[m];
-#pragma unroll
-                for (int c = 0; c < VEC; ++c) {
-                    const float vown = HAS_V ? V.a[c] : 0.f;
-                    float un, vn;
-                    state_update<OPT, PLAIN>(a, PLAIN ? G.a[c] : G.a[c] * sc, U.a[c], vown, vown, un, vn);
-                    U.a[c] = un;
-                    V.a[c] = vn;
-                }
-                acc.st(1, m, q, U);
-                if constexpr (HAS_V) acc.st(2, m, q, V);
-                if constexpr (DIAG) gg = sum_sq<VEC>(G);
-            }
-            wn.add(DIAG_G, m, gg);
+            const FV<VEC> G = acc.ldg(m, q);
+            FV<VEC> U = acc.ld(1, m, q), V{}, un, vn;
+            if constexpr (HAS_V) V = acc.ld(2, m, q);
+            state_update<OPT, PLAIN, VEC>(a, G, PLAIN ? 1.f : sscale[m], U, V, V, un, vn);
+            acc.st(1, m, q, un);
+            if constexpr (HAS_V) acc.st(2, m, q, vn);
+            if constexpr (DIAG) wn.add(DIAG_G, m, sum_sq<VEC>(G));
         }
         FV<VEC> mu{}, mv{};
-        if (active) {
-            if constexpr (SU) mu = mean_over_workers<VEC, MT>(acc, 1, q);
-            if constexpr (SV) mv = mean_over_workers<VEC, MT>(acc, 2, q);
-        }
+        if constexpr (SU) mu = mean_over_workers<VEC, MT, OPT != OPT_SGDM>(acc, 1, q);
+        if constexpr (SV) mv = mean_over_workers<VEC, MT, OPT != OPT_SGDM>(acc, 2, q);
         // parameters
 #pragma unroll
         for (int m = 0; m < MT; ++m) {
-            float dd = 0.f, xx = 0.f;
-            if (active) {
-                FV<VEC> X = acc.ld(0, m, q), U = mu, V = mv, D;
-                if constexpr (!SU) U = acc.ld(1, m, q);
-                if constexpr (OPT == OPT_ADAM && !SV) V = acc.ld(2, m, q);
-#pragma unroll
-                for (int c = 0; c < VEC; ++c) {
-                    D.a[c] = direction<OPT>(a, U.a[c], V.a[c]);
-                    X.a[c] = apply_step(a, X.a[c], D.a[c]);
-                }
-                acc.st(0, m, q, X);
-                if constexpr (SU) acc.st(1, m, q, mu);
-                if constexpr (SV) acc.st(2, m, q, mv);
-                if constexpr (DIAG) {
-                    dd = sum_sq<VEC>(D);
-                    xx = sum_sq<VEC>(X);
-                }
-            }
-            wn.add(DIAG_D, m, dd);
-            if constexpr (!SX) wn.add(DIAG_X, m, xx);
+            FV<VEC> X = acc.ld(0, m, q), U = mu, V = mv;
+            if constexpr (!SU) U = acc.ld(1, m, q);
+            if constexpr (OPT == OPT_ADAM && !SV) V = acc.ld(2, m, q);
+            const FV<VEC> D = minus_direction<OPT, PLAIN, VEC>(a, U, V);
+            X = apply_step<VEC, OPT != OPT_SGDM>(a, X, D);
+            acc.st(0, m, q, X);
+            if constexpr (SU) acc.st(1, m, q, mu);
+            if constexpr (SV) acc.st(2, m, q, mv);
+            if constexpr (DIAG) wn.add(DIAG_D, m, sum_sq<VEC>(D));
+            if constexpr (DIAG && !SX) wn.add(DIAG_X, m, sum_sq<VEC>(X));
         }
         if constexpr (SX) {
-            float xx = 0.f;
-            if (active) {
-                const FV<VEC> mx = mean_over_workers<VEC, MT>(acc, 0, q);
+            const FV<VEC> mx = mean_over_workers<VEC, MT, OPT != OPT_SGDM>(acc, 0, q);
 #pragma unroll
-                for (int m = 0; m < MT; ++m) acc.st(0, m, q, mx);
-                if constexpr (DIAG) xx = sum_sq<VEC>(mx);
+            for (int m = 0; m < MT; ++m) {
+                acc.st(0, m, q, mx);
+                if constexpr (DIAG) wn.add(DIAG_X, m, sum_sq<VEC>(mx));
             }
-#pragma unroll
-            for (int m = 0; m < MT; ++m) wn.add(DIAG_X, m, xx);
         }
     }
 }
@@ -660,10 +719,10 @@ desloc_step_kernel(const __grid_constant__ StepArgs a) {
     const int esize = arr == 3 ? static_cast<int>(sizeof(GT)) : 4;
     const int slot = arr == 3 ? L::g_off(m) : L::f_off(arr, m);
     uint32_t phases = 0;  // bit s: parity of the phase barrier s completes next
-    // No factor on the gradient and no coordinate clip -- the common case -- takes a copy of the
-    // inner loop without them (three instructions of about forty per coordinate: with eight
-    // workers at sustained clocks 0.4-0.7 % of the step).  The fallback paths keep the one form.
-    const bool plain = a.gscale == nullptr && a.rho > 3.4028235e38f;   // rho = +inf: clip off
+    // No factor on the gradient, no coordinate clip and an epsilon whose square is a normal number -- the
+    // common case -- take a copy of the inner loop without the instructions for these.  The fallback paths
+    // keep the one form.
+    const bool plain = plain_step(a);
     // Work items: parts of a chunk, of all MT replicas or (MT = 1: a single worker, local steps) of
     // replica blockIdx.y.  One item per block as launched (fewer than 2^31); a smaller grid
     // strides over the rest.

@@ -29,9 +29,9 @@
 //   bulk copies, 512-element tiles, no pipeline, 6-8 blocks/SM         25.76 ms  1.055
 // ("copy" = the device-to-device copy bandwidth of the same GPU; these are single-tensor
 // experiments with the pointers in the kernel parameters).  In the library, with the tensor
-// list's pointer look-up on every block's path, the pipelined form is the robust one: a run
-// of 8 tiles per block through two buffers gives 26.1 ms (1.04) on the 218-tensor list,
-// local and sync steps alike.
+// list's pointer look-up on every block's path, tiles of all replicas need the pipelined form: a run
+// of 8 tiles per block through two buffers gives 26.1 ms (1.04) on the 218-tensor list.  Local
+// steps take one replica per block, three tiles in buffers of their own: 25.5 ms (1.06).
 //
 // DIAG instantiations also accumulate, from values already in registers, the squared L2 norms
 // of the gradient as read, of the update d_t and of the new parameters per (worker, chunk):

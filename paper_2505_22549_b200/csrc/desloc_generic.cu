@@ -390,7 +390,7 @@ desloc_step_generic_kernel(const __grid_constant__ StepArgs a) {
             const int n4 = ch.count >> 2;
             // (no gradient factor and no coordinate clip, the common case: a copy of the loop
             // without them -- this kernel is bound by instruction issue)
-            if (plain_step(a)) {
+            if (plain_step<OPT>(a)) {
                 for (int p = tid; DIAG ? (p - lane < n4) : (p < n4); p += BLOCK_THREADS)
                     generic_position<OPT, GT, POST, MASK, 4, DIAG, true>(a, sp, sscale, static_cast<long long>(p) * 4,
                                                                         p < n4, wd);

@@ -136,9 +136,10 @@ struct StepArgs {
     float cbound;     // ADOPT normalised-gradient bound, +inf when off
 };
 
-// No factor on the gradient, coordinate clip off (rho = +inf), epsilon^2 a normal number.
+// No factor on the gradient, coordinate clip off (rho = +inf), epsilon^2 (not SGDM's) a normal number.
+template <int OPT>
 __device__ __forceinline__ bool plain_step(const StepArgs &a) {
-    return a.gscale == nullptr && a.rho > 3.4028235e38f && a.lam2 >= 1.17549435e-38f;
+    return a.gscale == nullptr && a.rho > 3.4028235e38f && (OPT == OPT_SGDM || a.lam2 >= 1.17549435e-38f);
 }
 
 // item / parts by a multiplication (the division is twenty instructions of every thread): exact for
@@ -722,7 +723,7 @@ desloc_step_kernel(const __grid_constant__ StepArgs a) {
     // No factor on the gradient, no coordinate clip and an epsilon whose square is a normal number -- the
     // common case -- take a copy of the inner loop without the instructions for these.  The fallback paths
     // keep the one form.
-    const bool plain = plain_step(a);
+    const bool plain = plain_step<OPT>(a);
     // Work items: parts of a chunk, of all MT replicas or (MT = 1: a single worker, local steps) of
     // replica blockIdx.y.  One item per block as launched (fewer than 2^31); a smaller grid
     // strides over the rest.

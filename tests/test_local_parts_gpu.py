@@ -37,3 +37,14 @@ def test_averaging_steps_at_part_and_tile_edges(opt, gd, M, numel):
                     clip_rho=1.5, adopt_norm_clip=(opt == "adopt"), eps=1e-3, seed=M)
     top = 3 if opt == "sgdm" else 7
     check(run_both(w, 2, align=4, v_init=0.25, forced_masks=[top, 1]))
+
+
+@pytest.mark.parametrize("opt", ["adam", "adopt", "sgdm"])
+@pytest.mark.parametrize("M", [2, 4, 12])
+@pytest.mark.parametrize("eps", [0.0, 1e-22, 1.2e-19, 1e-8])
+def test_epsilon_whose_square_is_no_normal_number(opt, M, eps):
+    """The square of epsilon is zero, a denormal number, or just a normal one: the last two decide between two forms of
+    1/sqrt.  v starts at 0.25, so that epsilon 0 is defined."""
+    w = di.Workload("eps", opt, M, (700_000, 513), "bf16", "normal1", lr=1e-2, eps=eps, beta2=0.99, seed=M)
+    top = 3 if opt == "sgdm" else 7
+    check(run_both(w, 3, align=4, v_init=0.25, forced_masks=[0, top, 0]))

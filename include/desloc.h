@@ -187,7 +187,8 @@ DESLOC_API int desloc_step_normclip(desloc_ctx *ctx, int64_t t, float lr_t, floa
 /*
  * Gradient norms ||g^m||_2 and clip factors of the latest desloc_step_normclip() into the host
  * arrays norms_out[M], scales_out[M] (either may be NULL).  Copies on `stream` and waits for
- * it: this call synchronises.
+ * it: this call synchronises.  DESLOC_E_DEVICE_WAIT, like the two read-outs below, if a bounded wait
+ * on the device has run out: the sums are incomplete then, whatever the output holds.
  */
 DESLOC_API int desloc_get_grad_norms(desloc_ctx *ctx, float *norms_out, float *scales_out,
                                      void *stream);

@@ -230,6 +230,10 @@ int cuda_fail(desloc_ctx *ctx, cudaError_t e) {
     return DESLOC_E_CUDA;
 }
 
+// A block of an earlier kernel of this context gave up waiting for its copies: what it should have
+// updated or summed up is incomplete.
+bool wait_ran_out(const desloc_ctx *ctx) { return *static_cast<volatile int *>(ctx->h_err) != 0; }
+
 void free_ctx(desloc_ctx *ctx) {
     if (!ctx) return;
     free_worker_res(ctx->res);
@@ -285,8 +289,7 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
     if (rc != DESLOC_OK) return rc;
     for (int64_t i = 0; i < ctx->nptr; ++i)
         if (!grads[i]) return DESLOC_E_NULL;
-    // a block of an earlier step gave up waiting for its tile: that step is incomplete
-    if (*static_cast<volatile int *>(ctx->h_err) != 0) return DESLOC_E_DEVICE_WAIT;
+    if (wait_ran_out(ctx)) return DESLOC_E_DEVICE_WAIT;
 
     int dev_before = -1;
     cudaError_t e = cudaGetDevice(&dev_before);
@@ -614,12 +617,14 @@ int desloc_get_diag_norms(desloc_ctx *ctx, float *per_tensor_out, float *total_o
                                   ctx->res.d_out, ctx->res.d_out + per, st);
     if (e == cudaSuccess) ctx->launches += 1;
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e == cudaSuccess) {
+    const bool valid = e == cudaSuccess && !wait_ran_out(ctx);
+    if (valid) {
         if (per_tensor_out) std::memcpy(per_tensor_out, ctx->res.h_out, per * sizeof(float));
         if (total_out) std::memcpy(total_out, ctx->res.h_out + per, rows * sizeof(float));
     }
     if (dev_before != ctx->device) cudaSetDevice(dev_before);
-    return e == cudaSuccess ? DESLOC_OK : cuda_fail(ctx, e);
+    if (e != cudaSuccess) return cuda_fail(ctx, e);
+    return valid ? DESLOC_OK : DESLOC_E_DEVICE_WAIT;
 }
 
 int desloc_step_host(desloc_ctx *ctx, int64_t t, float lr_t, float clip_bound_t,
@@ -673,7 +678,8 @@ int desloc_get_grad_norms(desloc_ctx *ctx, float *norms_out, float *scales_out, 
         e = cudaMemcpyAsync(scales_out, ctx->res.d_norms + ctx->cfg.M, bytes, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (dev_before != ctx->device) cudaSetDevice(dev_before);
-    return e == cudaSuccess ? DESLOC_OK : cuda_fail(ctx, e);
+    if (e != cudaSuccess) return cuda_fail(ctx, e);
+    return wait_ran_out(ctx) ? DESLOC_E_DEVICE_WAIT : DESLOC_OK;
 }
 
 int desloc_rel_change(desloc_ctx *ctx, int32_t array, const float *const *then, float *out,
@@ -700,13 +706,11 @@ int desloc_rel_change(desloc_ctx *ctx, int32_t array, const float *const *then, 
             ctx->res.d_partial, ctx->res.d_out + at, ctx->d_err, ctx->wait_limit, st);
     if (e == cudaSuccess) ctx->launches += 2;
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e == cudaSuccess && *static_cast<volatile int *>(ctx->h_err) != 0) {
-        if (dev_before != ctx->device) cudaSetDevice(dev_before);
-        return DESLOC_E_DEVICE_WAIT;
-    }
-    if (e == cudaSuccess) std::memcpy(out, ctx->res.h_out + at, static_cast<size_t>(ctx->cfg.M) * sizeof(float));
+    const bool valid = e == cudaSuccess && !wait_ran_out(ctx);
+    if (valid) std::memcpy(out, ctx->res.h_out + at, static_cast<size_t>(ctx->cfg.M) * sizeof(float));
     if (dev_before != ctx->device) cudaSetDevice(dev_before);
-    return e == cudaSuccess ? DESLOC_OK : cuda_fail(ctx, e);
+    if (e != cudaSuccess) return cuda_fail(ctx, e);
+    return valid ? DESLOC_OK : DESLOC_E_DEVICE_WAIT;
 }
 
 int desloc_set_workers(desloc_ctx *ctx, int32_t M_new, int32_t first_new, float *const *x,

@@ -58,3 +58,30 @@ def test_a_wait_that_runs_out_is_reported_and_nothing_is_stored(name):
     assert np.array_equal(st.to_numpy(st.x), ref.to_numpy(ref.x))
     assert not np.array_equal(st.to_numpy(st.x), after[0])
     eng.close(); eng2.close()
+
+
+@pytest.mark.parametrize("gd", ["bf16", "f32"])
+def test_read_outs_after_a_wait_that_ran_out_say_so(gd):
+    """Norms whose partial sums were never written are no norms: every read-out reports the failure, and works again once
+    it is cleared."""
+    import paper_2505_22549_b200 as d
+    w = di.Workload("readouts", "adam", 2, (70_000, 4096, 33), gd, "normal1", lr=1e-2, K=(1, 1, 1), seed=2)
+    dev = torch.device("cuda:0")
+    for step, read in ((lambda e, t, g: e.step_normclip(t, 1e-3, g, 1.0), lambda e: e.grad_norms()),
+                       (lambda e, t, g: e.step_diag(t, 1e-3, g), lambda e: e.diag_norms()),
+                       (lambda e, t, g: e.step_diag(t, 1e-3, g, max_norm=1.0), lambda e: e.grad_norms())):
+        st = State(w, dev)
+        eng = make_engine(d, w, st)
+        st.fill_grads(0)
+        d.desloc_testing_set_staging(eng.ctx, 0)
+        step(eng, 0, st.views(st.g))
+        assert np.all(np.isfinite(np.concatenate([np.ravel(a) for a in read(eng)])))
+        d.desloc_testing_set_wait_limit(eng.ctx, 0)
+        step(eng, 1, st.views(st.g))
+        with pytest.raises(d.DeslocError) as e:
+            read(eng)
+        assert e.value.status == d.DESLOC_E_DEVICE_WAIT
+        d.desloc_testing_set_wait_limit(eng.ctx, -1)
+        step(eng, 2, st.views(st.g))
+        read(eng)
+        eng.close()

@@ -75,9 +75,14 @@ class DesLoc:
         """Check a set of gradient tensors once and return a handle every step method accepts in
         place of the nested lists: a loop that reuses its gradient buffers then pays no
         per-step marshalling.  The handle keeps the tensors alive."""
+        if isinstance(grads, BoundGrads):
+            return grads
         n = self.M * len(self.numel)
-        array = (ctypes.c_void_p * n).from_buffer_copy((ctypes.c_void_p * n).from_address(self._grad_address(grads)))
-        return BoundGrads(array, grads)
+        # (a table of its own: another thread may be inside a step, which reads the buffer of self._table with
+        # the interpreter's lock released)
+        table = _native.Table(self.numel, self.M)
+        address = self._fill(table, grads, self.grad_dtype, 0, _GRAD_MISFIT)
+        return BoundGrads((ctypes.c_void_p * n).from_buffer_copy((ctypes.c_void_p * n).from_address(address)), grads)
 
     def _grad_address(self, grads) -> int:
         """Address of the array of gradient pointers, good until the next call of this method."""

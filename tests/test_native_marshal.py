@@ -41,3 +41,19 @@ def test_misfits_are_refused(native, spoil):
         table.fill(lists, 0, 0, "misfit")
     assert table.fill(good(), 0, 0, "misfit")
     assert table.fill([[1, 2], [3, 4]], 0, 0, "misfit") is None      # not tensors: the caller says so
+
+
+def test_binding_gradients_leaves_the_table_of_a_running_step_alone():
+    """A step reads its pointers with the interpreter's lock released; a thread that binds the next gradients meanwhile must
+    not write into the same buffer."""
+    import paper_2505_22549_b200 as d
+    eng = d.DesLoc.__new__(d.DesLoc)                       # no context: marshalling only
+    eng.ctx, eng.M, eng.numel, eng.grad_dtype = None, 2, [4, 6], d.DESLOC_F32
+    eng._tables()
+    lists = lambda: [[torch.zeros(4), torch.zeros(6)] for _ in range(2)]
+    first, second = lists(), lists()
+    at = eng._grad_address(first)
+    bound = eng.bind_grads(second)
+    want = lambda nested: [t.data_ptr() for row in nested for t in row]
+    assert list((ctypes.c_void_p * 4).from_address(at)) == want(first)
+    assert list(bound.array) == want(second) and eng.bind_grads(bound) is bound

@@ -79,9 +79,14 @@ void table_dealloc(PyObject *o) {
     Py_TYPE(o)->tp_free(o);
 }
 
+bool as_pointer(PyObject *o, void **out) {
+    *out = o == Py_None ? nullptr : PyLong_AsVoidPtr(o);
+    return !(*out == nullptr && PyErr_Occurred());
+}
+
 // fill(nested, kind, where, message) -> address of the pointer array [workers * tensors], row m = worker m.
 // kind: 0 = fp32, 1 = bf16.  where: 0 = any device, 1 = host only.  A tensor that does not fit raises
-// ValueError(message).  Returns None, and checks nothing, if an element is no torch tensor.
+// ValueError(message).  Returns None at the first element that is no torch.Tensor: the caller marshals the lists then.
 PyObject *table_fill(PyObject *o, PyObject *const *args, Py_ssize_t nargs) {
     Table *self = reinterpret_cast<Table *>(o);
     if (nargs != 4) {
@@ -139,7 +144,21 @@ PyObject *table_fill(PyObject *o, PyObject *const *args, Py_ssize_t nargs) {
     return PyLong_FromVoidPtr(self->ptrs->data());
 }
 
+// set(addresses) -> address of the pointer array, which holds them now: for what fill() leaves to the caller.
+PyObject *table_set(PyObject *o, PyObject *list) {
+    Table *self = reinterpret_cast<Table *>(o);
+    PyObject *seq = PySequence_Fast(list, "addresses must be a sequence");
+    if (!seq) return nullptr;
+    const Py_ssize_t n = PySequence_Fast_GET_SIZE(seq);
+    bool ok = static_cast<size_t>(n) == self->ptrs->size();
+    if (!ok) PyErr_SetString(PyExc_ValueError, "need one address per worker and tensor");
+    for (Py_ssize_t i = 0; ok && i < n; ++i) ok = as_pointer(PySequence_Fast_GET_ITEM(seq, i), &(*self->ptrs)[i]);
+    Py_DECREF(seq);
+    return ok ? PyLong_FromVoidPtr(self->ptrs->data()) : nullptr;
+}
+
 PyMethodDef table_methods[] = {
+    {"set", table_set, METH_O, nullptr},
     {"fill", reinterpret_cast<PyCFunction>(reinterpret_cast<void *>(table_fill)), METH_FASTCALL, nullptr},
     {nullptr, nullptr, 0, nullptr}};
 
@@ -158,10 +177,6 @@ bool as_float(PyObject *o, float *out) {
     if (v == -1.0 && PyErr_Occurred()) return false;
     *out = static_cast<float>(v);
     return true;
-}
-bool as_pointer(PyObject *o, void **out) {
-    *out = o == Py_None ? nullptr : PyLong_AsVoidPtr(o);
-    return !(*out == nullptr && PyErr_Occurred());
 }
 
 // (context, t, lr, clip bound, max_norm, pointer array, device, which) -> sync mask, or a negative status.

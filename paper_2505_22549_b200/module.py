@@ -91,10 +91,22 @@ class DesLoc:
         return self._fill(self._table, grads, self.grad_dtype, 0, _GRAD_MISFIT)
 
     def _fill(self, table, nested, kind: int, where: int, misfit: str) -> int:
-        """Checks and marshals nested lists of tensors into the buffer of `table`; its address."""
+        """Checks and marshals nested lists of tensors into the buffer of `table`; its address.  Objects that are no
+        torch.Tensor but answer the same questions go one by one."""
+        if not isinstance(nested, (list, tuple)):
+            nested = [list(row) for row in nested]
         address = table.fill(nested, kind, where, misfit)
         if address is None:
-            raise ValueError(misfit + " (not a torch.Tensor)")
+            want = torch.bfloat16 if kind == B.DESLOC_BF16 else torch.float32
+            ptrs = []
+            for row in nested:
+                for t, n in zip(row, self.numel):
+                    if t.dtype != want or t.numel() != n or not t.is_contiguous() or (where == 1 and t.is_cuda):
+                        raise ValueError(misfit)
+                    ptrs.append(t.data_ptr())
+            if len(ptrs) != self.M * len(self.numel):
+                raise ValueError("need one gradient list per worker")
+            address = table.set(ptrs)
         return address
 
     def _raise(self, status: int, where: str):

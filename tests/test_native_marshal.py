@@ -57,3 +57,29 @@ def test_binding_gradients_leaves_the_table_of_a_running_step_alone():
     want = lambda nested: [t.data_ptr() for row in nested for t in row]
     assert list((ctypes.c_void_p * 4).from_address(at)) == want(first)
     assert list(bound.array) == want(second) and eng.bind_grads(bound) is bound
+
+
+class _Like:
+    """Answers what a step asks of a gradient, but is no torch.Tensor."""
+
+    def __init__(self, t):
+        self.t, self.dtype, self.is_cuda = t, t.dtype, t.is_cuda
+        self.numel, self.is_contiguous, self.data_ptr = t.numel, t.is_contiguous, t.data_ptr
+
+
+@pytest.mark.parametrize("where", [0, 1])
+def test_objects_like_tensors_are_taken(where):
+    import paper_2505_22549_b200 as d
+    eng = d.DesLoc.__new__(d.DesLoc)
+    eng.ctx, eng.M, eng.numel, eng.grad_dtype = None, 2, [4, 6], d.DESLOC_F32
+    eng._tables()
+    real = [[torch.zeros(4), torch.zeros(6)] for _ in range(2)]
+    like = [[real[0][0], _Like(real[0][1])], [_Like(t) for t in real[1]]]
+    want = [t.data_ptr() for row in real for t in row]
+    for nested in (like, tuple(like), (row for row in like)):
+        at = eng._fill(eng._table, nested, d.DESLOC_F32, where, "misfit")
+        assert list((ctypes.c_void_p * 4).from_address(at)) == want
+    for spoiled in ([like[0], [_Like(torch.zeros(5)), like[1][1]]], [like[0], [_Like(torch.zeros(4).bfloat16()), like[1][1]]],
+                    like[:1], [like[0], like[1][:1]]):
+        with pytest.raises(ValueError):
+            eng._fill(eng._table, spoiled, d.DESLOC_F32, where, "misfit")

@@ -61,7 +61,8 @@ def _build_native(force: bool) -> None:
     dirs = ce.include_paths() + [sysconfig.get_paths()["include"], os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include")]
     tmp, stamp = NATIVE + f".tmp{os.getpid()}", os.path.join(OBJ, "_native.stamp")
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
-           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}"]
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
+           f'-DDESLOC_TORCH_VERSION="{torch.__version__}"']
     cmd += [a for d in dirs for a in ("-isystem", d)] + [NATIVE_SRC, "-L", libs]
     cmd += ["-ltorch_python", "-ltorch_cpu", "-ltorch", "-lc10_cuda", "-lc10"]
     h = hashlib.sha256(" ".join(cmd + [torch.__version__, sys.version]).encode())

@@ -371,5 +371,10 @@ PyMODINIT_FUNC PyInit__native(void) {
         Py_DECREF(m);
         return nullptr;
     }
+    // This module reads torch's own objects, whose layout is that of one build: module.py compares.
+    if (PyModule_AddStringConstant(m, "torch_version", DESLOC_TORCH_VERSION) < 0) {
+        Py_DECREF(m);
+        return nullptr;
+    }
     return m;
 }

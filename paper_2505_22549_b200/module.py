@@ -13,6 +13,9 @@ try:
 except ImportError as e:
     raise ImportError(f"the native part of this module is missing ({e}): build it with "
                       "`python -m paper_2505_22549_b200.build`") from e
+if _native.torch_version != str(torch.__version__):
+    raise ImportError(f"the native part of this module was built for torch {_native.torch_version}, this is torch "
+                      f"{torch.__version__}: build it again with `python -m paper_2505_22549_b200.build`")
 
 _entry = lambda f: ctypes.cast(f, ctypes.c_void_p).value
 _native.bind(*(_entry(getattr(B.raw_lib(), "desloc_" + n))

@@ -83,3 +83,14 @@ def test_objects_like_tensors_are_taken(where):
                     like[:1], [like[0], like[1][:1]]):
         with pytest.raises(ValueError):
             eng._fill(eng._table, spoiled, d.DESLOC_F32, where, "misfit")
+
+
+def test_a_module_built_for_another_torch_is_refused():
+    """It reads torch's objects directly: another build's layout would be misread in silence."""
+    import os
+    import subprocess
+    import sys
+    code = "import torch; torch.__version__ = '0.0.1'\nimport paper_2505_22549_b200.module"
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True,
+                       cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
+    assert r.returncode != 0 and "was built for torch" in r.stderr and "paper_2505_22549_b200.build" in r.stderr

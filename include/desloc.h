@@ -154,7 +154,8 @@ DESLOC_API int desloc_step(desloc_ctx *ctx, int64_t t, float lr_t, float clip_bo
  *                are to overlap with compute), same indexing and dtype as for desloc_step().
  *   dev_grads  : host array of M*num_tensors DEVICE pointers to caller-owned staging buffers
  *                of the same sizes; they receive the copies and are what the kernels read.
- * The tensor list is cut into up to 8 groups, of falling size; each group's gradients are copied on a stream
+ * The tensor list is cut into up to 8 groups, of falling size (inside a tensor, where a large
+ * one would make a group too long); each group's gradients are copied on a stream
  * the context owns (tensors adjacent in both host and device memory go as one copy) and the
  * group's part of the step is launched on `stream` as soon as its copies have landed, so all
  * but the last group's compute hides behind the transfers.  The copies wait for work already

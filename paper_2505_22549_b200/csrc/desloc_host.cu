@@ -54,7 +54,7 @@ using desloc::validate_config;
 namespace {
 
 constexpr int kSlots = 8;  // staging slots for per-step gradient pointer tables
-constexpr int kHostGroups = 8;  // most groups that desloc_step_host is pipelined in, and
+constexpr size_t kHostGroups = 8;  // most groups that desloc_step_host is pipelined in, and
 constexpr int64_t kHostSplit = 1600000;   // the fewest parameters worth splitting again
 
 struct Slot {
@@ -64,10 +64,11 @@ struct Slot {
     bool in_flight = false;     // `done` has been recorded behind the first kernel that reads the table
 };
 
-// desloc_step_host: tensor groups whose copies and kernels are pipelined
+// desloc_step_host: groups whose copies and kernels are pipelined
 struct HostGroup {
-    int32_t k0, k1;   // tensors [k0, k1)
-    int64_t c0, c1;   // tiles   [c0, c1)
+    int64_t c0, c1;   // chunks [c0, c1)
+    int32_t k0, k1;   // of tensors k0 .. k1,
+    int64_t e0, e1;   // the first one from element e0 on, the last one up to element e1
 };
 
 // Everything that depends on the worker count M (re-made by desloc_set_workers): the pointer
@@ -112,6 +113,37 @@ void free_worker_res(WorkerRes &r) {
     r = WorkerRes();
 }
 
+// Groups of desloc_step_host(): three quarters of what is left, each time.  A group's kernel takes a ninth of
+// its copies' time, so it hides behind the next group's even at a quarter of the size, and the last group,
+// whose kernel nothing hides, is small.  A copy costs 6 us beside its bytes, one per worker and group at
+// best: below 1.6 M parameters that is more than the kernel.  A group ends with a tensor where that
+// makes it no longer than seven eighths of what is left, else inside one, at the end of a chunk: a list whose
+// last tensor is large would otherwise be one group, with nothing hidden.  (25 M parameters x 4 workers in 29
+// tensors: 3817 us with eight equal groups of whole tensors, 3774 us with three; the copies alone 3690.)
+void plan_host_groups(std::vector<HostGroup> &groups, const std::vector<desloc::Chunk> &chunks, const int64_t *numel,
+                      int64_t total) {
+    groups.clear();
+    int64_t left = total, acc = 0;
+    HostGroup g{0, 0, 0, 0, 0, 0};
+    for (size_t c = 0; c < chunks.size(); ++c) {
+        const desloc::Chunk &ch = chunks[c];
+        const int64_t end = ch.start + ch.count, rest = numel[ch.tensor] - end;
+        acc += ch.count;
+        const bool split = groups.size() + 1 < kHostGroups && (left > kHostSplit || (rest == 0 && groups.empty()));
+        const bool enough = 4 * acc >= 3 * left && (rest == 0 || 8 * (acc + rest) > 7 * left);
+        if (c + 1 < chunks.size() && !(split && enough)) continue;
+        g.c1 = static_cast<int64_t>(c) + 1;
+        g.k1 = ch.tensor;
+        g.e1 = end;
+        groups.push_back(g);
+        g.c0 = g.c1;
+        g.k0 = rest > 0 ? ch.tensor : ch.tensor + 1;
+        g.e0 = rest > 0 ? end : 0;
+        left -= acc;
+        acc = 0;
+    }
+}
+
 // Allocates and fills the M-dependent resources; the device must be current.  May throw
 // std::bad_alloc (host vectors).
 cudaError_t make_worker_res(WorkerRes &r, int M, const int64_t *numel, int num_tensors, int64_t total,
@@ -125,29 +157,9 @@ cudaError_t make_worker_res(WorkerRes &r, int M, const int64_t *numel, int num_t
     std::vector<desloc::Chunk> chunks(static_cast<size_t>(nchunks));
     desloc::fill_chunks(numel, num_tensors, chunk_elems, chunks.data(), heads.data());
     std::vector<long long> tstart(static_cast<size_t>(num_tensors) + 1, 0);
-    r.groups.clear();
-    {
-        // Tensor groups for desloc_step_host: three quarters of what is left, each time.  A group's kernel
-        // takes a ninth of its copies' time, so it hides behind the next group's even at a quarter of the size, and
-        // the last group, whose kernel nothing hides, is small.  A copy costs 6 us beside its bytes, one per
-        // worker and group at best: below 1.6 M parameters that is more than the kernel.  (25 M parameters x
-        // 4 workers: 3817 us with eight equal groups, 3774 us with three; the copies alone 3690.)
-        int64_t left = total, acc = 0, c0 = 0;
-        int32_t k0 = 0;
-        for (int32_t k = 0; k < num_tensors; ++k) {
-            tstart[k + 1] = tstart[k] + desloc::chunks_of(numel[k], chunk_elems, heads[k]);
-            acc += numel[k];
-            const int done_groups = static_cast<int>(r.groups.size());
-            const bool split = done_groups < kHostGroups - 1 && (done_groups == 0 || left > kHostSplit);
-            if (k == num_tensors - 1 || (split && 4 * acc >= 3 * left)) {
-                r.groups.push_back({k0, k + 1, c0, tstart[k + 1]});
-                k0 = k + 1;
-                c0 = tstart[k + 1];
-                left -= acc;
-                acc = 0;
-            }
-        }
-    }
+    for (int32_t k = 0; k < num_tensors; ++k)
+        tstart[k + 1] = tstart[k] + desloc::chunks_of(numel[k], chunk_elems, heads[k]);
+    plan_host_groups(r.groups, chunks, numel, total);
     r.nchunks = nchunks;
     r.chunk_elems = chunk_elems;
     cudaError_t e0 = cudaMalloc(&r.d_chunks, chunks.size() * sizeof(desloc::Chunk));
@@ -393,18 +405,20 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
                 for (int m = 0; m < c.M && e == cudaSuccess; ++m) {
                     // merge tensors that are adjacent on both sides into one copy
                     int32_t k = grp.k0;
-                    while (k < grp.k1 && e == cudaSuccess) {
+                    while (k <= grp.k1 && e == cudaSuccess) {
                         const int64_t i0 = static_cast<int64_t>(m) * c.num_tensors + k;
-                        const char *hp = static_cast<const char *>(host_grads[i0]);
-                        char *dp = static_cast<char *>(const_cast<void *>(grads[i0]));
-                        size_t bytes = static_cast<size_t>(ctx->numel[k]) * gsz;
+                        const size_t from = k == grp.k0 ? static_cast<size_t>(grp.e0) * gsz : 0;
+                        const auto to = [&](int32_t kk) { return static_cast<size_t>(kk == grp.k1 ? grp.e1 : ctx->numel[kk]) * gsz; };
+                        const char *hp = static_cast<const char *>(host_grads[i0]) + from;
+                        char *dp = static_cast<char *>(const_cast<void *>(grads[i0])) + from;
+                        size_t bytes = to(k) - from;
                         int32_t k2 = k + 1;
-                        while (k2 < grp.k1) {
+                        while (k2 <= grp.k1) {
                             const int64_t i2 = static_cast<int64_t>(m) * c.num_tensors + k2;
                             if (static_cast<const char *>(host_grads[i2]) != hp + bytes ||
                                 static_cast<const char *>(grads[i2]) != dp + bytes)
                                 break;
-                            bytes += static_cast<size_t>(ctx->numel[k2]) * gsz;
+                            bytes += to(k2);
                             ++k2;
                         }
                         e = cudaMemcpyAsync(dp, hp, bytes, cudaMemcpyHostToDevice, ctx->copy_stream);
@@ -559,7 +573,7 @@ int desloc_create(desloc_ctx **out, const desloc_config *cfg, float *const *x, f
     }
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_entry, cudaEventDisableTiming);
-    for (int i = 0; i < kHostGroups && e == cudaSuccess; ++i)
+    for (size_t i = 0; i < kHostGroups && e == cudaSuccess; ++i)
         e = cudaEventCreateWithFlags(&ctx->ev_group[i], cudaEventDisableTiming);
     if (e == cudaSuccess) {
         try {

@@ -22,14 +22,22 @@ def test_sizes_where_the_split_changes(M, opt, gd, tiles, extra):
     check(run_both(w, 2, align=4, v_init=0.25, forced_masks=[top, 0]))
 
 
-def test_host_gradients_in_groups_of_falling_size():
-    """Forty tensors of 0.3 M parameters: 9 M, 2.25 M of the 3 M left, and the rest; the groups together give the plain step."""
+@pytest.mark.parametrize("numel,launches,M", [
+    # three quarters of what is left each time, as long as that is more than 1.6 M
+    ((300_000 + 3,) * 40, 3, 3),                   # 9 M, 2.25 M of the 3 M left, and the rest
+    ((1_000_000,) * 3 + (7_000_001,), 3, 2),       # 7.5 M, 1.9 M and the rest: both cuts inside the last tensor
+    ((2_000_003, 2_999_999), 2, 3),                # 3.75 M and the rest
+    ((3_200_005,), 2, 2), ((1_500_000,), 1, 2),    # one tensor: 2.4 M and the rest, or too small to cut
+    ((2_400_000, 700_000, 70_000), 2, 12),         # ends with the first tensor
+])
+def test_host_gradients_in_groups_of_falling_size(numel, launches, M):
+    """The groups together give the plain step, and there are as many as the sizes ask for."""
     import numpy as np
     import torch
     import paper_2505_22549_b200 as d
     from _util import State, f32r
     from test_parity_gpu import make_engine
-    w = di.Workload("groups", "adam", 3, (300_000 + 3,) * 40, "bf16", "student_t3", lr=1e-2, K=(2, 3, 4), seed=1)
+    w = di.Workload("groups", "adam", M, numel, "bf16", "student_t3", lr=1e-2, K=(2, 3, 4), seed=1)
     dev = torch.device("cuda:0")
     a, b = State(w, dev), State(w, dev)
     ea, eb = make_engine(d, w, a), make_engine(d, w, b)
@@ -45,5 +53,5 @@ def test_host_gradients_in_groups_of_falling_size():
     torch.cuda.synchronize()
     for pa, pb in ((a.x, b.x), (a.u, b.u), (a.v, b.v)):
         assert np.array_equal(a.to_numpy(pa), b.to_numpy(pb))
-    assert eb.launches() == 4 * 3 and ea.launches() == 4
+    assert eb.launches() == 4 * launches and ea.launches() == 4
     ea.close(); eb.close()

@@ -38,6 +38,35 @@ __host__ __device__ constexpr int gen_batch(int per_worker, int budget) {
     return b < 2 ? 1 : (b < 4 ? 2 : 4);
 }
 
+template <int N>
+struct Count {
+    static constexpr int value = N;
+};
+
+// Calls batch(Count<N>, m0, n) for all M workers in order: n <= N workers from m0 on.  WHOLE: every n is its
+// batch's N (the last workers by halves), known to the compiler, else only the last n is less.  The kernels with
+// norms are faster the first way (their shuffles keep the loads of a batch together), the others the second.
+template <int B, bool WHOLE, typename F>
+__device__ __forceinline__ void for_batches(int M, const F &batch) {
+    if constexpr (WHOLE) {
+        int m0 = 0;
+#pragma unroll 1
+        for (; m0 + B <= M; m0 += B) batch(Count<B>{}, m0, B);
+        if constexpr (B > 2) {
+            if (m0 + 2 <= M) {
+                batch(Count<2>{}, m0, 2);
+                m0 += 2;
+            }
+        }
+        if constexpr (B > 1) {
+            if (m0 < M) batch(Count<1>{}, m0, 1);
+        }
+    } else {
+#pragma unroll 1
+        for (int m0 = 0; m0 < M; m0 += B) batch(Count<B>{}, m0, M - m0);
+    }
+}
+
 // Sum of N workers' values as a binary tree.
 template <int VEC, int N>
 __device__ __forceinline__ FV<VEC> sum_of(const FV<VEC> (&v)[N]) {
@@ -85,17 +114,17 @@ struct WorkerSum {
         }
         return r;
     }
-    // A batch of B consecutive workers (B a power of two) of which the first n exist.  A full
-    // batch is summed as a binary tree first (exact when its values are equal) and enters the
-    // running sum as one value; a partial batch enters value by value.
-    template <int B>
-    __device__ __forceinline__ void add_batch(const FV<VEC> (&v)[B], int n) {
-        static_assert((B & (B - 1)) == 0, "batches are powers of two");
-        if (n >= B) {
-            add(sum_of<VEC, B>(v));
+    // The first n of N consecutive workers, in batches of B (a power of two).  A full batch is summed as a binary tree
+    // first (exact when its values are equal) and enters the running sum as one value; a shorter one enters
+    // value by value.
+    template <int B, int N>
+    __device__ __forceinline__ void add_batch(const FV<VEC> (&v)[N], int n) {
+        static_assert((B & (B - 1)) == 0 && N <= B, "batches are powers of two");
+        if (N == B && n >= B) {
+            add(sum_of<VEC, N>(v));
         } else {
 #pragma unroll
-            for (int j = 0; j < B; ++j)
+            for (int j = 0; j < N; ++j)
                 if (j < n) add(v[j]);
         }
     }
@@ -108,52 +137,67 @@ struct WorkerSum {
 template <int VEC, bool SX, bool SU, bool SV>
 __device__ __forceinline__ void means_of_workers(char *const (*sp)[GEN_MAX_M], int M, long long e,
                                                  bool active, FV<VEC> &xb, FV<VEC> &ub, FV<VEC> &vb) {
-    constexpr int NS = (SX ? 1 : 0) + (SU ? 1 : 0) + (SV ? 1 : 0);
-    constexpr int NB = NS == 1 ? 4 : 2;
-    WorkerSum<VEC> ax, au, av;
-    ax.clear(); au.clear(); av.clear();
-    int m0 = 0;
+    if constexpr ((SX ? 1 : 0) + (SU ? 1 : 0) + (SV ? 1 : 0) == 1) {
+        // One array: the last batch in the same loop as the full ones.  (A loop of full batches and one of
+        // single workers behind it was up to 15 % slower at 100 M parameters x workers, all counts and types.)
+        constexpr int ARR = SX ? 0 : SU ? 1 : 2;
+        WorkerSum<VEC> sum;
+        sum.clear();
 #pragma unroll 1
-    for (; m0 + 4 <= M; m0 += 4) {
-        FV<VEC> px[4 / NB], pu[4 / NB], pv[4 / NB];   // sums of NB workers
+        for (int m0 = 0; m0 < M; m0 += 4) {
+            FV<VEC> v[4];
 #pragma unroll
-        for (int h = 0; h < 4 / NB; ++h) {
-            FV<VEC> bx[NB], bu[NB], bv[NB];
+            for (int j = 0; j < 4; ++j)
+                if (active && m0 + j < M) v[j] = ld_f32<VEC>(sp[ARR][m0 + j], e);
+            if (active) sum.template add_batch<4, 4>(v, M - m0);
+        }
+        (SX ? xb : SU ? ub : vb) = sum.mean(M);
+    } else {
+        WorkerSum<VEC> ax, au, av;
+        ax.clear(); au.clear(); av.clear();
+        int m0 = 0;
+#pragma unroll 1
+        for (; m0 + 4 <= M; m0 += 4) {
+            FV<VEC> px[2], pu[2], pv[2];   // sums of two workers
 #pragma unroll
-            for (int j = 0; j < NB; ++j) {
+            for (int h = 0; h < 2; ++h) {
+                FV<VEC> bx[2], bu[2], bv[2];
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    if (active) {
+                        if constexpr (SX) bx[j] = ld_f32<VEC>(sp[0][m0 + h * 2 + j], e);
+                        if constexpr (SU) bu[j] = ld_f32<VEC>(sp[1][m0 + h * 2 + j], e);
+                        if constexpr (SV) bv[j] = ld_f32<VEC>(sp[2][m0 + h * 2 + j], e);
+                    }
+                }
                 if (active) {
-                    if constexpr (SX) bx[j] = ld_f32<VEC>(sp[0][m0 + h * NB + j], e);
-                    if constexpr (SU) bu[j] = ld_f32<VEC>(sp[1][m0 + h * NB + j], e);
-                    if constexpr (SV) bv[j] = ld_f32<VEC>(sp[2][m0 + h * NB + j], e);
+                    if constexpr (SX) px[h] = sum_of<VEC, 2>(bx);
+                    if constexpr (SU) pu[h] = sum_of<VEC, 2>(bu);
+                    if constexpr (SV) pv[h] = sum_of<VEC, 2>(bv);
                 }
             }
             if (active) {
-                if constexpr (SX) px[h] = sum_of<VEC, NB>(bx);
-                if constexpr (SU) pu[h] = sum_of<VEC, NB>(bu);
-                if constexpr (SV) pv[h] = sum_of<VEC, NB>(bv);
+                if constexpr (SX) ax.add(sum_of<VEC, 2>(px));
+                if constexpr (SU) au.add(sum_of<VEC, 2>(pu));
+                if constexpr (SV) av.add(sum_of<VEC, 2>(pv));
             }
         }
-        if (active) {
-            if constexpr (SX) ax.add(sum_of<VEC, 4 / NB>(px));
-            if constexpr (SU) au.add(sum_of<VEC, 4 / NB>(pu));
-            if constexpr (SV) av.add(sum_of<VEC, 4 / NB>(pv));
-        }
-    }
 #pragma unroll 1
-    for (; m0 < M; ++m0) {
-        if (active) {
-            FV<VEC> bx, bu, bv;
-            if constexpr (SX) bx = ld_f32<VEC>(sp[0][m0], e);
-            if constexpr (SU) bu = ld_f32<VEC>(sp[1][m0], e);
-            if constexpr (SV) bv = ld_f32<VEC>(sp[2][m0], e);
-            if constexpr (SX) ax.add(bx);
-            if constexpr (SU) au.add(bu);
-            if constexpr (SV) av.add(bv);
+        for (; m0 < M; ++m0) {
+            if (active) {
+                FV<VEC> bx, bu, bv;
+                if constexpr (SX) bx = ld_f32<VEC>(sp[0][m0], e);
+                if constexpr (SU) bu = ld_f32<VEC>(sp[1][m0], e);
+                if constexpr (SV) bv = ld_f32<VEC>(sp[2][m0], e);
+                if constexpr (SX) ax.add(bx);
+                if constexpr (SU) au.add(bu);
+                if constexpr (SV) av.add(bv);
+            }
         }
+        if constexpr (SX) xb = ax.mean(M);
+        if constexpr (SU) ub = au.mean(M);
+        if constexpr (SV) vb = av.mean(M);
     }
-    if constexpr (SX) xb = ax.mean(M);
-    if constexpr (SU) ub = au.mean(M);
-    if constexpr (SV) vb = av.mean(M);
 }
 
 // Diagnostics with a runtime worker count: a warp reduces each (kind, worker) value at once
@@ -195,14 +239,14 @@ __device__ __forceinline__ void generic_position(const StepArgs &a, char *const 
         FV<VEC> xb{}, ub{}, vb{};
         means_of_workers<VEC, SX, SU, SV>(sp, M, e, active, xb, ub, vb);
         constexpr bool NEED_V = OPT != OPT_SGDM && (!SV || OPT == OPT_ADOPT);
-                constexpr int B0 = gen_batch(worker_regs<OPT, GT>(!SX, !SU, NEED_V), GEN_BUDGET);
+        constexpr int B0 = gen_batch(worker_regs<OPT, GT>(!SX, !SU, NEED_V), GEN_BUDGET);
         constexpr int B = (OPT == OPT_ADOPT && B0 > 2) ? 2 : B0;  // ADOPT's normaliser needs more registers
-#pragma unroll 1
-        for (int m0 = 0; m0 < M; m0 += B) {
-            FV<VEC> G[B], X[B], U[B], V[B];
+        for_batches<B, DIAG>(M, [&](auto count, int m0, int n) {
+            constexpr int N = decltype(count)::value;
+            FV<VEC> G[N], X[N], U[N], V[N];
 #pragma unroll
-            for (int b = 0; b < B; ++b) {
-                if (active && m0 + b < M) {
+            for (int b = 0; b < N; ++b) {
+                if (active && b < n) {
                     G[b] = ld_grad<VEC, GT>(sp[3][m0 + b], e);
                     if constexpr (!SX) X[b] = ld_f32<VEC>(sp[0][m0 + b], e);
                     if constexpr (!SU) U[b] = ld_f32<VEC>(sp[1][m0 + b], e);
@@ -210,8 +254,8 @@ __device__ __forceinline__ void generic_position(const StepArgs &a, char *const 
                 }
             }
 #pragma unroll
-            for (int b = 0; b < B; ++b) {
-                if (m0 + b < M) {
+            for (int b = 0; b < N; ++b) {
+                if (b < n) {
                     float gg = 0.f, dd = 0.f, xx = 0.f;
                     if (active) {
                         gg = sum_sq<VEC>(G[b]);
@@ -234,19 +278,19 @@ __device__ __forceinline__ void generic_position(const StepArgs &a, char *const 
                     wd.add(DIAG_X, m0 + b, xx);
                 }
             }
-        }
+        });
     } else {
         using P = PostPlan<OPT, MASK>;
         WorkerSum<VEC> au, av, ax;
         au.clear(); av.clear(); ax.clear();
         constexpr int BA = gen_batch(worker_regs<OPT, GT>(!P::D_NEEDS_MEAN, true, OPT != OPT_SGDM), GEN_BUDGET);
         // phase A: states (and x where d_t needs no mean)
-#pragma unroll 1
-        for (int m0 = 0; m0 < M; m0 += BA) {
-            FV<VEC> G[BA], U[BA], V[BA], X[BA];
+        for_batches<BA, DIAG>(M, [&](auto count, int m0, int n) {
+            constexpr int N = decltype(count)::value;
+            FV<VEC> G[N], U[N], V[N], X[N];
 #pragma unroll
-            for (int b = 0; b < BA; ++b) {
-                if (active && m0 + b < M) {
+            for (int b = 0; b < N; ++b) {
+                if (active && b < n) {
                     G[b] = ld_grad<VEC, GT>(sp[3][m0 + b], e);
                     U[b] = ld_f32<VEC>(sp[1][m0 + b], e);
                     if constexpr (OPT != OPT_SGDM) V[b] = ld_f32<VEC>(sp[2][m0 + b], e);
@@ -254,8 +298,8 @@ __device__ __forceinline__ void generic_position(const StepArgs &a, char *const 
                 }
             }
 #pragma unroll
-            for (int b = 0; b < BA; ++b) {
-                if (m0 + b < M) {
+            for (int b = 0; b < N; ++b) {
+                if (b < n) {
                     float gg = 0.f, dd = 0.f, xx = 0.f;
                     if (active) {
                         gg = sum_sq<VEC>(G[b]);
@@ -288,29 +332,29 @@ __device__ __forceinline__ void generic_position(const StepArgs &a, char *const 
                 }
             }
             if (active) {
-                if constexpr (P::SU) au.template add_batch<BA>(U, M - m0);
-                if constexpr (P::SV) av.template add_batch<BA>(V, M - m0);
-                if constexpr (P::SX && !P::D_NEEDS_MEAN) ax.template add_batch<BA>(X, M - m0);
+                if constexpr (P::SU) au.template add_batch<BA, N>(U, n);
+                if constexpr (P::SV) av.template add_batch<BA, N>(V, n);
+                if constexpr (P::SX && !P::D_NEEDS_MEAN) ax.template add_batch<BA, N>(X, n);
             }
-        }
+        });
         const FV<VEC> mu = au.mean(M), mv = av.mean(M);
         if constexpr (P::D_NEEDS_MEAN) {
             // phase B: parameter step with the averaged states
             constexpr int BB = gen_batch(4 + ((P::KEEP_U || P::KEEP_V) ? 4 : 0), GEN_BUDGET);
-#pragma unroll 1
-            for (int m0 = 0; m0 < M; m0 += BB) {
-                FV<VEC> X[BB], K[BB];
+            for_batches<BB, DIAG>(M, [&](auto count, int m0, int n) {
+                constexpr int N = decltype(count)::value;
+                FV<VEC> X[N], K[N];
 #pragma unroll
-                for (int b = 0; b < BB; ++b) {
-                    if (active && m0 + b < M) {
+                for (int b = 0; b < N; ++b) {
+                    if (active && b < n) {
                         X[b] = ld_f32<VEC>(sp[0][m0 + b], e);
                         if constexpr (P::KEEP_U) K[b] = ld_f32<VEC>(sp[1][m0 + b], e);
                         if constexpr (P::KEEP_V) K[b] = ld_f32<VEC>(sp[2][m0 + b], e);
                     }
                 }
 #pragma unroll
-                for (int b = 0; b < BB; ++b) {
-                    if (m0 + b < M) {
+                for (int b = 0; b < N; ++b) {
+                    if (b < n) {
                         float dd = 0.f, xx = 0.f;
                         if (active) {
                             FV<VEC> vn{};
@@ -331,9 +375,9 @@ __device__ __forceinline__ void generic_position(const StepArgs &a, char *const 
                     }
                 }
                 if constexpr (P::SX) {
-                    if (active) ax.template add_batch<BB>(X, M - m0);
+                    if (active) ax.template add_batch<BB, N>(X, n);
                 }
-            }
+            });
         }
         if constexpr (P::SX || (!P::D_NEEDS_MEAN && P::SV)) {
             const FV<VEC> mx = ax.mean(M);
@@ -362,8 +406,6 @@ desloc_step_generic_kernel(const __grid_constant__ StepArgs a) {
     // exactly one chunk per block (this kernel does not stride: with a chunk loop around the
     // same body the compiler needs spill slots)
     const long long c = blockIdx.x;
-    begin_and_let_next_begin();
-    wait_for_earlier_kernels();
     if (c < a.nchunks) {
         const Chunk ch = a.chunks[c];
         int mis = 0;

@@ -393,7 +393,7 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
             if (ctx->prepared.size() < ctx->prepared.capacity()) ctx->prepared.push_back(plan.fn);
         }
         if (!host_grads) {
-            e = desloc::launch_kernel(plan.fn, capped(plan), plan.threads, plan.smem, stream, params, true);
+            e = desloc::launch_kernel(plan.fn, capped(plan), plan.threads, plan.smem, stream, params, plan.overlap);
             if (e == cudaSuccess) ctx->launches += 1;
         } else {
             // The device gradient buffers may still be read by earlier work on `stream`.

@@ -232,6 +232,7 @@ struct LaunchPlan {
     int threads = BLOCK_THREADS;
     int parts = 1, part_elems = 0;   // blocks that share a chunk, and elements of it for each
     bool direct = false;  // too small to gain from staging: update straight from global memory
+    bool overlap = true;  // may begin while the kernel in front of it still runs (not the runtime-M kernel)
 };
 
 // Launches of at most this many blocks of single-tile chunks (two per SM of a B200: one wave)
@@ -252,7 +253,9 @@ inline cudaError_t prepare_launch(const LaunchPlan &p) {
 // Launches `fn`.  overlap: the kernel may begin while the one in front of it in the stream still runs
 // (see begin_and_let_next_begin); also under capture, where it becomes an edge of the graph.  Measured
 // on B200: a graph window of 16 dependent steps on 4096 parameters 28.0 us instead of 43.0, a 5 M-parameter
-// step of four workers 82.0 us instead of 85.7, 135 M parameters 2044 us instead of 2050.
+// step of four workers 82.0 us instead of 85.7, 135 M parameters 2044 us instead of 2050.  The runtime-M
+// kernel neither begins early nor lets others: its blocks are few and long, and those of the next step crowded
+// onto the SMs this one left free (24 workers x 125 K parameters, 123 blocks: 23.9 us instead of 14.4).
 inline cudaError_t launch_kernel(const void *fn, dim3 grid, unsigned threads, size_t smem, cudaStream_t stream,
                                  void **params, bool overlap) {
     cudaLaunchConfig_t lc{};
@@ -282,7 +285,7 @@ inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, long long n
     const bool generic = !local && c.M > MAX_MT && (c.M > MAX_TILE_MT || post || diag);
     p.fn = generic ? lookup_generic_kernel(c.opt, post, bf16, static_cast<int>(kmask), diag)
                    : lookup_step_kernel(c.opt, post, bf16, c.M, static_cast<int>(kmask), diag);
-    p.strides = !generic;
+    p.strides = p.overlap = !generic;
     const int mt = local ? 1 : c.M;
     p.grid = nchunks;
     if (!generic) {

@@ -36,7 +36,9 @@ def _check_norms(st, got_per, got_tot, arrays, what):
 @pytest.mark.parametrize("name,M", [("cfg2_adam_135m", 4), ("cfg3_adopt_360m", 8),
                                     ("cfg5_sgdm_desloc", 8), ("cfg4_adam_1p7b", 1),
                                     ("cfg5_adam_desloc", 5), ("cfg2_adam_135m", 12),
-                                    ("cfg3_adopt_360m", 11), ("cfg5_sgdm_desloc", 2)])
+                                    ("cfg3_adopt_360m", 11), ("cfg5_sgdm_desloc", 2),
+                                    # the last one to three workers of a batch of four, or of two
+                                    ("cfg5_sgdm_desloc", 19), ("cfg2_adam_135m", 18), ("cfg3_adopt_360m", 17)])
 @pytest.mark.parametrize("post", [False, True])
 @pytest.mark.parametrize("align,g_shift", [(4, None), (1, None), (8, 4)])
 def test_diag_step_norms_match_oracle_and_state_matches_plain_step(name, M, post, align, g_shift):

@@ -28,7 +28,6 @@ constexpr int GEN_MAX_M = 256;    // worker pointers staged per chunk (= the con
 // 0.85; fp64 worker sums 0.87 and IEEE sqrt / division instead of the hardware reciprocal
 // square root 0.87 (this kernel is bound by instruction issue: ~75 instructions per
 // worker-coordinate with those, ~45 without).
-constexpr int GEN_MIN_BLOCKS = 3;   // 80 registers per thread
 constexpr int GEN_BUDGET = 24;      // registers a batch of workers may hold in flight
 
 // Workers per batch of the update loops: what fits in `budget` registers -- 1, 2 or 4 (a power
@@ -395,7 +394,7 @@ __device__ __forceinline__ void generic_position(const StepArgs &a, char *const 
 }
 
 template <int OPT, typename GT, bool POST, int MASK, bool DIAG>
-__global__ void __launch_bounds__(BLOCK_THREADS, GEN_MIN_BLOCKS)
+__global__ void __launch_bounds__(BLOCK_THREADS, GENERIC_MIN_BLOCKS)
 desloc_step_generic_kernel(const __grid_constant__ StepArgs a) {
     __shared__ char *sp[4][GEN_MAX_M];
     __shared__ float sscale[GEN_MAX_M];

@@ -271,6 +271,22 @@ inline cudaError_t launch_kernel(const void *fn, dim3 grid, unsigned threads, si
     return cudaLaunchKernelExC(&lc, fn, params);
 }
 
+// Nine to sixteen workers, a problem of few single-tile chunks: the runtime-M kernel has three places for a chunk
+// per SM where the tiles have two, and needs a round of blocks less for some counts.  It is the faster one there,
+// measured over all counts of workers, optimizers and types with 350 to 420 chunks by 1.1 to 1.75 (nine workers, 350
+// chunks, u averaged: 11.9 us instead of 19.7), with 600 to 870 by 1.0 to 1.4, beyond, with one array
+// averaged, by 0.97 to 1.13; ADOPT with several arrays averaged and more than a round of blocks: 0.87 to 1.3, not taken.
+// For as many rounds it is the faster one where one array of three is averaged (with more than a chunk per SM, 1.0
+// to 1.47; from 13 workers on not in the second round, 0.87 to 1.05).
+inline bool generic_fills_rounds_better(const desloc_config &c, uint32_t mask, long long nchunks, int64_t chunk_elems) {
+    if (chunk_elems > GENERIC_CHUNK_ELEMS || nchunks <= NUM_SMS) return false;
+    const long long tile_slots = static_cast<long long>(NUM_SMS) * step_min_blocks(c.opt, c.M, c.grad_dtype == DESLOC_BF16);
+    const long long slots = static_cast<long long>(NUM_SMS) * GENERIC_MIN_BLOCKS, rounds = (nchunks + slots - 1) / slots;
+    const bool fewer = rounds < (nchunks + tile_slots - 1) / tile_slots;
+    if ((mask & (mask - 1)) == 0 && (fewer || (c.opt != DESLOC_SGDM && (rounds == 1 || c.M <= 12)))) return true;
+    return fewer && (rounds == 1 || (rounds == 2 && c.opt != DESLOC_ADOPT));
+}
+
 inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, long long nchunks, int64_t chunk_elems,
                               bool diag) {
     LaunchPlan p;
@@ -282,7 +298,8 @@ inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, long long n
     // More than eight workers: tiles of all replicas up to sixteen, the runtime-M kernel beyond, for the
     // post-average ordering and for the norm diagnostics.  All-sync steps of sixteen workers (Adam, bf16
     // gradients): 6.52 TB/s in tiles, 6.29 in the runtime-M kernel; nine workers 6.2 and 5.89.
-    const bool generic = !local && c.M > MAX_MT && (c.M > MAX_TILE_MT || post || diag);
+    const bool generic = !local && c.M > MAX_MT &&
+                         (c.M > MAX_TILE_MT || post || diag || generic_fills_rounds_better(c, kmask, nchunks, chunk_elems));
     p.fn = generic ? lookup_generic_kernel(c.opt, post, bf16, static_cast<int>(kmask), diag)
                    : lookup_step_kernel(c.opt, post, bf16, c.M, static_cast<int>(kmask), diag);
     p.strides = p.overlap = !generic;

@@ -50,6 +50,7 @@ constexpr int MAX_TILE_MT = 16;    // ... for the pre-average sync steps without
 constexpr int DIAG_G = 0, DIAG_X = 1, DIAG_D = 2, DIAG_KINDS = 3;
 constexpr int REDUCE_CHUNK_ELEMS = BLOCK_THREADS * 16;  // chunks of the reduction kernels (4096)
 constexpr int GENERIC_CHUNK_ELEMS = 1024;               // chunks of contexts with M > MAX_MT
+constexpr int GENERIC_MIN_BLOCKS = 3;                   // blocks per SM of the runtime-M kernel (80 registers)
 constexpr int DRAIN_WAIT_LIMIT = 1 << 22;               // bound on the wait for copies in flight
 
 // Elements per tile and worker for a kernel that holds mt replicas per tile: bulk copies of 2 KB per

@@ -29,3 +29,13 @@ def test_chunks_in_several_parts(M, opt, gd, align, max_blocks, g_shift):
     masks = [3 if opt == "sgdm" else 7, 2]
     check(run_both(_workload(opt, gd, M, numel), 2, align=align, forced_masks=masks, v_init=0.5, max_blocks=max_blocks,
                    g_shift=g_shift))
+
+
+@pytest.mark.parametrize("M,opt,gd", [(9, "adam", "bf16"), (16, "adopt", "f32"), (12, "sgdm", "bf16")])
+@pytest.mark.parametrize("chunks", [148, 149, 296, 297, 444, 445, 593, 888, 889, 1183])
+def test_sizes_where_the_runtime_kernel_takes_over(M, opt, gd, chunks):
+    """Single-tile chunks of 1024 elements: between one round of tiles (296 blocks) and one of the runtime-M kernel (444), and
+    so on for more rounds, the latter runs."""
+    w = _workload(opt, gd, M, (1024 * chunks - 5,))
+    masks = [3 if opt == "sgdm" else 7, 2]
+    check(run_both(w, 2, forced_masks=masks, v_init=0.5))

@@ -10,7 +10,6 @@
 #include <cstring>
 #include <limits>
 #include <new>
-#include <utility>
 #include <vector>
 
 #include "../../include/desloc_testing.h"
@@ -47,12 +46,6 @@ const void *lookup_step_kernel(int opt, bool post, bool bf16, int mt, int mask, 
     return nullptr;
 }
 
-const void *lookup_own_kernel(int opt, bool post, bool bf16, int mt, int mask) {
-    if (opt == OPT_ADAM) return lookup_adam_own(post, bf16, mt, mask);
-    if (opt == OPT_ADOPT) return lookup_adopt_own(post, bf16, mt, mask);
-    return opt == OPT_SGDM ? lookup_sgdm_own(post, bf16, mt, mask) : nullptr;
-}
-
 }  // namespace desloc
 
 using desloc::mask_at;
@@ -85,7 +78,6 @@ struct WorkerRes {
     int64_t nchunks = 0;
     int64_t chunk_elems = 0;             // longest chunk of the plan
     long long *d_tstart = nullptr;       // [num_tensors + 1] first tile of every tensor
-    std::vector<int64_t> heads;          // [num_tensors] elements of the short first chunk
     std::vector<HostGroup> groups;
     void **d_tables = nullptr;  // [3][nptr] x, u, v
     Slot slots[kSlots];
@@ -170,7 +162,6 @@ cudaError_t make_worker_res(WorkerRes &r, int M, const int64_t *numel, int num_t
     plan_host_groups(r.groups, chunks, numel, total);
     r.nchunks = nchunks;
     r.chunk_elems = chunk_elems;
-    r.heads.swap(heads);
     cudaError_t e0 = cudaMalloc(&r.d_chunks, chunks.size() * sizeof(desloc::Chunk));
     if (e0 == cudaSuccess)
         e0 = cudaMemcpy(r.d_chunks, chunks.data(), chunks.size() * sizeof(desloc::Chunk), cudaMemcpyHostToDevice);
@@ -230,7 +221,6 @@ struct desloc_ctx {
     int next_slot = 0;
     int cur_slot = -1;           // slot holding the table equal to last_grads
     std::vector<const void *> last_grads;
-    bool last_off = false;       // desloc::grads_off_layout() of them
     cudaStream_t last_stream = nullptr;
     int64_t counters[4] = {0, 0, 0, 0};
     int64_t launches = 0;
@@ -290,7 +280,6 @@ int stage_grads(desloc_ctx *ctx, const void *const *grads, cudaStream_t stream, 
     cudaError_t e = cudaMemcpyAsync(s.dev, s.host, bytes, cudaMemcpyHostToDevice, stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e);
     std::memcpy(ctx->last_grads.data(), grads, bytes);
-    ctx->last_off = desloc::grads_off_layout(ctx->cfg, ctx->total_elems, grads, ctx->res.heads.data());
     ctx->cur_slot = ctx->next_slot;
     ctx->next_slot = (ctx->next_slot + 1) % kSlots;
     ctx->last_stream = stream;
@@ -365,10 +354,7 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
             d_gscale = ctx->res.d_norms + c.M;
         }
 
-        const bool off_layout = inline_g ? desloc::grads_off_layout(c, ctx->total_elems, grads, ctx->res.heads.data())
-                                         : ctx->last_off;
-        const desloc::LaunchPlan plan =
-            desloc::plan_launch(c, mask, ctx->res.nchunks, ctx->res.chunk_elems, diag, off_layout);
+        const desloc::LaunchPlan plan = desloc::plan_launch(c, mask, ctx->res.nchunks, ctx->res.chunk_elems, diag);
         if (!plan.fn) {
             rc = DESLOC_E_INVALID;
             break;
@@ -445,7 +431,7 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
                 a.chunks = ctx->res.d_chunks + grp.c0;
                 a.nchunks = grp.c1 - grp.c0;
                 a.diag_chunk0 = grp.c0;
-                const desloc::LaunchPlan gp = desloc::plan_launch(c, mask, a.nchunks, ctx->res.chunk_elems, diag, off_layout);
+                const desloc::LaunchPlan gp = desloc::plan_launch(c, mask, a.nchunks, ctx->res.chunk_elems, diag);
                 desloc::fill_plan(a, gp);
                 if (ctx->staging_mode >= 0) a.direct = ctx->staging_mode;
                 // (no overlap: this kernel also depends on the other stream's copies)
@@ -787,7 +773,7 @@ int desloc_set_workers(desloc_ctx *ctx, int32_t M_new, int32_t first_new, float 
     int rc = DESLOC_OK;
     if (e == cudaSuccess) {
         free_worker_res(ctx->res);
-        ctx->res = std::move(fresh);
+        ctx->res = fresh;
         ctx->last_grads.assign(static_cast<size_t>(nptr_new), nullptr);  // capacity reserved above
         ctx->cfg.M = M_new;
         ctx->nptr = nptr_new;

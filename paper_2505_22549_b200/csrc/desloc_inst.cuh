@@ -45,23 +45,6 @@ const void *lookup_unit(bool bf16, int mt, int mask) {
     return lookup_sync<OPT, POST, DIAG>(bf16, mt, mask);
 }
 
-// The OWN kernels of an optimizer: MT = 1 (mask 0), 2 and 4, without norms.
-template <int OPT, bool POST, typename GT, int MT, int... I>
-const void *pick_own(int mask, std::integer_sequence<int, I...>) {
-    static const void *const tbl[] = {
-        reinterpret_cast<const void *>(&desloc_step_kernel<OPT, 1 + I, MT, GT, POST, false, true>)...};
-    return mask >= 1 && mask <= static_cast<int>(sizeof...(I)) ? tbl[mask - 1] : nullptr;
-}
-template <int OPT, typename GT>
-const void *lookup_own(bool post, int mt, int mask) {
-    if (mask == 0)   // (the same code for either ordering)
-        return mt == 1 ? reinterpret_cast<const void *>(&desloc_step_kernel<OPT, 0, 1, GT, false, false, true>) : nullptr;
-    using Seq = std::make_integer_sequence<int, OPT == OPT_SGDM ? 3 : 7>;
-    if (mt == 2) return post ? pick_own<OPT, true, GT, 2>(mask, Seq{}) : pick_own<OPT, false, GT, 2>(mask, Seq{});
-    if (mt == 4) return post ? pick_own<OPT, true, GT, 4>(mask, Seq{}) : pick_own<OPT, false, GT, 4>(mask, Seq{});
-    return nullptr;
-}
-
 #define DESLOC_DECLARE_UNIT(name) const void *lookup_##name(bool bf16, int mt, int mask)
 DESLOC_DECLARE_UNIT(adam_pre);
 DESLOC_DECLARE_UNIT(adam_m9);    // MT = 9..12, pre-average
@@ -82,8 +65,5 @@ DESLOC_DECLARE_UNIT(adopt_post_diag);
 DESLOC_DECLARE_UNIT(sgdm_pre_diag);
 DESLOC_DECLARE_UNIT(sgdm_post_diag);
 #undef DESLOC_DECLARE_UNIT
-const void *lookup_adam_own(bool post, bool bf16, int mt, int mask);
-const void *lookup_adopt_own(bool post, bool bf16, int mt, int mask);
-const void *lookup_sgdm_own(bool post, bool bf16, int mt, int mask);
 
 }  // namespace desloc

@@ -287,24 +287,8 @@ inline bool generic_fills_rounds_better(const desloc_config &c, uint32_t mask, l
     return fewer && (rounds == 1 || (rounds == 2 && c.opt != DESLOC_ADOPT));
 }
 
-// Do the gradients of at least a quarter of the parameters lie where the copy engine cannot take them, behind the short
-// first chunks of `heads` elements?  (grads: [M][num_tensors])
-inline bool grads_off_layout(const desloc_config &c, int64_t total, const void *const *grads, const int64_t *heads) {
-    const int64_t size = c.grad_dtype == DESLOC_BF16 ? 2 : 4;
-    int64_t off = 0;
-    for (int32_t k = 0; k < c.num_tensors; ++k) {
-        const uintptr_t head = static_cast<uintptr_t>(heads[k] * size);
-        uintptr_t bits = 0;
-        for (int32_t m = 0; m < c.M; ++m)
-            bits |= reinterpret_cast<uintptr_t>(grads[static_cast<int64_t>(m) * c.num_tensors + k]) + head;
-        if ((bits & 15u) != 0) off += c.numel[k];
-    }
-    return off >= (total + 3) / 4;
-}
-
-// off_layout: see grads_off_layout().
 inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, long long nchunks, int64_t chunk_elems,
-                              bool diag, bool off_layout) {
+                              bool diag) {
     LaunchPlan p;
     // The mean of one replica is the replica: M = 1 always runs the local kernel.
     const uint32_t kmask = (c.M == 1) ? 0u : mask;
@@ -314,31 +298,20 @@ inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, long long n
     // More than eight workers: tiles of all replicas up to sixteen, the runtime-M kernel beyond, for the
     // post-average ordering and for the norm diagnostics.  All-sync steps of sixteen workers (Adam, bf16
     // gradients): 6.52 TB/s in tiles, 6.29 in the runtime-M kernel; nine workers 6.2 and 5.89.
-    const int mt = local ? 1 : c.M;
-    const int64_t replicas = local ? c.M : 1;
-    // Gradients that the copy engine cannot take and more than four rounds of blocks of the tile kernel.  Sixteen
-    // workers, 60 M parameters in all, averaging: 270 us in the runtime-M kernel, which reads with 128-bit accesses,
-    // 404 in tiles, which then read two elements at a time.
-    const bool off_many = off_layout && mt <= MAX_TILE_MT &&
-                          nchunks * replicas * parts_for(chunk_elems, c.opt, mt, bf16) >
-                              4LL * NUM_SMS * step_min_blocks(c.opt, mt, bf16);
     const bool generic = !local && c.M > MAX_MT &&
-                         (c.M > MAX_TILE_MT || post || diag || off_many ||
-                          generic_fills_rounds_better(c, kmask, nchunks, chunk_elems));
+                         (c.M > MAX_TILE_MT || post || diag || generic_fills_rounds_better(c, kmask, nchunks, chunk_elems));
     p.fn = generic ? lookup_generic_kernel(c.opt, post, bf16, static_cast<int>(kmask), diag)
                    : lookup_step_kernel(c.opt, post, bf16, c.M, static_cast<int>(kmask), diag);
     p.strides = p.overlap = !generic;
+    const int mt = local ? 1 : c.M;
     p.grid = nchunks;
     if (!generic) {
         const int64_t tile = tile_elems(c.opt, mt, bf16), tiles = (chunk_elems + tile - 1) / tile;
+        const int64_t replicas = local ? c.M : 1;
         // (the diagnostics write one partial sum per chunk: their blocks take whole chunks)
         const int64_t parts = diag ? 1 : parts_for(nchunks * replicas, chunk_elems, c.opt, mt, bf16);
         p.parts = static_cast<int>(parts);
         p.part_elems = static_cast<int>((tiles + parts - 1) / parts * tile);
-        if (off_many && !diag) {
-            const void *const own = lookup_own_kernel(c.opt, post, bf16, mt, static_cast<int>(kmask));
-            if (own) p.fn = own;
-        }
         p.threads = step_threads(c.opt, mt, bf16);
         p.smem = step_smem_bytes(c.opt, mt, bf16, p.part_elems);
         p.smem_limit = step_smem_bytes(c.opt, mt, bf16, most_part_elems(c.opt, mt, bf16));

@@ -40,8 +40,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <type_traits>
-
 namespace desloc {
 
 constexpr int OPT_ADAM = 0, OPT_ADOPT = 1, OPT_SGDM = 2;
@@ -351,7 +349,7 @@ __device__ __forceinline__ float mean_of(const float (&s)[MT]) {
 // that of the exact pair (about one ulp of the quotient), not its bits.
 __device__ __forceinline__ float rsqrt_1ulp(float a) {
     const float y = rsqrtf(a);
-    const float r = y * fmaf(a * y, -0.5f * y, 1.5f);   // (halving y, not a: half of a denormal number may round)
+    const float r = y * fmaf(-0.5f * (a * y), y, 1.5f);   // (in this order: half of a denormal number may round, a * y is none)
     return a > 0.f && a < 3.0e38f ? r : y;   // keep the limits (1/0 = inf, 1/inf = 0) free of NaN
 }
 
@@ -364,7 +362,7 @@ __device__ __forceinline__ FV<VEC> rsqrt_1ulp(const FV<VEC> &a) {
         FV<VEC> y;
 #pragma unroll
         for (int c = 0; c < VEC; ++c) asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y.a[c]) : "f"(a.a[c]));
-        r = vmul<VEC, P>(y, vfma<VEC, P>(vmul<VEC, P>(a, y), vmul<VEC, P>(y, splat<VEC>(-0.5f)), splat<VEC>(1.5f)));
+        r = vmul<VEC, P>(y, vfma<VEC, P>(vmul<VEC, P>(vmul<VEC, P>(a, y), splat<VEC>(-0.5f)), y, splat<VEC>(1.5f)));
 #pragma unroll
         for (int c = 0; c < VEC; ++c) r.a[c] = a.a[c] < 3.0e38f ? r.a[c] : y.a[c];
     } else {
@@ -692,43 +690,11 @@ __host__ __device__ constexpr int step_min_blocks(int opt, int mt, bool bf16) {
     return room < 2 ? 2 : room > 4 ? 4 : room;
 }
 
-// OWN kernels, for gradients laid out so that the copy engine cannot take them while it can take the state (bf16 gradients
-// 8 bytes off the state's layout, any gradients in packed buckets): each thread copies those of its own
-// coordinates into the tile, in one access per worker or element by element.  Measured against the whole chunk straight
-// from global memory, local steps of 60 M parameters x workers: 207 us instead of 247 at 8 bytes off, 209 instead
-// of 315 at 2.  (Kernels of their own, for large problems: the code beside the plain tile loop cost problems of a few
-// rounds of blocks 5-8 %, at the same registers.)
-template <int MT, typename GT, int VEC>
-__device__ __forceinline__ void copy_own_grads(char *const (*sp)[MT], char *tile, int stride, long long tile_first, int q,
-                                               bool wide) {
-    using Raw = std::conditional_t<sizeof(GT) == 2, unsigned short, unsigned>;
-    using Wide = std::conditional_t<VEC * sizeof(GT) == 16, uint4, std::conditional_t<VEC * sizeof(GT) == 8, uint2, unsigned>>;
-    static_assert(VEC * sizeof(GT) == sizeof(Wide), "two or four gradients");
-    // (all loads in front of all stores: one latency for the tile)
-    union {
-        Wide w;
-        Raw r[VEC];
-    } v[MT];
-#pragma unroll
-    for (int m = 0; m < MT; ++m) {
-        const char *src = sp[3][m] + (tile_first + q * VEC) * static_cast<long long>(sizeof(GT));
-        if (wide) {
-            v[m].w = *reinterpret_cast<const Wide *>(src);
-        } else {
-#pragma unroll
-            for (int c = 0; c < VEC; ++c) v[m].r[c] = reinterpret_cast<const Raw *>(src)[c];
-        }
-    }
-#pragma unroll
-    for (int m = 0; m < MT; ++m)
-        *reinterpret_cast<Wide *>(tile + m * stride + q * VEC * static_cast<int>(sizeof(GT))) = v[m].w;
-}
-
 // A chunk is a run of consecutive tiles of one tensor.  The block looks its pointers up
 // once, then streams the tiles through a ring of S buffers: while tile k is updated in
 // place, tiles k + 1 .. k + S - 1 are already landing; when tile k's copy back has left its
 // buffer, tile k + S is requested into it.
-template <int OPT, int MASK, int MT, typename GT, bool POST, bool DIAG, bool OWN = false>
+template <int OPT, int MASK, int MT, typename GT, bool POST, bool DIAG>
 __global__ void __launch_bounds__(step_threads(OPT, MT, sizeof(GT) == 2), step_min_blocks(OPT, MT, sizeof(GT) == 2))
 desloc_step_kernel(const __grid_constant__ StepArgs a) {
     constexpr int THREADS = step_threads(OPT, MT, sizeof(GT) == 2);
@@ -790,11 +756,6 @@ desloc_step_kernel(const __grid_constant__ StepArgs a) {
         const uintptr_t need = (arr == 3 && sizeof(GT) == 2) ? 7u : 15u;
         unsigned off = ((reinterpret_cast<uintptr_t>(p) & 15u) != 0 ? 1u : 0u) |
                        ((reinterpret_cast<uintptr_t>(p) & need) != 0 ? 2u : 0u);
-        if constexpr (OWN) {
-            // bit 2: the state misses them; bit 3: the gradients of a thread in one access miss theirs
-            if (arr != 3) off |= (off & 1u) << 2;
-            else if ((reinterpret_cast<uintptr_t>(p) & (VEC * sizeof(GT) - 1)) != 0) off |= 8u;
-        }
         if constexpr (4 * MT <= 32) {
             // all owners are lanes of the first warp: one reduction there, one barrier for the block
             if (tid < 32) {
@@ -804,14 +765,12 @@ desloc_step_kernel(const __grid_constant__ StepArgs a) {
             __syncthreads();   // (the barriers exist, too)
             off = misfit;
         } else {
-            static_assert(!OWN, "these kernels have all owners in one warp");
             const int any1 = __syncthreads_or(off & 1u), any2 = __syncthreads_or(off & 2u);
             off = (any1 ? 1u : 0u) | (any2 ? 2u : 0u);
         }
         // (a tile needs a byte count that is a multiple of 16, too: only a chunk's last tile can miss that, and
         // is then updated straight from global memory, like every tile of a chunk whose pointers are unaligned)
-        const bool own_grads = OWN && (off & 5u) == 1u;
-        const bool unaligned = !own_grads && (off & 1u) != 0, wide_ok = (off & 2u) == 0;
+        const bool unaligned = (off & 1u) != 0, wide_ok = (off & 2u) == 0;
         const int ntiles = (count + T - 1) / T;
         // (a launch of a single wave of single-tile chunks has nothing to overlap: staging would
         // only add the copy engine's round trip to every step of a latency-bound problem)
@@ -819,13 +778,13 @@ desloc_step_kernel(const __grid_constant__ StepArgs a) {
         // request tile k (< staged) into its buffer: every owner its own slice, one arrival
         auto request = [&](int k) {
             const int cnt = min(T, count - k * T);
-            if (owner && !(own_grads && arr == 3))
+            if (owner)
                 bulk_load(tile_mem + (k % S) * L::BYTES + slot, p + static_cast<long long>(k) * T * esize,
                           static_cast<uint32_t>(cnt * esize), &bar[k % S]);
             if (tid == 0)
                 asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
                              :: "r"(smem_u32(&bar[k % S])),
-                                "r"(static_cast<uint32_t>(MT * cnt * ((own_grads ? 0 : static_cast<int>(sizeof(GT))) + 4 * L::NS)))
+                                "r"(static_cast<uint32_t>(MT * cnt * (static_cast<int>(sizeof(GT)) + 4 * L::NS)))
                              : "memory");
         };
         wait_for_earlier_kernels();
@@ -841,12 +800,6 @@ desloc_step_kernel(const __grid_constant__ StepArgs a) {
             const int cnt = min(T, count - k * T);
             // Every thread waits for the tile itself and touches its own coordinates only, so one barrier
             // per tile is enough: behind the updates, in front of the copies back.
-            if constexpr (OWN) {
-                // (in front of the wait: the tile's copies hide the latency)
-                if (own_grads && tid * VEC < cnt)
-                    copy_own_grads<MT, GT, VEC>(sp, tile_mem + st * L::BYTES, L::GB, static_cast<long long>(k) * T, tid,
-                                                (off & 8u) == 0);
-            }
             const bool landed = bar_wait(&bar[st], (phases >> st) & 1u, a.wait_limit);
             const SmemAcc<OPT, MT, GT, T, VEC> acc{tile_mem + st * L::BYTES};
             if (landed && tid * VEC < cnt) {
@@ -923,9 +876,6 @@ __host__ __device__ constexpr int step_smem_bytes(int opt, int mt, bool bf16, in
 // with or without the norm diagnostics (MT = 1 exists for mask 0 only, and mask 0 for MT = 1).
 // Returns nullptr for combinations that do not exist.
 const void *lookup_step_kernel(int opt, bool post, bool bf16, int mt, int mask, bool diag);
-
-// OWN instantiations (without norms): MT = 1 (mask 0), 2 and 4; nullptr for others.
-const void *lookup_own_kernel(int opt, bool post, bool bf16, int mt, int mask);
 
 // Runtime-M kernel for the sync steps of M > MAX_MT that have no tile kernel.
 const void *lookup_generic_kernel(int opt, bool post, bool bf16, int mask, bool diag);

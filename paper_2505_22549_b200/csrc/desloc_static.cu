@@ -80,8 +80,7 @@ extern "C" DESLOC_API int desloc_step_static(const desloc_config *cfg, float *co
     if (rc != DESLOC_OK) return rc;
     if (!x || !u || !grads) return DESLOC_E_NULL;
     if (cfg->opt != DESLOC_SGDM && !v) return DESLOC_E_NULL;
-    int64_t total = 0;
-    rc = desloc::validate_numel(cfg, &total);
+    rc = desloc::validate_numel(cfg, nullptr);
     if (rc != DESLOC_OK) return rc;
     if (t < 0 || cuda_device < 0 || cuda_device >= kMaxDevices) return DESLOC_E_RANGE;
     rc = desloc::validate_step(cfg, lr_t, clip_bound_t);
@@ -99,8 +98,7 @@ extern "C" DESLOC_API int desloc_step_static(const desloc_config *cfg, float *co
     const int64_t nchunks = desloc::count_chunks(cfg->numel, cfg->num_tensors, chunk_elems, g_heads);
     if (nchunks > kMaxChunks) return DESLOC_E_TOO_LARGE;
     const uint32_t mask = desloc::mask_at(cfg, t);
-    const desloc::LaunchPlan plan = desloc::plan_launch(*cfg, mask, nchunks, chunk_elems, false,
-                                                          desloc::grads_off_layout(*cfg, total, grads, g_heads));
+    const desloc::LaunchPlan plan = desloc::plan_launch(*cfg, mask, nchunks, chunk_elems, false);
     if (!plan.fn) return DESLOC_E_INVALID;
 
     int dev_before = -1;

@@ -349,7 +349,7 @@ __device__ __forceinline__ float mean_of(const float (&s)[MT]) {
 // that of the exact pair (about one ulp of the quotient), not its bits.
 __device__ __forceinline__ float rsqrt_1ulp(float a) {
     const float y = rsqrtf(a);
-    const float r = y * fmaf(-0.5f * (a * y), y, 1.5f);   // (in this order: half of a denormal number may round, a * y is none)
+    const float r = y * fmaf(a * y, -0.5f * y, 1.5f);   // (halving y, not a: half of a denormal number may round)
     return a > 0.f && a < 3.0e38f ? r : y;   // keep the limits (1/0 = inf, 1/inf = 0) free of NaN
 }
 
@@ -362,7 +362,7 @@ __device__ __forceinline__ FV<VEC> rsqrt_1ulp(const FV<VEC> &a) {
         FV<VEC> y;
 #pragma unroll
         for (int c = 0; c < VEC; ++c) asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y.a[c]) : "f"(a.a[c]));
-        r = vmul<VEC, P>(y, vfma<VEC, P>(vmul<VEC, P>(vmul<VEC, P>(a, y), splat<VEC>(-0.5f)), y, splat<VEC>(1.5f)));
+        r = vmul<VEC, P>(y, vfma<VEC, P>(vmul<VEC, P>(vmul<VEC, P>(a, splat<VEC>(-0.5f)), y), y, splat<VEC>(1.5f)));
 #pragma unroll
         for (int c = 0; c < VEC; ++c) r.a[c] = a.a[c] < 3.0e38f ? r.a[c] : y.a[c];
     } else {

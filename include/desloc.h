@@ -128,7 +128,9 @@ DESLOC_API int desloc_create(desloc_ctx **out, const desloc_config *cfg, float *
  *   grads        : host array of M*num_tensors DEVICE pointers (same indexing as x) to
  *                  gradients of cfg.grad_dtype; read-only; may differ from call to call.
  *   stream       : a cudaStream_t (NULL = default stream).  The call only enqueues work and
- *                  never synchronises the device.
+ *                  never synchronises the device.  (A kernel launched behind a step with programmatic
+ *                  stream serialization must wait for its dependency before it reads x, u or v: steps let
+ *                  the kernel behind them begin early.)
  *   mask_out     : if not NULL receives the sync mask that was applied.
  * Errors: a failed launch is returned by this call; an asynchronous execution error surfaces
  * in a later call or at the caller's next synchronisation.
@@ -279,7 +281,8 @@ DESLOC_API int64_t desloc_get_launch_count(const desloc_ctx *ctx);
  *        it -- for x and for every array laid out like x (the same element offsets in a
  *        buffer of its own).  A gradient laid out differently may end up 8 or 2 bytes off a
  *        16-byte boundary after the cut; such chunks are updated straight from global memory
- *        (128-bit accesses, or coordinate by coordinate), correctly but more slowly.
+ *        (128-bit accesses, or coordinate by coordinate), correctly but more slowly, and where
+ *        they are many the launch is planned for that.
  * desloc_plan_chunks_at() with the x pointers given to desloc_create() is the table that context
  * works from; desloc_plan_chunks() is the same with x0 = NULL.
  */
@@ -288,12 +291,12 @@ DESLOC_API int64_t desloc_plan_chunks_at(const int64_t *numel, int32_t num_tenso
 DESLOC_API int64_t desloc_plan_chunks(const int64_t *numel, int32_t num_tensors, int64_t chunk_elems,
                                       int64_t *out, int64_t cap);
 
-/* Elements per chunk -- the run of tiles one thread block streams through, for all workers -- of
-   a context created from cfg (M, numel and num_tensors are read).  A tile is 1024 elements for
-   M <= 2, 512 for M = 3..8 (M > 8: 1024-element chunks, no tiles); a chunk is up to 8 tiles
-   on a large problem, fewer on a small one (so many that the blocks of an averaging step come
-   in full rounds).  Negative desloc_status on bad
-   input. */
+/* Elements per chunk of a context created from cfg (M, numel and num_tensors are read): a multiple
+   of 1024 elements for M <= 2 and M > 8, of 512 for M = 3..8, up to eight of these on a large problem,
+   fewer on a small one (for M = 3..8 so many that the blocks of an averaging step come in full rounds).  On
+   averaging steps a thread block takes a chunk, or a part of one, of all workers (M > 16, and some
+   variants and sizes from M = 9 on: a kernel without tiles); on local steps a part of a chunk of one
+   worker.  Negative desloc_status on bad input. */
 DESLOC_API int64_t desloc_chunk_elems(const desloc_config *cfg);
 
 /*

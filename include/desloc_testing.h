@@ -12,9 +12,9 @@ extern "C" {
 #endif
 
 /*
- * Cap the grid of the step kernels of this context at max_blocks thread blocks (0 = no cap, the
- * default: one block per chunk).  With a cap the blocks stride over the chunks (the runtime-M
- * kernel for sync steps of more than eight workers ignores the cap).  Results do not
+ * Cap the grid of the step kernels of this context at max_blocks thread blocks, per worker on local
+ * steps (0 = no cap, the default: one block per chunk or part of one).  With a cap the blocks stride over
+ * the parts (the runtime-M kernel ignores the cap).  Results do not
  * depend on it; the tests use it to run the striding path, which the default launch never takes
  * below 2^31 chunks.  DESLOC_E_RANGE for a negative value.
  */
@@ -22,8 +22,9 @@ DESLOC_API int desloc_testing_set_max_blocks(desloc_ctx *ctx, int64_t max_blocks
 
 /*
  * Whether the step kernels stage their tiles through shared memory: -1 = the library decides (the
- * default: a launch of at most two blocks per SM of single-tile chunks skips the staging, since
- * it has nothing to overlap), 0 = stage whenever alignment allows, 1 = never (every chunk is
+ * default: a launch of at most two blocks per SM of single tiles -- seven on local steps -- skips the
+ * staging, since it has nothing to overlap, and so do blocks that take whole chunks because the gradients
+ * cannot be staged), 0 = stage whenever alignment allows (but for those whole chunks), 1 = never (every chunk is
  * updated straight from global memory).  Results do not depend on it.  DESLOC_E_RANGE for other
  * values.
  */

@@ -10,6 +10,7 @@
 #include <cstring>
 #include <limits>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "../../include/desloc_testing.h"
@@ -78,6 +79,7 @@ struct WorkerRes {
     int64_t nchunks = 0;
     int64_t chunk_elems = 0;             // longest chunk of the plan
     long long *d_tstart = nullptr;       // [num_tensors + 1] first tile of every tensor
+    std::vector<int64_t> heads;          // [num_tensors] elements of the short first chunk
     std::vector<HostGroup> groups;
     void **d_tables = nullptr;  // [3][nptr] x, u, v
     Slot slots[kSlots];
@@ -162,6 +164,7 @@ cudaError_t make_worker_res(WorkerRes &r, int M, const int64_t *numel, int num_t
     plan_host_groups(r.groups, chunks, numel, total);
     r.nchunks = nchunks;
     r.chunk_elems = chunk_elems;
+    r.heads.swap(heads);
     cudaError_t e0 = cudaMalloc(&r.d_chunks, chunks.size() * sizeof(desloc::Chunk));
     if (e0 == cudaSuccess)
         e0 = cudaMemcpy(r.d_chunks, chunks.data(), chunks.size() * sizeof(desloc::Chunk), cudaMemcpyHostToDevice);
@@ -221,6 +224,7 @@ struct desloc_ctx {
     int next_slot = 0;
     int cur_slot = -1;           // slot holding the table equal to last_grads
     std::vector<const void *> last_grads;
+    desloc::GradLayout last_layout = desloc::GradLayout::FIT;   // of them
     cudaStream_t last_stream = nullptr;
     int64_t counters[4] = {0, 0, 0, 0};
     int64_t launches = 0;
@@ -280,6 +284,7 @@ int stage_grads(desloc_ctx *ctx, const void *const *grads, cudaStream_t stream, 
     cudaError_t e = cudaMemcpyAsync(s.dev, s.host, bytes, cudaMemcpyHostToDevice, stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e);
     std::memcpy(ctx->last_grads.data(), grads, bytes);
+    ctx->last_layout = desloc::grad_layout(ctx->cfg, grads, ctx->res.heads.data());
     ctx->cur_slot = ctx->next_slot;
     ctx->next_slot = (ctx->next_slot + 1) % kSlots;
     ctx->last_stream = stream;
@@ -354,7 +359,10 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
             d_gscale = ctx->res.d_norms + c.M;
         }
 
-        const desloc::LaunchPlan plan = desloc::plan_launch(c, mask, ctx->res.nchunks, ctx->res.chunk_elems, diag);
+        const desloc::GradLayout layout =
+            inline_g ? desloc::grad_layout(c, grads, ctx->res.heads.data()) : ctx->last_layout;
+        const desloc::LaunchPlan plan =
+            desloc::plan_launch(c, mask, ctx->res.nchunks, ctx->res.chunk_elems, diag, max_norm > 0.f, layout);
         if (!plan.fn) {
             rc = DESLOC_E_INVALID;
             break;
@@ -376,7 +384,7 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
         a.err = ctx->d_err;
         a.wait_limit = ctx->wait_limit;
         desloc::fill_plan(a, plan);
-        if (ctx->staging_mode >= 0) a.direct = ctx->staging_mode;
+        if (ctx->staging_mode >= 0 && !plan.whole) a.direct = ctx->staging_mode;
 
         void *params[] = {&a};
         const auto capped = [ctx](const desloc::LaunchPlan &lp) {
@@ -431,9 +439,9 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
                 a.chunks = ctx->res.d_chunks + grp.c0;
                 a.nchunks = grp.c1 - grp.c0;
                 a.diag_chunk0 = grp.c0;
-                const desloc::LaunchPlan gp = desloc::plan_launch(c, mask, a.nchunks, ctx->res.chunk_elems, diag);
+                const desloc::LaunchPlan gp = desloc::plan_launch(c, mask, a.nchunks, ctx->res.chunk_elems, diag, false, layout);
                 desloc::fill_plan(a, gp);
-                if (ctx->staging_mode >= 0) a.direct = ctx->staging_mode;
+                if (ctx->staging_mode >= 0 && !gp.whole) a.direct = ctx->staging_mode;
                 // (no overlap: this kernel also depends on the other stream's copies)
                 e = desloc::launch_kernel(gp.fn, capped(gp), gp.threads, gp.smem, stream, params, false);
                 if (e == cudaSuccess) ctx->launches += 1;
@@ -773,7 +781,7 @@ int desloc_set_workers(desloc_ctx *ctx, int32_t M_new, int32_t first_new, float 
     int rc = DESLOC_OK;
     if (e == cudaSuccess) {
         free_worker_res(ctx->res);
-        ctx->res = fresh;
+        ctx->res = std::move(fresh);
         ctx->last_grads.assign(static_cast<size_t>(nptr_new), nullptr);  // capacity reserved above
         ctx->cfg.M = M_new;
         ctx->nptr = nptr_new;

@@ -232,6 +232,7 @@ struct LaunchPlan {
     int threads = BLOCK_THREADS;
     int parts = 1, part_elems = 0;   // blocks that share a chunk, and elements of it for each
     bool direct = false;  // too small to gain from staging: update straight from global memory
+    bool whole = false;   // a block takes a whole chunk, straight from global memory: no shared memory to stage in
     bool overlap = true;  // may begin while the kernel in front of it still runs (not the runtime-M kernel)
 };
 
@@ -287,8 +288,30 @@ inline bool generic_fills_rounds_better(const desloc_config &c, uint32_t mask, l
     return fewer && (rounds == 1 || (rounds == 2 && c.opt != DESLOC_ADOPT));
 }
 
+// How the gradients lie towards the copy engine, which takes 16-byte aligned pieces: FIT, or at least a quarter of
+// the parameters have gradients that it cannot take, most of these (bf16) 8-byte aligned -- OFF -- or less -- NARROW.
+// fp32 gradients are FIT or OFF.  heads: elements of the short first chunks; grads: [M][num_tensors].
+enum class GradLayout { FIT, OFF, NARROW };
+inline GradLayout grad_layout(const desloc_config &c, const void *const *grads, const int64_t *heads) {
+    const bool bf16 = c.grad_dtype == DESLOC_BF16;
+    int64_t total = 0, off = 0, narrow = 0;
+    // (no plan for fewer elements than this asks: the look at 1088 pointers takes 6 us)
+    for (int32_t k = 0; k < c.num_tensors; ++k) total += c.numel[k];
+    if (total * c.M < (1 << 21)) return GradLayout::FIT;
+    for (int32_t k = 0; k < c.num_tensors; ++k) {
+        const uintptr_t head = static_cast<uintptr_t>(heads[k]) * (bf16 ? 2 : 4);
+        uintptr_t bits = 0;
+        for (int32_t m = 0; m < c.M; ++m)
+            bits |= reinterpret_cast<uintptr_t>(grads[static_cast<int64_t>(m) * c.num_tensors + k]) + head;
+        if ((bits & 15u) != 0) off += c.numel[k];
+        if (bf16 && (bits & 7u) != 0) narrow += c.numel[k];
+    }
+    if (off < total - off - off - off) return GradLayout::FIT;
+    return narrow > off - narrow ? GradLayout::NARROW : GradLayout::OFF;
+}
+
 inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, long long nchunks, int64_t chunk_elems,
-                              bool diag) {
+                              bool diag, bool scaled, GradLayout layout) {
     LaunchPlan p;
     // The mean of one replica is the replica: M = 1 always runs the local kernel.
     const uint32_t kmask = (c.M == 1) ? 0u : mask;
@@ -298,26 +321,38 @@ inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, long long n
     // More than eight workers: tiles of all replicas up to sixteen, the runtime-M kernel beyond, for the
     // post-average ordering and for the norm diagnostics.  All-sync steps of sixteen workers (Adam, bf16
     // gradients): 6.52 TB/s in tiles, 6.29 in the runtime-M kernel; nine workers 6.2 and 5.89.
+    const int mt = local ? 1 : c.M;
+    const int64_t replicas = local ? c.M : 1;
+    // Gradients that the copy engine cannot take, in problems of more than four rounds of blocks (smaller ones are served
+    // from L2 and gain nothing).  Measured with 60 M parameters x workers, Adam, gradients 8 bytes off the state's layout:
+    // whole chunks per block, nothing staged, for one replica (247 -> 213 us) and two (272 -> 222); the runtime-M
+    // kernel, which reads with 128-bit accesses, for nine workers and more (sixteen: 404 -> 258 us; where the
+    // accesses are narrow anyway, from thirteen on: 595 -> 470).
+    const bool off_many = layout != GradLayout::FIT && mt <= MAX_TILE_MT &&
+                          nchunks * replicas * parts_for(chunk_elems, c.opt, mt, bf16) >
+                              4LL * NUM_SMS * step_min_blocks(c.opt, mt, bf16);
+    const bool off_generic = off_many && ((bf16 && layout == GradLayout::OFF) || mt > 12);
     const bool generic = !local && c.M > MAX_MT &&
-                         (c.M > MAX_TILE_MT || post || diag || generic_fills_rounds_better(c, kmask, nchunks, chunk_elems));
+                         (c.M > MAX_TILE_MT || post || diag || off_generic ||
+                          generic_fills_rounds_better(c, kmask, nchunks, chunk_elems));
     p.fn = generic ? lookup_generic_kernel(c.opt, post, bf16, static_cast<int>(kmask), diag)
                    : lookup_step_kernel(c.opt, post, bf16, c.M, static_cast<int>(kmask), diag);
     p.strides = p.overlap = !generic;
-    const int mt = local ? 1 : c.M;
     p.grid = nchunks;
     if (!generic) {
         const int64_t tile = tile_elems(c.opt, mt, bf16), tiles = (chunk_elems + tile - 1) / tile;
-        const int64_t replicas = local ? c.M : 1;
+        // (with a factor on the gradients, behind norm clipping, whole chunks were 3-6 % slower)
+        const bool whole = p.whole = off_many && layout == GradLayout::OFF && mt <= 2 && !diag && !scaled;
         // (the diagnostics write one partial sum per chunk: their blocks take whole chunks)
-        const int64_t parts = diag ? 1 : parts_for(nchunks * replicas, chunk_elems, c.opt, mt, bf16);
+        const int64_t parts = diag || whole ? 1 : parts_for(nchunks * replicas, chunk_elems, c.opt, mt, bf16);
         p.parts = static_cast<int>(parts);
         p.part_elems = static_cast<int>((tiles + parts - 1) / parts * tile);
         p.threads = step_threads(c.opt, mt, bf16);
-        p.smem = step_smem_bytes(c.opt, mt, bf16, p.part_elems);
+        p.smem = whole ? 0 : step_smem_bytes(c.opt, mt, bf16, p.part_elems);
         p.smem_limit = step_smem_bytes(c.opt, mt, bf16, most_part_elems(c.opt, mt, bf16));
         p.grid = nchunks * parts;
         if (local) p.grid_y = static_cast<unsigned>(c.M);
-        p.direct = p.grid * replicas <= (local ? LOCAL_WAVE : DIRECT_GRID) && p.part_elems <= (local || mt > MAX_MT ? tile : plan_tile_elems(mt));
+        p.direct = whole || (p.grid * replicas <= (local ? LOCAL_WAVE : DIRECT_GRID) && p.part_elems <= (local || mt > MAX_MT ? tile : plan_tile_elems(mt)));
     }
     return p;
 }

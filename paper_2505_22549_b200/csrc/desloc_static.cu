@@ -98,7 +98,8 @@ extern "C" DESLOC_API int desloc_step_static(const desloc_config *cfg, float *co
     const int64_t nchunks = desloc::count_chunks(cfg->numel, cfg->num_tensors, chunk_elems, g_heads);
     if (nchunks > kMaxChunks) return DESLOC_E_TOO_LARGE;
     const uint32_t mask = desloc::mask_at(cfg, t);
-    const desloc::LaunchPlan plan = desloc::plan_launch(*cfg, mask, nchunks, chunk_elems, false);
+    const desloc::LaunchPlan plan = desloc::plan_launch(*cfg, mask, nchunks, chunk_elems, false, false,
+                                                          desloc::grad_layout(*cfg, grads, g_heads));
     if (!plan.fn) return DESLOC_E_INVALID;
 
     int dev_before = -1;

@@ -6,7 +6,7 @@
 With --gpus N > 1 and no torchrun environment the program starts N ranks of itself (one per
 GPU); under torchrun it is one of the ranks.  After the headline workload (default: workload 4)
 the single-GPU run times every other workload of the benchmark definition and reports them in
-"all_configs".
+"all_configs", a second line of JSON on standard error.
 
 One "step" is one call of desloc_step(): the whole hot path (clip, desynced averaging,
 optimizer update for all M worker replicas) over the full synthetic parameter/gradient set.
@@ -514,12 +514,39 @@ def run_ours(args, w):
             "graph_window": graph_info,
             "cpu_baseline": {k: cpu[k] for k in ("value", "unit", "cores", "kind", "sample",
                                                  "single_thread") if k in cpu},
-            "e2e": e2e, "gpu_launches": launches, "clocks": clocks, "all_configs": all_configs,
+            "e2e": e2e, "gpu_launches": launches, "clocks": clocks,
         }
-        print(json.dumps(line), flush=True)
+        # One short line on standard output; the other workloads' tables, ten times as long, go to standard error.
+        if all_configs is not None:
+            print(json.dumps({"all_configs": all_configs}), file=sys.stderr, flush=True)
+        print(result_line(line), flush=True)
     if world > 1:
         dist.destroy_process_group()
     return 0
+
+
+def _short(v):
+    """Floats to six significant digits."""
+    if isinstance(v, float):
+        return float(f"{v:.6g}")
+    if isinstance(v, dict):
+        return {k: _short(x) for k, x in v.items()}
+    return [_short(x) for x in v] if isinstance(v, list) else v
+
+
+MAX_LINE = 4000   # bytes: what reads the end of the output only must still see all of it
+
+
+def result_line(line):
+    """The result as one line of JSON of at most MAX_LINE bytes: if it is longer, breakdowns leave it, in this order."""
+    line = _short(line)
+    out = json.dumps(line)
+    for key in ("normclip_step", "diag_step", "by_mask", "graph_window", "roofline"):
+        if len(out) <= MAX_LINE:
+            break
+        line = {k: v for k, v in line.items() if k != key}
+        out = json.dumps(line)
+    return out
 
 
 # DRAM bytes (read + write) per algorithmic byte of one launch of the local-step kernel, from
@@ -584,7 +611,7 @@ def run_e2e(args, w, eng, G, X, offs, dev, world, barrier):
             "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": last[1] * 4, "steps": steps,
             "ms_per_step": ms / steps,
             "note": "desloc_step_host: gradients copied from pinned host memory every step, "
-                    "pipelined with the step in 8 tensor groups; result slice read back"
+                    "pipelined with the step in up to 8 groups of falling size; result slice read back"
                     + ("" if share else " (one host buffer re-sent for each worker)")}
 
 

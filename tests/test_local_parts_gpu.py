@@ -1,4 +1,4 @@
-"""Local steps (nothing averaged) run one replica per block, a chunk cut into parts of three or four 512-element tiles, or
+"""Local steps (nothing averaged) run one replica per block, a chunk cut into parts of up to three 512-element tiles, or
 single tiles straight from global memory where one wave of blocks covers the problem: sizes around those edges against the
 oracle."""
 import pytest

@@ -13,18 +13,19 @@ extern "C" {
 
 /*
  * Cap the grid of the step kernels of this context at max_blocks thread blocks, per worker on local
- * steps (0 = no cap, the default: one block per chunk or part of one).  With a cap the blocks stride over
- * the parts (the runtime-M kernel ignores the cap).  Results do not
+ * steps (0 = no cap, the default: one block per chunk or part of one).  With a cap every size runs in the tile
+ * kernels, whose blocks stride over the parts (the runtime-M kernel ignores the cap).  Results do not
  * depend on it; the tests use it to run the striding path, which the default launch never takes
  * below 2^31 chunks.  DESLOC_E_RANGE for a negative value.
  */
 DESLOC_API int desloc_testing_set_max_blocks(desloc_ctx *ctx, int64_t max_blocks);
 
 /*
- * Whether the step kernels stage their tiles through shared memory: -1 = the library decides (the
- * default: a launch of at most two blocks per SM of single tiles -- seven on local steps -- skips the
- * staging, since it has nothing to overlap, and so do blocks that take whole chunks because the gradients
- * cannot be staged), 0 = stage whenever alignment allows (but for those whole chunks), 1 = never (every chunk is
+ * Whether the tile kernels stage their tiles through shared memory: -1 = the library decides (the default:
+ * small and mid-sized problems do not run in tile kernels at all, and of the launches that do, one of at most two
+ * blocks per SM of single tiles -- seven on local steps -- skips the staging, since it has nothing to overlap, and
+ * so do blocks that take whole chunks because the gradients cannot be staged), 0 = tile kernels for every size,
+ * staged whenever alignment allows (but for those whole chunks), 1 = tile kernels that never stage (every chunk is
  * updated straight from global memory).  Results do not depend on it.  DESLOC_E_RANGE for other
  * values.
  */

@@ -361,8 +361,9 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
 
         const desloc::GradLayout layout =
             inline_g ? desloc::grad_layout(c, grads, ctx->res.heads.data()) : ctx->last_layout;
-        const desloc::LaunchPlan plan =
-            desloc::plan_launch(c, mask, ctx->res.nchunks, ctx->res.chunk_elems, diag, max_norm > 0.f, layout);
+        const bool lanes_ok = ctx->staging_mode < 0 && ctx->max_blocks == 0;
+        const desloc::LaunchPlan plan = desloc::plan_launch(c, mask, ctx->res.nchunks, ctx->res.chunk_elems, diag,
+                                                            max_norm > 0.f, layout, lanes_ok);
         if (!plan.fn) {
             rc = DESLOC_E_INVALID;
             break;
@@ -439,7 +440,7 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
                 a.chunks = ctx->res.d_chunks + grp.c0;
                 a.nchunks = grp.c1 - grp.c0;
                 a.diag_chunk0 = grp.c0;
-                const desloc::LaunchPlan gp = desloc::plan_launch(c, mask, a.nchunks, ctx->res.chunk_elems, diag, false, layout);
+                const desloc::LaunchPlan gp = desloc::plan_launch(c, mask, a.nchunks, ctx->res.chunk_elems, diag, false, layout, lanes_ok);
                 desloc::fill_plan(a, gp);
                 if (ctx->staging_mode >= 0 && !gp.whole) a.direct = ctx->staging_mode;
                 // (no overlap: this kernel also depends on the other stream's copies)

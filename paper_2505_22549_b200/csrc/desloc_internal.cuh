@@ -9,7 +9,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "../../include/desloc.h"
-#include "desloc_kernels.cuh"
+#include "desloc_lanes.cuh"
 
 namespace desloc {
 
@@ -221,6 +221,11 @@ inline void fill_hyper(StepArgs &a, const desloc_config &c, float lr_t, float cl
     a.part_elems = 0;
 }
 
+inline const void *lookup_lanes_kernel(int opt, bool post, bool bf16, int mt, int mask) {
+    return opt == OPT_ADAM ? lookup_lanes_adam(post, bf16, mt, mask)
+           : opt == OPT_ADOPT ? lookup_lanes_adopt(post, bf16, mt, mask) : lookup_lanes_sgdm(post, bf16, mt, mask);
+}
+
 // Which kernel a step of this configuration runs, and over how many blocks.
 struct LaunchPlan {
     const void *fn = nullptr;
@@ -310,8 +315,18 @@ inline GradLayout grad_layout(const desloc_config &c, const void *const *grads, 
     return narrow > off - narrow ? GradLayout::NARROW : GradLayout::OFF;
 }
 
+// The most coordinates (parameters times workers) of a step with mt replicas that runs with these in the lanes of a warp.
+// Measured with the arrays cold in L2 (Adam, ADOPT, SGDM, both gradient types): local steps of 0.25 to 16 million
+// 0.82 to 0.99 of the tile kernel's time, of a hundred million at the power cap 1.02 to 1.03; two workers up to five
+// million 0.68 to 1.01, four 0.53 to 1.03 (mean 0.85); eight up to 2.4 million 0.39 to 1.03, 3.2 million 0.91 to 1.08; three, and five
+// to seven, of which lanes are idle, up to 1.6 million 0.5 to 1.0, 2.4 million 1.0 to 1.2.
+inline int64_t lanes_most(int mt) {
+    return mt == 1 ? 12000000 : mt == 2 || mt == 4 ? 5000000 : mt == 8 ? 3000000 : 1600000;
+}
+
+// lanes_ok: (false in tests of the tile kernels)
 inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, long long nchunks, int64_t chunk_elems,
-                              bool diag, bool scaled, GradLayout layout) {
+                              bool diag, bool scaled, GradLayout layout, bool lanes_ok = true) {
     LaunchPlan p;
     // The mean of one replica is the replica: M = 1 always runs the local kernel.
     const uint32_t kmask = (c.M == 1) ? 0u : mask;
@@ -323,6 +338,18 @@ inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, long long n
     // gradients): 6.52 TB/s in tiles, 6.29 in the runtime-M kernel; nine workers 6.2 and 5.89.
     const int mt = local ? 1 : c.M;
     const int64_t replicas = local ? c.M : 1;
+    // (chunks times chunk length: no fewer coordinates than there are, so that a list of very many tiny tensors, most of
+    // whose work items would be empty, stays with the tiles)
+    if (lanes_ok && !diag && mt <= MAX_MT && nchunks * chunk_elems * c.M <= lanes_most(mt)) {
+        p.fn = lookup_lanes_kernel(c.opt, post, bf16, mt, static_cast<int>(kmask));
+        p.part_elems = lanes_part_elems(mt);
+        p.parts = static_cast<int>((chunk_elems + p.part_elems - 1) / p.part_elems);
+        p.threads = LANES_THREADS;
+        p.grid = nchunks * p.parts;
+        if (local) p.grid_y = static_cast<unsigned>(c.M);
+        p.strides = false;
+        return p;
+    }
     // Gradients that the copy engine cannot take, in problems of more than four rounds of blocks (smaller ones are served
     // from L2 and gain nothing).  Measured with 60 M parameters x workers, Adam, gradients 8 bytes off the state's layout:
     // whole chunks per block, nothing staged, for one replica (247 -> 213 us) and two (272 -> 222); the runtime-M

@@ -331,15 +331,20 @@ __device__ __forceinline__ float compensated_mean(const float (&s)[MT]) {
     return div_by_count(hi, lo, static_cast<float>(MT), 1.f / MT);
 }
 
+// The sum of up to eight values as their mean.
+template <int MT>
+__device__ __forceinline__ float div_sum(float t) {
+    if constexpr ((MT & (MT - 1)) == 0) return t * (1.f / MT);   // exact
+    else return div_by_count(t, 0.f, static_cast<float>(MT), 1.f / MT);
+}
+
 template <int MT>
 __device__ __forceinline__ float mean_of(const float (&s)[MT]) {
     if constexpr (MT > MAX_MT) {
         static_assert(MT <= MAX_TILE_MT, "three or four trees of four, and up to three more");
         return compensated_mean<MT>(s);
     } else {
-        const float t = tree_sum<0, MT, MT>(s);
-        if constexpr ((MT & (MT - 1)) == 0) return t * (1.f / MT);   // exact
-        else return div_by_count(t, 0.f, static_cast<float>(MT), 1.f / MT);
+        return div_sum<MT>(tree_sum<0, MT, MT>(s));
     }
 }
 

@@ -1,0 +1,205 @@
+// The step of small and mid-sized problems: a thread per worker and four coordinates, the replicas of a
+// coordinate in the lanes of one warp.
+//
+// Bound: latency up to about a million coordinates (parameters times workers), then HBM.  What a tile
+// kernel spends on such a problem is a chain: the copy engine's round trip, or, straight from global memory, one
+// round trip per worker (a worker's stores stand in front of the next one's loads), and rounds of few large
+// blocks.  Here a thread requests all it needs at once -- x, u, v and g of its four coordinates, 128 bits at a
+// time -- and the worker means are shuffles: no shared memory, no barrier, twelve blocks of four warps per SM.
+// Sums have the order of the tile kernels (tree_sum): same bits.
+//
+// Measured on B200, Adam, bf16 gradients, per step of a graph of dependent steps (before: the tile kernels).  One array
+// averaged: eight workers x 4096 parameters 1.7 us (5.2), x 110 K 3.7 (5.6), x 280 K 8.1 (11.5); four x 20 K 1.7 (3.3),
+// x 280 K 4.0 (7.3); two x 4096 1.4 (2.0), x 560 K 4.0 (5.6).  Local steps: four x 4096 1.5 us (1.7),
+// x 200 K 3.1 (4.4), x 400 K 5.0 (7.1).  With the arrays cold in L2: four x 250 K, local 5.8 us (6.6), all
+// averaged 6.6 (9.0).
+#pragma once
+#include <utility>
+
+#include "desloc_kernels.cuh"
+
+namespace desloc {
+
+// Four coordinates of one worker within a piece of `cnt`: side by side (WIDE, 128-bit accesses), or `step` apart.
+template <bool WIDE>
+struct Quad {
+    int e, step, cnt;
+    bool live;   // (lanes of no worker read and write nothing)
+    __device__ __forceinline__ bool has(int j) const { return live && (WIDE ? e : e + j * step) < cnt; }
+    __device__ __forceinline__ FV<4> ld(const float *p) const {
+        FV<4> r = splat<4>(0.f);
+        if constexpr (WIDE) {
+            if (has(0)) r = ld_f32<4>(reinterpret_cast<const char *>(p), e);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (has(j)) r.a[j] = p[e + j * step];
+        }
+        return r;
+    }
+    template <typename GT>
+    __device__ __forceinline__ FV<4> ldg(const char *p) const {
+        FV<4> r = splat<4>(0.f);
+        if constexpr (WIDE) {
+            if (has(0)) r = ld_grad<4, GT>(p, e);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (has(j)) r.a[j] = ld_grad<1, GT>(p, e + j * step).a[0];
+        }
+        return r;
+    }
+    __device__ __forceinline__ void st(float *p, const FV<4> &v) const {
+        if constexpr (WIDE) {
+            if (has(0)) st_f32<4>(reinterpret_cast<char *>(p), e, v);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (has(j)) p[e + j * step] = v.a[j];
+        }
+    }
+};
+
+// One worker's arrays from the first coordinate of a piece on.
+template <int OPT, typename GT>
+struct Replica {
+    float *x, *u, *v;
+    const char *g;
+    __device__ __forceinline__ Replica(const StepArgs &a, long long idx, long long start)
+        : x(a.x[idx] + start), u(a.u[idx] + start), v(OPT != OPT_SGDM ? a.v[idx] + start : nullptr),
+          g(static_cast<const char *>(grad_ptr(a, idx)) + start * static_cast<long long>(sizeof(GT))) {}
+    // 16-byte aligned states, and gradients as wide as four of them
+    __device__ __forceinline__ bool wide_ok() const {
+        return ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(v) |
+                 (reinterpret_cast<uintptr_t>(g) << (sizeof(GT) == 2 ? 1 : 0))) & 15u) == 0;
+    }
+};
+
+// A thread's four coordinates through the step, from and to global memory; mean(values) replaces each array of
+// `values` by its worker means.  All threads that share a mean call it together.
+template <int OPT, int MASK, typename GT, bool POST, bool PLAIN, bool WIDE, typename Mean>
+__device__ __forceinline__ void update_quad(const StepArgs &a, float sc, const Quad<WIDE> &q, const Replica<OPT, GT> &w,
+                                            const Mean &mean) {
+    constexpr bool SX = MASK & SYNC_X, SU = MASK & SYNC_U, HAS_V = OPT != OPT_SGDM, P = OPT != OPT_SGDM;
+    constexpr bool SV = (MASK & SYNC_V) && HAS_V;
+    FV<4> X = q.ld(w.x), U = q.ld(w.u), V{}, un, vn;
+    if constexpr (HAS_V) V = q.ld(w.v);
+    const FV<4> G = q.template ldg<GT>(w.g);
+    if constexpr (!POST) {
+        const FV<4> vown = V;
+        constexpr int KU = SX ? 1 : 0, KV = KU + (SU ? 1 : 0), N = KV + (SV ? 1 : 0);
+        if constexpr (N > 0) {
+            FV<4> s[N];
+            if constexpr (SX) s[0] = X;
+            if constexpr (SU) s[KU] = U;
+            if constexpr (SV) s[KV] = V;
+            mean(s);
+            if constexpr (SX) X = s[0];
+            if constexpr (SU) U = s[KU];
+            if constexpr (SV) V = s[KV];
+        }
+        state_update<OPT, PLAIN, 4>(a, G, sc, U, V, vown, un, vn);
+        X = apply_step<4, P>(a, X, minus_direction<OPT, PLAIN, 4>(a, un, vn));
+    } else {
+        state_update<OPT, PLAIN, 4>(a, G, sc, U, V, V, un, vn);
+        constexpr int KV = SU ? 1 : 0, N = KV + (SV ? 1 : 0);
+        if constexpr (N > 0) {
+            FV<4> s[N];
+            if constexpr (SU) s[0] = un;
+            if constexpr (SV) s[KV] = vn;
+            mean(s);
+            if constexpr (SU) un = s[0];
+            if constexpr (SV) vn = s[KV];
+        }
+        X = apply_step<4, P>(a, X, minus_direction<OPT, PLAIN, 4>(a, un, vn));
+        if constexpr (SX) {
+            FV<4> s[1] = {X};
+            mean(s);
+            X = s[0];
+        }
+    }
+    q.st(w.x, X);
+    q.st(w.u, un);
+    if constexpr (HAS_V) q.st(w.v, vn);
+}
+
+// Work item: a run of a chunk, of all MT replicas (of replica blockIdx.y for MT = 1, the local step of any worker
+// count).  A worker has 32 / lanes_groups(MT) lanes of every warp.  Five to seven workers take eight groups, of which some
+// idle: a sum over eight is three shuffles, a sum over six, of the values one by one, six -- all-sync steps of six
+// workers x 270 K parameters 10.7 us against 12.0 with 30 busy lanes.  Three workers have three groups: x 530 K 10.0
+// against 10.5 with four.
+constexpr int LANES_THREADS = 128;
+__host__ __device__ constexpr int lanes_groups(int mt) { return mt <= 4 ? mt : 8; }
+__host__ __device__ constexpr int lanes_part_elems(int mt) { return LANES_THREADS / 32 * 4 * (32 / lanes_groups(mt)); }
+
+template <int OPT, int MASK, int MT, typename GT, bool POST>
+__global__ void __launch_bounds__(LANES_THREADS, 10) desloc_lanes_kernel(const __grid_constant__ StepArgs a) {
+    constexpr int G = lanes_groups(MT), LW = 32 / G;   // lanes of a worker
+    begin_and_let_next_begin();
+    const unsigned c = item_chunk(a, blockIdx.x);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int part0 = static_cast<int>(blockIdx.x - c * a.parts) * a.part_elems + warp * (4 * LW);
+    const Chunk ch = a.chunks[c];
+    const int cnt = min(ch.count - part0, 4 * LW);
+    if (cnt <= 0) return;   // (of the whole warp)
+    const int own = lane / LW, lx = lane - own * LW;
+    const int m = MT == 1 ? static_cast<int>(blockIdx.y) : min(own, MT - 1);
+    const Replica<OPT, GT> w(a, static_cast<long long>(m) * a.nt + ch.tensor, ch.start + part0);
+    const bool live = own < MT, wide = __all_sync(0xffffffffu, w.wide_ok() && (cnt & 3) == 0);
+    const auto mean = [&](auto &arrays) {
+        if constexpr (MT > 1) {
+#pragma unroll
+            for (auto &v : arrays) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if constexpr ((G & (G - 1)) == 0) {
+                        // a butterfly adds in tree_sum's order (a sum's two sides may change places, and adding -0
+                        // for a worker that is not there changes nothing)
+                        float t = live ? v.a[j] : -0.f;
+#pragma unroll
+                        for (int o = LW; o < 32; o *= 2) t += __shfl_xor_sync(0xffffffffu, t, o);
+                        v.a[j] = div_sum<MT>(t);
+                    } else {
+                        float s[MT];
+#pragma unroll
+                        for (int k = 0; k < MT; ++k) s[k] = __shfl_sync(0xffffffffu, v.a[j], k * LW + lx);
+                        v.a[j] = mean_of<MT>(s);
+                    }
+                }
+            }
+        }
+    };
+    wait_for_earlier_kernels();
+    const float sc = a.gscale ? a.gscale[m] : 1.f;
+    if (wide) {
+        const Quad<true> q{4 * lx, 1, cnt, live};
+        if (plain_step<OPT>(a)) update_quad<OPT, MASK, GT, POST, true>(a, sc, q, w, mean);
+        else update_quad<OPT, MASK, GT, POST, false>(a, sc, q, w, mean);
+    } else {
+        const Quad<false> q{lx, LW, cnt, live};
+        update_quad<OPT, MASK, GT, POST, false>(a, sc, q, w, mean);
+    }
+}
+
+template <int OPT, typename GT, bool POST, int NMASK, int... I>
+const void *pick_lanes(int mt, int mask, std::integer_sequence<int, I...>) {
+    static const void *const tbl[] = {
+        reinterpret_cast<const void *>(&desloc_lanes_kernel<OPT, 1 + I % NMASK, 2 + I / NMASK, GT, POST>)...};
+    if (mt < 2 || mt > MAX_MT || mask < 1 || mask > NMASK) return nullptr;
+    return tbl[(mt - 2) * NMASK + mask - 1];
+}
+
+template <int OPT, typename GT>
+const void *lookup_lanes(bool post, int mt, int mask) {
+    constexpr int NMASK = OPT == OPT_SGDM ? 3 : 7;
+    using Seq = std::make_integer_sequence<int, (MAX_MT - 1) * NMASK>;
+    if (mask == 0) return reinterpret_cast<const void *>(&desloc_lanes_kernel<OPT, 0, 1, GT, false>);
+    return post ? pick_lanes<OPT, GT, true, NMASK>(mt, mask, Seq{}) : pick_lanes<OPT, GT, false, NMASK>(mt, mask, Seq{});
+}
+
+// One unit per optimizer.  Mask 0 is the one-replica kernel, whatever mt; else mt in 2..MAX_MT.
+const void *lookup_lanes_adam(bool post, bool bf16, int mt, int mask);
+const void *lookup_lanes_adopt(bool post, bool bf16, int mt, int mask);
+const void *lookup_lanes_sgdm(bool post, bool bf16, int mt, int mask);
+
+}  // namespace desloc

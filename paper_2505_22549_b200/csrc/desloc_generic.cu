@@ -23,20 +23,6 @@ namespace desloc {
 namespace {
 
 constexpr int GEN_MAX_M = 256;    // worker pointers staged per chunk (= the context's limit)
-// Measured on B200 (134.5 M parameters x 16 workers, fraction of the copy bandwidth on all-sync
-// steps): three blocks per SM with small batches 0.96; two blocks with batches twice as large
-// 0.85; fp64 worker sums 0.87 and IEEE sqrt / division instead of the hardware reciprocal
-// square root 0.87 (this kernel is bound by instruction issue: ~75 instructions per
-// worker-coordinate with those, ~45 without).
-constexpr int GEN_BUDGET = 24;      // registers a batch of workers may hold in flight
-
-// Workers per batch of the update loops: what fits in `budget` registers -- 1, 2 or 4 (a power
-// of two, so that a full batch can be summed as a tree).
-__host__ __device__ constexpr int gen_batch(int per_worker, int budget) {
-    const int b = budget / per_worker;
-    return b < 2 ? 1 : (b < 4 ? 2 : 4);
-}
-
 template <int N>
 struct Count {
     static constexpr int value = N;
@@ -238,7 +224,7 @@ __device__ __forceinline__ void generic_position(const StepArgs &a, char *const 
         FV<VEC> xb{}, ub{}, vb{};
         means_of_workers<VEC, SX, SU, SV>(sp, M, e, active, xb, ub, vb);
         constexpr bool NEED_V = OPT != OPT_SGDM && (!SV || OPT == OPT_ADOPT);
-        constexpr int B0 = gen_batch(worker_regs<OPT, GT>(!SX, !SU, NEED_V), GEN_BUDGET);
+        constexpr int B0 = gen_batch(worker_regs<OPT, GT>(!SX, !SU, NEED_V));
         constexpr int B = (OPT == OPT_ADOPT && B0 > 2) ? 2 : B0;  // ADOPT's normaliser needs more registers
         for_batches<B, DIAG>(M, [&](auto count, int m0, int n) {
             constexpr int N = decltype(count)::value;
@@ -282,7 +268,7 @@ __device__ __forceinline__ void generic_position(const StepArgs &a, char *const 
         using P = PostPlan<OPT, MASK>;
         WorkerSum<VEC> au, av, ax;
         au.clear(); av.clear(); ax.clear();
-        constexpr int BA = gen_batch(worker_regs<OPT, GT>(!P::D_NEEDS_MEAN, true, OPT != OPT_SGDM), GEN_BUDGET);
+        constexpr int BA = PostBatch<OPT, MASK, GT>::STATES;
         // phase A: states (and x where d_t needs no mean)
         for_batches<BA, DIAG>(M, [&](auto count, int m0, int n) {
             constexpr int N = decltype(count)::value;
@@ -339,7 +325,7 @@ __device__ __forceinline__ void generic_position(const StepArgs &a, char *const 
         const FV<VEC> mu = au.mean(M), mv = av.mean(M);
         if constexpr (P::D_NEEDS_MEAN) {
             // phase B: parameter step with the averaged states
-            constexpr int BB = gen_batch(4 + ((P::KEEP_U || P::KEEP_V) ? 4 : 0), GEN_BUDGET);
+            constexpr int BB = PostBatch<OPT, MASK, GT>::PARAMS;
             for_batches<BB, DIAG>(M, [&](auto count, int m0, int n) {
                 constexpr int N = decltype(count)::value;
                 FV<VEC> X[N], K[N];

@@ -402,7 +402,7 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
             if (ctx->prepared.size() < ctx->prepared.capacity()) ctx->prepared.push_back(plan.fn);
         }
         if (!host_grads) {
-            e = desloc::launch_kernel(plan.fn, capped(plan), plan.threads, plan.smem, stream, params, plan.overlap);
+            e = desloc::launch_kernel(plan.fn, capped(plan), dim3(plan.threads, plan.threads_y), plan.smem, stream, params, plan.overlap);
             if (e == cudaSuccess) ctx->launches += 1;
         } else {
             // The device gradient buffers may still be read by earlier work on `stream`.
@@ -444,7 +444,7 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
                 desloc::fill_plan(a, gp);
                 if (ctx->staging_mode >= 0 && !gp.whole) a.direct = ctx->staging_mode;
                 // (no overlap: this kernel also depends on the other stream's copies)
-                e = desloc::launch_kernel(gp.fn, capped(gp), gp.threads, gp.smem, stream, params, false);
+                e = desloc::launch_kernel(gp.fn, capped(gp), dim3(gp.threads, gp.threads_y), gp.smem, stream, params, false);
                 if (e == cudaSuccess) ctx->launches += 1;
             }
         }

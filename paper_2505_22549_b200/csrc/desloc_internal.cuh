@@ -9,7 +9,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "../../include/desloc.h"
-#include "desloc_lanes.cuh"
+#include "desloc_crowd.cuh"
 
 namespace desloc {
 
@@ -221,6 +221,11 @@ inline void fill_hyper(StepArgs &a, const desloc_config &c, float lr_t, float cl
     a.part_elems = 0;
 }
 
+inline const void *lookup_crowd_kernel(int opt, bool post, bool bf16, int kind, int mask) {
+    return opt == OPT_ADAM ? lookup_crowd_adam(post, bf16, kind, mask)
+           : opt == OPT_ADOPT ? lookup_crowd_adopt(post, bf16, kind, mask) : lookup_crowd_sgdm(post, bf16, kind, mask);
+}
+
 inline const void *lookup_lanes_kernel(int opt, bool post, bool bf16, int mt, int mask) {
     return opt == OPT_ADAM ? lookup_lanes_adam(post, bf16, mt, mask)
            : opt == OPT_ADOPT ? lookup_lanes_adopt(post, bf16, mt, mask) : lookup_lanes_sgdm(post, bf16, mt, mask);
@@ -234,15 +239,16 @@ struct LaunchPlan {
     bool strides = true;  // a smaller grid may stride over the work items (not the runtime-M kernel)
     int smem = 0;         // dynamic shared memory of the launch
     int smem_limit = 0;   // of any launch of this kernel
-    int threads = BLOCK_THREADS;
+    int threads = BLOCK_THREADS, threads_y = 1;
     int parts = 1, part_elems = 0;   // blocks that share a chunk, and elements of it for each
     bool direct = false;  // too small to gain from staging: update straight from global memory
     bool whole = false;   // a block takes a whole chunk, straight from global memory: no shared memory to stage in
     bool overlap = true;  // may begin while the kernel in front of it still runs (not the runtime-M kernel)
 };
 
-// Launches of at most this many blocks of single-tile chunks (two per SM of a B200: one wave)
-// skip the staging.  Measured on the 4096-parameter, two-worker workload: 3.08 us per step in a
+// Steps with norm diagnostics (small problems without them run in desloc_lanes_kernel and desloc_crowd_kernel): launches
+// of at most this many blocks of single-tile chunks (two per SM of a B200: one wave)
+// skip the staging.  Measured on 4096 parameters and two workers: 3.08 us per step in a
 // CUDA graph of 16 steps against 3.34 us staged.
 constexpr long long DIRECT_GRID = 2 * NUM_SMS;
 // One-replica kernel: at most seven blocks of one tile per SM go straight to global memory.
@@ -262,11 +268,11 @@ inline cudaError_t prepare_launch(const LaunchPlan &p) {
 // step of four workers 82.0 us instead of 85.7, 135 M parameters 2044 us instead of 2050.  The runtime-M
 // kernel neither begins early nor lets others: its blocks are few and long, and those of the next step crowded
 // onto the SMs this one left free (24 workers x 125 K parameters, 123 blocks: 23.9 us instead of 14.4).
-inline cudaError_t launch_kernel(const void *fn, dim3 grid, unsigned threads, size_t smem, cudaStream_t stream,
+inline cudaError_t launch_kernel(const void *fn, dim3 grid, dim3 threads, size_t smem, cudaStream_t stream,
                                  void **params, bool overlap) {
     cudaLaunchConfig_t lc{};
     lc.gridDim = grid;
-    lc.blockDim = dim3(threads);
+    lc.blockDim = threads;
     lc.dynamicSmemBytes = smem;
     lc.stream = stream;
     cudaLaunchAttribute at{};
@@ -324,6 +330,14 @@ inline int64_t lanes_most(int mt) {
     return mt == 1 ? 12000000 : mt == 2 || mt == 4 ? 5000000 : mt == 8 ? 3000000 : 1600000;
 }
 
+// The same of averaging steps of more than eight workers that run in desloc_crowd_kernel.  Measured, as above: nine and ten workers
+// up to a million 0.42 to 0.9, 1.6 million 0.73 to 1.1; 12 to 16 up to 2.4 million 0.29 to 1.04 (3.2 million 0.8 to 1.15); 24 and
+// 32 up to four million 0.15 to 0.95 (six 0.75 to 1.16); 64 up to eight million 0.1 to 0.94 (15: 1.1 to 1.4); 128 and 256 up
+// to ten million 0.03 to 0.82 (15: 0.7 to 1.2).
+inline int64_t crowd_most(int mt) {
+    return mt < 12 ? 1500000 : mt <= 16 ? 2500000 : mt <= 32 ? 4000000 : mt <= 64 ? 8000000 : 10000000;
+}
+
 // lanes_ok: (false in tests of the tile kernels)
 inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, long long nchunks, int64_t chunk_elems,
                               bool diag, bool scaled, GradLayout layout, bool lanes_ok = true) {
@@ -347,6 +361,21 @@ inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, long long n
         p.threads = LANES_THREADS;
         p.grid = nchunks * p.parts;
         if (local) p.grid_y = static_cast<unsigned>(c.M);
+        p.strides = false;
+        return p;
+    }
+    if (lanes_ok && !diag && mt > MAX_MT && nchunks * chunk_elems * c.M <= crowd_most(mt)) {
+        const int L = crowd_lanes(c.M), threads = c.M * L;
+        p.part_elems = 4 * L;
+        p.parts = static_cast<int>((chunk_elems + p.part_elems - 1) / p.part_elems);
+        p.grid = nchunks * p.parts;
+        const int kind = threads > 512 ? CROWD_1024 : threads > 256 ? CROWD_512
+                         : p.grid <= crowd_min_blocks(CROWD_FEW) * NUM_SMS ? CROWD_FEW : CROWD_256;
+        p.fn = lookup_crowd_kernel(c.opt, post, bf16, kind, static_cast<int>(kmask));
+        p.threads = L;
+        p.threads_y = c.M;
+        p.smem = crowd_smem_bytes(c.opt, bf16, c.M);
+        p.smem_limit = crowd_smem_limit(kind);
         p.strides = false;
         return p;
     }
@@ -379,7 +408,7 @@ inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, long long n
         p.smem_limit = step_smem_bytes(c.opt, mt, bf16, most_part_elems(c.opt, mt, bf16));
         p.grid = nchunks * parts;
         if (local) p.grid_y = static_cast<unsigned>(c.M);
-        p.direct = whole || (p.grid * replicas <= (local ? LOCAL_WAVE : DIRECT_GRID) && p.part_elems <= (local || mt > MAX_MT ? tile : plan_tile_elems(mt)));
+        p.direct = whole || (p.grid * replicas <= (local ? LOCAL_WAVE : DIRECT_GRID) && p.part_elems <= (local ? tile : plan_tile_elems(mt)));
     }
     return p;
 }

@@ -431,6 +431,26 @@ struct PostPlan {
     static constexpr bool KEEP_V = D_NEEDS_MEAN && OPT == OPT_ADAM && !SV;   // Adam, u synced only
 };
 
+// Workers per batch of the runtime-M kernel's update loops: what fits in `budget` registers -- 1, 2 or 4 (a power
+// of two, so that a full batch can be summed as a tree).  Measured on B200 (134.5 M parameters x 16 workers, fraction of
+// the copy bandwidth on all-sync steps): three blocks per SM with small batches 0.96; two blocks with batches twice as large
+// 0.85; fp64 worker sums 0.87 and IEEE sqrt / division instead of the hardware reciprocal
+// square root 0.87 (this kernel is bound by instruction issue: ~75 instructions per
+// worker-coordinate with those, ~45 without).
+constexpr int GEN_BUDGET = 24;      // registers a batch of workers may hold in flight
+__host__ __device__ constexpr int gen_batch(int per_worker, int budget = GEN_BUDGET) {
+    const int b = budget / per_worker;
+    return b < 2 ? 1 : (b < 4 ? 2 : 4);
+}
+// Post-average ordering, more than eight workers: how many values enter the sums of the states, and of x, as one tree.
+template <int OPT, int MASK, typename GT>
+struct PostBatch {
+    using P = PostPlan<OPT, MASK>;
+    static constexpr int STATES = gen_batch(worker_regs<OPT, GT>(!P::D_NEEDS_MEAN, true, OPT != OPT_SGDM));
+    static constexpr int PARAMS = gen_batch(4 + ((P::KEEP_U || P::KEEP_V) ? 4 : 0));   // where d_t needs a mean
+    static constexpr int X = P::D_NEEDS_MEAN ? PARAMS : STATES;
+};
+
 
 // ---- where a tile lives -----------------------------------------------------------------------
 // Position q of a thread covers VEC consecutive elements.  Both accessors expose the same four

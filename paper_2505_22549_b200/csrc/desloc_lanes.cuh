@@ -5,14 +5,13 @@
 // kernel spends on such a problem is a chain: the copy engine's round trip, or, straight from global memory, one
 // round trip per worker (a worker's stores stand in front of the next one's loads), and rounds of few large
 // blocks.  Here a thread requests all it needs at once -- x, u, v and g of its four coordinates, 128 bits at a
-// time -- and the worker means are shuffles: no shared memory, no barrier, twelve blocks of four warps per SM.
+// time -- and the worker means are shuffles: no barrier, ten blocks of four warps per SM.
 // Sums have the order of the tile kernels (tree_sum): same bits.
 //
-// Measured on B200, Adam, bf16 gradients, per step of a graph of dependent steps (before: the tile kernels).  One array
-// averaged: eight workers x 4096 parameters 1.7 us (5.2), x 110 K 3.7 (5.6), x 280 K 8.1 (11.5); four x 20 K 1.7 (3.3),
-// x 280 K 4.0 (7.3); two x 4096 1.4 (2.0), x 560 K 4.0 (5.6).  Local steps: four x 4096 1.5 us (1.7),
-// x 200 K 3.1 (4.4), x 400 K 5.0 (7.1).  With the arrays cold in L2: four x 250 K, local 5.8 us (6.6), all
-// averaged 6.6 (9.0).
+// Measured on B200, Adam, bf16 gradients, per step of a graph of dependent steps, the arrays cold in L2 from 0.25 million
+// coordinates on (before: the tile kernels).  One array averaged: eight workers x 7.5 K parameters 1.8 us (4.8), x 125 K 6.5
+// (9.8), x 300 K 12.6 (17.4); four x 15 K 1.7 (2.8); two x 250 K 3.7 (5.4).  Four x 250 K, all averaged, 6.5 (9.1).
+// Local steps: four x 2.5 K 1.5 us (1.7), x 250 K 5.8 (6.6), x 400 K 8.0 (9.5), x 1.25 M 21.9 (22.7).
 #pragma once
 #include <utility>
 
@@ -75,49 +74,103 @@ struct Replica {
     }
 };
 
-// A thread's four coordinates through the step, from and to global memory; mean(values) replaces each array of
-// `values` by its worker means.  All threads that share a mean call it together.
-template <int OPT, int MASK, typename GT, bool POST, bool PLAIN, bool WIDE, typename Mean>
-__device__ __forceinline__ void update_quad(const StepArgs &a, float sc, const Quad<WIDE> &q, const Replica<OPT, GT> &w,
-                                            const Mean &mean) {
+// Where the loads of a thread land: array k (x, u, v, and fp32 gradients as the fourth) at `p + k * stride`.  128-bit loads
+// go there past L1 (cp.async): in registers' place, the bytes in flight need room in L1, and behind a kernel
+// that left most of the SM to shared memory, as the tile kernels do, there are 28 KB of it -- local steps of four workers x 1.25 M
+// parameters took 26.0 us then instead of 21.9, with loads that allocate no lines 24.9, this way 22.1 behind either.
+struct Landing {
+    float *p;
+    int stride;
+    __device__ __forceinline__ void load(int k, const float *src) const {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
+                     :: "r"(static_cast<uint32_t>(__cvta_generic_to_shared(p + k * stride))), "l"(src) : "memory");
+    }
+    __device__ __forceinline__ FV<4> get(int k) const { return ld_f32<4>(reinterpret_cast<const char *>(p + k * stride), 0); }
+};
+template <int OPT, typename GT>
+__host__ __device__ constexpr int landing_arrays() { return (OPT == OPT_SGDM ? 2 : 3) + (sizeof(GT) == 4 ? 1 : 0); }
+
+// A thread's four coordinates through the step, out of the arrays `from` and back to the same ones, which to() gives.
+// mean(values, arrays) replaces values[i], of array arrays::at(i) (0 x, 1 u, 2 v), by their worker means; all threads that
+// share a mean call it together.
+template <int... A>
+struct Arrays {
+    static constexpr int N = sizeof...(A);
+    static __device__ constexpr int at(int i) {
+        constexpr int a[] = {A...};
+        return a[i];
+    }
+};
+template <int OPT, int MASK, typename GT, bool POST, bool PLAIN, bool WIDE, typename Mean, typename Where>
+__device__ __forceinline__ void update_quad(const StepArgs &a, float sc, const Quad<WIDE> &q, const Landing &land,
+                                            const Replica<OPT, GT> &from, const Where &to, const Mean &mean) {
     constexpr bool SX = MASK & SYNC_X, SU = MASK & SYNC_U, HAS_V = OPT != OPT_SGDM, P = OPT != OPT_SGDM;
     constexpr bool SV = (MASK & SYNC_V) && HAS_V;
-    FV<4> X = q.ld(w.x), U = q.ld(w.u), V{}, un, vn;
-    if constexpr (HAS_V) V = q.ld(w.v);
-    const FV<4> G = q.template ldg<GT>(w.g);
+    FV<4> X{}, U{}, V{}, G{}, un, vn;
+    if constexpr (WIDE) {
+        if (q.has(0)) {
+            land.load(0, from.x + q.e);
+            land.load(1, from.u + q.e);
+            if constexpr (HAS_V) land.load(2, from.v + q.e);
+            if constexpr (sizeof(GT) == 4) land.load(HAS_V ? 3 : 2, reinterpret_cast<const float *>(from.g) + q.e);
+            else G = ld_grad<4, GT>(from.g, q.e);
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            X = land.get(0);
+            U = land.get(1);
+            if constexpr (HAS_V) V = land.get(2);
+            if constexpr (sizeof(GT) == 4) G = land.get(HAS_V ? 3 : 2);
+        }
+    } else {
+        X = q.ld(from.x);
+        U = q.ld(from.u);
+        if constexpr (HAS_V) V = q.ld(from.v);
+        G = q.template ldg<GT>(from.g);
+    }
     if constexpr (!POST) {
         const FV<4> vown = V;
-        constexpr int KU = SX ? 1 : 0, KV = KU + (SU ? 1 : 0), N = KV + (SV ? 1 : 0);
-        if constexpr (N > 0) {
-            FV<4> s[N];
-            if constexpr (SX) s[0] = X;
-            if constexpr (SU) s[KU] = U;
-            if constexpr (SV) s[KV] = V;
-            mean(s);
-            if constexpr (SX) X = s[0];
-            if constexpr (SU) U = s[KU];
-            if constexpr (SV) V = s[KV];
+        // (one case per subset of the three arrays)
+        if constexpr (SX && SU && SV) {
+            FV<4> s[3] = {X, U, V};
+            mean(s, Arrays<0, 1, 2>{});
+            X = s[0]; U = s[1]; V = s[2];
+        } else if constexpr (SX && SU) {
+            FV<4> s[2] = {X, U};
+            mean(s, Arrays<0, 1>{});
+            X = s[0]; U = s[1];
+        } else if constexpr (SX && SV) {
+            FV<4> s[2] = {X, V};
+            mean(s, Arrays<0, 2>{});
+            X = s[0]; V = s[1];
+        } else if constexpr (SU && SV) {
+            FV<4> s[2] = {U, V};
+            mean(s, Arrays<1, 2>{});
+            U = s[0]; V = s[1];
+        } else if constexpr (SX || SU || SV) {
+            FV<4> s[1] = {SX ? X : SU ? U : V};
+            mean(s, Arrays<SX ? 0 : SU ? 1 : 2>{});
+            (SX ? X : SU ? U : V) = s[0];
         }
         state_update<OPT, PLAIN, 4>(a, G, sc, U, V, vown, un, vn);
         X = apply_step<4, P>(a, X, minus_direction<OPT, PLAIN, 4>(a, un, vn));
     } else {
         state_update<OPT, PLAIN, 4>(a, G, sc, U, V, V, un, vn);
-        constexpr int KV = SU ? 1 : 0, N = KV + (SV ? 1 : 0);
-        if constexpr (N > 0) {
-            FV<4> s[N];
-            if constexpr (SU) s[0] = un;
-            if constexpr (SV) s[KV] = vn;
-            mean(s);
-            if constexpr (SU) un = s[0];
-            if constexpr (SV) vn = s[KV];
+        if constexpr (SU && SV) {
+            FV<4> s[2] = {un, vn};
+            mean(s, Arrays<1, 2>{});
+            un = s[0]; vn = s[1];
+        } else if constexpr (SU || SV) {
+            FV<4> s[1] = {SU ? un : vn};
+            mean(s, Arrays<SU ? 1 : 2>{});
+            (SU ? un : vn) = s[0];
         }
         X = apply_step<4, P>(a, X, minus_direction<OPT, PLAIN, 4>(a, un, vn));
         if constexpr (SX) {
             FV<4> s[1] = {X};
-            mean(s);
+            mean(s, Arrays<0>{});
             X = s[0];
         }
     }
+    const Replica<OPT, GT> w = to();
     q.st(w.x, X);
     q.st(w.u, un);
     if constexpr (HAS_V) q.st(w.v, vn);
@@ -145,8 +198,10 @@ __global__ void __launch_bounds__(LANES_THREADS, 10) desloc_lanes_kernel(const _
     const int own = lane / LW, lx = lane - own * LW;
     const int m = MT == 1 ? static_cast<int>(blockIdx.y) : min(own, MT - 1);
     const Replica<OPT, GT> w(a, static_cast<long long>(m) * a.nt + ch.tensor, ch.start + part0);
+    __shared__ float4 landing[landing_arrays<OPT, GT>()][LANES_THREADS];
+    const Landing land{reinterpret_cast<float *>(&landing[0][threadIdx.x]), 4 * LANES_THREADS};
     const bool live = own < MT, wide = __all_sync(0xffffffffu, w.wide_ok() && (cnt & 3) == 0);
-    const auto mean = [&](auto &arrays) {
+    const auto mean = [&](auto &arrays, auto) {
         if constexpr (MT > 1) {
 #pragma unroll
             for (auto &v : arrays) {
@@ -173,11 +228,11 @@ __global__ void __launch_bounds__(LANES_THREADS, 10) desloc_lanes_kernel(const _
     const float sc = a.gscale ? a.gscale[m] : 1.f;
     if (wide) {
         const Quad<true> q{4 * lx, 1, cnt, live};
-        if (plain_step<OPT>(a)) update_quad<OPT, MASK, GT, POST, true>(a, sc, q, w, mean);
-        else update_quad<OPT, MASK, GT, POST, false>(a, sc, q, w, mean);
+        if (plain_step<OPT>(a)) update_quad<OPT, MASK, GT, POST, true>(a, sc, q, land, w, [&] { return w; }, mean);
+        else update_quad<OPT, MASK, GT, POST, false>(a, sc, q, land, w, [&] { return w; }, mean);
     } else {
         const Quad<false> q{lx, LW, cnt, live};
-        update_quad<OPT, MASK, GT, POST, false>(a, sc, q, w, mean);
+        update_quad<OPT, MASK, GT, POST, false>(a, sc, q, land, w, [&] { return w; }, mean);
     }
 }
 

@@ -182,7 +182,7 @@ extern "C" DESLOC_API int desloc_step_static(const desloc_config *cfg, float *co
         void *params[] = {&a};
         e = desloc::prepare_launch(plan);
         if (e == cudaSuccess)
-            e = desloc::launch_kernel(plan.fn, dim3(static_cast<unsigned>(plan.grid), plan.grid_y), plan.threads, plan.smem, st, params, plan.overlap);
+            e = desloc::launch_kernel(plan.fn, dim3(static_cast<unsigned>(plan.grid), plan.grid_y), dim3(plan.threads, plan.threads_y), plan.smem, st, params, plan.overlap);
         if (e != cudaSuccess) { rc = DESLOC_E_CUDA; break; }
     } while (false);
     if (rc == DESLOC_E_CUDA) (void)cudaGetLastError();

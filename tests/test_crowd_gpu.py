@@ -1,0 +1,35 @@
+"""Averaging steps of more than eight workers on small problems: against the oracle, and bit for bit against the tile kernels (up to
+sixteen workers) and the runtime-M kernel, whose sums have the same order."""
+import numpy as np
+import pytest
+
+import desloc_inputs as di
+from test_parity_gpu import check, run_both
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("M", [9, 11, 12, 16, 17, 32, 33, 64, 65, 128, 129, 256])
+@pytest.mark.parametrize("opt,gd,rho,align,g_shift", [("adam", "bf16", 0.0, 4, 0), ("adopt", "f32", 1.5, 1, 0),
+                                                      ("sgdm", "bf16", 0.0, 8, 4), ("adam", "f32", 1.5, 8, 1)])
+@pytest.mark.parametrize("post", [False, True])
+def test_every_mask_at_the_edges_of_a_piece(M, opt, gd, rho, align, g_shift, post):
+    piece = 64 if M < 12 else 32 if M <= 32 else 16
+    numel = (1, 2, 3, piece - 1, piece, piece + 1, piece + 4, 2 * piece, 516, 1031)
+    masks = list(range(1, 4 if opt == "sgdm" else 8))
+    w = di.Workload("crowd", opt, M, numel, gd, "normal1", beta1=0.9, beta2=0.99, eps=1e-2, lr=1e-2, weight_decay=0.05,
+                    clip_rho=rho, adopt_norm_clip=(opt == "adopt"), seed=M)
+    kw = dict(align=align, g_shift=g_shift, forced_masks=masks, v_init=0.25, post=post)
+    crowd, other = run_both(w, len(masks), **kw), run_both(w, len(masks), staging=0, **kw)
+    check(crowd)
+    check(other)
+    for name in ("gx", "gu") + (("gv",) if crowd["gv"] is not None else ()):
+        assert np.array_equal(crowd[name].view(np.uint32), other[name].view(np.uint32)), name
+
+
+@pytest.mark.parametrize("M,opt,gd,n", [(12, "adam", "bf16", 60_000), (16, "sgdm", "f32", 156_001), (24, "adopt", "bf16", 165_888),
+                                        (64, "adam", "f32", 124_929)])
+def test_more_blocks_than_fit_at_once(M, opt, gd, n):
+    w = di.Workload("crowd", opt, M, (n,), gd, "student_t3", lr=1e-2, clip_rho=1.5, eps=1e-3,
+                    adopt_norm_clip=(opt == "adopt"), seed=M)
+    check(run_both(w, 2, align=4, v_init=0.25, forced_masks=[3 if opt == "sgdm" else 7, 2]))

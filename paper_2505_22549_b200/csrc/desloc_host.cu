@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "../../include/desloc_testing.h"
+#include "desloc_hostcopy.cuh"
 #include "desloc_inst.cuh"
 #include "desloc_internal.cuh"
 #include "desloc_norms.cuh"
@@ -292,6 +293,32 @@ int stage_grads(desloc_ctx *ctx, const void *const *grads, cudaStream_t stream, 
     return DESLOC_OK;
 }
 
+// The gradients of a small problem as contiguous pieces that a kernel can read where they are, in pinned host memory;
+// false where there are too many bytes or pieces, or some of them in memory that only the copy engine reaches.
+bool gather_host_runs(const desloc_ctx *ctx, const void *const *host_grads, const void *const *grads, desloc::HostRuns &runs) {
+    const desloc_config &c = ctx->cfg;
+    const size_t gsz = c.grad_dtype == DESLOC_BF16 ? 2 : 4;
+    if (ctx->total_elems > desloc::HOST_KERNEL_BYTES / static_cast<int64_t>(gsz) / c.M) return false;
+    const char *from = nullptr;
+    char *to = nullptr;
+    size_t bytes = 0;
+    const auto flush = [&] { return bytes == 0 || (runs.add(from, to, bytes) && desloc::device_reads_host(from, bytes)); };
+    for (int64_t i = 0; i < ctx->nptr; ++i) {
+        const char *hp = static_cast<const char *>(host_grads[i]);
+        char *dp = static_cast<char *>(const_cast<void *>(grads[i]));
+        const size_t n = static_cast<size_t>(ctx->numel[i % c.num_tensors]) * gsz;
+        if (bytes != 0 && hp == from + bytes && dp == to + bytes) {
+            bytes += n;
+            continue;
+        }
+        if (!flush()) return false;
+        from = hp;
+        to = dp;
+        bytes = n;
+    }
+    return flush();
+}
+
 // max_norm > 0: norm-based clipping first (two reduction launches), then the step.
 // diag: the step kernel also accumulates the per-chunk sums of squares of g, x_{t+1} and d_t.
 // host_grads != nullptr: the gradients are first copied from host memory into `grads` (device),
@@ -401,8 +428,18 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
             }
             if (ctx->prepared.size() < ctx->prepared.capacity()) ctx->prepared.push_back(plan.fn);
         }
-        if (!host_grads) {
-            e = desloc::launch_kernel(plan.fn, capped(plan), dim3(plan.threads, plan.threads_y), plan.smem, stream, params, plan.overlap);
+        bool on_device = !host_grads;
+        if (host_grads) {
+            desloc::HostRuns runs;
+            if (gather_host_runs(ctx, host_grads, grads, runs)) {
+                e = desloc::launch_host_copy(runs, stream);
+                if (e == cudaSuccess) ctx->launches += 1;
+                on_device = true;
+            }
+        }
+        if (on_device) {
+            if (e == cudaSuccess)
+                e = desloc::launch_kernel(plan.fn, capped(plan), dim3(plan.threads, plan.threads_y), plan.smem, stream, params, plan.overlap);
             if (e == cudaSuccess) ctx->launches += 1;
         } else {
             // The device gradient buffers may still be read by earlier work on `stream`.

@@ -29,6 +29,7 @@ struct Entry {
     decltype(&desloc_step_diag) step_diag = nullptr;
     decltype(&desloc_rel_change) rel_change = nullptr;
     decltype(&desloc_get_diag_norms) diag_norms = nullptr;
+    decltype(&desloc_step_host) step_host = nullptr;
 } g_entry;
 
 struct Table {
@@ -237,6 +238,33 @@ PyObject *call_step_masked(PyObject *, PyObject *const *args, Py_ssize_t nargs) 
     return PyLong_FromLong(rc);
 }
 
+// (context, t, lr, clip bound, host pointer array, device pointer array, device) -> sync mask, or a negative status
+PyObject *call_step_host(PyObject *, PyObject *const *args, Py_ssize_t nargs) {
+    void *ctx = nullptr, *from = nullptr, *to = nullptr;
+    int64_t t = 0, device = 0;
+    float lr = 0.f, bound = 0.f;
+    if (nargs != 7) {
+        PyErr_SetString(PyExc_TypeError, "step_host(ctx, t, lr, clip_bound, host_grads, dev_grads, device)");
+        return nullptr;
+    }
+    if (!as_pointer(args[0], &ctx) || !as_int64(args[1], &t) || !as_float(args[2], &lr) || !as_float(args[3], &bound) ||
+        !as_pointer(args[4], &from) || !as_pointer(args[5], &to) || !as_int64(args[6], &device))
+        return nullptr;
+    uint32_t mask = 0;
+    int rc = 0;
+    try {
+        void *stream = c10::cuda::getCurrentCUDAStream(static_cast<c10::DeviceIndex>(device)).stream();
+        Py_BEGIN_ALLOW_THREADS
+        rc = g_entry.step_host(static_cast<desloc_ctx *>(ctx), t, lr, bound, static_cast<const void *const *>(from),
+                               static_cast<void *const *>(to), stream, &mask);
+        Py_END_ALLOW_THREADS
+    } catch (const std::exception &e) {
+        PyErr_SetString(PyExc_RuntimeError, e.what());
+        return nullptr;
+    }
+    return PyLong_FromLong(rc == DESLOC_OK ? static_cast<long>(mask) : rc);
+}
+
 // A list of n floats.
 PyObject *float_list(const float *v, size_t n) {
     PyObject *list = PyList_New(static_cast<Py_ssize_t>(n));
@@ -328,16 +356,17 @@ PyObject *call_diag_norms(PyObject *, PyObject *const *args, Py_ssize_t nargs) {
     return both;
 }
 
-// bind(addresses of desloc_step, _step_masked, _step_normclip, _step_diag, _rel_change, _get_diag_norms)
+// bind(addresses of desloc_step, _step_masked, _step_normclip, _step_diag, _rel_change, _get_diag_norms, _step_host)
 PyObject *bind_entries(PyObject *, PyObject *args) {
-    unsigned long long a[6];
-    if (!PyArg_ParseTuple(args, "KKKKKK", &a[0], &a[1], &a[2], &a[3], &a[4], &a[5])) return nullptr;
+    unsigned long long a[7];
+    if (!PyArg_ParseTuple(args, "KKKKKKK", &a[0], &a[1], &a[2], &a[3], &a[4], &a[5], &a[6])) return nullptr;
     g_entry.step = reinterpret_cast<decltype(g_entry.step)>(a[0]);
     g_entry.step_masked = reinterpret_cast<decltype(g_entry.step_masked)>(a[1]);
     g_entry.step_normclip = reinterpret_cast<decltype(g_entry.step_normclip)>(a[2]);
     g_entry.step_diag = reinterpret_cast<decltype(g_entry.step_diag)>(a[3]);
     g_entry.rel_change = reinterpret_cast<decltype(g_entry.rel_change)>(a[4]);
     g_entry.diag_norms = reinterpret_cast<decltype(g_entry.diag_norms)>(a[5]);
+    g_entry.step_host = reinterpret_cast<decltype(g_entry.step_host)>(a[6]);
     Py_RETURN_NONE;
 }
 
@@ -349,6 +378,7 @@ PyCFunction fast(F f) {
 PyMethodDef methods[] = {{"bind", bind_entries, METH_VARARGS, nullptr},
                          {"step", fast(call_step), METH_FASTCALL, nullptr},
                          {"step_masked", fast(call_step_masked), METH_FASTCALL, nullptr},
+                         {"step_host", fast(call_step_host), METH_FASTCALL, nullptr},
                          {"diag_norms", fast(call_diag_norms), METH_FASTCALL, nullptr},
                          {"rel_change", fast(call_rel_change), METH_FASTCALL, nullptr},
                          {nullptr, nullptr, 0, nullptr}};

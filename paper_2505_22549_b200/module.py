@@ -19,7 +19,7 @@ if _native.torch_version != str(torch.__version__):
 
 _entry = lambda f: ctypes.cast(f, ctypes.c_void_p).value
 _native.bind(*(_entry(getattr(B.raw_lib(), "desloc_" + n))
-               for n in ("step", "step_masked", "step_normclip", "step_diag", "rel_change", "get_diag_norms")))
+               for n in ("step", "step_masked", "step_normclip", "step_diag", "rel_change", "get_diag_norms", "step_host")))
 
 _GRAD_MISFIT = "gradient tensor of wrong dtype, size or layout"
 _SNAP_MISFIT = "snapshot tensor of wrong dtype, size or layout"
@@ -176,10 +176,10 @@ class DesLoc:
     def step_host(self, t: int, lr: float, host_grads, dev_grads, clip_bound: float = 0.0) -> int:
         """Step t with gradients in (pinned) host tensors; dev_grads are device staging tensors."""
         hp = self._fill(self._table2, host_grads, self.grad_dtype, 1, _HOST_MISFIT)
-        n = self.M * len(self.numel)
-        at = lambda address: (ctypes.c_void_p * n).from_address(address)
-        stream = torch.cuda.current_stream(self.device).cuda_stream
-        return B.desloc_step_host(self.ctx, t, lr, clip_bound, at(hp), at(self._grad_address(dev_grads)), stream)
+        r = _native.step_host(self.ctx, t, lr, clip_bound, hp, self._grad_address(dev_grads), self._index)
+        if r < 0:
+            self._raise(r, "desloc_step_host")
+        return r
 
     def step_masked(self, mask: int, lr: float, grads, clip_bound: float = 0.0) -> None:
         r = _native.step_masked(self.ctx, mask, lr, clip_bound, self._grad_address(grads), self._index)

@@ -291,9 +291,9 @@ DESLOC_API int64_t desloc_plan_chunks_at(const int64_t *numel, int32_t num_tenso
 DESLOC_API int64_t desloc_plan_chunks(const int64_t *numel, int32_t num_tensors, int64_t chunk_elems,
                                       int64_t *out, int64_t cap);
 
-/* Elements per chunk of a context created from cfg (M, numel and num_tensors are read): a multiple
+/* Elements per chunk of a context created from cfg (M, numel, num_tensors, opt and grad_dtype are read): a multiple
    of 1024 elements for M <= 2 and M > 8, of 512 for M = 3..8, up to eight of these on a large problem,
-   fewer on a small one (for M = 3..8 so many that the blocks of an averaging step come in full rounds).  On
+   fewer on a small one (for M = 3..8, as opt and grad_dtype have it, so many that the blocks of an averaging step come in full rounds).  On
    averaging steps a thread block takes a chunk, or a part of one, of all workers (M > 16, and some
    variants and sizes from M = 9 on: a kernel without tiles); on local steps a part of a chunk of one
    worker.  Negative desloc_status on bad input. */

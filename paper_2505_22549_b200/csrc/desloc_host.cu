@@ -149,11 +149,11 @@ void plan_host_groups(std::vector<HostGroup> &groups, const std::vector<desloc::
 
 // Allocates and fills the M-dependent resources; the device must be current.  May throw
 // std::bad_alloc (host vectors).
-cudaError_t make_worker_res(WorkerRes &r, int M, const int64_t *numel, int num_tensors, int64_t total,
+cudaError_t make_worker_res(WorkerRes &r, const desloc_config &cfg, int M, const int64_t *numel, int num_tensors, int64_t total,
                             int64_t nrchunks, bool has_v, float *const *x, float *const *u,
                             float *const *v) {
     // tile plan for this worker count
-    const int64_t chunk_elems = desloc::chunk_elems_for(M, numel, num_tensors);
+    const int64_t chunk_elems = desloc::chunk_elems_for(cfg, M);
     std::vector<int64_t> heads(static_cast<size_t>(num_tensors));
     for (int32_t k = 0; k < num_tensors; ++k) heads[k] = desloc::head_elems(x[k], numel[k]);
     const int64_t nchunks = desloc::count_chunks(numel, num_tensors, chunk_elems, heads.data());
@@ -526,7 +526,7 @@ int64_t desloc_chunk_elems(const desloc_config *cfg) {
     if (cfg->M < 1 || cfg->M > DESLOC_MAX_M || cfg->num_tensors < 1) return DESLOC_E_RANGE;
     for (int32_t k = 0; k < cfg->num_tensors; ++k)
         if (cfg->numel[k] < 1) return DESLOC_E_RANGE;
-    return desloc::chunk_elems_for(cfg->M, cfg->numel, cfg->num_tensors);
+    return desloc::chunk_elems_for(*cfg, cfg->M);
 }
 
 int64_t desloc_plan_chunks_at(const int64_t *numel, int32_t num_tensors, int64_t chunk_elems,
@@ -583,7 +583,7 @@ int desloc_create(desloc_ctx **out, const desloc_config *cfg, float *const *x, f
     // the step kernels' made no measurable difference, and this way the norms do not depend on
     // where the buffers are)
     const int64_t nrchunks = desloc::count_chunks(cfg->numel, cfg->num_tensors, desloc::REDUCE_CHUNK_ELEMS);
-    if (!desloc::grid_fits(cfg->M, cfg->numel, cfg->num_tensors)) return DESLOC_E_RANGE;
+    if (!desloc::grid_fits(*cfg, cfg->M)) return DESLOC_E_RANGE;
 
     desloc_ctx *ctx = new (std::nothrow) desloc_ctx();
     if (!ctx) return DESLOC_E_NOMEM;
@@ -623,7 +623,7 @@ int desloc_create(desloc_ctx **out, const desloc_config *cfg, float *const *x, f
         e = cudaEventCreateWithFlags(&ctx->ev_group[i], cudaEventDisableTiming);
     if (e == cudaSuccess) {
         try {
-            e = make_worker_res(ctx->res, cfg->M, ctx->numel.data(), cfg->num_tensors, total, nrchunks,
+            e = make_worker_res(ctx->res, ctx->cfg, cfg->M, ctx->numel.data(), cfg->num_tensors, total, nrchunks,
                                 cfg->opt != DESLOC_SGDM, x, u, v);
         } catch (const std::bad_alloc &) {
             e = cudaErrorMemoryAllocation;
@@ -779,7 +779,7 @@ int desloc_set_workers(desloc_ctx *ctx, int32_t M_new, int32_t first_new, float 
     const bool has_v = ctx->cfg.opt != DESLOC_SGDM;
     if (has_v && !v) return DESLOC_E_NULL;
     if (M_new < 1 || M_new > DESLOC_MAX_M || first_new < 0 || first_new > M_new) return DESLOC_E_RANGE;
-    if (!desloc::grid_fits(M_new, ctx->numel.data(), ctx->cfg.num_tensors)) return DESLOC_E_RANGE;
+    if (!desloc::grid_fits(ctx->cfg, M_new)) return DESLOC_E_RANGE;
     const int nt = ctx->cfg.num_tensors;
     const int64_t nptr_new = static_cast<int64_t>(M_new) * nt;
     for (int64_t i = 0; i < nptr_new; ++i) {
@@ -795,7 +795,7 @@ int desloc_set_workers(desloc_ctx *ctx, int32_t M_new, int32_t first_new, float 
     WorkerRes fresh;
     if (e == cudaSuccess) {
         try {
-            e = make_worker_res(fresh, M_new, ctx->numel.data(), nt, ctx->total_elems, ctx->nrchunks, has_v, x, u, v);
+            e = make_worker_res(fresh, ctx->cfg, M_new, ctx->numel.data(), nt, ctx->total_elems, ctx->nrchunks, has_v, x, u, v);
             if (ctx->last_grads.capacity() < static_cast<size_t>(nptr_new))
                 ctx->last_grads.reserve(static_cast<size_t>(nptr_new));  // may throw; no state changed yet
         } catch (const std::bad_alloc &) {

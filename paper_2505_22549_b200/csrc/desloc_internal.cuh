@@ -88,26 +88,39 @@ constexpr int NUM_SMS = 148;   // of a B200
 // 8 * 8 rounds of blocks takes the run that fills its last round -- as few rounds of at most 8 tiles as
 // it needs, and the shortest run that does with these.  All-sync steps, Adam, bf16 gradients, against
 // the first rule: eight workers, 400 K parameters 16.2 us instead of 22.7, 700 K 27.3 (32.1), 2 M 72.3 (80.2), 5 M 164.8
-// (172.2); four workers, 1 M 19.5 (21.1), 2 M 36.2 (39.3).
-inline int64_t chunk_elems_for(int32_t M, const int64_t *numel, int32_t num_tensors) {
+// (172.2); four workers, 1 M 19.5 (21.1), 2 M 36.2 (39.3).  A tensor costs a block more for its short first chunk
+// (head_elems), and how many blocks are in a round depends on optimizer and gradient type: without both, models of 47
+// tensors, x averaged, cold in L2, took eight workers x 690 K parameters 35.8 us (now 31.6), x 1 M 46.3 (39.9), with fp32 gradients
+// and ADOPT x 690 K 35.3 (28.7), six x 920 K 35.3 (29.6).
+constexpr int64_t ALIGN_PHASE_ELEMS = 512;
+inline int64_t chunk_elems_for(int opt, bool bf16, int32_t M, const int64_t *numel, int32_t num_tensors) {
     const int64_t T = M <= MAX_MT ? plan_tile_elems(M) : GENERIC_CHUNK_ELEMS;
     const int64_t most = M <= MAX_MT ? max_tiles_per_chunk(M) : 8;
-    int64_t tiles = 0;
-    for (int32_t k = 0; k < num_tensors; ++k) tiles += (numel[k] + T - 1) / T;
+    int64_t tiles = 0, heads = 0;
+    for (int32_t k = 0; k < num_tensors; ++k) {
+        tiles += (numel[k] + T - 1) / T;
+        heads += numel[k] > ALIGN_PHASE_ELEMS ? 1 : 0;
+    }
     int64_t per_chunk = tiles / (4 * NUM_SMS);
     if (M > 2 && M <= MAX_MT) {
-        const int64_t slots = static_cast<int64_t>(NUM_SMS) * step_min_blocks(OPT_ADAM, M, true);
+        const int64_t slots = static_cast<int64_t>(NUM_SMS) * step_min_blocks(opt, M, bf16);
         // chunks of t tiles, a tensor's last one half full on average
-        const auto chunks_with = [&](int64_t t) { return (tiles + num_tensors * (t - 1) / 2 + t - 1) / t; };
-        const int64_t rounds = (chunks_with(most) + slots - 1) / slots;
+        const auto chunks_with = [&](int64_t t) { return (tiles + num_tensors * (t - 1) / 2 + t - 1) / t + heads; };
+        // (at most eight of the kernel's own tiles: ADOPT, eight workers, fp32 gradients, 1.5 M parameters in a round of long
+        // chunks 62 us, in two of shorter ones 57)
+        const int64_t limit = tile_elems(opt, M, bf16) < T ? most / 2 : most;
+        const int64_t rounds = (chunks_with(limit) + slots - 1) / slots;
         if (tiles > 2 * slots && rounds <= 8) {
             per_chunk = 1;
-            while (per_chunk < most && chunks_with(per_chunk) > rounds * slots) ++per_chunk;
+            while (per_chunk < limit && chunks_with(per_chunk) > rounds * slots) ++per_chunk;
         }
     }
     if (per_chunk < 1) per_chunk = 1;
     if (per_chunk > most) per_chunk = most;
     return per_chunk * T;
+}
+inline int64_t chunk_elems_for(const desloc_config &c, int32_t M) {
+    return chunk_elems_for(c.opt, c.grad_dtype == DESLOC_BF16, M, c.numel, c.num_tensors);
 }
 
 // Where the copy engine's 2 KB pieces start matters: measured on B200, tiles that begin 256 or
@@ -122,7 +135,6 @@ inline int64_t chunk_elems_for(int32_t M, const int64_t *numel, int32_t num_tens
 // offsets can lose its 16-byte alignment by the cut; where it keeps 8 bytes, the chunk is
 // updated with 128-bit accesses from global memory (0.66-0.86 of the copy bandwidth), else
 // coordinate by coordinate.
-constexpr int64_t ALIGN_PHASE_ELEMS = 512;
 inline int64_t head_elems(const void *x0, int64_t numel) {
     const uintptr_t a = reinterpret_cast<uintptr_t>(x0);
     if ((a & 3u) != 0) return 0;
@@ -168,9 +180,9 @@ inline int64_t parts_for(int64_t items, int64_t chunk_elems, int opt, int mt, bo
 
 // One thread block per part of a chunk and worker on a local step, one per chunk on the others: does
 // the largest grid of a context with M workers fit, whatever the first chunks are cut to?
-inline bool grid_fits(int32_t M, const int64_t *numel, int32_t num_tensors) {
-    const int64_t nchunks = count_chunks(numel, num_tensors, chunk_elems_for(M, numel, num_tensors)) + num_tensors;
-    const int64_t chunk_elems = chunk_elems_for(M, numel, num_tensors);
+inline bool grid_fits(const desloc_config &c, int32_t M) {
+    const int64_t chunk_elems = chunk_elems_for(c, M);
+    const int64_t nchunks = count_chunks(c.numel, c.num_tensors, chunk_elems) + c.num_tensors;
     const int64_t per_chunk = M * parts_for(chunk_elems, OPT_ADAM, 1, true);
     return nchunks <= 0x7fffffffLL / per_chunk;
 }

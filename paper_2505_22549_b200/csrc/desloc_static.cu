@@ -93,7 +93,7 @@ extern "C" DESLOC_API int desloc_step_static(const desloc_config *cfg, float *co
         if (cfg->opt != DESLOC_SGDM && !v[i]) return DESLOC_E_NULL;
     }
     std::lock_guard<std::mutex> lock(g_mutex);
-    const int64_t chunk_elems = desloc::chunk_elems_for(cfg->M, cfg->numel, cfg->num_tensors);
+    const int64_t chunk_elems = desloc::chunk_elems_for(*cfg, cfg->M);
     for (int32_t k = 0; k < cfg->num_tensors; ++k) g_heads[k] = desloc::head_elems(x[k], cfg->numel[k]);
     const int64_t nchunks = desloc::count_chunks(cfg->numel, cfg->num_tensors, chunk_elems, g_heads);
     if (nchunks > kMaxChunks) return DESLOC_E_TOO_LARGE;

@@ -1,0 +1,31 @@
+"""Chunk lengths of mid-sized problems of three to eight workers: with the short first chunks that tensors off a 2 KB boundary get, the
+blocks of an averaging step come in full rounds, and a round is as many blocks as the optimizer and the gradient type leave room for."""
+import numpy as np
+import pytest
+
+import paper_2505_22549_b200.binding as B
+
+
+def model(width, layers=5):
+    w = width
+    kv, f = w // 3, w * 8 // 3
+    return [w * 3 * w] + [w * w, w * kv, w * kv, w * w, f * w, f * w, w * f, w, w] * layers + [w]
+
+
+def blocks(M, opt, gd, numel, off):
+    cfg = B.make_config(M, numel, opt, gd, 0.9, 0.99, 1e-8, 0.0, 0.0, 1, 1, 1, 0)
+    length = B.desloc_chunk_elems(cfg)
+    at = np.cumsum([0] + [-(-n // 4) * 4 for n in numel])[:-1] * 4 + (1 << 30) + off
+    return length, B.desloc_plan_chunks(numel, length, cap=0, x0=[int(a) for a in at])[0]
+
+
+@pytest.mark.parametrize("M,opt,gd,per_sm", [(8, "adam", "bf16", 2), (6, "adam", "bf16", 2), (6, "sgdm", "bf16", 3), (8, "adopt", "f32", 3),
+                                             (4, "adam", "bf16", 4), (3, "adam", "f32", 4)])
+@pytest.mark.parametrize("width", [97, 104, 128, 150])
+def test_blocks_come_in_full_rounds(M, opt, gd, per_sm, width):
+    length, n = blocks(M, opt, gd, model(width), 16)
+    most = 2048 if (M, gd) == (8, "f32") else 4096
+    assert length % 512 == 0 and 512 <= length <= most
+    slots = 148 * per_sm
+    # no round for a few blocks (the rule takes every tensor's last chunk as half full, so that a list can be off by some)
+    assert n <= slots or n % slots == 0 or n % slots > 0.4 * slots

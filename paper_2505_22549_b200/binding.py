@@ -109,6 +109,8 @@ _lib.desloc_testing_set_max_blocks.restype = ctypes.c_int
 _lib.desloc_testing_set_max_blocks.argtypes = [_P, ctypes.c_int64]
 _lib.desloc_testing_set_staging.restype = ctypes.c_int
 _lib.desloc_testing_set_staging.argtypes = [_P, ctypes.c_int32]
+_lib.desloc_testing_kernel_of.restype = ctypes.c_int32
+_lib.desloc_testing_kernel_of.argtypes = [ctypes.POINTER(DeslocConfig), ctypes.c_uint32, ctypes.c_int64]
 _lib.desloc_testing_set_wait_limit.restype = ctypes.c_int
 _lib.desloc_testing_set_wait_limit.argtypes = [_P, ctypes.c_int32]
 _lib.desloc_plan_chunks.restype = ctypes.c_int64
@@ -325,6 +327,14 @@ def desloc_testing_set_staging(ctx: int, mode: int) -> None:
     rc = _lib.desloc_testing_set_staging(ctx, int(mode))
     if rc != DESLOC_OK:
         raise DeslocError(rc, "desloc_testing_set_staging")
+
+
+def desloc_testing_kernel_of(cfg: DeslocConfig, mask: int, nchunks: int) -> str:
+    """Test hook (include/desloc_testing.h): which kernel a step of so many chunks runs."""
+    n = int(_lib.desloc_testing_kernel_of(ctypes.byref(cfg), mask, int(nchunks)))
+    if n < 0:
+        raise DeslocError(n, "desloc_testing_kernel_of")
+    return ("tiles", "runtime_m", "lanes", "crowd")[n]
 
 
 def desloc_testing_set_wait_limit(ctx: int, polls: int) -> None:

@@ -319,6 +319,15 @@ bool gather_host_runs(const desloc_ctx *ctx, const void *const *host_grads, cons
     return flush();
 }
 
+// Raises the kernel's shared-memory limit, once per kernel and context (the attribute call costs a microsecond that a
+// latency-bound step notices).
+cudaError_t prepare_once(desloc_ctx *ctx, const desloc::LaunchPlan &plan) {
+    if (std::find(ctx->prepared.begin(), ctx->prepared.end(), plan.fn) != ctx->prepared.end()) return cudaSuccess;
+    const cudaError_t e = desloc::prepare_launch(plan);
+    if (e == cudaSuccess && ctx->prepared.size() < ctx->prepared.capacity()) ctx->prepared.push_back(plan.fn);
+    return e;
+}
+
 // max_norm > 0: norm-based clipping first (two reduction launches), then the step.
 // diag: the step kernel also accumulates the per-chunk sums of squares of g, x_{t+1} and d_t.
 // host_grads != nullptr: the gradients are first copied from host memory into `grads` (device),
@@ -419,15 +428,6 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
             const bool cap = lp.strides && ctx->max_blocks > 0 && lp.grid > ctx->max_blocks;
             return dim3(static_cast<unsigned>(cap ? ctx->max_blocks : lp.grid), lp.grid_y);
         };
-        // (once per kernel: the attribute call costs a microsecond that a latency-bound step notices)
-        if (std::find(ctx->prepared.begin(), ctx->prepared.end(), plan.fn) == ctx->prepared.end()) {
-            e = desloc::prepare_launch(plan);
-            if (e != cudaSuccess) {
-                rc = cuda_fail(ctx, e);
-                break;
-            }
-            if (ctx->prepared.size() < ctx->prepared.capacity()) ctx->prepared.push_back(plan.fn);
-        }
         bool on_device = !host_grads;
         if (host_grads) {
             desloc::HostRuns runs;
@@ -438,13 +438,22 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
             }
         }
         if (on_device) {
+            if (e == cudaSuccess) e = prepare_once(ctx, plan);
             if (e == cudaSuccess)
                 e = desloc::launch_kernel(plan.fn, capped(plan), dim3(plan.threads, plan.threads_y), plan.smem, stream, params, plan.overlap);
             if (e == cudaSuccess) ctx->launches += 1;
         } else {
+            // A group of chunks may run in another kernel than the whole list would.  All are planned and prepared
+            // before the first one is launched: a kernel that is refused leaves the state as it was.
+            desloc::LaunchPlan plans[kHostGroups];
+            for (size_t gi = 0; gi < ctx->res.groups.size() && e == cudaSuccess; ++gi) {
+                const HostGroup &grp = ctx->res.groups[gi];
+                plans[gi] = desloc::plan_launch(c, mask, grp.c1 - grp.c0, ctx->res.chunk_elems, diag, false, layout, lanes_ok);
+                e = plans[gi].fn ? prepare_once(ctx, plans[gi]) : cudaErrorInvalidDeviceFunction;
+            }
             // The device gradient buffers may still be read by earlier work on `stream`.
             const size_t gsz = c.grad_dtype == DESLOC_BF16 ? 2 : 4;
-            e = cudaEventRecord(ctx->ev_entry, stream);
+            if (e == cudaSuccess) e = cudaEventRecord(ctx->ev_entry, stream);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->copy_stream, ctx->ev_entry, 0);
             for (size_t gi = 0; gi < ctx->res.groups.size() && e == cudaSuccess; ++gi) {
                 const HostGroup &grp = ctx->res.groups[gi];
@@ -477,7 +486,7 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
                 a.chunks = ctx->res.d_chunks + grp.c0;
                 a.nchunks = grp.c1 - grp.c0;
                 a.diag_chunk0 = grp.c0;
-                const desloc::LaunchPlan gp = desloc::plan_launch(c, mask, a.nchunks, ctx->res.chunk_elems, diag, false, layout, lanes_ok);
+                const desloc::LaunchPlan &gp = plans[gi];
                 desloc::fill_plan(a, gp);
                 if (ctx->staging_mode >= 0 && !gp.whole) a.direct = ctx->staging_mode;
                 // (no overlap: this kernel also depends on the other stream's copies)
@@ -874,6 +883,14 @@ int desloc_testing_set_wait_limit(desloc_ctx *ctx, int32_t polls) {
     ctx->wait_limit = polls < 0 ? desloc::DEFAULT_WAIT_LIMIT : polls;
     if (polls < 0) *static_cast<volatile int *>(ctx->h_err) = 0;
     return DESLOC_OK;
+}
+
+int32_t desloc_testing_kernel_of(const desloc_config *cfg, uint32_t mask, int64_t nchunks) {
+    if (!cfg || !cfg->numel) return DESLOC_E_NULL;
+    if (validate_config(cfg) != DESLOC_OK || (mask & ~7u) || nchunks < 1) return DESLOC_E_INVALID;
+    const desloc::LaunchPlan p = desloc::plan_launch(*cfg, mask, nchunks, desloc::chunk_elems_for(*cfg, cfg->M), false, false,
+                                                     desloc::GradLayout::FIT);
+    return p.fn ? static_cast<int32_t>(p.kernel) : DESLOC_E_INVALID;
 }
 
 int desloc_last_cuda_error(const desloc_ctx *ctx) { return ctx ? ctx->last_cuda_error : 0; }

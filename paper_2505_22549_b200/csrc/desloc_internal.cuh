@@ -244,7 +244,9 @@ inline const void *lookup_lanes_kernel(int opt, bool post, bool bf16, int mt, in
 }
 
 // Which kernel a step of this configuration runs, and over how many blocks.
+enum class Kernel { TILES, RUNTIME_M, LANES, CROWD };
 struct LaunchPlan {
+    Kernel kernel = Kernel::TILES;
     const void *fn = nullptr;
     long long grid = 0;       // blocks in x
     unsigned grid_y = 1;      // one-replica kernel: workers
@@ -367,6 +369,7 @@ inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, long long n
     // (chunks times chunk length: no fewer coordinates than there are, so that a list of very many tiny tensors, most of
     // whose work items would be empty, stays with the tiles)
     if (lanes_ok && !diag && mt <= MAX_MT && nchunks * chunk_elems * c.M <= lanes_most(mt)) {
+        p.kernel = Kernel::LANES;
         p.fn = lookup_lanes_kernel(c.opt, post, bf16, mt, static_cast<int>(kmask));
         p.part_elems = lanes_part_elems(mt);
         p.parts = static_cast<int>((chunk_elems + p.part_elems - 1) / p.part_elems);
@@ -383,6 +386,7 @@ inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, long long n
         p.grid = nchunks * p.parts;
         const int kind = threads > 512 ? CROWD_1024 : threads > 256 ? CROWD_512
                          : p.grid <= crowd_min_blocks(CROWD_FEW) * NUM_SMS ? CROWD_FEW : CROWD_256;
+        p.kernel = Kernel::CROWD;
         p.fn = lookup_crowd_kernel(c.opt, post, bf16, kind, static_cast<int>(kmask));
         p.threads = L;
         p.threads_y = c.M;
@@ -403,6 +407,7 @@ inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, long long n
     const bool generic = !local && c.M > MAX_MT &&
                          (c.M > MAX_TILE_MT || post || diag || off_generic ||
                           generic_fills_rounds_better(c, kmask, nchunks, chunk_elems));
+    p.kernel = generic ? Kernel::RUNTIME_M : Kernel::TILES;
     p.fn = generic ? lookup_generic_kernel(c.opt, post, bf16, static_cast<int>(kmask), diag)
                    : lookup_step_kernel(c.opt, post, bf16, c.M, static_cast<int>(kmask), diag);
     p.strides = p.overlap = !generic;

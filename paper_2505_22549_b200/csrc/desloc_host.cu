@@ -295,28 +295,12 @@ int stage_grads(desloc_ctx *ctx, const void *const *grads, cudaStream_t stream, 
 
 // The gradients of a small problem as contiguous pieces that a kernel can read where they are, in pinned host memory;
 // false where there are too many bytes or pieces, or some of them in memory that only the copy engine reaches.
-bool gather_host_runs(const desloc_ctx *ctx, const void *const *host_grads, const void *const *grads, desloc::HostRuns &runs) {
+bool host_runs_of(const desloc_ctx *ctx, const void *const *host_grads, const void *const *grads, desloc::HostRuns &runs) {
     const desloc_config &c = ctx->cfg;
-    const size_t gsz = c.grad_dtype == DESLOC_BF16 ? 2 : 4;
-    if (ctx->total_elems > desloc::HOST_KERNEL_BYTES / static_cast<int64_t>(gsz) / c.M) return false;
-    const char *from = nullptr;
-    char *to = nullptr;
-    size_t bytes = 0;
-    const auto flush = [&] { return bytes == 0 || (runs.add(from, to, bytes) && desloc::device_reads_host(from, bytes)); };
-    for (int64_t i = 0; i < ctx->nptr; ++i) {
-        const char *hp = static_cast<const char *>(host_grads[i]);
-        char *dp = static_cast<char *>(const_cast<void *>(grads[i]));
-        const size_t n = static_cast<size_t>(ctx->numel[i % c.num_tensors]) * gsz;
-        if (bytes != 0 && hp == from + bytes && dp == to + bytes) {
-            bytes += n;
-            continue;
-        }
-        if (!flush()) return false;
-        from = hp;
-        to = dp;
-        bytes = n;
-    }
-    return flush();
+    const int64_t gsz = c.grad_dtype == DESLOC_BF16 ? 2 : 4;
+    return ctx->total_elems <= desloc::HOST_KERNEL_BYTES / gsz / c.M &&
+           desloc::gather_host_runs(host_grads, grads, ctx->nptr, c.numel, c.num_tensors, static_cast<size_t>(gsz), runs,
+                                    desloc::device_reads_host);
 }
 
 // Raises the kernel's shared-memory limit, once per kernel and context (the attribute call costs a microsecond that a
@@ -431,7 +415,7 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
         bool on_device = !host_grads;
         if (host_grads) {
             desloc::HostRuns runs;
-            if (gather_host_runs(ctx, host_grads, grads, runs)) {
+            if (host_runs_of(ctx, host_grads, grads, runs)) {
                 e = desloc::launch_host_copy(runs, stream);
                 if (e == cudaSuccess) ctx->launches += 1;
                 on_device = true;

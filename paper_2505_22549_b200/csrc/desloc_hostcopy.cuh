@@ -26,6 +26,34 @@ struct HostRuns {
     }
 };
 
+// host[i], dev[i]: n pieces of numel[i mod nt] elements, merged where they follow one another on both sides.  readable(from, bytes)
+// is asked once per run, and only when all of them have found room: asked as they came, a list of 72 pieces put 64 questions
+// to the driver at every step before it went by copies all the same (time of the calling thread alone: the copies' 290 us hide it).
+template <typename Readable>
+bool gather_host_runs(const void *const *host, const void *const *dev, int64_t n, const int64_t *numel, int32_t nt, size_t elem_bytes,
+                      HostRuns &runs, const Readable &readable) {
+    const char *from = nullptr;
+    char *to = nullptr;
+    size_t bytes = 0;
+    for (int64_t i = 0; i < n; ++i) {
+        const char *hp = static_cast<const char *>(host[i]);
+        char *dp = static_cast<char *>(const_cast<void *>(dev[i]));
+        const size_t len = static_cast<size_t>(numel[i % nt]) * elem_bytes;
+        if (bytes != 0 && hp == from + bytes && dp == to + bytes) {
+            bytes += len;
+            continue;
+        }
+        if (bytes != 0 && !runs.add(from, to, bytes)) return false;
+        from = hp;
+        to = dp;
+        bytes = len;
+    }
+    if (bytes != 0 && !runs.add(from, to, bytes)) return false;
+    for (int i = 0; i < runs.n; ++i)
+        if (!readable(runs.src[i], runs.bytes[i])) return false;
+    return true;
+}
+
 // Can a kernel read all of these bytes at the addresses the host uses?  (Every byte page-locked host memory that is mapped there.)
 bool device_reads_host(const void *p, size_t bytes);
 

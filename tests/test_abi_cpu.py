@@ -51,6 +51,18 @@ def test_header_is_plain_c_and_a_c_program_links(d, tmp_path):
     assert "abi_check: ok" in r.stdout
 
 
+def test_host_gradients_are_counted_before_the_driver_is_asked(tmp_path):
+    """Pieces of host gradients: merged where they touch, at most 64, no question about any of a longer list."""
+    import subprocess
+    csrc = os.path.join(ROOT, "paper_2505_22549_b200", "csrc")
+    exe = str(tmp_path / "host_runs_check")
+    cuda = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")
+    subprocess.check_call(["g++", "-std=c++17", "-Wall", "-Wextra", "-Werror", "-isystem", cuda, "-I", csrc,
+                           os.path.join(ROOT, "tests", "c_abi", "host_runs_check.cpp"), "-o", exe])
+    r = subprocess.run([exe], capture_output=True, text=True)
+    assert r.returncode == 0 and "host_runs_check: ok" in r.stdout, r.stdout + r.stderr
+
+
 def test_sync_mask_matches_oracle_schedule(d):
     for opt, oid in (("adam", oracle.ADAM), ("adopt", oracle.ADOPT), ("sgdm", oracle.SGDM)):
         for K in [(4, 8, 16), (1, 1, 1), (16, 64, 256), (0, 0, 0), (3, 0, 7), (256, 768, 1536)]:

@@ -78,7 +78,7 @@ struct HostGroup {
 struct WorkerRes {
     desloc::Chunk *d_chunks = nullptr;   // tiles of the step kernels
     int64_t nchunks = 0;
-    int64_t chunk_elems = 0;             // longest chunk of the plan
+    desloc::ChunkSet set;                // all of them
     long long *d_tstart = nullptr;       // [num_tensors + 1] first tile of every tensor
     std::vector<int64_t> heads;          // [num_tensors] elements of the short first chunk
     std::vector<HostGroup> groups;
@@ -156,7 +156,8 @@ cudaError_t make_worker_res(WorkerRes &r, const desloc_config &cfg, int M, const
     const int64_t chunk_elems = desloc::chunk_elems_for(cfg, M);
     std::vector<int64_t> heads(static_cast<size_t>(num_tensors));
     for (int32_t k = 0; k < num_tensors; ++k) heads[k] = desloc::head_elems(x[k], numel[k]);
-    const int64_t nchunks = desloc::count_chunks(numel, num_tensors, chunk_elems, heads.data());
+    r.set = desloc::chunk_set(numel, num_tensors, chunk_elems, heads.data());
+    const int64_t nchunks = r.set.n;
     std::vector<desloc::Chunk> chunks(static_cast<size_t>(nchunks));
     desloc::fill_chunks(numel, num_tensors, chunk_elems, chunks.data(), heads.data());
     std::vector<long long> tstart(static_cast<size_t>(num_tensors) + 1, 0);
@@ -164,7 +165,6 @@ cudaError_t make_worker_res(WorkerRes &r, const desloc_config &cfg, int M, const
         tstart[k + 1] = tstart[k] + desloc::chunks_of(numel[k], chunk_elems, heads[k]);
     plan_host_groups(r.groups, chunks, numel, total);
     r.nchunks = nchunks;
-    r.chunk_elems = chunk_elems;
     r.heads.swap(heads);
     cudaError_t e0 = cudaMalloc(&r.d_chunks, chunks.size() * sizeof(desloc::Chunk));
     if (e0 == cudaSuccess)
@@ -382,8 +382,7 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
         const desloc::GradLayout layout =
             inline_g ? desloc::grad_layout(c, grads, ctx->res.heads.data()) : ctx->last_layout;
         const bool lanes_ok = ctx->staging_mode < 0 && ctx->max_blocks == 0;
-        const desloc::LaunchPlan plan = desloc::plan_launch(c, mask, ctx->res.nchunks, ctx->res.chunk_elems, diag,
-                                                            max_norm > 0.f, layout, lanes_ok);
+        const desloc::LaunchPlan plan = desloc::plan_launch(c, mask, ctx->res.set, diag, max_norm > 0.f, layout, lanes_ok);
         if (!plan.fn) {
             rc = DESLOC_E_INVALID;
             break;
@@ -432,7 +431,9 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
             desloc::LaunchPlan plans[kHostGroups];
             for (size_t gi = 0; gi < ctx->res.groups.size() && e == cudaSuccess; ++gi) {
                 const HostGroup &grp = ctx->res.groups[gi];
-                plans[gi] = desloc::plan_launch(c, mask, grp.c1 - grp.c0, ctx->res.chunk_elems, diag, false, layout, lanes_ok);
+                desloc::ChunkSet set = ctx->res.set;
+                set.n = grp.c1 - grp.c0;
+                plans[gi] = desloc::plan_launch(c, mask, set, diag, false, layout, lanes_ok);
                 e = plans[gi].fn ? prepare_once(ctx, plans[gi]) : cudaErrorInvalidDeviceFunction;
             }
             // The device gradient buffers may still be read by earlier work on `stream`.
@@ -869,11 +870,13 @@ int desloc_testing_set_wait_limit(desloc_ctx *ctx, int32_t polls) {
     return DESLOC_OK;
 }
 
-int32_t desloc_testing_kernel_of(const desloc_config *cfg, uint32_t mask, int64_t nchunks) {
+int32_t desloc_testing_kernel_of(const desloc_config *cfg, uint32_t mask, int64_t nchunks, int64_t *blocks) {
     if (!cfg || !cfg->numel) return DESLOC_E_NULL;
-    if (validate_config(cfg) != DESLOC_OK || (mask & ~7u) || nchunks < 1) return DESLOC_E_INVALID;
-    const desloc::LaunchPlan p = desloc::plan_launch(*cfg, mask, nchunks, desloc::chunk_elems_for(*cfg, cfg->M), false, false,
-                                                     desloc::GradLayout::FIT);
+    if (validate_config(cfg) != DESLOC_OK || (mask & ~7u) || nchunks < 0) return DESLOC_E_INVALID;
+    desloc::ChunkSet set = desloc::chunk_set(cfg->numel, cfg->num_tensors, desloc::chunk_elems_for(*cfg, cfg->M));
+    if (nchunks > 0) set.n = nchunks;
+    const desloc::LaunchPlan p = desloc::plan_launch(*cfg, mask, set, false, false, desloc::GradLayout::FIT);
+    if (blocks) *blocks = p.grid * p.grid_y;
     return p.fn ? static_cast<int32_t>(p.kernel) : DESLOC_E_INVALID;
 }
 

@@ -156,6 +156,29 @@ inline int64_t count_chunks(const int64_t *numel, int32_t num_tensors, int64_t c
     return n;
 }
 
+// The chunks of a launch, as its plan sees them.
+struct ChunkSet {
+    int64_t n = 0;
+    int64_t length = 0;     // of a whole chunk,
+    int64_t longest = 0;    // and of the longest one that there is: a list of small tensors has none of whole length
+    bool sparse = false;    // (see chunk_set)
+};
+inline ChunkSet chunk_set(const int64_t *numel, int32_t num_tensors, int64_t chunk_elems, const int64_t *heads = nullptr) {
+    ChunkSet s{count_chunks(numel, num_tensors, chunk_elems, heads), chunk_elems, 0, false};
+    int64_t total = 0;
+    for (int32_t k = 0; k < num_tensors; ++k) {
+        const int64_t head = heads ? heads[k] : 0, rest = numel[k] - head;
+        const int64_t most = rest < chunk_elems ? rest : chunk_elems;
+        s.longest = s.longest > most ? s.longest : most;
+        s.longest = s.longest > head ? s.longest : head;
+        total += numel[k];
+    }
+    // Blocks of the one-replica kernel (desloc_lanes_kernel) that would stand three quarters empty.
+    const int64_t part = lanes_part_elems(1);
+    s.sparse = 4 * total < s.n * ((s.longest + part - 1) / part) * part;
+    return s;
+}
+
 // Blocks that share a chunk of all mt replicas (of one, for mt = 1).
 inline int64_t parts_for(int64_t chunk_elems, int opt, int mt, bool bf16) {
     const int64_t most = most_part_elems(opt, mt, bf16);
@@ -265,6 +288,8 @@ struct LaunchPlan {
 // skip the staging.  Measured on 4096 parameters and two workers: 3.08 us per step in a
 // CUDA graph of 16 steps against 3.34 us staged.
 constexpr long long DIRECT_GRID = 2 * NUM_SMS;
+// Blocks of desloc_lanes_kernel that are resident at once.
+constexpr long long LANES_WAVE = 10 * NUM_SMS;
 // One-replica kernel: at most seven blocks of one tile per SM go straight to global memory.
 constexpr long long LOCAL_WAVE = 7 * NUM_SMS;
 
@@ -352,10 +377,22 @@ inline int64_t crowd_most(int mt) {
     return mt < 12 ? 1500000 : mt <= 16 ? 2500000 : mt <= 32 ? 4000000 : mt <= 64 ? 8000000 : 10000000;
 }
 
+// A part of a chunk per block, as many as the longest chunk has.  (With as many as a chunk of whole length has, lists of small
+// tensors launched 2 to 64 times the blocks that had work, a nanosecond each: 200 tensors of 78 elements x 12 workers, averaged,
+// 7.6 us where the tiles took 4.8; 38 of 16 elements x 128 workers, local, 11.1 and 6.1.)
+inline void plan_parts(LaunchPlan &p, const ChunkSet &chunks, int part_elems) {
+    p.part_elems = part_elems;
+    p.parts = static_cast<int>((chunks.longest + part_elems - 1) / part_elems);
+    p.grid = chunks.n * p.parts;
+    p.strides = false;
+}
+
 // lanes_ok: (false in tests of the tile kernels)
-inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, long long nchunks, int64_t chunk_elems,
+inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, const ChunkSet &chunks,
                               bool diag, bool scaled, GradLayout layout, bool lanes_ok = true) {
     LaunchPlan p;
+    const long long nchunks = chunks.n;
+    const int64_t chunk_elems = chunks.length;
     // The mean of one replica is the replica: M = 1 always runs the local kernel.
     const uint32_t kmask = (c.M == 1) ? 0u : mask;
     const bool post = (c.flags & DESLOC_FLAG_POST_AVERAGE) != 0;
@@ -366,24 +403,24 @@ inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, long long n
     // gradients): 6.52 TB/s in tiles, 6.29 in the runtime-M kernel; nine workers 6.2 and 5.89.
     const int mt = local ? 1 : c.M;
     const int64_t replicas = local ? c.M : 1;
-    // (chunks times chunk length: no fewer coordinates than there are, so that a list of very many tiny tensors, most of
-    // whose work items would be empty, stays with the tiles)
+    // (chunks times chunk length: no fewer coordinates than there are, so that a list of very many tiny tensors
+    // stays with the tiles)
     if (lanes_ok && !diag && mt <= MAX_MT && nchunks * chunk_elems * c.M <= lanes_most(mt)) {
-        p.kernel = Kernel::LANES;
-        p.fn = lookup_lanes_kernel(c.opt, post, bf16, mt, static_cast<int>(kmask));
-        p.part_elems = lanes_part_elems(mt);
-        p.parts = static_cast<int>((chunk_elems + p.part_elems - 1) / p.part_elems);
-        p.threads = LANES_THREADS;
-        p.grid = nchunks * p.parts;
-        if (local) p.grid_y = static_cast<unsigned>(c.M);
-        p.strides = false;
-        return p;
+        plan_parts(p, chunks, lanes_part_elems(mt));
+        // (Sparse lists, see chunk_set, of more than a wave of blocks: 0.54 to 1.75 of the tiles' time, on average 1.05.  Those
+        // with a fourth of the room filled and more 0.49 to 1.3, on average 0.77.)
+        if (!(local && chunks.sparse && p.grid * c.M > LANES_WAVE)) {
+            p.kernel = Kernel::LANES;
+            p.fn = lookup_lanes_kernel(c.opt, post, bf16, mt, static_cast<int>(kmask));
+            p.threads = LANES_THREADS;
+            if (local) p.grid_y = static_cast<unsigned>(c.M);
+            return p;
+        }
+        p = LaunchPlan();
     }
     if (lanes_ok && !diag && mt > MAX_MT && nchunks * chunk_elems * c.M <= crowd_most(mt)) {
         const int L = crowd_lanes(c.M), threads = c.M * L;
-        p.part_elems = 4 * L;
-        p.parts = static_cast<int>((chunk_elems + p.part_elems - 1) / p.part_elems);
-        p.grid = nchunks * p.parts;
+        plan_parts(p, chunks, 4 * L);
         const int kind = threads > 512 ? CROWD_1024 : threads > 256 ? CROWD_512
                          : p.grid <= crowd_min_blocks(CROWD_FEW) * NUM_SMS ? CROWD_FEW : CROWD_256;
         p.kernel = Kernel::CROWD;
@@ -392,7 +429,6 @@ inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, long long n
         p.threads_y = c.M;
         p.smem = crowd_smem_bytes(c.opt, bf16, c.M);
         p.smem_limit = crowd_smem_limit(kind);
-        p.strides = false;
         return p;
     }
     // Gradients that the copy engine cannot take, in problems of more than four rounds of blocks (smaller ones are served

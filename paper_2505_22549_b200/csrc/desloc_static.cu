@@ -95,11 +95,11 @@ extern "C" DESLOC_API int desloc_step_static(const desloc_config *cfg, float *co
     std::lock_guard<std::mutex> lock(g_mutex);
     const int64_t chunk_elems = desloc::chunk_elems_for(*cfg, cfg->M);
     for (int32_t k = 0; k < cfg->num_tensors; ++k) g_heads[k] = desloc::head_elems(x[k], cfg->numel[k]);
-    const int64_t nchunks = desloc::count_chunks(cfg->numel, cfg->num_tensors, chunk_elems, g_heads);
+    const desloc::ChunkSet set = desloc::chunk_set(cfg->numel, cfg->num_tensors, chunk_elems, g_heads);
+    const int64_t nchunks = set.n;
     if (nchunks > kMaxChunks) return DESLOC_E_TOO_LARGE;
     const uint32_t mask = desloc::mask_at(cfg, t);
-    const desloc::LaunchPlan plan = desloc::plan_launch(*cfg, mask, nchunks, chunk_elems, false, false,
-                                                          desloc::grad_layout(*cfg, grads, g_heads));
+    const desloc::LaunchPlan plan = desloc::plan_launch(*cfg, mask, set, false, false, desloc::grad_layout(*cfg, grads, g_heads));
     if (!plan.fn) return DESLOC_E_INVALID;
 
     int dev_before = -1;

@@ -27,6 +27,18 @@ def test_every_mask_at_the_edges_of_a_piece(M, opt, gd, rho, align, g_shift, pos
         assert np.array_equal(crowd[name].view(np.uint32), other[name].view(np.uint32)), name
 
 
+@pytest.mark.parametrize("M", [9, 12, 33, 129])
+@pytest.mark.parametrize("opt,gd,post", [("adam", "bf16", False), ("adopt", "f32", True)])
+@pytest.mark.parametrize("numel", [(2, 1, 3), (16, 5, 15, 17), (65, 7, 64, 63)])
+def test_lists_of_small_tensors_have_fewer_parts(M, opt, gd, post, numel):
+    w = di.Workload("crowd", opt, M, numel, gd, "normal1", beta2=0.99, eps=1e-2, lr=1e-2, adopt_norm_clip=(opt == "adopt"), seed=M)
+    kw = dict(align=4, forced_masks=[7, 1], v_init=0.25, post=post)
+    crowd, other = run_both(w, 2, **kw), run_both(w, 2, staging=0, **kw)
+    check(crowd)
+    for name in ("gx", "gu", "gv"):
+        assert np.array_equal(crowd[name].view(np.uint32), other[name].view(np.uint32)), name
+
+
 @pytest.mark.parametrize("M,opt,gd,n", [(12, "adam", "bf16", 60_000), (16, "sgdm", "f32", 156_001), (24, "adopt", "bf16", 165_888),
                                         (64, "adam", "f32", 124_929)])
 def test_more_blocks_than_fit_at_once(M, opt, gd, n):

@@ -40,7 +40,7 @@ def run(M, opt, gd, numel, post, kernels):
     cfg = d.make_config(M, numel, opt, gd, eps=1e-3, flags=_flags(d, w, post))
     chunks = [-(-n // d.desloc_chunk_elems(cfg)) for n in numel]
     mask = 3 if opt == "sgdm" else 7
-    assert tuple(d.desloc_testing_kernel_of(cfg, mask, n) for n in (sum(chunks), *chunks)) == kernels
+    assert tuple(d.desloc_testing_kernel_of(cfg, mask, n)[0] for n in (sum(chunks), *chunks)) == kernels
     ea, eb = make_engine(d, w, a, post), make_engine(d, w, b, post)
     host = [torch.empty(b.nflat, dtype=b.g[0].dtype).pin_memory() for _ in range(M)]
     views = [[h[o:o + n] for o, n in zip(b.offs, numel)] for h in host]

@@ -30,6 +30,15 @@ def test_every_mask_at_the_edges_of_a_piece(M, opt, gd, rho, post, align, g_shif
     both_ways(w, len(masks), align=align, g_shift=g_shift, forced_masks=masks, v_init=0.25, post=post)
 
 
+@pytest.mark.parametrize("M", [1, 2, 3, 4, 5, 8])
+@pytest.mark.parametrize("opt,gd,align", [("adam", "bf16", 4), ("sgdm", "f32", 1)])
+@pytest.mark.parametrize("numel", [(2, 1, 3), (64, 5, 63, 65, 64), (161, 7, 160, 159, 256, 257)])
+def test_lists_of_small_tensors_have_fewer_parts(M, opt, gd, align, numel):
+    masks = [3 if opt == "sgdm" else 7, 0, 1]
+    w = di.Workload("lanes", opt, M, numel, gd, "normal1", beta2=0.99, eps=1e-2, lr=1e-2, seed=M)
+    both_ways(w, len(masks), align=align, forced_masks=masks, v_init=0.25)
+
+
 @pytest.mark.parametrize("M,opt,gd,n", [(8, "adam", "bf16", 374784), (8, "adam", "bf16", 374785), (3, "sgdm", "f32", 532480),
                                         (2, "adopt", "bf16", 2490368), (4, "adam", "f32", 1249280)])
 def test_sizes_on_either_side_of_the_tile_kernels(M, opt, gd, n):

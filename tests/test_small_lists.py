@@ -1,0 +1,31 @@
+"""Lists of small tensors: no thread block without work beside those of chunks that end short."""
+import pytest
+
+import paper_2505_22549_b200.binding as B
+
+
+def plan(M, numel, opt, mask):
+    return B.desloc_testing_kernel_of(B.make_config(M, numel, opt, "bf16"), mask)
+
+
+@pytest.mark.parametrize("M,count,size,local,averaging", [
+    # coordinates of a worker per block: 512 on local steps; 256, 160, 128, 64 for two, three, four, five to eight workers;
+    # 64, 32, 16 for nine, twelve, from 33 workers on
+    (1, 100, 5, 1, 1), (2, 56, 200, 1, 1), (2, 30, 257, 1, 2), (3, 30, 161, 1, 2), (4, 56, 200, 1, 2), (5, 200, 73, 1, 2),
+    (8, 200, 64, 1, 1), (8, 20, 511, 1, 8), (9, 100, 28, 1, 1), (12, 200, 78, 1, 3), (24, 100, 600, 2, 19), (64, 38, 200, 1, 13),
+    (128, 70, 2, 1, 1), (256, 38, 17, 1, 2),
+])
+def test_as_many_blocks_as_have_work(M, count, size, local, averaging):
+    kernel, blocks = plan(M, [size] * count, "sgdm", 0)
+    assert kernel == "tiles" or blocks == count * M * local       # (sparse lists: see below)
+    assert kernel == "lanes" or 4 * size < 512 * local and count * M > 1480
+    if M > 1:
+        assert plan(M, [size] * count, "sgdm", 3) == ("lanes" if M <= 8 else "crowd", count * averaging)
+
+
+@pytest.mark.parametrize("M,numel,kernel", [
+    (128, [600] + [2] * 46, "tiles"), (128, [600] + [300] * 46, "lanes"),    # three quarters of the blocks' room empty, or less
+    (15, [600] + [2] * 46, "lanes"),                                         # no more than fit at once: 1480
+])
+def test_sparse_lists_stay_with_the_tiles(M, numel, kernel):
+    assert plan(M, numel, "adam", 0)[0] == kernel

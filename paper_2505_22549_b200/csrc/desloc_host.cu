@@ -71,6 +71,7 @@ struct HostGroup {
     int64_t c0, c1;   // chunks [c0, c1)
     int32_t k0, k1;   // of tensors k0 .. k1,
     int64_t e0, e1;   // the first one from element e0 on, the last one up to element e1
+    int64_t elems;    // in all
 };
 
 // Everything that depends on the worker count M (re-made by desloc_set_workers): the pointer
@@ -127,7 +128,7 @@ void plan_host_groups(std::vector<HostGroup> &groups, const std::vector<desloc::
                       int64_t total) {
     groups.clear();
     int64_t left = total, acc = 0;
-    HostGroup g{0, 0, 0, 0, 0, 0};
+    HostGroup g{0, 0, 0, 0, 0, 0, 0};
     for (size_t c = 0; c < chunks.size(); ++c) {
         const desloc::Chunk &ch = chunks[c];
         const int64_t end = ch.start + ch.count, rest = numel[ch.tensor] - end;
@@ -138,6 +139,7 @@ void plan_host_groups(std::vector<HostGroup> &groups, const std::vector<desloc::
         g.c1 = static_cast<int64_t>(c) + 1;
         g.k1 = ch.tensor;
         g.e1 = end;
+        g.elems = acc;
         groups.push_back(g);
         g.c0 = g.c1;
         g.k0 = rest > 0 ? ch.tensor : ch.tensor + 1;
@@ -433,6 +435,7 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
                 const HostGroup &grp = ctx->res.groups[gi];
                 desloc::ChunkSet set = ctx->res.set;
                 set.n = grp.c1 - grp.c0;
+                set.total = grp.elems;
                 plans[gi] = desloc::plan_launch(c, mask, set, diag, false, layout, lanes_ok);
                 e = plans[gi].fn ? prepare_once(ctx, plans[gi]) : cudaErrorInvalidDeviceFunction;
             }

@@ -161,21 +161,17 @@ struct ChunkSet {
     int64_t n = 0;
     int64_t length = 0;     // of a whole chunk,
     int64_t longest = 0;    // and of the longest one that there is: a list of small tensors has none of whole length
-    bool sparse = false;    // (see chunk_set)
+    int64_t total = 0;      // of all
 };
 inline ChunkSet chunk_set(const int64_t *numel, int32_t num_tensors, int64_t chunk_elems, const int64_t *heads = nullptr) {
-    ChunkSet s{count_chunks(numel, num_tensors, chunk_elems, heads), chunk_elems, 0, false};
-    int64_t total = 0;
+    ChunkSet s{count_chunks(numel, num_tensors, chunk_elems, heads), chunk_elems, 0, 0};
     for (int32_t k = 0; k < num_tensors; ++k) {
         const int64_t head = heads ? heads[k] : 0, rest = numel[k] - head;
         const int64_t most = rest < chunk_elems ? rest : chunk_elems;
         s.longest = s.longest > most ? s.longest : most;
         s.longest = s.longest > head ? s.longest : head;
-        total += numel[k];
+        s.total += numel[k];
     }
-    // Blocks of the one-replica kernel (desloc_lanes_kernel) that would stand three quarters empty.
-    const int64_t part = lanes_part_elems(1);
-    s.sparse = 4 * total < s.n * ((s.longest + part - 1) / part) * part;
     return s;
 }
 
@@ -407,9 +403,12 @@ inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, const Chunk
     // stays with the tiles)
     if (lanes_ok && !diag && mt <= MAX_MT && nchunks * chunk_elems * c.M <= lanes_most(mt)) {
         plan_parts(p, chunks, lanes_part_elems(mt));
-        // (Sparse lists, see chunk_set, of more than a wave of blocks: 0.54 to 1.75 of the tiles' time, on average 1.05.  Those
-        // with a fourth of the room filled and more 0.49 to 1.3, on average 0.77.)
-        if (!(local && chunks.sparse && p.grid * c.M > LANES_WAVE)) {
+        // Local steps of lists whose chunks differ so much in length that three quarters of the blocks' room is empty, in more
+        // than a wave: 0.73 to 1.19 of the tiles' time, 1.04 on average; SGDM, which has the least to load, with 55 % of it
+        // empty, 0.91 to 1.69, 1.2 on average.  With more of the room filled 0.68 to 1.14, 0.89 on average.  Where a block takes a
+        // whole chunk there is one for each, as there would be of tiles: 0.49 to 1.06.
+        const bool sparse = p.parts > 1 && 20 * chunks.total < (c.opt == OPT_SGDM ? 9 : 5) * p.grid * p.part_elems;
+        if (!(local && sparse && p.grid * c.M > LANES_WAVE)) {
             p.kernel = Kernel::LANES;
             p.fn = lookup_lanes_kernel(c.opt, post, bf16, mt, static_cast<int>(kmask));
             p.threads = LANES_THREADS;

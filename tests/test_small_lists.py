@@ -16,16 +16,16 @@ def plan(M, numel, opt, mask):
     (128, 70, 2, 1, 1), (256, 38, 17, 1, 2),
 ])
 def test_as_many_blocks_as_have_work(M, count, size, local, averaging):
-    kernel, blocks = plan(M, [size] * count, "sgdm", 0)
-    assert kernel == "tiles" or blocks == count * M * local       # (sparse lists: see below)
-    assert kernel == "lanes" or 4 * size < 512 * local and count * M > 1480
+    assert plan(M, [size] * count, "sgdm", 0) == ("lanes", count * M * local)
     if M > 1:
         assert plan(M, [size] * count, "sgdm", 3) == ("lanes" if M <= 8 else "crowd", count * averaging)
 
 
-@pytest.mark.parametrize("M,numel,kernel", [
-    (128, [600] + [2] * 46, "tiles"), (128, [600] + [300] * 46, "lanes"),    # three quarters of the blocks' room empty, or less
-    (15, [600] + [2] * 46, "lanes"),                                         # no more than fit at once: 1480
+@pytest.mark.parametrize("M,numel,opt,kernel", [
+    (128, [600] + [2] * 46, "adam", "tiles"), (128, [600] + [300] * 46, "adam", "lanes"),    # three quarters of the blocks' room empty, or less
+    (128, [600] + [470] * 46, "sgdm", "lanes"), (128, [600] + [450] * 46, "sgdm", "tiles"),  # 55 % of it
+    (128, [500] + [2] * 46, "sgdm", "lanes"),                                                # a block to each chunk
+    (15, [600] + [2] * 46, "adam", "lanes"), (16, [600] + [2] * 46, "adam", "tiles"),        # a wave of 1480, or more
 ])
-def test_sparse_lists_stay_with_the_tiles(M, numel, kernel):
-    assert plan(M, numel, "adam", 0)[0] == kernel
+def test_sparse_lists_stay_with_the_tiles(M, numel, opt, kernel):
+    assert plan(M, numel, opt, 0)[0] == kernel

@@ -873,12 +873,12 @@ int desloc_testing_set_wait_limit(desloc_ctx *ctx, int32_t polls) {
     return DESLOC_OK;
 }
 
-int32_t desloc_testing_kernel_of(const desloc_config *cfg, uint32_t mask, int64_t nchunks, int64_t *blocks) {
+int32_t desloc_testing_kernel_of(const desloc_config *cfg, uint32_t mask, int64_t nchunks, int32_t layout, int64_t *blocks) {
     if (!cfg || !cfg->numel) return DESLOC_E_NULL;
-    if (validate_config(cfg) != DESLOC_OK || (mask & ~7u) || nchunks < 0) return DESLOC_E_INVALID;
+    if (validate_config(cfg) != DESLOC_OK || (mask & ~7u) || nchunks < 0 || layout < 0 || layout > 2) return DESLOC_E_INVALID;
     desloc::ChunkSet set = desloc::chunk_set(cfg->numel, cfg->num_tensors, desloc::chunk_elems_for(*cfg, cfg->M));
     if (nchunks > 0) set.n = nchunks;
-    const desloc::LaunchPlan p = desloc::plan_launch(*cfg, mask, set, false, false, desloc::GradLayout::FIT);
+    const desloc::LaunchPlan p = desloc::plan_launch(*cfg, mask, set, false, false, static_cast<desloc::GradLayout>(layout));
     if (blocks) *blocks = p.grid * p.grid_y;
     return p.fn ? static_cast<int32_t>(p.kernel) : DESLOC_E_INVALID;
 }

@@ -29,3 +29,16 @@ def test_blocks_come_in_full_rounds(M, opt, gd, per_sm, width):
     slots = 148 * per_sm
     # no round for a few blocks (the rule takes every tensor's last chunk as half full, so that a list can be off by some)
     assert n <= slots or n % slots == 0 or n % slots > 0.4 * slots
+
+
+@pytest.mark.parametrize("M,opt,gd,layout,finest", [(7, "adopt", "f32", 1, True), (7, "adopt", "bf16", 2, True), (7, "adopt", "bf16", 1, False),
+                                                    (7, "adopt", "f32", 0, False)])
+def test_gradients_that_nothing_wide_takes_leave_no_block_idle(M, opt, gd, layout, finest):
+    """100 tensors of seven tiles: one round of blocks with a chunk each would leave a third of the chip idle; a tile to a
+    block where the gradients are read coordinate by coordinate."""
+    numel = [3448] * 100
+    cfg = B.make_config(M, numel, opt, gd)
+    chunks, length = B.desloc_plan_chunks(numel, B.desloc_chunk_elems(cfg), cap=0)[0], B.desloc_chunk_elems(cfg)
+    kernel, blocks = B.desloc_testing_kernel_of(cfg, 7, 0, layout)
+    assert kernel == "tiles"
+    assert (blocks == chunks * (length // 512)) == finest

@@ -21,6 +21,14 @@ def test_gradients_off_the_states_layout(M, opt, gd, g_shift):
     check(run_both(w, 4, align=8, forced_masks=[0, top, 2, 1], v_init=0.25, g_shift=g_shift, staging=0))
 
 
+@pytest.mark.parametrize("M,opt,gd,g_shift", [(7, "adopt", "f32", 1), (8, "adam", "f32", 2), (6, "adam", "bf16", 1), (3, "sgdm", "f32", 3)])
+@pytest.mark.parametrize("numel", [(3448,) * 100 + (372_003,), (2_100_000 // 3, 511, 1025)])
+def test_mid_sized_problems_off_the_states_layout(M, opt, gd, g_shift, numel):
+    w = di.Workload("layouts", opt, M, numel, gd, "student_t3", lr=1e-2, clip_rho=1.5, beta2=0.99, eps=1e-2,
+                    adopt_norm_clip=(opt == "adopt"), seed=M)
+    check(run_both(w, 2, align=4, forced_masks=[3 if opt == "sgdm" else 7, 2], v_init=0.25, g_shift=g_shift))
+
+
 @pytest.mark.parametrize("M,opt,gd,g_shift", [(1, "adam", "bf16", 4), (1, "sgdm", "f32", 1), (2, "adam", "f32", 1),
                                               (2, "sgdm", "bf16", 4), (4, "adopt", "bf16", 4), (4, "adam", "bf16", 3),
                                               (12, "sgdm", "bf16", 4), (16, "adam", "bf16", 1), (16, "adam", "bf16", 4)])

@@ -403,12 +403,13 @@ inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, const Chunk
     // stays with the tiles)
     if (lanes_ok && !diag && mt <= MAX_MT && nchunks * chunk_elems * c.M <= lanes_most(mt)) {
         plan_parts(p, chunks, lanes_part_elems(mt));
-        // Local steps of lists whose chunks differ so much in length that three quarters of the blocks' room is empty, in more
-        // than a wave: 0.73 to 1.19 of the tiles' time, 1.04 on average; SGDM, which has the least to load, with 55 % of it
-        // empty, 0.91 to 1.69, 1.2 on average.  With more of the room filled 0.68 to 1.14, 0.89 on average.  Where a block takes a
-        // whole chunk there is one for each, as there would be of tiles: 0.49 to 1.06.
-        const bool sparse = p.parts > 1 && 20 * chunks.total < (c.opt == OPT_SGDM ? 9 : 5) * p.grid * p.part_elems;
-        if (!(local && sparse && p.grid * c.M > LANES_WAVE)) {
+        // Local steps of long lists whose chunks differ so much in length that most of the blocks' room is empty.  More than four
+        // waves of chunks, three quarters of the room empty: 0.96 to 1.25 of the tiles' time, 1.09 on average (fewer chunks 0.54 to
+        // 1.15, 0.87; more of the room filled 0.49 to 1.14, 0.82).  SGDM, which has the least to load, two waves and 55 %: 0.95 to
+        // 1.75, 1.3 on average (else 0.58 to 1.37, 0.9).  Where a block takes a whole chunk there is one for each, as there
+        // would be of tiles: 0.49 to 1.06.
+        const bool sgdm = c.opt == OPT_SGDM, sparse = p.parts > 1 && 20 * chunks.total < (sgdm ? 9 : 5) * p.grid * p.part_elems;
+        if (!(local && sparse && nchunks * c.M > (sgdm ? 2 : 4) * LANES_WAVE)) {
             p.kernel = Kernel::LANES;
             p.fn = lookup_lanes_kernel(c.opt, post, bf16, mt, static_cast<int>(kmask));
             p.threads = LANES_THREADS;

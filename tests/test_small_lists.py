@@ -25,7 +25,8 @@ def test_as_many_blocks_as_have_work(M, count, size, local, averaging):
     (128, [600] + [2] * 46, "adam", "tiles"), (128, [600] + [300] * 46, "adam", "lanes"),    # three quarters of the blocks' room empty, or less
     (128, [600] + [470] * 46, "sgdm", "lanes"), (128, [600] + [450] * 46, "sgdm", "tiles"),  # 55 % of it
     (128, [500] + [2] * 46, "sgdm", "lanes"),                                                # a block to each chunk
-    (15, [600] + [2] * 46, "adam", "lanes"), (16, [600] + [2] * 46, "adam", "tiles"),        # a wave of 1480, or more
+    (125, [600] + [2] * 46, "adopt", "lanes"), (126, [600] + [2] * 46, "adopt", "tiles"),    # four waves of 1480 chunks, or more
+    (62, [600] + [2] * 46, "sgdm", "lanes"), (63, [600] + [2] * 46, "sgdm", "tiles"),        # two
 ])
 def test_sparse_lists_stay_with_the_tiles(M, numel, opt, kernel):
     assert plan(M, numel, opt, 0)[0] == kernel

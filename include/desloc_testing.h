@@ -26,8 +26,8 @@ DESLOC_API int desloc_testing_set_max_blocks(desloc_ctx *ctx, int64_t max_blocks
  * blocks per SM of single tiles -- seven on local steps -- skips the staging, since it has nothing to overlap, and
  * so do blocks that take whole chunks because the gradients cannot be staged), 0 = tile kernels for every size,
  * staged whenever alignment allows (but for those whole chunks), 1 = tile kernels that never stage (every chunk is
- * updated straight from global memory).  Results do not depend on it.  DESLOC_E_RANGE for other
- * values.
+ * updated straight from global memory), 2 = tile kernels (or the runtime-M kernel) for every size, staged as the library
+ * decides.  Results do not depend on it.  DESLOC_E_RANGE for other values.
  */
 DESLOC_API int desloc_testing_set_staging(desloc_ctx *ctx, int32_t mode);
 

@@ -324,7 +324,8 @@ def desloc_chunk_elems(cfg: DeslocConfig) -> int:
 
 
 def desloc_testing_set_staging(ctx: int, mode: int) -> None:
-    """Test hook (include/desloc_testing.h): -1 the library decides, 0 always stage, 1 never."""
+    """Test hook (include/desloc_testing.h): -1 the library decides; tile kernels for every size that
+    0 always stage, 1 never, 2 as the library decides."""
     rc = _lib.desloc_testing_set_staging(ctx, int(mode))
     if rc != DESLOC_OK:
         raise DeslocError(rc, "desloc_testing_set_staging")

@@ -234,7 +234,7 @@ struct desloc_ctx {
     int last_cuda_error = 0;
     bool diag_valid = false;        // a diagnostics step has run since the workers last changed
     int64_t max_blocks = 0;         // test hook: cap on the grid (0 = one block per work item)
-    int staging_mode = -1;          // test hook: -1 the library decides, 0 always stage, 1 never
+    int staging_mode = -1;          // test hook: -1 the library decides; tile kernels that 0 always stage, 1 never, 2 as decided
     std::vector<const void *> prepared;  // kernels whose shared-memory limit this context has raised
     cudaStream_t copy_stream = nullptr;
     cudaEvent_t ev_entry = nullptr;
@@ -316,9 +316,9 @@ cudaError_t prepare_once(desloc_ctx *ctx, const desloc::LaunchPlan &plan) {
 
 // max_norm > 0: norm-based clipping first (two reduction launches), then the step.
 // diag: the step kernel also accumulates the per-chunk sums of squares of g, x_{t+1} and d_t.
-// host_grads != nullptr: the gradients are first copied from host memory into `grads` (device),
-// tensor group by tensor group on the context's copy stream, each group's kernel starting as
-// soon as its copies have landed.
+// host_grads != nullptr: the gradients are first brought from host memory into `grads` (device): by a kernel on `stream`
+// where host_runs_of() allows it, else tensor group by tensor group on the context's copy stream, each group's
+// kernel starting as soon as its copies have landed.
 int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
              const void *const *grads, cudaStream_t stream, float max_norm = 0.f,
              const void *const *host_grads = nullptr, bool diag = false) {
@@ -406,7 +406,8 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
         a.err = ctx->d_err;
         a.wait_limit = ctx->wait_limit;
         desloc::fill_plan(a, plan);
-        if (ctx->staging_mode >= 0 && !plan.whole) a.direct = ctx->staging_mode;
+        const bool forced = ctx->staging_mode == 0 || ctx->staging_mode == 1;
+        if (forced && !plan.whole) a.direct = ctx->staging_mode;
 
         void *params[] = {&a};
         const auto capped = [ctx](const desloc::LaunchPlan &lp) {
@@ -476,7 +477,7 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
                 a.diag_chunk0 = grp.c0;
                 const desloc::LaunchPlan &gp = plans[gi];
                 desloc::fill_plan(a, gp);
-                if (ctx->staging_mode >= 0 && !gp.whole) a.direct = ctx->staging_mode;
+                if (forced && !gp.whole) a.direct = ctx->staging_mode;
                 // (no overlap: this kernel also depends on the other stream's copies)
                 e = desloc::launch_kernel(gp.fn, capped(gp), dim3(gp.threads, gp.threads_y), gp.smem, stream, params, false);
                 if (e == cudaSuccess) ctx->launches += 1;
@@ -861,7 +862,7 @@ int desloc_testing_set_max_blocks(desloc_ctx *ctx, int64_t max_blocks) {
 
 int desloc_testing_set_staging(desloc_ctx *ctx, int32_t mode) {
     if (!ctx) return DESLOC_E_NULL;
-    if (mode < -1 || mode > 1) return DESLOC_E_RANGE;
+    if (mode < -1 || mode > 2) return DESLOC_E_RANGE;
     ctx->staging_mode = mode;
     return DESLOC_OK;
 }

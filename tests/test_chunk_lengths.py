@@ -1,5 +1,6 @@
 """Chunk lengths of mid-sized problems of three to eight workers: with the short first chunks that tensors off a 2 KB boundary get, the
-blocks of an averaging step come in full rounds, and a round is as many blocks as the optimizer and the gradient type leave room for."""
+blocks of an averaging step come in few rounds, none of them for a few blocks, and a round is as many blocks as the
+optimizer and the gradient type leave room for."""
 import numpy as np
 import pytest
 
@@ -22,13 +23,30 @@ def blocks(M, opt, gd, numel, off):
 @pytest.mark.parametrize("M,opt,gd,per_sm", [(8, "adam", "bf16", 2), (6, "adam", "bf16", 2), (6, "sgdm", "bf16", 3), (8, "adopt", "f32", 3),
                                              (4, "adam", "bf16", 4), (3, "adam", "f32", 4)])
 @pytest.mark.parametrize("width", [97, 104, 128, 150])
-def test_blocks_come_in_full_rounds(M, opt, gd, per_sm, width):
+def test_no_round_is_for_a_few_blocks(M, opt, gd, per_sm, width):
     length, n = blocks(M, opt, gd, model(width), 16)
     most = 2048 if (M, gd) == (8, "f32") else 4096
     assert length % 512 == 0 and 512 <= length <= most
     slots = 148 * per_sm
-    # no round for a few blocks (the rule takes every tensor's last chunk as half full, so that a list can be off by some)
+    # (the rule takes every tensor's last chunk as half full, so that a list can be off by some)
     assert n <= slots or n % slots == 0 or n % slots > 0.4 * slots
+
+
+@pytest.mark.parametrize("M,opt,gd,per_sm", [(8, "adam", "bf16", 2), (6, "adam", "bf16", 2), (6, "sgdm", "bf16", 3), (8, "adopt", "f32", 3),
+                                             (4, "adam", "bf16", 4), (3, "adam", "f32", 4)])
+@pytest.mark.parametrize("width", [104, 112, 128, 150, 176])
+def test_few_rounds_wherever_the_tensors_lie(M, opt, gd, per_sm, width):
+    """Tensors packed from 16 bytes behind a 2 KB boundary, packed from one, and each on one (no short first chunks: the rule,
+    which knows no addresses, counts them all the same): the rounds that chunks of the greatest length need, or one more, where
+    many tensors end in chunks that the rule takes for half full."""
+    numel, slots, most = model(width), 148 * per_sm, 2048 if (M, gd) == (8, "f32") else 4096
+    assert sum(-(-n // 512) for n in numel) > 2 * slots            # (what the rule asks for)
+    length, packed = blocks(M, opt, gd, numel, 16)
+    rounds = lambda n: -(-n // slots)
+    at = np.cumsum([0] + [-(-n // 4) * 4 for n in numel])[:-1] * 4 + (1 << 30) + 16
+    longest = B.desloc_plan_chunks(numel, most, cap=0, x0=[int(a) for a in at])[0]
+    for n in (packed, blocks(M, opt, gd, numel, 0)[1], B.desloc_plan_chunks(numel, length, cap=0)[0]):
+        assert rounds(n) <= rounds(longest) + 1
 
 
 @pytest.mark.parametrize("M,opt,gd,layout,finest", [(7, "adopt", "f32", 1, True), (7, "adopt", "bf16", 2, True), (7, "adopt", "bf16", 1, False),
@@ -42,3 +60,10 @@ def test_gradients_that_nothing_wide_takes_leave_no_block_idle(M, opt, gd, layou
     kernel, blocks = B.desloc_testing_kernel_of(cfg, 7, 0, layout)
     assert kernel == "tiles"
     assert (blocks == chunks * (length // 512)) == finest
+
+
+def test_what_no_context_accepts_counts_as_adam_and_fp32():
+    numel = model(128)
+    want = B.desloc_chunk_elems(B.make_config(8, numel, "adam", "f32"))
+    assert want != B.desloc_chunk_elems(B.make_config(8, numel, "sgdm", "bf16"))
+    assert B.desloc_chunk_elems(B.make_config(8, numel, 7, 9)) == want

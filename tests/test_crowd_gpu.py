@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 
 import desloc_inputs as di
-from test_parity_gpu import check, run_both
+from test_parity_gpu import _lib, check, run_both
 
 pytestmark = pytest.mark.gpu
 
@@ -17,6 +17,8 @@ def test_every_mask_at_the_edges_of_a_piece(M, opt, gd, rho, align, g_shift, pos
     piece = 64 if M < 12 else 32 if M <= 32 else 16
     numel = (1, 2, 3, piece - 1, piece, piece + 1, piece + 4, 2 * piece, 516, 1031)
     masks = list(range(1, 4 if opt == "sgdm" else 8))
+    cfg = _lib().make_config(M, numel, opt, gd)
+    assert all(_lib().desloc_testing_kernel_of(cfg, mask)[0] == "crowd" for mask in masks)
     w = di.Workload("crowd", opt, M, numel, gd, "normal1", beta1=0.9, beta2=0.99, eps=1e-2, lr=1e-2, weight_decay=0.05,
                     clip_rho=rho, adopt_norm_clip=(opt == "adopt"), seed=M)
     kw = dict(align=align, g_shift=g_shift, forced_masks=masks, v_init=0.25, post=post)
@@ -39,9 +41,19 @@ def test_lists_of_small_tensors_have_fewer_parts(M, opt, gd, post, numel):
         assert np.array_equal(crowd[name].view(np.uint32), other[name].view(np.uint32)), name
 
 
-@pytest.mark.parametrize("M,opt,gd,n", [(12, "adam", "bf16", 60_000), (16, "sgdm", "f32", 156_001), (24, "adopt", "bf16", 165_888),
-                                        (64, "adam", "f32", 124_929)])
+@pytest.mark.parametrize("M,opt,gd,n", [(12, "adam", "bf16", 190_000), (16, "sgdm", "f32", 140_001), (24, "adopt", "bf16", 150_000),
+                                        (64, "adam", "f32", 110_003), (128, "adopt", "f32", 60_000), (256, "adam", "bf16", 30_001)])
 def test_more_blocks_than_fit_at_once(M, opt, gd, n):
+    d = _lib()
+    top = 3 if opt == "sgdm" else 7
+    kernel, blocks = d.desloc_testing_kernel_of(d.make_config(M, [n], opt, gd, flags=1 if opt == "adopt" else 0), top)
+    # (64 warps an SM at most)
+    lanes = 16 if M < 12 else 8 if M <= 32 else 4
+    assert kernel == "crowd" and blocks > 148 * (64 // -(-M * lanes // 32))
     w = di.Workload("crowd", opt, M, (n,), gd, "student_t3", lr=1e-2, clip_rho=1.5, eps=1e-3,
                     adopt_norm_clip=(opt == "adopt"), seed=M)
-    check(run_both(w, 2, align=4, v_init=0.25, forced_masks=[3 if opt == "sgdm" else 7, 2]))
+    kw = dict(align=4, v_init=0.25, forced_masks=[top, 2])
+    crowd, other = run_both(w, 2, **kw), run_both(w, 2, staging=2, **kw)
+    check(crowd)
+    for name in ("gx", "gu") + (("gv",) if crowd["gv"] is not None else ()):
+        assert np.array_equal(crowd[name].view(np.uint32), other[name].view(np.uint32)), name

@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("M,numel,separate,pinned,by_kernel", [
     (2, (1,), False, True, True), (3, (4095, 17, 8193, 1), False, True, True), (4, (2053, 64, 7), True, True, True),
     (8, (4096 + 31,), False, False, False),                 # pageable
-    (8, (33,) * 9, True, True, False),                      # 72 pieces
+    (8, (33,) * 9, True, True, False), (8, (33,) * 8 + (99,), True, True, False),      # 72 pieces
 ])
 def test_host_gradients_of_small_problems(gd, shift_h, shift_d, M, numel, separate, pinned, by_kernel):
     w = di.Workload("hostcopy", "adam", M, numel, gd, "normal1", lr=1e-2, K=(2, 3, 4), eps=1e-3, seed=1)
@@ -38,8 +38,8 @@ def test_host_gradients_of_small_problems(gd, shift_h, shift_d, M, numel, separa
         before = eb.launches()
         assert ea.step(t, f32r(w.lr), a.views(a.g)) == eb.step_host(t, f32r(w.lr), host, b.views(b.g))
         torch.cuda.synchronize()
-        if by_kernel:
-            assert eb.launches() == before + 2          # the copies and the step
+        # by the kernel, the copies and the step; else the step alone, in two groups where a tensor ends at three quarters
+        assert eb.launches() == before + (2 if by_kernel or numel == (33,) * 9 else 1)
         for m in range(M):
             for x, y in zip(a.views(a.g)[m], b.views(b.g)[m]):
                 assert torch.equal(x, y)

@@ -20,12 +20,14 @@ def _valid(st):
                                     ("cfg5_sgdm_desloc", 3), ("cfg2_adam_135m", 12),
                                     ("cfg2_adam_135m", 1)])
 @pytest.mark.parametrize("align", [4, 1])
-def test_normclip_step_matches_oracle(name, M, align):
+@pytest.mark.parametrize("staging", [-1, 0, 1])      # the kernels of small problems; tiles, as large ones run, and not staged
+def test_normclip_step_matches_oracle(name, M, align, staging):
     import paper_2505_22549_b200 as d
     w = di.mini(di.WORKLOADS[name], T=12).replace(M=M, K=(2, 3, 4))
     dev = torch.device("cuda:0")
     st = State(w, dev, align=align)
     eng = make_engine(d, w, st)
+    d.desloc_testing_set_staging(eng.ctx, staging)
     ox, ou = st.to_numpy(st.x), st.to_numpy(st.u)
     ov = st.to_numpy(st.v) if st.v is not None else None
     ocfg = oracle_cfg(w)
@@ -61,7 +63,8 @@ def test_normclip_step_matches_oracle(name, M, align):
 
 
 @pytest.mark.parametrize("M", [2, 8])
-def test_normclip_with_fp32_gradients(M):
+@pytest.mark.parametrize("staging", [-1, 0])
+def test_normclip_with_fp32_gradients(M, staging):
     """fp32 gradients take their own wide path in the sum-of-squares kernel: full chunks, ragged
     tails and misaligned tensors."""
     import paper_2505_22549_b200 as d
@@ -71,6 +74,7 @@ def test_normclip_with_fp32_gradients(M):
     for align in (4, 1):
         st = State(w, dev, align=align)
         eng = make_engine(d, w, st)
+        d.desloc_testing_set_staging(eng.ctx, staging)
         ox, ou, ov = st.to_numpy(st.x), st.to_numpy(st.u), st.to_numpy(st.v)
         valid = _valid(st)
         for t in range(6):

@@ -43,7 +43,7 @@ def run_both(w, T, align=4, byte_shift=0, post=False, v_init=0.0, identical=Fals
     if max_blocks:
         d.desloc_testing_set_max_blocks(eng.ctx, max_blocks)   # blocks stride over the chunks
     if staging is not None:
-        d.desloc_testing_set_staging(eng.ctx, staging)         # 0: always stage, 1: never
+        d.desloc_testing_set_staging(eng.ctx, staging)         # tile kernels that 0: always stage, 1: never, 2: as decided
     ox, ou = st.to_numpy(st.x), st.to_numpy(st.u)
     ov = st.to_numpy(st.v) if st.v is not None else None
     ocfg = oracle_cfg(w, oracle.FLAG_POST_AVERAGE if post else 0)
@@ -104,7 +104,7 @@ def test_cfg1_adam_n4096_full_run():
 @pytest.mark.parametrize("staging", [0, 1])
 def test_every_mask_on_ragged_tensors(opt, M, gd, staging):
     """Tensors of 1..9 elements, one chunk + 1, odd sizes; all 8 sync patterns in turn, twice.
-    A problem this small would skip the staging by itself: it is run staged (tiles through
+    A problem this small would not run in the tile kernels by itself: they run it staged (tiles through
     shared memory wherever alignment allows) and unstaged (everything straight from global
     memory)."""
     numel = (1, 2, 3, 4, 5, 7, 8, 9, 4095, 4096, 4097, 8191, 12289, 31)
@@ -119,10 +119,11 @@ def test_every_mask_on_ragged_tensors(opt, M, gd, staging):
 
 
 def test_small_launches_skip_the_staging_and_give_the_same_bits():
-    """The library's own choice (no staging for a single wave of single-tile chunks) against
-    both forced modes: the arithmetic per coordinate is the same, so are the bits."""
+    """The library's own choice (replicas in the lanes of a warp) against tile kernels as it would launch them (no
+    staging for a single wave of single-tile chunks) and in both forced modes: the arithmetic per coordinate is the
+    same, so are the bits."""
     w = di.Workload("small", "adam", 4, (4096, 1000, 37), "bf16", "normal1", lr=1e-2, K=(2, 3, 4), seed=5)
-    runs = [run_both(w, 8, staging=mode) for mode in (None, 0, 1)]
+    runs = [run_both(w, 8, staging=mode) for mode in (None, 0, 1, 2)]
     for r in runs:
         check(r)
     for r in runs[1:]:
@@ -148,9 +149,11 @@ def test_post_average_ordering(opt, M):
 
 @pytest.mark.parametrize("opt", ["adam", "adopt", "sgdm"])
 @pytest.mark.parametrize("M,post", [(9, False), (16, False), (16, True), (33, True), (64, False), (256, False)])
-def test_many_workers_runtime_m_path(opt, M, post):
-    """More workers than the register-resident kernels hold (M > 8): runtime-M kernel on sync
-    steps, per-worker items on local steps; up to the largest M a context accepts."""
+@pytest.mark.parametrize("staging", [None, 2])
+def test_many_workers_runtime_m_path(opt, M, post, staging):
+    """More workers than the register-resident kernels hold (M > 8): a block of all replicas (staging None), tiles up to
+    sixteen workers and the runtime-M kernel beyond on sync steps, per-worker items on local steps; up to the
+    largest M a context accepts."""
     numel = (3, 4096, 4101, 777)
     nmask = 4 if opt == "sgdm" else 8
     masks = list(range(nmask)) + [nmask - 1, 0]
@@ -158,7 +161,7 @@ def test_many_workers_runtime_m_path(opt, M, post):
                     eps=1e-2, lr=1e-2, weight_decay=0.01, clip_rho=2.0,
                     adopt_norm_clip=(opt == "adopt"), seed=11 + M)
     for align in (4, 1):
-        res = run_both(w, len(masks), align=align, forced_masks=masks, post=post, v_init=0.5)
+        res = run_both(w, len(masks), align=align, forced_masks=masks, post=post, v_init=0.5, staging=staging)
         check(res)
 
 
@@ -343,7 +346,8 @@ def test_step_host_equals_step_with_device_gradients(name):
     ea.close(); eb.close()
 
 
-def test_guard_bands_around_every_tensor_stay_untouched():
+@pytest.mark.parametrize("staging", [-1, 0, 1])
+def test_guard_bands_around_every_tensor_stay_untouched(staging):
     """Each element is written by exactly one thread and nothing outside a tensor is touched:
     tensors are laid out with up to 15 elements of padding between them (and 32 in front and
     behind), filled with a sentinel that must survive every kind of step."""
@@ -372,6 +376,7 @@ def test_guard_bands_around_every_tensor_stay_untouched():
         eng = d.DesLoc(views(X), views(U), views(V) if opt != "sgdm" else None, opt=opt,
                        grad_dtype="bf16", clip_rho=1.0, K=(2, 3, 4),
                        flags=d.DESLOC_FLAG_ADOPT_NORM_CLIP if opt == "adopt" else 0)
+        d.desloc_testing_set_staging(eng.ctx, staging)
         inside = torch.zeros(total, dtype=torch.bool, device=dev)
         for o, n in zip(offs, numel):
             inside[o:o + n] = True

@@ -15,11 +15,12 @@ pytestmark = pytest.mark.gpu
     (16, "adam", "bf16", 196), (12, "adopt", "f32", 593), (9, "sgdm", "bf16", 1200),
 ])
 @pytest.mark.parametrize("extra", [0, -7])
-def test_sizes_where_the_split_changes(M, opt, gd, tiles, extra):
+@pytest.mark.parametrize("staging", [None, 2])       # 2: the smaller ones in tiles, too
+def test_sizes_where_the_split_changes(M, opt, gd, tiles, extra, staging):
     w = di.Workload("rounds", opt, M, (512 * tiles + extra,), gd, "student_t3", lr=1e-2, weight_decay=0.05, clip_rho=1.5,
                     adopt_norm_clip=(opt == "adopt"), eps=1e-3, seed=M)
     top = 3 if opt == "sgdm" else 7
-    check(run_both(w, 2, align=4, v_init=0.25, forced_masks=[top, 0]))
+    check(run_both(w, 2, align=4, v_init=0.25, forced_masks=[top, 0], staging=staging))
 
 
 @pytest.mark.parametrize("numel,launches,M", [

@@ -156,12 +156,17 @@ DESLOC_API int desloc_step(desloc_ctx *ctx, int64_t t, float lr_t, float clip_bo
  *                are to overlap with compute), same indexing and dtype as for desloc_step().
  *   dev_grads  : host array of M*num_tensors DEVICE pointers to caller-owned staging buffers
  *                of the same sizes; they receive the copies and are what the kernels read.
- * The tensor list is cut into up to 8 groups, of falling size (inside a tensor, where a large
+ * Up to 4 MB of gradients in at most 64 pieces (tensors adjacent in both host and device memory
+ * are one piece), all of it page-locked memory that the device reads at the host's addresses
+ * (cudaMallocHost; cudaHostRegister and cudaHostAlloc where these map it): one kernel on `stream`
+ * reads them from there into dev_grads, and the step follows it on `stream`, two launches in all.
+ * Else the tensor list is cut into up to 8 groups, of falling size (inside a tensor, where a large
  * one would make a group too long); each group's gradients are copied on a stream
- * the context owns (tensors adjacent in both host and device memory go as one copy) and the
+ * the context owns (a copy per piece) and the
  * group's part of the step is launched on `stream` as soon as its copies have landed, so all
- * but the last group's compute hides behind the transfers.  The copies wait for work already
- * enqueued on `stream`.  Not available under stream capture (DESLOC_E_INVALID).
+ * but the last group's compute hides behind the transfers.  Either way the gradients are fetched
+ * behind the work already enqueued on `stream`, and host_grads may be written again when that
+ * stream has come past the step.  Not available under stream capture (DESLOC_E_INVALID).
  */
 DESLOC_API int desloc_step_host(desloc_ctx *ctx, int64_t t, float lr_t, float clip_bound_t,
                                 const void *const *host_grads, void *const *dev_grads,
@@ -291,9 +296,11 @@ DESLOC_API int64_t desloc_plan_chunks_at(const int64_t *numel, int32_t num_tenso
 DESLOC_API int64_t desloc_plan_chunks(const int64_t *numel, int32_t num_tensors, int64_t chunk_elems,
                                       int64_t *out, int64_t cap);
 
-/* Elements per chunk of a context created from cfg (M, numel, num_tensors, opt and grad_dtype are read): a multiple
+/* Elements per chunk of a context created from cfg (M, numel, num_tensors, opt and grad_dtype are read; an opt or grad_dtype
+   that desloc_create() refuses counts as Adam or fp32): a multiple
    of 1024 elements for M <= 2 and M > 8, of 512 for M = 3..8, up to eight of these on a large problem,
-   fewer on a small one (for M = 3..8, as opt and grad_dtype have it, so many that the blocks of an averaging step come in full rounds).  On
+   fewer on a small one (for M = 3..8, as opt and grad_dtype have it, so many that the blocks of an averaging step come in few
+   rounds, with a short first chunk counted for every tensor of more than 512 elements, wherever it will lie).  On
    averaging steps a thread block takes a chunk, or a part of one, of all workers (M > 16, and some
    variants and sizes from M = 9 on: a kernel without tiles); on local steps a part of a chunk of one
    worker.  Negative desloc_status on bad input. */

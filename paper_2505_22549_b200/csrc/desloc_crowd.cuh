@@ -55,7 +55,8 @@ __device__ __forceinline__ float column_mean(const float *column, int T, int M) 
 }
 
 // Lanes of a worker, threads of a block and blocks per SM.  FEW: blocks that all fit at once four to an SM, where
-// the registers are better spent than on more blocks (12 x 40 K: 4.2 us against 4.5).
+// the registers are better spent than on more blocks (12 x 40 K: 4.2 us against 4.5; 2320 lists of 9 to 64 workers: with
+// CROWD_256 0.91 to 1.26 of the time, 1.017 on average).
 __host__ __device__ constexpr int crowd_lanes(int M) { return M < 12 ? 16 : M <= 32 ? 8 : 4; }
 constexpr int CROWD_FEW = 0, CROWD_256 = 1, CROWD_512 = 2, CROWD_1024 = 3;
 __host__ __device__ constexpr int crowd_threads(int kind) { return kind <= CROWD_256 ? 256 : kind == CROWD_512 ? 512 : 1024; }

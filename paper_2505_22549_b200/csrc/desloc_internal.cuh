@@ -363,7 +363,8 @@ inline GradLayout grad_layout(const desloc_config &c, const void *const *grads, 
 // Measured with the arrays cold in L2 (Adam, ADOPT, SGDM, both gradient types): local steps of 0.25 to 16 million
 // 0.82 to 0.99 of the tile kernel's time, of a hundred million at the power cap 1.02 to 1.03; two workers up to five
 // million 0.68 to 1.01, four 0.53 to 1.03 (mean 0.85); eight up to 2.4 million 0.39 to 1.03, 3.2 million 0.91 to 1.08; three, and five
-// to seven, of which lanes are idle, up to 1.6 million 0.5 to 1.0, 2.4 million 1.0 to 1.2.
+// to seven, of which lanes are idle, up to 1.6 million 0.5 to 1.0, 2.4 million 1.0 to 1.2.  (Lists of up to 200 tensors: up to
+// 1.1 where the tiles fill a round of blocks exactly, 5 of 3591 above 1.04.)
 inline int64_t lanes_most(int mt) {
     return mt == 1 ? 12000000 : mt == 2 || mt == 4 ? 5000000 : mt == 8 ? 3000000 : 1600000;
 }

@@ -102,17 +102,21 @@ desloc_crowd_kernel(const __grid_constant__ StepArgs a) {
 #pragma unroll
         for (int i = 0; i < N; ++i) s[i] = q.ld(means + i * T);
     };
+    const Quad<true> q4{4 * lx, 1, cnt, true};
+    const auto mean4 = [&](auto &s, auto arrays) { mean_of_arrays(q4, s, arrays, !POST); };
+    if (wide && plain_step<OPT>(a)) {   // (the common form: nothing but its loads behind the wait)
+        wait_for_earlier_kernels();
+        update_quad<OPT, MASK, GT, POST, true, true>(a, 1.f, q4, land, w, replica, mean4);
+        return;
+    }
     wait_for_earlier_kernels();
     const float sc = a.gscale ? a.gscale[m] : 1.f;
     if (wide) {
-        const Quad<true> q{4 * lx, 1, cnt, true};
-        const auto mean = [&](auto &s, auto arrays) { mean_of_arrays(q, s, arrays, !POST); };
-        if (plain_step<OPT>(a)) update_quad<OPT, MASK, GT, POST, true>(a, sc, q, land, w, replica, mean);
-        else update_quad<OPT, MASK, GT, POST, false>(a, sc, q, land, w, replica, mean);
+        update_quad<OPT, MASK, GT, POST, false, true>(a, sc, q4, land, w, replica, mean4);
     } else {
         const Quad<false> q{lx, L, cnt, true};
         const auto mean = [&](auto &s, auto arrays) { mean_of_arrays(q, s, arrays, false); };
-        update_quad<OPT, MASK, GT, POST, false>(a, sc, q, land, w, replica, mean);
+        update_quad<OPT, MASK, GT, POST, false, false>(a, sc, q, land, w, replica, mean);
     }
 }
 

@@ -289,6 +289,8 @@ struct LaunchPlan {
 constexpr long long DIRECT_GRID = 2 * NUM_SMS;
 // Blocks of desloc_lanes_kernel that are resident at once.
 constexpr long long LANES_WAVE = 10 * NUM_SMS;
+// As many that their loads (8 KB a block) find room in the 28 KB of L1 that a kernel with much shared memory leaves behind.
+constexpr long long LANES_FEW = 3 * NUM_SMS;
 // One-replica kernel: at most seven blocks of one tile per SM go straight to global memory.
 constexpr long long LOCAL_WAVE = 7 * NUM_SMS;
 
@@ -418,6 +420,7 @@ inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, const Chunk
             p.fn = lookup_lanes_kernel(c.opt, post, bf16, mt, static_cast<int>(kmask));
             p.threads = LANES_THREADS;
             if (local) p.grid_y = static_cast<unsigned>(c.M);
+            p.direct = p.grid * p.grid_y <= LANES_FEW;
             return p;
         }
         p = LaunchPlan();

@@ -9,7 +9,7 @@
 // Sums have the order of the tile kernels (tree_sum): same bits.
 //
 // Measured on B200, Adam, bf16 gradients, per step of a graph of dependent steps, the arrays cold in L2 from 0.25 million
-// coordinates on (before: the tile kernels).  One array averaged: eight workers x 7.5 K parameters 1.8 us (4.8), x 125 K 6.5
+// coordinates on, without the short way behind the wait at the kernel's end (before: the tile kernels).  One array averaged: eight workers x 7.5 K parameters 1.8 us (4.8), x 125 K 6.5
 // (9.8), x 300 K 12.6 (17.4); four x 15 K 1.7 (2.8); two x 250 K 3.7 (5.4).  Four x 250 K, all averaged, 6.5 (9.1).
 // Local steps: four x 2.5 K 1.5 us (1.7), x 250 K 5.8 (6.6), x 400 K 8.0 (9.5), x 1.25 M 21.9 (22.7).
 #pragma once
@@ -101,13 +101,21 @@ struct Arrays {
         return a[i];
     }
 };
-template <int OPT, int MASK, typename GT, bool POST, bool PLAIN, bool WIDE, typename Mean, typename Where>
+// REGS: loads into registers -- a shared-memory round trip less (0.07 us of a step), where a few blocks per SM leave L1 room enough.
+template <int OPT, int MASK, typename GT, bool POST, bool PLAIN, bool WIDE, bool REGS = false, typename Mean, typename Where>
 __device__ __forceinline__ void update_quad(const StepArgs &a, float sc, const Quad<WIDE> &q, const Landing &land,
                                             const Replica<OPT, GT> &from, const Where &to, const Mean &mean) {
     constexpr bool SX = MASK & SYNC_X, SU = MASK & SYNC_U, HAS_V = OPT != OPT_SGDM, P = OPT != OPT_SGDM;
     constexpr bool SV = (MASK & SYNC_V) && HAS_V;
     FV<4> X{}, U{}, V{}, G{}, un, vn;
-    if constexpr (WIDE) {
+    if constexpr (WIDE && REGS) {
+        if (q.has(0)) {
+            X = ld_f32<4>(reinterpret_cast<const char *>(from.x), q.e);
+            U = ld_f32<4>(reinterpret_cast<const char *>(from.u), q.e);
+            if constexpr (HAS_V) V = ld_f32<4>(reinterpret_cast<const char *>(from.v), q.e);
+            G = ld_grad<4, GT>(from.g, q.e);
+        }
+    } else if constexpr (WIDE) {
         if (q.has(0)) {
             land.load(0, from.x + q.e);
             land.load(1, from.u + q.e);
@@ -224,15 +232,29 @@ __global__ void __launch_bounds__(LANES_THREADS, 10) desloc_lanes_kernel(const _
             }
         }
     };
+    // What follows the wait is a latency-bound step's whole time: the common forms have it to themselves, every branch in front.  A step
+    // of a graph of dependent ones, 4096 parameters x 2 workers, fp32 gradients: 1.06 us instead of 1.35 (loads through shared memory, branches
+    // behind the wait); with the branches in front alone 1.21, with the registers alone 1.28; 1.02 us a kernel that loads and stores x.
+    const auto stay = [&] { return w; };
+    if (wide && plain_step<OPT>(a)) {
+        const Quad<true> q{4 * lx, 1, cnt, live};
+        if (a.direct) {
+            wait_for_earlier_kernels();
+            update_quad<OPT, MASK, GT, POST, true, true, true>(a, 1.f, q, land, w, stay, mean);
+        } else {
+            wait_for_earlier_kernels();
+            update_quad<OPT, MASK, GT, POST, true, true>(a, 1.f, q, land, w, stay, mean);
+        }
+        return;
+    }
     wait_for_earlier_kernels();
     const float sc = a.gscale ? a.gscale[m] : 1.f;
     if (wide) {
         const Quad<true> q{4 * lx, 1, cnt, live};
-        if (plain_step<OPT>(a)) update_quad<OPT, MASK, GT, POST, true>(a, sc, q, land, w, [&] { return w; }, mean);
-        else update_quad<OPT, MASK, GT, POST, false>(a, sc, q, land, w, [&] { return w; }, mean);
+        update_quad<OPT, MASK, GT, POST, false, true>(a, sc, q, land, w, stay, mean);
     } else {
         const Quad<false> q{lx, LW, cnt, live};
-        update_quad<OPT, MASK, GT, POST, false>(a, sc, q, land, w, [&] { return w; }, mean);
+        update_quad<OPT, MASK, GT, POST, false, false>(a, sc, q, land, w, stay, mean);
     }
 }
 

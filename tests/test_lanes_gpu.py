@@ -53,3 +53,15 @@ def test_sizes_on_either_side_of_the_tile_kernels(M, opt, gd, n):
     w = di.Workload("lanes", opt, M, (n,), gd, "student_t3", lr=1e-2, clip_rho=1.5, eps=1e-3,
                     adopt_norm_clip=(opt == "adopt"), seed=M)
     both_ways(w, 2, masks_in_lanes=[0] if n in (374785, 375297, 1249280) else [top, 0], align=4, v_init=0.25, forced_masks=[top, 0])
+
+
+# 444 blocks load into registers, 445 through shared memory: pieces of 512 coordinates of one worker, of 128 of four, 64 of eight (the last
+# ragged; a first chunk off a 2 KB boundary adds a block)
+@pytest.mark.parametrize("M,opt,gd,blocks", [(1, "adam", "bf16", 512), (3, "adopt", "f32", 512), (4, "adam", "f32", 128), (8, "sgdm", "bf16", 64)])
+@pytest.mark.parametrize("more", [-516, -4, 4, 129])
+def test_loads_on_either_side_of_the_registers(M, opt, gd, blocks, more):
+    local = blocks == 512
+    n = 444 * blocks // (M if local else 1) + more
+    masks = [0] if local else [3 if opt == "sgdm" else 7, 1]
+    w = di.Workload("lanes", opt, M, (n,), gd, "normal1", eps=1e-2, lr=1e-2, weight_decay=0.05, seed=M)
+    both_ways(w, len(masks), align=4, forced_masks=masks, v_init=0.25)

@@ -185,7 +185,7 @@ DESLOC_API int desloc_step_masked(desloc_ctx *ctx, uint32_t mask, float lr_t, fl
  * appendix gives the bound on the gradient's L2 norm, 1.0, in its rho column); Algorithms 1-3
  * only have the coordinate-wise clip.  Costs one more read of the gradients: two reduction
  * launches (per-chunk partial sums in fp32, per-worker totals in fp64, fixed order, no
- * atomics) ahead of the step kernel, all enqueued on `stream` without host synchronisation.
+ * atomics), or one for up to 131072 parameters in few tensors, ahead of the step kernel, all enqueued on `stream` without host synchronisation.
  * max_norm must be > 0 and finite.  Other arguments as desloc_step().
  */
 DESLOC_API int desloc_step_normclip(desloc_ctx *ctx, int64_t t, float lr_t, float clip_bound_t,

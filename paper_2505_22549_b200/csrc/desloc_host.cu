@@ -368,16 +368,17 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
         }
         const float *d_gscale = nullptr;
         if (max_norm > 0.f) {
-            e = desloc::launch_grad_norms(ctx->d_rchunks, ctx->nrchunks,
+            int n = 0;
+            e = desloc::launch_grad_norms(ctx->d_rchunks, ctx->nrchunks, ctx->total_elems,
                                           reinterpret_cast<const void *const *>(d_g), c.num_tensors,
                                           c.M, c.grad_dtype == DESLOC_BF16, max_norm,
                                           ctx->res.d_partial, ctx->res.d_norms, ctx->res.d_norms + c.M,
-                                          ctx->d_err, ctx->wait_limit, stream);
+                                          ctx->d_err, ctx->wait_limit, stream, &n);
             if (e != cudaSuccess) {
                 rc = cuda_fail(ctx, e);
                 break;
             }
-            ctx->launches += 2;
+            ctx->launches += n;
             d_gscale = ctx->res.d_norms + c.M;
         }
 

@@ -3,7 +3,7 @@
 // ||s_now - s_then||_2 / ||s_then||_2 (Section 5.1, "Metrics"), and the finalisation of the
 // per-tensor gradient / parameter / update norms a diagnostics step accumulated.
 //
-// All are two-stage and deterministic: stage 1 writes one fp32 partial per work item -- per-thread
+// All are deterministic and, but for the gradient norms of small problems, two-stage: stage 1 writes one fp32 partial per work item -- per-thread
 // sums of up to 128 squares, a shuffle tree, then the warp sums in order; stage 2 adds the
 // partials of a row in fp64 in a fixed pattern.  No atomics.
 #include "desloc_norms.cuh"
@@ -191,6 +191,13 @@ __device__ __forceinline__ void pad_row(float *row, long long n, long long strid
     __syncthreads();
 }
 
+// norm = sqrt(sum of squares), scale = min(1, max_norm / norm) (1 when max_norm <= 0).
+__device__ __forceinline__ void finish_norm(double ss, float max_norm, float *norm, float *scale) {
+    const double nrm = sqrt(ss);
+    *norm = static_cast<float>(nrm);
+    *scale = (max_norm > 0.f && nrm > static_cast<double>(max_norm)) ? static_cast<float>(static_cast<double>(max_norm) / nrm) : 1.f;
+}
+
 constexpr int FINAL_THREADS = 512;
 
 // norms[m] = ||g^m||_2, scales[m] = min(1, max_norm / norms[m]) (1 when max_norm <= 0).
@@ -203,13 +210,7 @@ norm_finalize_kernel(float *partial, long long n, long long stride, float max_no
     float *row = partial + m * stride;
     pad_row(row, n, stride);
     const double ss = row_sum_f64<true>(row, stride, sh);
-    if (threadIdx.x == 0) {
-        const double nrm = sqrt(ss);
-        norms[m] = static_cast<float>(nrm);
-        scales[m] = (max_norm > 0.f && nrm > static_cast<double>(max_norm))
-                        ? static_cast<float>(static_cast<double>(max_norm) / nrm)
-                        : 1.f;
-    }
+    if (threadIdx.x == 0) finish_norm(ss, max_norm, norms + m, scales + m);
 }
 
 __global__ void __launch_bounds__(FINAL_THREADS)
@@ -224,6 +225,89 @@ relchange_finalize_kernel(float *partial, long long n, long long stride, int M, 
     const double num = row_sum_f64<true>(row, stride, sh);
     const double den = row_sum_f64<true>(row2, stride, sh);
     if (threadIdx.x == 0) out[m] = static_cast<float>(sqrt(num) / sqrt(den));
+}
+
+// ---- small problems: gradient norms in one launch -------------------------------------------------
+// Bound: latency, and the launch (2 us of the host's time, as much as the kernel).  A cluster of eight blocks takes all of a worker's gradients: a
+// warp reads a piece of 1024 elements straight into registers, all of it at once, adds the lanes' fp32 sums (32 squares of a
+// piece) in fp64, and the blocks hand their sums to the first one through its shared memory.  A warp has one piece to read, of
+// lists of many tensors half a chunk or one: few wait for a second round trip.
+// A norm-clipped step of SGDM in a graph of dependent steps (before: two stages), bf16 gradients: one worker x 2 K parameters 2.7 us (4.3), x 131 K
+// 3.3 (4.9); four x 33 K 3.6 (5.2), x 120 K in 120 tensors 4.5 (7.2); from Python 5.4 (7.9), where the launch counts.  Rates of
+// change, which the host waits for either way, gained 1 us of 18 at best and lost as much with many tensors: not taken.
+constexpr int SMALL_THREADS = 512, SMALL_BLOCKS = 8, SMALL_PIECE = 1024, SMALL_PIECES = REDUCE_CHUNK_ELEMS / SMALL_PIECE;
+constexpr int SMALL_WARPS = SMALL_BLOCKS * SMALL_THREADS / 32;
+constexpr int64_t SMALL_BYTES = 4 << 20;   // of all workers
+
+__device__ __forceinline__ uint32_t first_block_addr(const void *shared) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(smem_u32(shared)));
+    return r;
+}
+
+template <int MODE>
+__global__ void __cluster_dims__(SMALL_BLOCKS, 1, 1) __launch_bounds__(SMALL_THREADS)
+small_norms_kernel(const Chunk *chunks, int nchunks, const void *const *g, int nt, float max_norm, float *norms, float *scales) {
+    using GT = std::conditional_t<MODE == RED_BF16, bf16_t, float>;
+    constexpr int ESZ = static_cast<int>(sizeof(GT)), PER = 16 / ESZ, ROUNDS = SMALL_PIECE / PER / 32;
+    __shared__ double warp_sums[SMALL_THREADS / 32];
+    __shared__ double block_sums[SMALL_BLOCKS];   // (the first block's)
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int m = static_cast<int>(blockIdx.x) / SMALL_BLOCKS, rank = static_cast<int>(blockIdx.x) % SMALL_BLOCKS;
+    begin_and_let_next_begin();
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // (do the blocks exist?  asked below)
+    // Half chunks or whole ones where there is not a warp for each piece of them.
+    const int at = rank * (SMALL_THREADS / 32) + warp;
+    const int share = nchunks <= SMALL_WARPS / 4 ? SMALL_PIECES : nchunks <= SMALL_WARPS / 2 ? 2 : 1;
+    const int c = at / share, part = REDUCE_CHUNK_ELEMS / share;
+    double total = 0.0;
+    int count = 0;
+    const char *p = nullptr;
+    if (c < nchunks) {
+        const Chunk ch = chunks[c];
+        const int e0 = (at - c * share) * part;
+        count = min(ch.count - e0, part);
+        p = reinterpret_cast<const char *>(g[static_cast<long long>(m) * nt + ch.tensor]) + (ch.start + e0) * static_cast<long long>(ESZ);
+    }
+    wait_for_earlier_kernels();
+#pragma unroll 1
+    for (int done = 0; done < count; done += SMALL_PIECE, p += SMALL_PIECE * ESZ) {
+        // 16-byte loads from the first boundary on; what lies around them element by element
+        const int n = min(count - done, SMALL_PIECE);
+        const uintptr_t addr = reinterpret_cast<uintptr_t>(p);
+        const bool can = addr % ESZ == 0;
+        const int head = can ? min(n, static_cast<int>((0 - addr) & 15u) / ESZ) : 0, wide = can ? (n - head) / PER : 0;
+        const uint4 *w = reinterpret_cast<const uint4 *>(p + head * ESZ);
+        uint4 v[ROUNDS];
+#pragma unroll
+        for (int r = 0; r < ROUNDS; ++r) v[r] = r * 32 + lane < wide ? w[r * 32 + lane] : make_uint4(0, 0, 0, 0);
+        float acc[2] = {0.f, 0.f};
+        for (int i = lane; i < n - wide * PER; i += 32) {
+            const float f = ld_grad<1, GT>(p, i < head ? i : i + wide * PER).a[0];
+            acc[0] = fmaf(f, f, acc[0]);
+        }
+#pragma unroll
+        for (int r = 0; r < ROUNDS; ++r) add_squares<MODE>(v[r], v[r], acc);
+        total += static_cast<double>(acc[0]) + acc[1];
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) total += __shfl_down_sync(0xffffffffu, total, off);
+    if (lane == 0) warp_sums[warp] = total;
+    __syncthreads();
+    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+#pragma unroll
+        for (int w = 0; w < SMALL_THREADS / 32; ++w) t += warp_sums[w];
+        asm volatile("st.shared::cluster.f64 [%0], %1;" :: "r"(first_block_addr(&block_sums[rank])), "d"(t) : "memory");
+    }
+    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (rank == 0 && threadIdx.x == 0) {
+        double t = 0.0;
+#pragma unroll
+        for (int r = 0; r < SMALL_BLOCKS; ++r) t += block_sums[r];
+        finish_norm(t, max_norm, norms + m, scales + m);
+    }
 }
 
 // dst^j[i] = mean over the M_src source replicas of src^m[i] (fp64 sum in the order
@@ -301,9 +385,17 @@ static cudaError_t launch_sumsq(const Chunk *chunks, long long nchunks, const vo
                   M, partial, *stride, err, wait_limit);
 }
 
-cudaError_t launch_grad_norms(const Chunk *chunks, long long nchunks, const void *const *g, int nt,
+cudaError_t launch_grad_norms(const Chunk *chunks, long long nchunks, int64_t elems, const void *const *g, int nt,
                               int M, bool bf16, float max_norm, float *partial, float *norms,
-                              float *scales, int *err, int wait_limit, cudaStream_t stream) {
+                              float *scales, int *err, int wait_limit, cudaStream_t stream, int *launches) {
+    // A piece, half a chunk or a chunk for each warp of a cluster.  Beyond 4 MB in all the two stages read no slower (16 workers x 129 K parameters,
+    // fp32, in 33 and 65 tensors, in a graph: 19.1 and 18.9 us in two stages, 20.0 and 20.2 in one; 2 bytes each 16.8 and 15.3, 15.7 and 14.1).
+    if (elems <= SMALL_WARPS * SMALL_PIECE && nchunks <= SMALL_WARPS && elems * M * (bf16 ? 2 : 4) <= SMALL_BYTES) {
+        *launches = 1;
+        return launch(bf16 ? small_norms_kernel<RED_BF16> : small_norms_kernel<RED_F32>, M * SMALL_BLOCKS, SMALL_THREADS, 0, stream, chunks,
+                      nchunks, g, nt, max_norm, norms, scales);
+    }
+    *launches = 2;
     long long items, stride;
     const cudaError_t e =
         bf16 ? launch_sumsq<RED_BF16>(chunks, nchunks, g, nullptr, nt, M, partial, &items, &stride, err, wait_limit, stream)

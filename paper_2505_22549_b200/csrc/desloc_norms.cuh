@@ -8,12 +8,13 @@ namespace desloc {
 inline long long reduce_row(long long items) { return (items + 3) & ~3LL; }
 
 // partial: scratch of at least M * reduce_row(nchunks) floats; norms, scales: [M] floats, all on the device.
-// scales[m] = min(1, max_norm / ||g^m||_2), or 1 when max_norm <= 0.  Two launches.
+// scales[m] = min(1, max_norm / ||g^m||_2), or 1 when max_norm <= 0.  elems: parameters of a worker; *launches: one (small
+// problems) or two.
 // err, wait_limit: the flag a block sets when its bounded wait for a bulk copy runs out, and the
 // bound (as for the step kernels).
-cudaError_t launch_grad_norms(const Chunk *chunks, long long nchunks, const void *const *g, int nt,
+cudaError_t launch_grad_norms(const Chunk *chunks, long long nchunks, int64_t elems, const void *const *g, int nt,
                               int M, bool bf16, float max_norm, float *partial, float *norms,
-                              float *scales, int *err, int wait_limit, cudaStream_t stream);
+                              float *scales, int *err, int wait_limit, cudaStream_t stream, int *launches);
 
 // partial: scratch of at least 2 * M * reduce_row(nchunks) floats; out[m] = ||now - then|| / ||then||
 // (out may be host memory that the device can write to).  Two launches.

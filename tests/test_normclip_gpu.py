@@ -173,3 +173,27 @@ def test_rel_change_matches_oracle(opt):
             with pytest.raises(d.DeslocError):
                 eng.rel_change(2, st.views(snaps[0]))
         eng.close()
+
+
+# (a cluster of eight blocks per worker up to 131072 elements and 128 chunks of 4096, beyond that two stages; half chunks from 33 chunks on, whole ones from 65)
+@pytest.mark.parametrize("gd", ["bf16", "f32"])
+@pytest.mark.parametrize("numel", [(1,), (7, 1, 9, 1024, 1023, 1025, 4096, 4097), (33,) * 128, (33,) * 129, (4000,) * 32, (3970,) * 33, (2049,) * 63, (2016,) * 65, (131072,), (131073,)])
+@pytest.mark.parametrize("align,shift", [(4, 0), (1, 0), (1, 1), (8, 5)])
+def test_sums_of_small_problems(gd, numel, align, shift):
+    """Norms against fp64 sums of the same arrays.  A lane adds up to 32 squares of a piece in fp32 (two stages: up to 128 and a tree), fp64
+    above: 32 (140) roundings of 6e-8 at most in a sum of positive numbers, half of that in its root."""
+    import paper_2505_22549_b200 as d
+    w = di.Workload("small_sums", "adam", 3, numel, gd, "normal1", lr=1e-2, K=(0, 0, 0), seed=5)
+    st = State(w, torch.device("cuda:0"), align=align, byte_shift=shift)
+    eng = make_engine(d, w, st)
+    valid = _valid(st)
+    bound = 4.5e-6
+    for t in range(2):
+        st.fill_grads(t)
+        g = st.to_numpy(st.g)[:, valid].astype(np.float64)
+        eng.step_normclip(t, 1e-2, st.views(st.g), 0.5)
+        n, s = eng.grad_norms()
+        want = np.sqrt((g * g).sum(axis=1))
+        assert np.allclose(n, want, rtol=bound, atol=0)
+        assert np.allclose(s, np.minimum(1.0, 0.5 / want), rtol=bound, atol=0)
+    eng.close()

@@ -362,21 +362,26 @@ inline GradLayout grad_layout(const desloc_config &c, const void *const *grads, 
 }
 
 // The most coordinates (parameters times workers) of a step with mt replicas that runs with these in the lanes of a warp.
-// Measured with the arrays cold in L2 (Adam, ADOPT, SGDM, both gradient types): local steps of 0.25 to 16 million
-// 0.82 to 0.99 of the tile kernel's time, of a hundred million at the power cap 1.02 to 1.03; two workers up to five
-// million 0.68 to 1.01, four 0.53 to 1.03 (mean 0.85); eight up to 2.4 million 0.39 to 1.03, 3.2 million 0.91 to 1.08; three, and five
-// to seven, of which lanes are idle, up to 1.6 million 0.5 to 1.0, 2.4 million 1.0 to 1.2.  (Lists of up to 200 tensors: up to
-// 1.1 where the tiles fill a round of blocks exactly, 5 of 3591 above 1.04.)
+// Measured with the arrays cold in L2, 4260 points of lists of 1 to 200 tensors (Adam, ADOPT, SGDM, both gradient types), against the tile
+// kernels: local steps of 2 to 7 million 0.91 to 0.95 of the time on average, of 10 to 15 million 0.97, of a hundred million at the power cap
+// 1.02 to 1.03; two workers 3 million 0.95, 4.6 million 1.02; four 5 to 7 million 0.98, 10 million 1.0; eight 3 to 5 million 0.8 to 0.9
+// (from 4.2 million on, behind one another from Python, 1.05 to 1.13), 10 million 1.07; three, and five to seven, of which lanes are idle, 1.5 million 0.7 to 0.9, 2.2 million 0.8 to 1.05, 5 million 1.02 to 1.06.
+// Counted by chunks times their length, as they were before, lists of many tensors left these kernels at half the size.  Averaging steps that
+// moved, 1400 other points, arrays cold and not: five to seven workers 0.86 of the time, eight 0.88; one in 50 is more than 5 % slower (up
+// to 1.35: a single round of blocks with three tiles each, exactly filled).
 inline int64_t lanes_most(int mt) {
-    return mt == 1 ? 12000000 : mt == 2 || mt == 4 ? 5000000 : mt == 8 ? 3000000 : 1600000;
+    return mt == 1 ? 16000000 : mt == 2 ? 5000000 : mt == 3 ? 1700000 : mt == 4 ? 7000000 : mt == 8 ? 3800000 : 2000000;
 }
 
 // The same of averaging steps of more than eight workers that run in desloc_crowd_kernel.  Measured, as above: nine and ten workers
-// up to a million 0.42 to 0.9, 1.6 million 0.73 to 1.1; 12 to 16 up to 2.4 million 0.29 to 1.04 (3.2 million 0.8 to 1.15); 24 and
-// 32 up to four million 0.15 to 0.95 (six 0.75 to 1.16); 64 up to eight million 0.1 to 0.94 (15: 1.1 to 1.4); 128 and 256 up
-// to ten million 0.03 to 0.82 (15: 0.7 to 1.2).
-inline int64_t crowd_most(int mt) {
-    return mt < 12 ? 1500000 : mt <= 16 ? 2500000 : mt <= 32 ? 4000000 : mt <= 64 ? 8000000 : 10000000;
+// 1.5 million 0.67 to 0.79, 2.2 million 0.9 to 0.97; 12 and 14 2.2 million 0.7 to 0.8, 3.2 million 0.87 to 0.98; 16 3.2 million 0.87, 4.6 million 1.0;
+// 20 and 24 3.2 million 0.67, 4.2 million 0.7, 5.6 million 0.9 (up to 1.2); 32 5.6 million 0.78, 10 million 0.9; 64 7 million 0.7, 10 million 0.98; 128 and
+// 256 up to ten million 0.03 to 0.82 (15: 0.7 to 1.2).  SGDM, which has the least to load, by itself: nine and ten 1.8 million 0.8, 2.4 million 1.13; 12 and
+// 14 2.4 million 0.72 to 1.28; 16 2.4 million 0.73, 3.2 million 1.09; 20 and 24 4.2 million 0.94, 5.6 million 1.03; 32 5.6 million 0.72, 10 million 1.03.
+// Steps that moved with the count by coordinates, 900 points: nine and ten workers 0.8 of the time, 12 and 14 0.8, 16 0.72; 1 in 50 more than 5 % slower.
+inline int64_t crowd_most(int opt, int mt) {
+    if (opt == OPT_SGDM) return mt < 12 ? 1590000 : mt < 16 ? 2300000 : mt == 16 ? 2500000 : mt <= 24 ? 4000000 : mt <= 32 ? 5500000 : mt <= 64 ? 8000000 : 10000000;
+    return mt < 12 ? 2100000 : mt < 16 ? 3100000 : mt == 16 ? 4200000 : mt <= 24 ? 4500000 : mt <= 32 ? 8000000 : 10000000;
 }
 
 // A part of a chunk per block, as many as the longest chunk has.  (With as many as a chunk of whole length has, lists of small
@@ -405,9 +410,9 @@ inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, const Chunk
     // gradients): 6.52 TB/s in tiles, 6.29 in the runtime-M kernel; nine workers 6.2 and 5.89.
     const int mt = local ? 1 : c.M;
     const int64_t replicas = local ? c.M : 1;
-    // (chunks times chunk length: no fewer coordinates than there are, so that a list of very many tiny tensors
-    // stays with the tiles)
-    if (lanes_ok && !diag && mt <= MAX_MT && nchunks * chunk_elems * c.M <= lanes_most(mt)) {
+    // (a launch may cover some of the chunks)
+    const int64_t coords = (chunks.total < nchunks * chunk_elems ? chunks.total : nchunks * chunk_elems) * c.M;
+    if (lanes_ok && !diag && mt <= MAX_MT && coords <= lanes_most(mt)) {
         plan_parts(p, chunks, lanes_part_elems(mt));
         // Local steps of long lists whose chunks differ so much in length that most of the blocks' room is empty.  More than four
         // waves of chunks, three quarters of the room empty: 0.96 to 1.25 of the tiles' time, 1.09 on average (fewer chunks 0.54 to
@@ -415,7 +420,9 @@ inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, const Chunk
         // 1.75, 1.3 on average (else 0.58 to 1.37, 0.9).  Where a block takes a whole chunk there is one for each, as there
         // would be of tiles: 0.49 to 1.06.
         const bool sgdm = c.opt == OPT_SGDM, sparse = p.parts > 1 && 20 * chunks.total < (sgdm ? 9 : 5) * p.grid * p.part_elems;
-        if (!(local && sparse && nchunks * c.M > (sgdm ? 2 : 4) * LANES_WAVE)) {
+        // Blocks for more than twice as many coordinates as the line allows, of lists of thousands of tensors: tiles, too.
+        const bool crowded = p.grid * p.part_elems * c.M > 2 * lanes_most(mt);
+        if (!crowded && !(local && sparse && nchunks * c.M > (sgdm ? 2 : 4) * LANES_WAVE)) {
             p.kernel = Kernel::LANES;
             p.fn = lookup_lanes_kernel(c.opt, post, bf16, mt, static_cast<int>(kmask));
             p.threads = LANES_THREADS;
@@ -425,18 +432,21 @@ inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, const Chunk
         }
         p = LaunchPlan();
     }
-    if (lanes_ok && !diag && mt > MAX_MT && nchunks * chunk_elems * c.M <= crowd_most(mt)) {
+    if (lanes_ok && !diag && mt > MAX_MT && coords <= crowd_most(c.opt, mt)) {
         const int L = crowd_lanes(c.M), threads = c.M * L;
         plan_parts(p, chunks, 4 * L);
-        const int kind = threads > 512 ? CROWD_1024 : threads > 256 ? CROWD_512
-                         : p.grid <= crowd_min_blocks(CROWD_FEW) * NUM_SMS ? CROWD_FEW : CROWD_256;
-        p.kernel = Kernel::CROWD;
-        p.fn = lookup_crowd_kernel(c.opt, post, bf16, kind, static_cast<int>(kmask));
-        p.threads = L;
-        p.threads_y = c.M;
-        p.smem = crowd_smem_bytes(c.opt, bf16, c.M);
-        p.smem_limit = crowd_smem_limit(kind);
-        return p;
+        if (p.grid * p.part_elems * c.M <= 2 * crowd_most(c.opt, mt)) {   // (else crowded, as above)
+            const int kind = threads > 512 ? CROWD_1024 : threads > 256 ? CROWD_512
+                             : p.grid <= crowd_min_blocks(CROWD_FEW) * NUM_SMS ? CROWD_FEW : CROWD_256;
+            p.kernel = Kernel::CROWD;
+            p.fn = lookup_crowd_kernel(c.opt, post, bf16, kind, static_cast<int>(kmask));
+            p.threads = L;
+            p.threads_y = c.M;
+            p.smem = crowd_smem_bytes(c.opt, bf16, c.M);
+            p.smem_limit = crowd_smem_limit(kind);
+            return p;
+        }
+        p = LaunchPlan();
     }
     // Gradients that the copy engine cannot take, in problems of more than four rounds of blocks (smaller ones are served
     // from L2 and gain nothing).  Measured with 60 M parameters x workers, Adam, gradients 8 bytes off the state's layout:

@@ -30,3 +30,15 @@ def test_as_many_blocks_as_have_work(M, count, size, local, averaging):
 ])
 def test_sparse_lists_stay_with_the_tiles(M, numel, opt, kernel):
     assert plan(M, numel, opt, 0)[0] == kernel
+
+
+@pytest.mark.parametrize("M,numel,kernel", [
+    # what counts are the coordinates, not the chunks: lists of many tensors as large as a single one
+    (16, [2_600] * 100, "crowd"), (16, [262_400], "crowd"), (16, [2_700] * 100, "runtime_m"), (6, [3_300] * 100, "lanes"), (6, [3_400] * 100, "tiles"),
+    (8, [4_700] * 100, "lanes"), (8, [4_800] * 100, "tiles"), (24, [1_870] * 100, "crowd"), (24, [1_900] * 100, "runtime_m"),
+    # blocks with room for twice the line: as many for each tiny tensor as for a whole chunk
+    (4, [300_000] + [2] * 1_200, "lanes"), (4, [300_000] + [2] * 1_300, "tiles"), (12, [100_000] + [2] * 400, "crowd"),
+    (12, [100_000] + [2] * 450, "tiles"),
+])
+def test_lists_are_counted_by_coordinates(M, numel, kernel):
+    assert plan(M, numel, "adam", 7)[0] == kernel

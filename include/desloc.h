@@ -162,8 +162,8 @@ DESLOC_API int desloc_step(desloc_ctx *ctx, int64_t t, float lr_t, float clip_bo
  * reads them from there into dev_grads, and the step follows it on `stream`, two launches in all.
  * Else the tensor list is cut into up to 8 groups, of falling size (inside a tensor, where a large
  * one would make a group too long); each group's gradients are copied on a stream
- * the context owns (a copy per piece) and the
- * group's part of the step is launched on `stream` as soon as its copies have landed, so all
+ * the context owns (a copy per piece, or, where the pieces are many and all of them page-locked memory as
+ * above, one kernel that reads them) and the group's part of the step is launched on `stream` as soon as its copies have landed, so all
  * but the last group's compute hides behind the transfers.  Either way the gradients are fetched
  * behind the work already enqueued on `stream`, and host_grads may be written again when that
  * stream has come past the step.  Not available under stream capture (DESLOC_E_INVALID).
@@ -269,7 +269,8 @@ DESLOC_API int desloc_destroy(desloc_ctx *ctx);
    distributed run of the same schedule would pay; Section 5.1 "Metrics"). */
 DESLOC_API int desloc_get_counters(const desloc_ctx *ctx, int64_t out[4]);
 
-/* Kernels launched by this context so far (one per step on the main path). */
+/* Kernels launched by this context so far (one per step on the main path; those that stand in for the copies of a
+   group of desloc_step_host() are not counted). */
 DESLOC_API int64_t desloc_get_launch_count(const desloc_ctx *ctx);
 
 /*

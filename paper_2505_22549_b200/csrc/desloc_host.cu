@@ -72,6 +72,7 @@ struct HostGroup {
     int32_t k0, k1;   // of tensors k0 .. k1,
     int64_t e0, e1;   // the first one from element e0 on, the last one up to element e1
     int64_t elems;    // in all
+    int64_t r0, r1;   // the same in chunks of the reduction kernels, the first and the last one in parts
 };
 
 // Everything that depends on the worker count M (re-made by desloc_set_workers): the pointer
@@ -94,6 +95,7 @@ struct WorkerRes {
     float *d_diag = nullptr;     // diagnostics step: [3][M][nchunks] per-chunk sums of squares
     // Results the host waits for go to its memory straight from the kernels, without a copy:
     // [3][M][num_tensors] per-tensor norms, [3][M] totals, [M] relative changes.
+    Slot host_slots[2];          // the same of addresses in host memory (desloc_step_host), staged on the copy stream
     float *h_out = nullptr;      // mapped pinned memory, and
     float *d_out = nullptr;      // the same as the kernels address it
 };
@@ -103,6 +105,8 @@ void free_worker_res(WorkerRes &r) {
         if (s.done) cudaEventDestroy(s.done);
         s = Slot();
     }
+    for (Slot &s : r.host_slots)
+        if (s.done) cudaEventDestroy(s.done);
     if (r.h_slots) cudaFreeHost(r.h_slots);
     if (r.d_slots) cudaFree(r.d_slots);
     if (r.d_chunks) cudaFree(r.d_chunks);
@@ -128,9 +132,11 @@ void plan_host_groups(std::vector<HostGroup> &groups, const std::vector<desloc::
                       int64_t total) {
     groups.clear();
     int64_t left = total, acc = 0;
-    HostGroup g{0, 0, 0, 0, 0, 0, 0};
+    HostGroup g{};
+    int64_t rstart = 0;   // first reduction chunk of the tensor
     for (size_t c = 0; c < chunks.size(); ++c) {
         const desloc::Chunk &ch = chunks[c];
+        if (c > 0 && ch.tensor != chunks[c - 1].tensor) rstart += desloc::chunks_of(numel[chunks[c - 1].tensor], desloc::REDUCE_CHUNK_ELEMS, 0);
         const int64_t end = ch.start + ch.count, rest = numel[ch.tensor] - end;
         acc += ch.count;
         const bool split = groups.size() + 1 < kHostGroups && (left > kHostSplit || (rest == 0 && groups.empty()));
@@ -140,8 +146,10 @@ void plan_host_groups(std::vector<HostGroup> &groups, const std::vector<desloc::
         g.k1 = ch.tensor;
         g.e1 = end;
         g.elems = acc;
+        g.r1 = rstart + (end + desloc::REDUCE_CHUNK_ELEMS - 1) / desloc::REDUCE_CHUNK_ELEMS;
         groups.push_back(g);
         g.c0 = g.c1;
+        g.r0 = rest > 0 ? rstart + end / desloc::REDUCE_CHUNK_ELEMS : g.r1;
         g.k0 = rest > 0 ? ch.tensor : ch.tensor + 1;
         g.e0 = rest > 0 ? end : 0;
         left -= acc;
@@ -199,10 +207,11 @@ cudaError_t make_worker_res(WorkerRes &r, const desloc_config &cfg, int M, const
                           cudaHostAllocMapped);
     if (e == cudaSuccess) e = cudaHostGetDevicePointer(reinterpret_cast<void **>(&r.d_out), r.h_out, 0);
     const size_t room = static_cast<size_t>(nptr + 15) & ~size_t{15};   // tables on 128-byte boundaries
-    if (e == cudaSuccess) e = cudaMallocHost(&r.h_slots, kSlots * room * sizeof(void *));
-    if (e == cudaSuccess) e = cudaMalloc(&r.d_slots, kSlots * room * sizeof(void *));
-    for (int i = 0; i < kSlots && e == cudaSuccess; ++i) {
-        Slot &s = r.slots[i];
+    constexpr int kAll = kSlots + 2;
+    if (e == cudaSuccess) e = cudaMallocHost(&r.h_slots, kAll * room * sizeof(void *));
+    if (e == cudaSuccess) e = cudaMalloc(&r.d_slots, kAll * room * sizeof(void *));
+    for (int i = 0; i < kAll && e == cudaSuccess; ++i) {
+        Slot &s = i < kSlots ? r.slots[i] : r.host_slots[i - kSlots];
         s.host = r.h_slots + i * room;
         s.dev = r.d_slots + i * room;
         e = cudaEventCreateWithFlags(&s.done, cudaEventDisableTiming);
@@ -226,6 +235,8 @@ struct desloc_ctx {
     WorkerRes res;
     int next_slot = 0;
     int cur_slot = -1;           // slot holding the table equal to last_grads
+    int cur_host = -1;           // the same of addresses in host memory
+    std::vector<const void *> last_host;
     std::vector<const void *> last_grads;
     desloc::GradLayout last_layout = desloc::GradLayout::FIT;   // of them
     cudaStream_t last_stream = nullptr;
@@ -300,9 +311,65 @@ int stage_grads(desloc_ctx *ctx, const void *const *grads, cudaStream_t stream, 
 bool host_runs_of(const desloc_ctx *ctx, const void *const *host_grads, const void *const *grads, desloc::HostRuns &runs) {
     const desloc_config &c = ctx->cfg;
     const int64_t gsz = c.grad_dtype == DESLOC_BF16 ? 2 : 4;
+    desloc::HostRange known;
     return ctx->total_elems <= desloc::HOST_KERNEL_BYTES / gsz / c.M &&
            desloc::gather_host_runs(host_grads, grads, ctx->nptr, c.numel, c.num_tensors, static_cast<size_t>(gsz), runs,
-                                    desloc::device_reads_host);
+                                    [&](const void *p, size_t bytes) { return desloc::device_reads_host(p, bytes, known); });
+}
+
+// The pieces of a group, contiguous on both sides, in order: piece(from, to, bytes) until it says no.
+template <typename Piece>
+bool for_pieces(const desloc_ctx *ctx, const HostGroup &grp, const void *const *host_grads, const void *const *grads, const Piece &piece) {
+    const desloc_config &c = ctx->cfg;
+    const size_t gsz = c.grad_dtype == DESLOC_BF16 ? 2 : 4;
+    const auto upto = [&](int32_t k) { return static_cast<size_t>(k == grp.k1 ? grp.e1 : ctx->numel[k]) * gsz; };
+    for (int m = 0; m < c.M; ++m) {
+        for (int32_t k = grp.k0; k <= grp.k1;) {
+            const int64_t i0 = static_cast<int64_t>(m) * c.num_tensors;
+            const size_t from = k == grp.k0 ? static_cast<size_t>(grp.e0) * gsz : 0;
+            const char *hp = static_cast<const char *>(host_grads[i0 + k]) + from;
+            char *dp = static_cast<char *>(const_cast<void *>(grads[i0 + k])) + from;
+            size_t bytes = upto(k) - from;
+            for (++k; k <= grp.k1 && static_cast<const char *>(host_grads[i0 + k]) == hp + bytes &&
+                      static_cast<const char *>(grads[i0 + k]) == dp + bytes; ++k)
+                bytes += upto(k);
+            if (!piece(hp, dp, bytes)) return false;
+        }
+    }
+    return true;
+}
+
+// Is a group brought by a kernel: many pieces, all of them in memory that the device reads?
+bool group_by_kernel(const desloc_ctx *ctx, const HostGroup &grp, const void *const *host_grads, const void *const *grads,
+                     desloc::HostRange &known) {
+    const int64_t bytes = grp.elems * ctx->cfg.M * (ctx->cfg.grad_dtype == DESLOC_BF16 ? 2 : 4);
+    int64_t pieces = 0;
+    for_pieces(ctx, grp, host_grads, grads, [&](const char *, char *, size_t) { return ++pieces != 0; });
+    return desloc::gather_pays(pieces, bytes) &&
+           for_pieces(ctx, grp, host_grads, grads, [&](const char *hp, char *, size_t n) { return desloc::device_reads_host(hp, n, known); });
+}
+
+// The table of host addresses on the device, for kernels on the copy stream.
+cudaError_t stage_host_table(desloc_ctx *ctx, const void *const *host_grads, const void *const **out) {
+    const size_t bytes = static_cast<size_t>(ctx->nptr) * sizeof(void *);
+    cudaError_t e = cudaSuccess;
+    if (ctx->cur_host < 0 || std::memcmp(ctx->last_host.data(), host_grads, bytes) != 0) {
+        const int next = ctx->cur_host == 0 ? 1 : 0;
+        Slot &s = ctx->res.host_slots[next];
+        if (s.in_flight) e = cudaEventSynchronize(s.done);   // (the copy of two tables ago)
+        if (e != cudaSuccess) return e;
+        s.in_flight = false;
+        ctx->cur_host = -1;
+        std::memcpy(s.host, host_grads, bytes);
+        e = cudaMemcpyAsync(s.dev, s.host, bytes, cudaMemcpyHostToDevice, ctx->copy_stream);
+        if (e == cudaSuccess) e = cudaEventRecord(s.done, ctx->copy_stream);
+        if (e != cudaSuccess) return e;
+        s.in_flight = true;
+        std::memcpy(ctx->last_host.data(), host_grads, bytes);
+        ctx->cur_host = next;
+    }
+    *out = reinterpret_cast<const void *const *>(ctx->res.host_slots[ctx->cur_host].dev);
+    return e;
 }
 
 // Raises the kernel's shared-memory limit, once per kernel and context (the attribute call costs a microsecond that a
@@ -442,33 +509,21 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
                 e = plans[gi].fn ? prepare_once(ctx, plans[gi]) : cudaErrorInvalidDeviceFunction;
             }
             // The device gradient buffers may still be read by earlier work on `stream`.
-            const size_t gsz = c.grad_dtype == DESLOC_BF16 ? 2 : 4;
             if (e == cudaSuccess) e = cudaEventRecord(ctx->ev_entry, stream);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->copy_stream, ctx->ev_entry, 0);
+            desloc::HostRange known;
             for (size_t gi = 0; gi < ctx->res.groups.size() && e == cudaSuccess; ++gi) {
                 const HostGroup &grp = ctx->res.groups[gi];
-                for (int m = 0; m < c.M && e == cudaSuccess; ++m) {
-                    // merge tensors that are adjacent on both sides into one copy
-                    int32_t k = grp.k0;
-                    while (k <= grp.k1 && e == cudaSuccess) {
-                        const int64_t i0 = static_cast<int64_t>(m) * c.num_tensors + k;
-                        const size_t from = k == grp.k0 ? static_cast<size_t>(grp.e0) * gsz : 0;
-                        const auto to = [&](int32_t kk) { return static_cast<size_t>(kk == grp.k1 ? grp.e1 : ctx->numel[kk]) * gsz; };
-                        const char *hp = static_cast<const char *>(host_grads[i0]) + from;
-                        char *dp = static_cast<char *>(const_cast<void *>(grads[i0])) + from;
-                        size_t bytes = to(k) - from;
-                        int32_t k2 = k + 1;
-                        while (k2 <= grp.k1) {
-                            const int64_t i2 = static_cast<int64_t>(m) * c.num_tensors + k2;
-                            if (static_cast<const char *>(host_grads[i2]) != hp + bytes ||
-                                static_cast<const char *>(grads[i2]) != dp + bytes)
-                                break;
-                            bytes += to(k2);
-                            ++k2;
-                        }
+                if (group_by_kernel(ctx, grp, host_grads, grads, known)) {
+                    desloc::HostGather hg{ctx->d_rchunks, grp.r0, grp.r1, nullptr, a.g, c.num_tensors, c.M, grp.k0, grp.k1, grp.e0, grp.e1,
+                                          c.grad_dtype == DESLOC_BF16 ? 2 : 4};
+                    e = stage_host_table(ctx, host_grads, &hg.src);
+                    if (e == cudaSuccess) e = desloc::launch_host_gather(hg, ctx->copy_stream);   // (in the copies' place, and not counted either)
+                } else {
+                    for_pieces(ctx, grp, host_grads, grads, [&](const char *hp, char *dp, size_t bytes) {
                         e = cudaMemcpyAsync(dp, hp, bytes, cudaMemcpyHostToDevice, ctx->copy_stream);
-                        k = k2;
-                    }
+                        return e == cudaSuccess;
+                    });
                 }
                 if (e == cudaSuccess) e = cudaEventRecord(ctx->ev_group[gi], ctx->copy_stream);
                 if (e == cudaSuccess) e = cudaStreamWaitEvent(stream, ctx->ev_group[gi], 0);
@@ -590,6 +645,7 @@ int desloc_create(desloc_ctx **out, const desloc_config *cfg, float *const *x, f
     try {
         ctx->numel.assign(cfg->numel, cfg->numel + cfg->num_tensors);
         ctx->last_grads.assign(static_cast<size_t>(nptr), nullptr);
+        ctx->last_host.assign(static_cast<size_t>(nptr), nullptr);
         ctx->prepared.reserve(64);   // steps never allocate: beyond this the attribute is simply set again
         rchunks.resize(static_cast<size_t>(nrchunks));
         desloc::fill_chunks(cfg->numel, cfg->num_tensors, desloc::REDUCE_CHUNK_ELEMS, rchunks.data());
@@ -616,7 +672,10 @@ int desloc_create(desloc_ctx **out, const desloc_config *cfg, float *const *x, f
         *ctx->h_err = 0;
         e = cudaHostGetDevicePointer(reinterpret_cast<void **>(&ctx->d_err), ctx->h_err, 0);
     }
-    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking);
+    // (ahead of the step's blocks: a kernel on this stream holds few of them, and the bus waits for it)
+    int least = 0, greatest = 0;
+    if (e == cudaSuccess) e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
+    if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&ctx->copy_stream, cudaStreamNonBlocking, greatest);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_entry, cudaEventDisableTiming);
     for (size_t i = 0; i < kHostGroups && e == cudaSuccess; ++i)
         e = cudaEventCreateWithFlags(&ctx->ev_group[i], cudaEventDisableTiming);
@@ -795,8 +854,9 @@ int desloc_set_workers(desloc_ctx *ctx, int32_t M_new, int32_t first_new, float 
     if (e == cudaSuccess) {
         try {
             e = make_worker_res(fresh, ctx->cfg, M_new, ctx->numel.data(), nt, ctx->total_elems, ctx->nrchunks, has_v, x, u, v);
-            if (ctx->last_grads.capacity() < static_cast<size_t>(nptr_new))
-                ctx->last_grads.reserve(static_cast<size_t>(nptr_new));  // may throw; no state changed yet
+            for (auto *last : {&ctx->last_grads, &ctx->last_host})
+                if (last->capacity() < static_cast<size_t>(nptr_new))
+                    last->reserve(static_cast<size_t>(nptr_new));  // may throw; no state changed yet
         } catch (const std::bad_alloc &) {
             e = cudaErrorMemoryAllocation;
         }
@@ -820,6 +880,8 @@ int desloc_set_workers(desloc_ctx *ctx, int32_t M_new, int32_t first_new, float 
         free_worker_res(ctx->res);
         ctx->res = std::move(fresh);
         ctx->last_grads.assign(static_cast<size_t>(nptr_new), nullptr);  // capacity reserved above
+        ctx->last_host.assign(static_cast<size_t>(nptr_new), nullptr);
+        ctx->cur_host = -1;
         ctx->cfg.M = M_new;
         ctx->nptr = nptr_new;
         ctx->next_slot = 0;

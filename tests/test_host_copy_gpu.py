@@ -46,3 +46,36 @@ def test_host_gradients_of_small_problems(gd, shift_h, shift_d, M, numel, separa
     for pa, pb in ((a.x, b.x), (a.u, b.u), (a.v, b.v)):
         assert np.array_equal(a.to_numpy(pa), b.to_numpy(pb))
     ea.close(); eb.close()
+
+
+@pytest.mark.parametrize("gd", ["bf16", "f32"])
+@pytest.mark.parametrize("shift_h,shift_d", [(0, 0), (1, 0), (3, 5)])
+@pytest.mark.parametrize("M,numel,separate,pinned", [
+    (3, (33, 4095, 4096, 4097, 8193) * 4 + (2_500_007,), True, True),        # a cut inside the last tensor
+    (2, (1_900_001,) + (7, 1, 4100) * 12 + (900_003,), True, True),          # inside the first, and the last
+    (12, (40_003,) * 9, False, True), (2, (33, 5000) * 16 + (2_100_000,), True, False),      # pageable: copies
+])
+def test_many_pieces_arrive_group_by_group(gd, shift_h, shift_d, M, numel, separate, pinned):
+    """Every byte of the pieces, nothing around them, and other addresses at every step."""
+    import paper_2505_22549_b200 as d
+    w = di.Workload("pieces", "sgdm", M, numel, gd, "normal1", lr=1e-2, K=(2, 3, 4), seed=2)
+    dev = torch.device("cuda:0")
+    st = State(w, dev, align=3, g_shift=shift_d)          # (elements in between that belong to nobody)
+    eng = make_engine(d, w, st)
+    dt, gen = st.g[0].dtype, torch.Generator().manual_seed(3)
+    inside = torch.from_numpy(st.valid_mask()).to(dev)
+    for t in range(4):
+        def pin(n):
+            h = torch.empty(n + shift_h + t, dtype=dt, pin_memory=pinned)[shift_h + t:]
+            return h.copy_(torch.randn(n, generator=gen))
+        flat = [pin(st.nflat + 1) for _ in range(M)]
+        host = [[pin(n) for n in numel] for _ in range(M)] if separate else [[f[o + 1:o + 1 + n] for o, n in zip(st.offs, numel)] for f in flat]
+        for g in st.g:
+            g.fill_(7.0)
+        eng.step_host(t, 1e-2, host, st.views(st.g))
+        torch.cuda.synchronize()
+        for m in range(M):
+            for x, y in zip(host[m], st.views(st.g)[m]):
+                assert torch.equal(x, y.cpu())
+            assert bool((st.g[m][~inside] == 7.0).all())
+    eng.close()

@@ -70,8 +70,12 @@ __host__ __device__ constexpr int crowd_smem_bytes(int opt, bool bf16, int M) {
 __host__ __device__ constexpr int crowd_smem_limit(int kind) { return 4 * crowd_threads(kind) * 16 + 3 * 4 * 16 * 4; }
 
 // Blocks of crowd_lanes(M) x M threads; a work item is 4 * crowd_lanes(M) coordinates of a chunk, of all replicas.
-template <int OPT, int MASK, typename GT, bool POST, int KIND>
-__global__ void __launch_bounds__(crowd_threads(KIND), crowd_min_blocks(KIND))
+// DIAG: also the sums of squares of gradient, new parameters and update, a partial sum per block, worker and kind, reduced by shuffles where they
+// arise; two thirds of the blocks, for the registers.  205 random lists of 9 to 64 workers, averaging steps with diagnostics (before: the
+// runtime-M kernel, which lets one block go over all workers of a chunk): up to 0.5 million coordinates 3.3 to 7 us (15 to 29), a million 14.5 (27.7),
+// two million 21 (38).
+template <int OPT, int MASK, typename GT, bool POST, int KIND, bool DIAG = false>
+__global__ void __launch_bounds__(crowd_threads(KIND), DIAG && KIND != CROWD_1024 ? crowd_min_blocks(KIND) * 2 / 3 : crowd_min_blocks(KIND))
 desloc_crowd_kernel(const __grid_constant__ StepArgs a) {
     extern __shared__ __align__(16) float pool[];
     begin_and_let_next_begin();
@@ -79,8 +83,23 @@ desloc_crowd_kernel(const __grid_constant__ StepArgs a) {
     const int part0 = static_cast<int>(blockIdx.x - c * a.parts) * a.part_elems;
     const Chunk ch = a.chunks[c];
     const int cnt = min(ch.count - part0, a.part_elems);
-    if (cnt <= 0) return;   // (of the whole block)
     const int M = a.M, L = blockDim.x, T = 4 * L, m = threadIdx.y, lx = threadIdx.x;
+    const auto put = [&](int kind, float v) {
+        a.diag[(static_cast<long long>(kind) * M + m) * a.diag_stride + blockIdx.x] = v;
+    };
+    if (cnt <= 0) {   // (of the whole block)
+        if (DIAG && lx == 0) {
+            wait_for_earlier_kernels();
+            for (int kind = 0; kind < DIAG_KINDS; ++kind) put(kind, 0.f);
+        }
+        return;
+    }
+    const auto norms = [&](int kind, float v) {
+        const int first = (m * L + lx) & ~31, there = M * L - first;   // (the last warp may be a part of one)
+        const unsigned lanes = there >= 32 ? 0xffffffffu : (1u << there) - 1;
+        for (int o = L / 2; o > 0; o /= 2) v += __shfl_down_sync(lanes, v, o, L);
+        if (lx == 0) put(kind, v);
+    };
     const auto replica = [&] { return Replica<OPT, GT>(a, static_cast<long long>(m) * a.nt + ch.tensor, ch.start + part0); };
     const Replica<OPT, GT> w = replica();
     const bool wide = __syncthreads_and(w.wide_ok() && (cnt & 3) == 0) != 0;
@@ -104,40 +123,45 @@ desloc_crowd_kernel(const __grid_constant__ StepArgs a) {
     };
     const Quad<true> q4{4 * lx, 1, cnt, true};
     const auto mean4 = [&](auto &s, auto arrays) { mean_of_arrays(q4, s, arrays, !POST); };
-    if (wide && plain_step<OPT>(a)) {   // (the common form: nothing but its loads behind the wait)
+    const Quad<false> q1{lx, L, cnt, true};
+    const auto mean1 = [&](auto &s, auto arrays) { mean_of_arrays(q1, s, arrays, false); };
+    if constexpr (DIAG) {
         wait_for_earlier_kernels();
-        update_quad<OPT, MASK, GT, POST, true, true>(a, 1.f, q4, land, w, replica, mean4);
-        return;
-    }
-    wait_for_earlier_kernels();
-    const float sc = a.gscale ? a.gscale[m] : 1.f;
-    if (wide) {
-        update_quad<OPT, MASK, GT, POST, false, true>(a, sc, q4, land, w, replica, mean4);
+        const float sc = a.gscale ? a.gscale[m] : 1.f;
+        if (wide) update_quad<OPT, MASK, GT, POST, false, true>(a, sc, q4, land, w, replica, mean4, norms);
+        else update_quad<OPT, MASK, GT, POST, false, false>(a, sc, q1, land, w, replica, mean1, norms);
     } else {
-        const Quad<false> q{lx, L, cnt, true};
-        const auto mean = [&](auto &s, auto arrays) { mean_of_arrays(q, s, arrays, false); };
-        update_quad<OPT, MASK, GT, POST, false, false>(a, sc, q, land, w, replica, mean);
+        if (wide && plain_step<OPT>(a)) {   // (the common form: nothing but its loads behind the wait)
+            wait_for_earlier_kernels();
+            update_quad<OPT, MASK, GT, POST, true, true>(a, 1.f, q4, land, w, replica, mean4);
+            return;
+        }
+        wait_for_earlier_kernels();
+        const float sc = a.gscale ? a.gscale[m] : 1.f;
+        if (wide) update_quad<OPT, MASK, GT, POST, false, true>(a, sc, q4, land, w, replica, mean4);
+        else update_quad<OPT, MASK, GT, POST, false, false>(a, sc, q1, land, w, replica, mean1);
     }
 }
 
-template <int OPT, typename GT, bool POST, int NMASK, int... I>
+template <int OPT, typename GT, bool POST, bool DIAG, int NMASK, int... I>
 const void *pick_crowd(int kind, int mask, std::integer_sequence<int, I...>) {
     static const void *const tbl[] = {
-        reinterpret_cast<const void *>(&desloc_crowd_kernel<OPT, 1 + I % NMASK, GT, POST, I / NMASK>)...};
+        reinterpret_cast<const void *>(&desloc_crowd_kernel<OPT, 1 + I % NMASK, GT, POST, I / NMASK, DIAG>)...};
     if (kind < CROWD_FEW || kind > CROWD_1024 || mask < 1 || mask > NMASK) return nullptr;
     return tbl[kind * NMASK + mask - 1];
 }
 
 template <int OPT, typename GT>
-const void *lookup_crowd(bool post, int kind, int mask) {
+const void *lookup_crowd(bool post, int kind, int mask, bool diag) {
     constexpr int NMASK = OPT == OPT_SGDM ? 3 : 7;
     using Seq = std::make_integer_sequence<int, 4 * NMASK>;
-    return post ? pick_crowd<OPT, GT, true, NMASK>(kind, mask, Seq{}) : pick_crowd<OPT, GT, false, NMASK>(kind, mask, Seq{});
+    if (diag) return post ? pick_crowd<OPT, GT, true, true, NMASK>(kind, mask, Seq{}) : pick_crowd<OPT, GT, false, true, NMASK>(kind, mask, Seq{});
+    return post ? pick_crowd<OPT, GT, true, false, NMASK>(kind, mask, Seq{}) : pick_crowd<OPT, GT, false, false, NMASK>(kind, mask, Seq{});
 }
 
 // One unit per optimizer.
-const void *lookup_crowd_adam(bool post, bool bf16, int kind, int mask);
-const void *lookup_crowd_adopt(bool post, bool bf16, int kind, int mask);
-const void *lookup_crowd_sgdm(bool post, bool bf16, int kind, int mask);
+const void *lookup_crowd_adam(bool post, bool bf16, int kind, int mask, bool diag);
+const void *lookup_crowd_adopt(bool post, bool bf16, int kind, int mask, bool diag);
+const void *lookup_crowd_sgdm(bool post, bool bf16, int kind, int mask, bool diag);
 
 }  // namespace desloc

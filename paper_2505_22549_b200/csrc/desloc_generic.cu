@@ -1,5 +1,5 @@
 // DES-LOC step for the worker counts and variants that have no tile kernel (M > 16; from nine workers on also
-// the post-average ordering and the norm diagnostics) on steps that average something.  Same update
+// the post-average ordering and the norm diagnostics) on steps that average something in problems too large for desloc_crowd_kernel.  Same update
 // as desloc_step_kernel, runtime M, compile-time mask.  Worker sums run in the order m = 0..M-1 as
 // compensated fp32 sums (see WorkerSum): exact for equal replicas, and within an ulp of a
 // sequential fp64 reference.

@@ -92,7 +92,7 @@ struct WorkerRes {
     float *d_norms = nullptr;    // [2][M]: gradient norms, clip factors
     void **h_snap = nullptr;     // pinned pointer table for desloc_rel_change
     void **d_snap = nullptr;
-    float *d_diag = nullptr;     // diagnostics step: [3][M][nchunks] per-chunk sums of squares
+    float *d_diag = nullptr;     // diagnostics step: [3][M][row] sums of squares, of a chunk each or, in desloc_crowd_kernel, of a part of one
     // Results the host waits for go to its memory straight from the kernels, without a copy:
     // [3][M][num_tensors] per-tensor norms, [3][M] totals, [M] relative changes.
     Slot host_slots[2];          // the same of addresses in host memory (desloc_step_host), staged on the copy stream
@@ -201,7 +201,12 @@ cudaError_t make_worker_res(WorkerRes &r, const desloc_config &cfg, int M, const
     if (e == cudaSuccess) e = cudaMallocHost(&r.h_snap, static_cast<size_t>(nptr) * sizeof(void *));
     if (e == cudaSuccess) e = cudaMalloc(&r.d_snap, static_cast<size_t>(nptr) * sizeof(void *));
     const size_t ndiag = static_cast<size_t>(desloc::DIAG_KINDS) * M;
-    if (e == cudaSuccess) e = cudaMalloc(&r.d_diag, ndiag * static_cast<size_t>(nchunks) * sizeof(float));
+    // (a partial sum per chunk, or per block of a chunk where averaging steps run in desloc_crowd_kernel)
+    desloc_config as = cfg;
+    as.M = M;
+    const desloc::LaunchPlan crowd = desloc::plan_launch(as, DESLOC_SYNC_X, r.set, true, false, desloc::GradLayout::FIT);
+    const int64_t row = crowd.kernel == desloc::Kernel::CROWD ? nchunks * crowd.parts : nchunks;
+    if (e == cudaSuccess) e = cudaMalloc(&r.d_diag, ndiag * static_cast<size_t>(row) * sizeof(float));
     if (e == cudaSuccess)
         e = cudaHostAlloc(reinterpret_cast<void **>(&r.h_out), (ndiag * (num_tensors + 1) + M) * sizeof(float),
                           cudaHostAllocMapped);
@@ -243,7 +248,8 @@ struct desloc_ctx {
     int64_t counters[4] = {0, 0, 0, 0};
     int64_t launches = 0;
     int last_cuda_error = 0;
-    bool diag_valid = false;        // a diagnostics step has run since the workers last changed
+    bool diag_valid = false;        // a diagnostics step has run since the workers last changed,
+    int diag_parts = 1;             // and left so many sums per chunk
     int64_t max_blocks = 0;         // test hook: cap on the grid (0 = one block per work item)
     int staging_mode = -1;          // test hook: -1 the library decides; tile kernels that 0 always stage, 1 never, 2 as decided
     std::vector<const void *> prepared;  // kernels whose shared-memory limit this context has raised
@@ -468,7 +474,8 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
             for (int64_t i = 0; i < ctx->nptr; ++i) a.g_inline[i] = grads[i];
         a.gscale = d_gscale;
         a.diag = diag ? ctx->res.d_diag : nullptr;
-        a.diag_stride = ctx->res.nchunks;
+        const int diag_parts = plan.kernel == desloc::Kernel::CROWD ? plan.parts : 1;
+        a.diag_stride = ctx->res.nchunks * diag_parts;
         a.diag_chunk0 = 0;
         desloc::fill_hyper(a, c, lr_t, clip_bound_t);
         a.err = ctx->d_err;
@@ -556,7 +563,10 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
                 s.in_flight = true;
             }
         }
-        if (diag) ctx->diag_valid = true;
+        if (diag) {
+            ctx->diag_valid = true;
+            ctx->diag_parts = diag_parts;
+        }
         ctx->counters[0] += 1;
         ctx->counters[1] += (mask & DESLOC_SYNC_X) ? 1 : 0;
         ctx->counters[2] += (mask & DESLOC_SYNC_U) ? 1 : 0;
@@ -731,7 +741,7 @@ int desloc_get_diag_norms(desloc_ctx *ctx, float *per_tensor_out, float *total_o
     if (e != cudaSuccess) return cuda_fail(ctx, e);
     const size_t rows = static_cast<size_t>(desloc::DIAG_KINDS) * c.M;
     const size_t per = rows * c.num_tensors;
-    e = desloc::launch_diag_norms(ctx->res.d_diag, ctx->res.nchunks, ctx->res.d_tstart, c.num_tensors, c.M,
+    e = desloc::launch_diag_norms(ctx->res.d_diag, ctx->res.nchunks, ctx->diag_parts, ctx->res.d_tstart, c.num_tensors, c.M,
                                   ctx->res.d_out, ctx->res.d_out + per, st);
     if (e == cudaSuccess) ctx->launches += 1;
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);

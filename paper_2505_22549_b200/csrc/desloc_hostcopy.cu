@@ -22,7 +22,7 @@ namespace {
 
 constexpr int COPY_THREADS = 128, COPY_UNITS = 4;
 constexpr uint32_t HOST_SLICE = COPY_THREADS * COPY_UNITS * 16;
-constexpr long long GATHER_BLOCKS = 64;   // four of them keep the bus busy where the pieces are long; the step's blocks run beside them
+constexpr long long GATHER_BLOCKS = 64;   // sixteen keep the bus busy where the pieces are long; the step's blocks run beside them
 
 // Units of U bytes from the first boundary on, what lies around them byte by byte, by THREADS threads.
 template <typename U, int THREADS>

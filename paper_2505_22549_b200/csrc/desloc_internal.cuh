@@ -255,9 +255,9 @@ inline void fill_hyper(StepArgs &a, const desloc_config &c, float lr_t, float cl
     a.part_elems = 0;
 }
 
-inline const void *lookup_crowd_kernel(int opt, bool post, bool bf16, int kind, int mask) {
-    return opt == OPT_ADAM ? lookup_crowd_adam(post, bf16, kind, mask)
-           : opt == OPT_ADOPT ? lookup_crowd_adopt(post, bf16, kind, mask) : lookup_crowd_sgdm(post, bf16, kind, mask);
+inline const void *lookup_crowd_kernel(int opt, bool post, bool bf16, int kind, int mask, bool diag) {
+    return opt == OPT_ADAM ? lookup_crowd_adam(post, bf16, kind, mask, diag)
+           : opt == OPT_ADOPT ? lookup_crowd_adopt(post, bf16, kind, mask, diag) : lookup_crowd_sgdm(post, bf16, kind, mask, diag);
 }
 
 inline const void *lookup_lanes_kernel(int opt, bool post, bool bf16, int mt, int mask) {
@@ -432,14 +432,14 @@ inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, const Chunk
         }
         p = LaunchPlan();
     }
-    if (lanes_ok && !diag && mt > MAX_MT && coords <= crowd_most(c.opt, mt)) {
+    if (lanes_ok && mt > MAX_MT && coords <= crowd_most(c.opt, mt)) {
         const int L = crowd_lanes(c.M), threads = c.M * L;
         plan_parts(p, chunks, 4 * L);
         if (p.grid * p.part_elems * c.M <= 2 * crowd_most(c.opt, mt)) {   // (else crowded, as above)
             const int kind = threads > 512 ? CROWD_1024 : threads > 256 ? CROWD_512
                              : p.grid <= crowd_min_blocks(CROWD_FEW) * NUM_SMS ? CROWD_FEW : CROWD_256;
             p.kernel = Kernel::CROWD;
-            p.fn = lookup_crowd_kernel(c.opt, post, bf16, kind, static_cast<int>(kmask));
+            p.fn = lookup_crowd_kernel(c.opt, post, bf16, kind, static_cast<int>(kmask), diag);
             p.threads = L;
             p.threads_y = c.M;
             p.smem = crowd_smem_bytes(c.opt, bf16, c.M);

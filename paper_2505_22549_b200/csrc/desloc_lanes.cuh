@@ -13,6 +13,7 @@
 // (9.8), x 300 K 12.6 (17.4); four x 15 K 1.7 (2.8); two x 250 K 3.7 (5.4).  Four x 250 K, all averaged, 6.5 (9.1).
 // Local steps: four x 2.5 K 1.5 us (1.7), x 250 K 5.8 (6.6), x 400 K 8.0 (9.5), x 1.25 M 21.9 (22.7).
 #pragma once
+#include <type_traits>
 #include <utility>
 
 #include "desloc_kernels.cuh"
@@ -47,6 +48,14 @@ struct Quad {
                 if (has(j)) r.a[j] = ld_grad<1, GT>(p, e + j * step).a[0];
         }
         return r;
+    }
+    __device__ __forceinline__ float sum_of_squares(const FV<4> &v) const {
+        if constexpr (WIDE) return has(0) ? sum_sq<4>(v) : 0.f;
+        float s = 0.f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (has(j)) s = fmaf(v.a[j], v.a[j], s);
+        return s;
     }
     __device__ __forceinline__ void st(float *p, const FV<4> &v) const {
         if constexpr (WIDE) {
@@ -101,10 +110,13 @@ struct Arrays {
         return a[i];
     }
 };
+// norms(kind, sum) in a step with diagnostics: a thread's sums of squares of the gradient as read, the update and the new parameters.
+struct NoNorms {};
 // REGS: loads into registers -- a shared-memory round trip less (0.07 us of a step), where a few blocks per SM leave L1 room enough.
-template <int OPT, int MASK, typename GT, bool POST, bool PLAIN, bool WIDE, bool REGS = false, typename Mean, typename Where>
+template <int OPT, int MASK, typename GT, bool POST, bool PLAIN, bool WIDE, bool REGS = false, typename Mean, typename Where, typename Norms = NoNorms>
 __device__ __forceinline__ void update_quad(const StepArgs &a, float sc, const Quad<WIDE> &q, const Landing &land,
-                                            const Replica<OPT, GT> &from, const Where &to, const Mean &mean) {
+                                            const Replica<OPT, GT> &from, const Where &to, const Mean &mean, const Norms &norms = {}) {
+    constexpr bool DIAG = !std::is_same_v<Norms, NoNorms>;
     constexpr bool SX = MASK & SYNC_X, SU = MASK & SYNC_U, HAS_V = OPT != OPT_SGDM, P = OPT != OPT_SGDM;
     constexpr bool SV = (MASK & SYNC_V) && HAS_V;
     FV<4> X{}, U{}, V{}, G{}, un, vn;
@@ -134,6 +146,12 @@ __device__ __forceinline__ void update_quad(const StepArgs &a, float sc, const Q
         if constexpr (HAS_V) V = q.ld(from.v);
         G = q.template ldg<GT>(from.g);
     }
+    if constexpr (DIAG) norms(DIAG_G, q.sum_of_squares(G));
+    const auto step = [&] {
+        const FV<4> D = minus_direction<OPT, PLAIN, 4>(a, un, vn);
+        if constexpr (DIAG) norms(DIAG_D, q.sum_of_squares(D));
+        X = apply_step<4, P>(a, X, D);
+    };
     if constexpr (!POST) {
         const FV<4> vown = V;
         // (one case per subset of the three arrays)
@@ -159,7 +177,7 @@ __device__ __forceinline__ void update_quad(const StepArgs &a, float sc, const Q
             (SX ? X : SU ? U : V) = s[0];
         }
         state_update<OPT, PLAIN, 4>(a, G, sc, U, V, vown, un, vn);
-        X = apply_step<4, P>(a, X, minus_direction<OPT, PLAIN, 4>(a, un, vn));
+        step();
     } else {
         state_update<OPT, PLAIN, 4>(a, G, sc, U, V, V, un, vn);
         if constexpr (SU && SV) {
@@ -171,13 +189,14 @@ __device__ __forceinline__ void update_quad(const StepArgs &a, float sc, const Q
             mean(s, Arrays<SU ? 1 : 2>{});
             (SU ? un : vn) = s[0];
         }
-        X = apply_step<4, P>(a, X, minus_direction<OPT, PLAIN, 4>(a, un, vn));
+        step();
         if constexpr (SX) {
             FV<4> s[1] = {X};
             mean(s, Arrays<0>{});
             X = s[0];
         }
     }
+    if constexpr (DIAG) norms(DIAG_X, q.sum_of_squares(X));
     const Replica<OPT, GT> w = to();
     q.st(w.x, X);
     q.st(w.u, un);
@@ -202,9 +221,9 @@ __global__ void __launch_bounds__(LANES_THREADS, 10) desloc_lanes_kernel(const _
     const int part0 = static_cast<int>(blockIdx.x - c * a.parts) * a.part_elems + warp * (4 * LW);
     const Chunk ch = a.chunks[c];
     const int cnt = min(ch.count - part0, 4 * LW);
-    if (cnt <= 0) return;   // (of the whole warp)
     const int own = lane / LW, lx = lane - own * LW;
     const int m = MT == 1 ? static_cast<int>(blockIdx.y) : min(own, MT - 1);
+    if (cnt <= 0) return;   // (of the whole warp)
     const Replica<OPT, GT> w(a, static_cast<long long>(m) * a.nt + ch.tensor, ch.start + part0);
     __shared__ float4 landing[landing_arrays<OPT, GT>()][LANES_THREADS];
     const Landing land{reinterpret_cast<float *>(&landing[0][threadIdx.x]), 4 * LANES_THREADS};

@@ -330,8 +330,8 @@ mean_fill_kernel(const Chunk *chunks, long long nchunks, const float *const *src
     }
 }
 
-// Norm diagnostics of a DIAG step.  partial[row * stride + c], row = kind * M + m, holds the sum of
-// squares of chunk c; tstart[k] .. tstart[k + 1] are the chunks of tensor k.  A block per (row,
+// Norm diagnostics of a DIAG step.  partial[row * stride + i], row = kind * M + m, holds the sum of
+// squares of part i % parts of chunk i / parts; tstart[k] .. tstart[k + 1] are the chunks of tensor k.  A block per (row,
 // tensor): fp64 sum of the tensor's chunks, its root as the per-tensor norm.  The first `rows` blocks
 // take a whole row each: the norm over the tensor list.  One launch, and both results go
 // straight to the host's memory.  (A warp per row and tensor spent 20 us in a row on the 6912 chunks of an
@@ -339,7 +339,7 @@ mean_fill_kernel(const Chunk *chunks, long long nchunks, const float *const *src
 constexpr int DIAG_THREADS = 256;
 
 __global__ void __launch_bounds__(DIAG_THREADS)
-diag_norms_kernel(const float *partial, long long stride, const long long *tstart, int nt, int rows, float *norms,
+diag_norms_kernel(const float *partial, long long stride, int parts, const long long *tstart, int nt, int rows, float *norms,
                   float *totals) {
     __shared__ double sh[DIAG_THREADS / 32];
     begin_and_let_next_begin();
@@ -348,7 +348,7 @@ diag_norms_kernel(const float *partial, long long stride, const long long *tstar
     const long long item = static_cast<long long>(blockIdx.x) - rows;
     const long long row = whole ? blockIdx.x : item / nt;
     const int k = static_cast<int>(item - row * nt);
-    const long long c0 = whole ? 0 : tstart[k], c1 = whole ? stride : tstart[k + 1];
+    const long long c0 = whole ? 0 : tstart[k] * parts, c1 = whole ? stride : tstart[k + 1] * parts;
     const double ss = row_sum_f64<false>(partial + row * stride + c0, c1 - c0, sh);
     if (threadIdx.x == 0) (whole ? totals + row : norms + item)[0] = static_cast<float>(sqrt(ss));
 }
@@ -415,11 +415,11 @@ cudaError_t launch_rel_change(const Chunk *chunks, long long nchunks, const floa
     return launch(relchange_finalize_kernel, M, FINAL_THREADS, 0, stream, partial, items, stride, M, out);
 }
 
-cudaError_t launch_diag_norms(const float *partial, long long stride, const long long *tstart,
+cudaError_t launch_diag_norms(const float *partial, long long nchunks, int parts, const long long *tstart,
                               int nt, int M, float *per_tensor, float *totals, cudaStream_t stream) {
     const int rows = DIAG_KINDS * M;
     const long long blocks = rows + static_cast<long long>(rows) * nt;
-    return launch(diag_norms_kernel, grid_for(blocks), DIAG_THREADS, 0, stream, partial, stride, tstart, nt, rows,
+    return launch(diag_norms_kernel, grid_for(blocks), DIAG_THREADS, 0, stream, partial, nchunks * parts, parts, tstart, nt, rows,
                   per_tensor, totals);
 }
 

@@ -151,3 +151,30 @@ def test_diag_fullsize_totals_on_workload_2():
     # coordinate; here just: positive, finite, far below the parameter norm
     assert np.all(per[2] > 0) and np.all(np.isfinite(per[2])) and np.all(per[2] < per[1])
     eng.close()
+
+
+@pytest.mark.parametrize("M", [9, 12, 16, 17, 18, 19, 33, 129])
+@pytest.mark.parametrize("opt,gd,post,align", [("adam", "bf16", False, 4), ("adopt", "f32", True, 1), ("sgdm", "bf16", True, 8), ("adam", "f32", False, 1)])
+def test_more_than_eight_workers_in_either_kernel(M, opt, gd, post, align):
+    """Averaging steps of small problems run in blocks of all replicas with diagnostics, too: the norms of the runtime-M kernel (sums of
+    up to 16 squares of a thread and a tree in fp32 there, of four here: 2e-6 apart at most), and its state bit for bit."""
+    import paper_2505_22549_b200 as d
+    piece = 64 if M < 12 else 32 if M <= 32 else 16
+    numel = (1, 3, piece - 1, piece, 2 * piece + 1, 516, 1031, 2049)
+    w = di.Workload("diag", opt, M, numel, gd, "normal1", beta2=0.99, eps=1e-2, lr=1e-2, weight_decay=0.05, clip_rho=1.5,
+                    adopt_norm_clip=(opt == "adopt"), K=(1, 2, 2), seed=M)
+    dev = torch.device("cuda:0")
+    a, b = (State(w, dev, align=align, v_init=0.25) for _ in range(2))
+    ea, eb = make_engine(d, w, a, post), make_engine(d, w, b, post)
+    d.desloc_testing_set_staging(eb.ctx, 0)
+    for t in range(3):
+        a.fill_grads(t)
+        for m in range(M):
+            b.g[m].copy_(a.g[m])
+        kw = dict(clip_bound=1.0, max_norm=10.0 if t == 2 else 0.0)
+        assert ea.step_diag(t, f32r(w.lr), a.views(a.g), **kw) == eb.step_diag(t, f32r(w.lr), b.views(b.g), **kw)
+        for x, y in zip(ea.diag_norms(), eb.diag_norms()):
+            assert np.allclose(x, y, rtol=2e-6, atol=0)
+    for pa, pb in ((a.x, b.x), (a.u, b.u)) + (((a.v, b.v),) if a.v is not None else ()):
+        assert np.array_equal(a.to_numpy(pa).view(np.uint32), b.to_numpy(pb).view(np.uint32))
+    ea.close(); eb.close()

@@ -238,7 +238,7 @@ DESLOC_API int desloc_get_diag_norms(desloc_ctx *ctx, float *per_tensor_out, flo
  * ||then^m||_2 over the whole tensor list (the rate-of-change measure of Section 5.1,
  * "Metrics", ||s_{t+K} - s_t|| / ||s_t||).  array: 0 = x, 1 = u, 2 = v.  then: host array of
  * M*num_tensors DEVICE pointers to the caller's fp32 snapshot (same shapes as the state).
- * out: host array [M].  Enqueues on `stream` and waits for it: this call synchronises.
+ * out: host array [M].  Enqueues on `stream` and waits for the result: what was on the stream before is complete then.
  */
 DESLOC_API int desloc_rel_change(desloc_ctx *ctx, int32_t array, const float *const *then,
                                  float *out, void *stream);

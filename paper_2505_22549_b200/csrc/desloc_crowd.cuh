@@ -23,7 +23,7 @@ namespace desloc {
 // Mean of column[0], column[T], ... column[(M - 1) T]: trees of B values (1, 2 or 4; what is left value by value) in a
 // compensated sum.
 template <int B>
-__device__ __forceinline__ float column_mean(const float *column, int T, int M) {
+__device__ __forceinline__ float column_mean(const float *column, int T, int M, float inv_m) {
     float sum = 0.f, err = 0.f;
     const auto add = [&](float x) {
         const float t = sum + x, bp = t - sum;
@@ -50,8 +50,7 @@ __device__ __forceinline__ float column_mean(const float *column, int T, int M) 
     }
     for (; m < M; ++m) add(column[m * T]);
     const float hi = sum + err, lo = err - (hi - sum);   // hi + lo = sum + err
-    const float mf = static_cast<float>(M);
-    return div_by_count(hi, lo, mf, 1.f / mf);
+    return div_by_count(hi, lo, static_cast<float>(M), inv_m);
 }
 
 // Lanes of a worker, threads of a block and blocks per SM.  FEW: blocks that all fit at once four to an SM, where
@@ -102,9 +101,13 @@ desloc_crowd_kernel(const __grid_constant__ StepArgs a) {
     };
     const auto replica = [&] { return Replica<OPT, GT>(a, static_cast<long long>(m) * a.nt + ch.tensor, ch.start + part0); };
     const Replica<OPT, GT> w = replica();
+    // (the stores' addresses: kept where there are registers for it)
+    const auto to = [&] { return KIND == CROWD_FEW ? w : replica(); };
     const bool wide = __syncthreads_and(w.wide_ok() && (cnt & 3) == 0) != 0;
     float *const means = pool + landing_arrays<OPT, GT>() * M * T;
     const Landing land{pool + m * T + 4 * lx, M * T};
+    float inv_m = 1.f / static_cast<float>(M);
+    asm volatile("" : "+f"(inv_m));   // (the division stays in front of the wait)
     const auto mean_of_arrays = [&](const auto &q, auto &s, auto arrays, bool landed) {
         using Batch = PostBatch<OPT, MASK, GT>;
         constexpr int N = arrays.N, B = !POST ? 4 : arrays.at(0) == 0 ? Batch::X : Batch::STATES;
@@ -115,7 +118,7 @@ desloc_crowd_kernel(const __grid_constant__ StepArgs a) {
         __syncthreads();
         for (int i = m * L + lx; i < N * T; i += M * L) {
             const int k = i / T, e = i - k * T;
-            if (e < cnt) means[i] = column_mean<B>(pool + arrays.at(k) * M * T + e, T, M);
+            if (e < cnt) means[i] = column_mean<B>(pool + arrays.at(k) * M * T + e, T, M, inv_m);
         }
         __syncthreads();
 #pragma unroll
@@ -128,18 +131,18 @@ desloc_crowd_kernel(const __grid_constant__ StepArgs a) {
     if constexpr (DIAG) {
         wait_for_earlier_kernels();
         const float sc = a.gscale ? a.gscale[m] : 1.f;
-        if (wide) update_quad<OPT, MASK, GT, POST, false, true>(a, sc, q4, land, w, replica, mean4, norms);
-        else update_quad<OPT, MASK, GT, POST, false, false>(a, sc, q1, land, w, replica, mean1, norms);
+        if (wide) update_quad<OPT, MASK, GT, POST, false, true>(a, sc, q4, land, w, to, mean4, norms);
+        else update_quad<OPT, MASK, GT, POST, false, false>(a, sc, q1, land, w, to, mean1, norms);
     } else {
         if (wide && plain_step<OPT>(a)) {   // (the common form: nothing but its loads behind the wait)
             wait_for_earlier_kernels();
-            update_quad<OPT, MASK, GT, POST, true, true>(a, 1.f, q4, land, w, replica, mean4);
+            update_quad<OPT, MASK, GT, POST, true, true>(a, 1.f, q4, land, w, to, mean4);
             return;
         }
         wait_for_earlier_kernels();
         const float sc = a.gscale ? a.gscale[m] : 1.f;
-        if (wide) update_quad<OPT, MASK, GT, POST, false, true>(a, sc, q4, land, w, replica, mean4);
-        else update_quad<OPT, MASK, GT, POST, false, false>(a, sc, q1, land, w, replica, mean1);
+        if (wide) update_quad<OPT, MASK, GT, POST, false, true>(a, sc, q4, land, w, to, mean4);
+        else update_quad<OPT, MASK, GT, POST, false, false>(a, sc, q1, land, w, to, mean1);
     }
 }
 

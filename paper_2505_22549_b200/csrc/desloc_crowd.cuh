@@ -130,6 +130,7 @@ desloc_crowd_kernel(const __grid_constant__ StepArgs a) {
     const auto mean1 = [&](auto &s, auto arrays) { mean_of_arrays(q1, s, arrays, false); };
     if constexpr (DIAG) {
         wait_for_earlier_kernels();
+        if (blockIdx.x == 0 && m == 0 && lx == 0) *a.diag_parts = a.parts;
         const float sc = a.gscale ? a.gscale[m] : 1.f;
         if (wide) update_quad<OPT, MASK, GT, POST, false, true>(a, sc, q4, land, w, to, mean4, norms);
         else update_quad<OPT, MASK, GT, POST, false, false>(a, sc, q1, land, w, to, mean1, norms);

@@ -441,8 +441,9 @@ desloc_step_generic_kernel(const __grid_constant__ StepArgs a) {
 #pragma unroll
                 for (int w = 0; w < BLOCK_THREADS / 32; ++w)
                     total += srows[(w * DIAG_KINDS + kind) * GEN_MAX_M + m];
-                a.diag[(static_cast<long long>(kind) * a.M + m) * a.diag_stride + a.diag_chunk0 + c] = total;
+                a.diag[(static_cast<long long>(kind) * a.M + m) * a.diag_stride + c] = total;
             }
+            if (c == 0 && tid == 0) *a.diag_parts = 1;
         }
     }
 }

@@ -93,7 +93,10 @@ struct WorkerRes {
     float *d_norms = nullptr;    // [2][M]: gradient norms, clip factors
     void **h_snap = nullptr;     // pinned pointer table for desloc_rel_change
     void **d_snap = nullptr;
-    float *d_diag = nullptr;     // diagnostics step: [3][M][row] sums of squares, of a chunk each or, in desloc_crowd_kernel, of a part of one
+    // Diagnostics step: [3][M][row] sums of squares, of a chunk each or, in desloc_crowd_kernel, of a part of one.  How many a chunk
+    // has is written beside them by the step that leaves them: the host does not see when a captured step runs.
+    float *d_diag = nullptr;
+    int *d_diag_parts = nullptr;
     // Results the host waits for go to its memory straight from the kernels, without a copy:
     // [3][M][num_tensors] per-tensor norms, [3][M] totals, [M] relative changes.
     Slot host_slots[2];          // the same of addresses in host memory (desloc_step_host), staged on the copy stream
@@ -207,7 +210,12 @@ cudaError_t make_worker_res(WorkerRes &r, const desloc_config &cfg, int M, const
     as.M = M;
     const desloc::LaunchPlan crowd = desloc::plan_launch(as, DESLOC_SYNC_X, r.set, true, false, desloc::GradLayout::FIT);
     const int64_t row = crowd.kernel == desloc::Kernel::CROWD ? nchunks * crowd.parts : nchunks;
-    if (e == cudaSuccess) e = cudaMalloc(&r.d_diag, ndiag * static_cast<size_t>(row) * sizeof(float));
+    static_assert(sizeof(int) == sizeof(float), "the number of parts lies behind the sums");
+    if (e == cudaSuccess) e = cudaMalloc(&r.d_diag, (ndiag * static_cast<size_t>(row) + 1) * sizeof(float));
+    if (e == cudaSuccess) {
+        r.d_diag_parts = reinterpret_cast<int *>(r.d_diag + ndiag * static_cast<size_t>(row));
+        e = cudaMemset(r.d_diag_parts, 0, sizeof(int));
+    }
     if (e == cudaSuccess)
         e = cudaHostAlloc(reinterpret_cast<void **>(&r.h_out), (ndiag * (num_tensors + 1) + M) * sizeof(float),
                           cudaHostAllocMapped);
@@ -222,6 +230,8 @@ cudaError_t make_worker_res(WorkerRes &r, const desloc_config &cfg, int M, const
         s.dev = r.d_slots + i * room;
         e = cudaEventCreateWithFlags(&s.done, cudaEventDisableTiming);
     }
+    // (memsets are asynchronous, and the caller's stream need not wait for this one)
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
     return e;
 }
 
@@ -249,8 +259,7 @@ struct desloc_ctx {
     int64_t counters[4] = {0, 0, 0, 0};
     int64_t launches = 0;
     int last_cuda_error = 0;
-    bool diag_valid = false;        // a diagnostics step has run since the workers last changed,
-    int diag_parts = 1;             // and left so many sums per chunk
+    bool diag_valid = false;        // a diagnostics step has run since the workers last changed
     int64_t max_blocks = 0;         // test hook: cap on the grid (0 = one block per work item)
     int staging_mode = -1;          // test hook: -1 the library decides; tile kernels that 0 always stage, 1 never, 2 as decided
     std::vector<const void *> prepared;  // kernels whose shared-memory limit this context has raised
@@ -496,9 +505,8 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
             for (int64_t i = 0; i < ctx->nptr; ++i) a.g_inline[i] = grads[i];
         a.gscale = d_gscale;
         a.diag = diag ? ctx->res.d_diag : nullptr;
-        const int diag_parts = plan.kernel == desloc::Kernel::CROWD ? plan.parts : 1;
-        a.diag_stride = ctx->res.nchunks * diag_parts;
-        a.diag_chunk0 = 0;
+        a.diag_stride = ctx->res.nchunks * (plan.kernel == desloc::Kernel::CROWD ? plan.parts : 1);
+        a.diag_parts = ctx->res.d_diag_parts;
         desloc::fill_hyper(a, c, lr_t, clip_bound_t);
         a.err = ctx->d_err;
         a.wait_limit = ctx->wait_limit;
@@ -559,7 +567,6 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
                 if (e != cudaSuccess) break;
                 a.chunks = ctx->res.d_chunks + grp.c0;
                 a.nchunks = grp.c1 - grp.c0;
-                a.diag_chunk0 = grp.c0;
                 const desloc::LaunchPlan &gp = plans[gi];
                 desloc::fill_plan(a, gp);
                 if (forced && !gp.whole) a.direct = ctx->staging_mode;
@@ -585,10 +592,7 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
                 s.in_flight = true;
             }
         }
-        if (diag) {
-            ctx->diag_valid = true;
-            ctx->diag_parts = diag_parts;
-        }
+        if (diag) ctx->diag_valid = true;
         ctx->counters[0] += 1;
         ctx->counters[1] += (mask & DESLOC_SYNC_X) ? 1 : 0;
         ctx->counters[2] += (mask & DESLOC_SYNC_U) ? 1 : 0;
@@ -764,7 +768,7 @@ int desloc_get_diag_norms(desloc_ctx *ctx, float *per_tensor_out, float *total_o
     const size_t rows = static_cast<size_t>(desloc::DIAG_KINDS) * c.M;
     const size_t per = rows * c.num_tensors;
     expect_results(ctx->res.h_out, per + rows);
-    e = desloc::launch_diag_norms(ctx->res.d_diag, ctx->res.nchunks, ctx->diag_parts, ctx->res.d_tstart, c.num_tensors, c.M,
+    e = desloc::launch_diag_norms(ctx->res.d_diag, ctx->res.nchunks, ctx->res.d_diag_parts, ctx->res.d_tstart, c.num_tensors, c.M,
                                   ctx->res.d_out, ctx->res.d_out + per, st);
     if (e == cudaSuccess) ctx->launches += 1;
     if (e == cudaSuccess) e = wait_for_results(ctx->res.h_out, per + rows, st);

@@ -117,8 +117,8 @@ struct StepArgs {
     const void *g_inline[INLINE_PTRS];   // small problems under stream capture (no table upload)
     const float *gscale;  // per-worker factor applied to g before the clip, or nullptr (= 1)
     float *diag;          // DIAG kernels: [DIAG_KINDS][M][diag_stride] partial sums of squares
-    long long diag_stride;  // chunks of the whole context (a launch may cover a sub-range)
-    long long diag_chunk0;  // index of chunks[0] within the context's chunk table
+    long long diag_stride;  // chunks of the whole context, times the sums that a chunk gets
+    int *diag_parts;        // that number: written by the step itself, which may be a captured one that runs at any time
     int *err;             // set to 1 when a bounded wait ran out (may be nullptr)
     int wait_limit;       // iterations a block polls for its tile before it gives up
     int direct;           // non-zero: no staging, every chunk straight from global memory (tiny launches)
@@ -882,7 +882,8 @@ desloc_step_kernel(const __grid_constant__ StepArgs a) {
 #pragma unroll
                 for (int w = 0; w < THREADS / 32; ++w) total += slots[tid * (THREADS / 32) + w];
                 const int kind = tid / MT, mm = tid - kind * MT;
-                a.diag[(static_cast<long long>(kind) * a.M + m0 + mm) * a.diag_stride + a.diag_chunk0 + c] = total;
+                a.diag[(static_cast<long long>(kind) * a.M + m0 + mm) * a.diag_stride + c] = total;
+                if (tid == 0 && m0 == 0 && c == 0) *a.diag_parts = 1;
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // before the copy engine writes there again
         }

@@ -330,8 +330,8 @@ mean_fill_kernel(const Chunk *chunks, long long nchunks, const float *const *src
     }
 }
 
-// Norm diagnostics of a DIAG step.  partial[row * stride + i], row = kind * M + m, holds the sum of
-// squares of part i % parts of chunk i / parts; tstart[k] .. tstart[k + 1] are the chunks of tensor k.  A block per (row,
+// Norm diagnostics of a DIAG step.  partial[row * nchunks * parts + i], row = kind * M + m, holds the sum of
+// squares of part i % parts of chunk i / parts (parts = *parts_of: of the step that ran last); tstart[k] .. tstart[k + 1] are the chunks of tensor k.  A block per (row,
 // tensor): fp64 sum of the tensor's chunks, its root as the per-tensor norm.  The first `rows` blocks
 // take a whole row each: the norm over the tensor list.  One launch, and both results go
 // straight to the host's memory.  (A warp per row and tensor spent 20 us in a row on the 6912 chunks of an
@@ -339,11 +339,13 @@ mean_fill_kernel(const Chunk *chunks, long long nchunks, const float *const *src
 constexpr int DIAG_THREADS = 256;
 
 __global__ void __launch_bounds__(DIAG_THREADS)
-diag_norms_kernel(const float *partial, long long stride, int parts, const long long *tstart, int nt, int rows, float *norms,
+diag_norms_kernel(const float *partial, long long nchunks, const int *parts_of, const long long *tstart, int nt, int rows, float *norms,
                   float *totals) {
     __shared__ double sh[DIAG_THREADS / 32];
     begin_and_let_next_begin();
     wait_for_earlier_kernels();
+    const int parts = *parts_of;
+    const long long stride = nchunks * parts;
     const bool whole = blockIdx.x < rows;
     const long long item = static_cast<long long>(blockIdx.x) - rows;
     const long long row = whole ? blockIdx.x : item / nt;
@@ -415,11 +417,11 @@ cudaError_t launch_rel_change(const Chunk *chunks, long long nchunks, const floa
     return launch(relchange_finalize_kernel, M, FINAL_THREADS, 0, stream, partial, items, stride, M, out);
 }
 
-cudaError_t launch_diag_norms(const float *partial, long long nchunks, int parts, const long long *tstart,
+cudaError_t launch_diag_norms(const float *partial, long long nchunks, const int *parts, const long long *tstart,
                               int nt, int M, float *per_tensor, float *totals, cudaStream_t stream) {
     const int rows = DIAG_KINDS * M;
     const long long blocks = rows + static_cast<long long>(rows) * nt;
-    return launch(diag_norms_kernel, grid_for(blocks), DIAG_THREADS, 0, stream, partial, nchunks * parts, parts, tstart, nt, rows,
+    return launch(diag_norms_kernel, grid_for(blocks), DIAG_THREADS, 0, stream, partial, nchunks, parts, tstart, nt, rows,
                   per_tensor, totals);
 }
 

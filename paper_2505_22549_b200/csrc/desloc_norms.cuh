@@ -22,10 +22,10 @@ cudaError_t launch_rel_change(const Chunk *chunks, long long nchunks, const floa
                               const float *const *then, int nt, int M, float *partial, float *out,
                               int *err, int wait_limit, cudaStream_t stream);
 
-// Norms of a diagnostics step: partial [DIAG_KINDS][M][nchunks * parts] sums of squares of the parts of a chunk,
+// Norms of a diagnostics step: partial [DIAG_KINDS][M][nchunks * *parts] sums of squares of the parts of a chunk,
 // tstart [nt + 1] first chunk of every tensor; writes per_tensor [DIAG_KINDS][M][nt] and totals
 // [DIAG_KINDS][M] (floats; may be host memory that the device can write to).  One launch.
-cudaError_t launch_diag_norms(const float *partial, long long nchunks, int parts, const long long *tstart,
+cudaError_t launch_diag_norms(const float *partial, long long nchunks, const int *parts, const long long *tstart,
                               int nt, int M, float *per_tensor, float *totals, cudaStream_t stream);
 
 // Every element of the m_dst destination replicas := mean over the m_src source replicas.

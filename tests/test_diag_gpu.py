@@ -178,3 +178,38 @@ def test_more_than_eight_workers_in_either_kernel(M, opt, gd, post, align):
     for pa, pb in ((a.x, b.x), (a.u, b.u)) + (((a.v, b.v),) if a.v is not None else ()):
         assert np.array_equal(a.to_numpy(pa).view(np.uint32), b.to_numpy(pb).view(np.uint32))
     ea.close(); eb.close()
+
+
+@pytest.mark.parametrize("M", [12, 16])
+def test_norms_are_those_of_the_step_that_ran_last(M):
+    """Averaging and local steps of these run in different kernels, which leave different numbers of partial sums.  A graph's replay
+    comes past no host code, and a captured step has not run: the read-out follows what ran on the device."""
+    import paper_2505_22549_b200 as d
+    w = di.Workload("replay", "adam", M, (3000, 1031), "f32", "normal1", beta2=0.99, eps=1e-2, lr=1e-2, K=(2, 2, 2), seed=M)
+    dev = torch.device("cuda:0")
+    a, b = (State(w, dev, v_init=0.25) for _ in range(2))
+    ea, eb = make_engine(d, w, a), make_engine(d, w, b)
+    for st in (a, b):
+        st.fill_grads(0)
+    run = lambda eng, st, t: eng.step_diag(t, 1e-2, st.views(st.g))
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        run(ea, a, 0), run(eb, b, 0)                        # (t = 0: everything averaged; t = 1: nothing)
+        for first, then in ((0, 1), (1, 0)):
+            run(ea, a, first), run(eb, b, first)
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=side):
+                run(ea, a, then)
+            assert ea.diag_norms() == eb.diag_norms()       # nothing of the captured step has run
+            run(ea, a, first), run(eb, b, first)
+            graph.replay(), run(eb, b, then)
+            assert ea.diag_norms() == eb.diag_norms()       # the replayed step was the last one
+            run(ea, a, first), run(eb, b, first)
+            assert ea.diag_norms() == eb.diag_norms()
+            graph.replay(), run(eb, b, then)
+            assert ea.diag_norms() == eb.diag_norms()
+            del graph
+    torch.cuda.synchronize()
+    assert np.array_equal(a.to_numpy(a.x), b.to_numpy(b.x))
+    ea.close(); eb.close()

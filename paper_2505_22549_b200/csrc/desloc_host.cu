@@ -4,7 +4,6 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <chrono>
 #include <cmath>
 #include <cstdint>
 #include <cstdlib>
@@ -19,6 +18,7 @@
 #include "desloc_inst.cuh"
 #include "desloc_internal.cuh"
 #include "desloc_norms.cuh"
+#include "desloc_readout.cuh"
 
 namespace desloc {
 
@@ -93,13 +93,13 @@ struct WorkerRes {
     float *d_norms = nullptr;    // [2][M]: gradient norms, clip factors
     void **h_snap = nullptr;     // pinned pointer table for desloc_rel_change
     void **d_snap = nullptr;
+    Slot host_slots[2];          // tables of addresses in host memory (desloc_step_host), staged on the copy stream
     // Diagnostics step: [3][M][row] sums of squares, of a chunk each or, in desloc_crowd_kernel, of a part of one.  How many a chunk
     // has is written beside them by the step that leaves them: the host does not see when a captured step runs.
     float *d_diag = nullptr;
     int *d_diag_parts = nullptr;
-    // Results the host waits for go to its memory straight from the kernels, without a copy:
-    // [3][M][num_tensors] per-tensor norms, [3][M] totals, [M] relative changes.
-    Slot host_slots[2];          // the same of addresses in host memory (desloc_step_host), staged on the copy stream
+    // Results the host waits for go to its memory straight from the kernels, without a copy: [3][M][num_tensors] per-tensor norms,
+    // [3][M] totals; [M] relative changes; a word behind either for the state of the wait flag.
     float *h_out = nullptr;      // mapped pinned memory, and
     float *d_out = nullptr;      // the same as the kernels address it
 };
@@ -217,7 +217,7 @@ cudaError_t make_worker_res(WorkerRes &r, const desloc_config &cfg, int M, const
         e = cudaMemset(r.d_diag_parts, 0, sizeof(int));
     }
     if (e == cudaSuccess)
-        e = cudaHostAlloc(reinterpret_cast<void **>(&r.h_out), (ndiag * (num_tensors + 1) + M) * sizeof(float),
+        e = cudaHostAlloc(reinterpret_cast<void **>(&r.h_out), (ndiag * (num_tensors + 1) + M + 2) * sizeof(float),
                           cudaHostAllocMapped);
     if (e == cudaSuccess) e = cudaHostGetDevicePointer(reinterpret_cast<void **>(&r.d_out), r.h_out, 0);
     const size_t room = static_cast<size_t>(nptr + 15) & ~size_t{15};   // tables on 128-byte boundaries
@@ -279,27 +279,6 @@ int cuda_fail(desloc_ctx *ctx, cudaError_t e) {
 // A block of an earlier kernel of this context gave up waiting for its copies: what it should have
 // updated or summed up is incomplete.
 bool wait_ran_out(const desloc_ctx *ctx) { return *static_cast<volatile int *>(ctx->h_err) != 0; }
-
-// Results that the last kernel of a call writes straight to the host's memory (WorkerRes::h_out), each value once: the calling thread looks for them
-// there, and asks the driver only when they keep it waiting (20 ms, or an error).  A launch and cudaStreamSynchronize() take 10.6 us until
-// the thread goes on, a launch and the look 7.1.  What is in front in the stream is complete when they are there.
-constexpr uint32_t kUnwritten = 0x7fb5eed5u;   // (a NaN that no conversion or root gives)
-
-void expect_results(float *v, size_t n) {
-    volatile uint32_t *p = reinterpret_cast<volatile uint32_t *>(v);
-    for (size_t i = 0; i < n; ++i) p[i] = kUnwritten;
-}
-
-cudaError_t wait_for_results(const float *v, size_t n, cudaStream_t stream) {
-    const volatile uint32_t *p = reinterpret_cast<const volatile uint32_t *>(v);
-    const auto until = std::chrono::steady_clock::now() + std::chrono::milliseconds(20);
-    unsigned looks = 0;
-    for (size_t i = 0; i < n; ++i) {
-        while (p[i] == kUnwritten)
-            if ((++looks & 1023u) == 0 && std::chrono::steady_clock::now() > until) return cudaStreamSynchronize(stream);
-    }
-    return cudaSuccess;
-}
 
 void free_ctx(desloc_ctx *ctx) {
     if (!ctx) return;
@@ -767,15 +746,16 @@ int desloc_get_diag_norms(desloc_ctx *ctx, float *per_tensor_out, float *total_o
     if (e != cudaSuccess) return cuda_fail(ctx, e);
     const size_t rows = static_cast<size_t>(desloc::DIAG_KINDS) * c.M;
     const size_t per = rows * c.num_tensors;
-    expect_results(ctx->res.h_out, per + rows);
+    float *const out = ctx->res.h_out;
+    desloc::expect_results(out, per + rows + 1);
     e = desloc::launch_diag_norms(ctx->res.d_diag, ctx->res.nchunks, ctx->res.d_diag_parts, ctx->res.d_tstart, c.num_tensors, c.M,
-                                  ctx->res.d_out, ctx->res.d_out + per, st);
+                                  ctx->res.d_out, ctx->res.d_out + per, ctx->d_err, ctx->res.d_out + per + rows, st);
     if (e == cudaSuccess) ctx->launches += 1;
-    if (e == cudaSuccess) e = wait_for_results(ctx->res.h_out, per + rows, st);
-    const bool valid = e == cudaSuccess && !wait_ran_out(ctx);
+    if (e == cudaSuccess) e = desloc::wait_for_results(out, per + rows + 1, [st] { return cudaStreamSynchronize(st); });
+    const bool valid = e == cudaSuccess && out[per + rows] == 0.f;
     if (valid) {
-        if (per_tensor_out) std::memcpy(per_tensor_out, ctx->res.h_out, per * sizeof(float));
-        if (total_out) std::memcpy(total_out, ctx->res.h_out + per, rows * sizeof(float));
+        if (per_tensor_out) std::memcpy(per_tensor_out, out, per * sizeof(float));
+        if (total_out) std::memcpy(total_out, out + per, rows * sizeof(float));
     }
     if (dev_before != ctx->device) cudaSetDevice(dev_before);
     if (e != cudaSuccess) return cuda_fail(ctx, e);
@@ -852,18 +832,19 @@ int desloc_rel_change(desloc_ctx *ctx, int32_t array, const float *const *then, 
     // The call ends when the kernels behind this copy have their results, so the pinned table is free again on return.
     std::memcpy(ctx->res.h_snap, then, tbytes);
     e = cudaMemcpyAsync(ctx->res.d_snap, ctx->res.h_snap, tbytes, cudaMemcpyHostToDevice, st);
-    const size_t at = static_cast<size_t>(desloc::DIAG_KINDS) * ctx->cfg.M * (ctx->cfg.num_tensors + 1);
-    expect_results(ctx->res.h_out + at, static_cast<size_t>(ctx->cfg.M));
+    const size_t M = static_cast<size_t>(ctx->cfg.M), at = desloc::DIAG_KINDS * M * (ctx->cfg.num_tensors + 1) + 1;
+    float *const change = ctx->res.h_out + at;
+    desloc::expect_results(change, M + 1);
     if (e == cudaSuccess)
         e = desloc::launch_rel_change(
             ctx->d_rchunks, ctx->nrchunks,
             reinterpret_cast<const float *const *>(ctx->res.d_tables + array * ctx->nptr),
             reinterpret_cast<const float *const *>(ctx->res.d_snap), ctx->cfg.num_tensors, ctx->cfg.M,
-            ctx->res.d_partial, ctx->res.d_out + at, ctx->d_err, ctx->wait_limit, st);
+            ctx->res.d_partial, ctx->res.d_out + at, ctx->res.d_out + at + M, ctx->d_err, ctx->wait_limit, st);
     if (e == cudaSuccess) ctx->launches += 2;
-    if (e == cudaSuccess) e = wait_for_results(ctx->res.h_out + at, static_cast<size_t>(ctx->cfg.M), st);
-    const bool valid = e == cudaSuccess && !wait_ran_out(ctx);
-    if (valid) std::memcpy(out, ctx->res.h_out + at, static_cast<size_t>(ctx->cfg.M) * sizeof(float));
+    if (e == cudaSuccess) e = desloc::wait_for_results(change, M + 1, [st] { return cudaStreamSynchronize(st); });
+    const bool valid = e == cudaSuccess && change[M] == 0.f;
+    if (valid) std::memcpy(out, change, M * sizeof(float));
     if (dev_before != ctx->device) cudaSetDevice(dev_before);
     if (e != cudaSuccess) return cuda_fail(ctx, e);
     return valid ? DESLOC_OK : DESLOC_E_DEVICE_WAIT;

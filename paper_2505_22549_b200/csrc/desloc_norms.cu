@@ -198,6 +198,15 @@ __device__ __forceinline__ void finish_norm(double ss, float max_norm, float *no
     *scale = (max_norm > 0.f && nrm > static_cast<double>(max_norm)) ? static_cast<float>(static_cast<double>(max_norm) / nrm) : 1.f;
 }
 
+// The last word of a read-out: has a bounded wait of a kernel in front run out?  Its flag lies in the host's memory: a block of its own, the first,
+// looks there and writes the word while the others add up (behind the sums of one of them: 2 us more).
+__device__ __forceinline__ void hand_over_flag(const int *err, float *word) {
+    if (threadIdx.x != 0) return;
+    const int flag = *reinterpret_cast<const volatile int *>(err);
+    __threadfence_system();   // what is complete for this thread is complete for the host that sees the word
+    *reinterpret_cast<volatile float *>(word) = flag != 0 ? 1.f : 0.f;
+}
+
 constexpr int FINAL_THREADS = 512;
 
 // norms[m] = ||g^m||_2, scales[m] = min(1, max_norm / norms[m]) (1 when max_norm <= 0).
@@ -214,11 +223,12 @@ norm_finalize_kernel(float *partial, long long n, long long stride, float max_no
 }
 
 __global__ void __launch_bounds__(FINAL_THREADS)
-relchange_finalize_kernel(float *partial, long long n, long long stride, int M, float *out) {
+relchange_finalize_kernel(float *partial, long long n, long long stride, int M, float *out, const int *err, float *ran_out) {
     __shared__ double sh[FINAL_THREADS / 32];
     begin_and_let_next_begin();
     wait_for_earlier_kernels();
-    const int m = blockIdx.x;
+    if (blockIdx.x == 0) return hand_over_flag(err, ran_out);
+    const int m = blockIdx.x - 1;
     float *row = partial + m * stride, *row2 = partial + (static_cast<long long>(M) + m) * stride;
     pad_row(row, n, stride);
     pad_row(row2, n, stride);
@@ -332,23 +342,24 @@ mean_fill_kernel(const Chunk *chunks, long long nchunks, const float *const *src
 
 // Norm diagnostics of a DIAG step.  partial[row * nchunks * parts + i], row = kind * M + m, holds the sum of
 // squares of part i % parts of chunk i / parts (parts = *parts_of: of the step that ran last); tstart[k] .. tstart[k + 1] are the chunks of tensor k.  A block per (row,
-// tensor): fp64 sum of the tensor's chunks, its root as the per-tensor norm.  The first `rows` blocks
-// take a whole row each: the norm over the tensor list.  One launch, and both results go
+// tensor): fp64 sum of the tensor's chunks, its root as the per-tensor norm.  In front of them `rows` blocks that
+// take a whole row each: the norm over the tensor list.  One launch, and all results go
 // straight to the host's memory.  (A warp per row and tensor spent 20 us in a row on the 6912 chunks of an
 // embedding; three partial sums per chunk, for shorter blocks in the step, made the step no faster.)
 constexpr int DIAG_THREADS = 256;
 
 __global__ void __launch_bounds__(DIAG_THREADS)
 diag_norms_kernel(const float *partial, long long nchunks, const int *parts_of, const long long *tstart, int nt, int rows, float *norms,
-                  float *totals) {
+                  float *totals, const int *err, float *ran_out) {
     __shared__ double sh[DIAG_THREADS / 32];
     begin_and_let_next_begin();
     wait_for_earlier_kernels();
-    const int parts = *parts_of;
+    if (blockIdx.x == 0) return hand_over_flag(err, ran_out);
+    const int parts = *parts_of, block = static_cast<int>(blockIdx.x) - 1;
     const long long stride = nchunks * parts;
-    const bool whole = blockIdx.x < rows;
-    const long long item = static_cast<long long>(blockIdx.x) - rows;
-    const long long row = whole ? blockIdx.x : item / nt;
+    const bool whole = block < rows;
+    const long long item = static_cast<long long>(block) - rows;
+    const long long row = whole ? block : item / nt;
     const int k = static_cast<int>(item - row * nt);
     const long long c0 = whole ? 0 : tstart[k] * parts, c1 = whole ? stride : tstart[k + 1] * parts;
     const double ss = row_sum_f64<false>(partial + row * stride + c0, c1 - c0, sh);
@@ -407,22 +418,23 @@ cudaError_t launch_grad_norms(const Chunk *chunks, long long nchunks, int64_t el
 }
 
 cudaError_t launch_rel_change(const Chunk *chunks, long long nchunks, const float *const *now,
-                              const float *const *then, int nt, int M, float *partial, float *out,
+                              const float *const *then, int nt, int M, float *partial, float *out, float *ran_out,
                               int *err, int wait_limit, cudaStream_t stream) {
     long long items, stride;
     const cudaError_t e = launch_sumsq<RED_CHANGE>(
         chunks, nchunks, reinterpret_cast<const void *const *>(now), reinterpret_cast<const void *const *>(then), nt, M,
         partial, &items, &stride, err, wait_limit, stream);
     if (e != cudaSuccess) return e;
-    return launch(relchange_finalize_kernel, M, FINAL_THREADS, 0, stream, partial, items, stride, M, out);
+    return launch(relchange_finalize_kernel, M + 1, FINAL_THREADS, 0, stream, partial, items, stride, M, out, err, ran_out);
 }
 
 cudaError_t launch_diag_norms(const float *partial, long long nchunks, const int *parts, const long long *tstart,
-                              int nt, int M, float *per_tensor, float *totals, cudaStream_t stream) {
+                              int nt, int M, float *per_tensor, float *totals, const int *err, float *ran_out,
+                              cudaStream_t stream) {
     const int rows = DIAG_KINDS * M;
-    const long long blocks = rows + static_cast<long long>(rows) * nt;
+    const long long blocks = 1 + rows + static_cast<long long>(rows) * nt;
     return launch(diag_norms_kernel, grid_for(blocks), DIAG_THREADS, 0, stream, partial, nchunks, parts, tstart, nt, rows,
-                  per_tensor, totals);
+                  per_tensor, totals, err, ran_out);
 }
 
 cudaError_t launch_mean_fill(const Chunk *chunks, long long nchunks, const float *const *src,

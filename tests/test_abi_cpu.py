@@ -63,6 +63,23 @@ def test_host_gradients_are_counted_before_the_driver_is_asked(tmp_path):
     assert r.returncode == 0 and "host_runs_check: ok" in r.stdout, r.stdout + r.stderr
 
 
+def _run_check(tmp_path, name, *objects):
+    """tests/c_abi/<name>.cpp, built with the library's own headers (and objects), says that it is ok."""
+    import subprocess
+    csrc = os.path.join(ROOT, "paper_2505_22549_b200", "csrc")
+    exe = str(tmp_path / name)
+    cuda = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")
+    subprocess.check_call(["g++", "-std=c++17", "-Wall", "-Wextra", "-Werror", "-pthread", "-isystem", cuda, "-I", csrc,
+                           os.path.join(ROOT, "tests", "c_abi", name + ".cpp"), *objects, "-o", exe])
+    r = subprocess.run([exe], capture_output=True, text=True)
+    assert r.returncode == 0 and name + ": ok" in r.stdout, r.stdout + r.stderr
+
+
+def test_read_outs_wait_for_the_state_of_the_wait_flag(tmp_path):
+    """Results that are there before the word that says whether they are complete are not handed out."""
+    _run_check(tmp_path, "readout_check")
+
+
 def test_sync_mask_matches_oracle_schedule(d):
     for opt, oid in (("adam", oracle.ADAM), ("adopt", oracle.ADOPT), ("sgdm", oracle.SGDM)):
         for K in [(4, 8, 16), (1, 1, 1), (16, 64, 256), (0, 0, 0), (3, 0, 7), (256, 768, 1536)]:

@@ -85,3 +85,38 @@ def test_read_outs_after_a_wait_that_ran_out_say_so(gd):
         step(eng, 2, st.views(st.g))
         read(eng)
         eng.close()
+
+
+@pytest.mark.parametrize("gd", ["bf16", "f32"])
+def test_a_reduction_whose_wait_ran_out_says_so(gd):
+    """More parameters than the norms of one launch take, and steps that have no bounded wait of their own: the wait that runs out is the
+    reduction's.  Norms and rates of change of incomplete sums are refused, time and again, and the next good ones are right."""
+    import paper_2505_22549_b200 as d
+    w = di.Workload("reductions", "adam", 2, (150_000, 4096, 33), gd, "normal1", lr=1e-2, K=(1, 1, 1), seed=3)
+    dev = torch.device("cuda:0")
+    st = State(w, dev)
+    eng = make_engine(d, w, st)
+    assert d.desloc_testing_kernel_of(d.make_config(2, w.numel, "adam", gd), 7)[0] == "lanes"
+    gv = st.views(st.g)
+    st.fill_grads(0)
+    eng.step_normclip(0, 1e-3, gv, 1.0)
+    norms, then = eng.grad_norms(), [[b.clone() for b in row] for row in st.views(st.x)]
+    for row in then:
+        for b in row:
+            b.mul_(0.5)
+    for _ in range(8):
+        d.desloc_testing_set_wait_limit(eng.ctx, 0)
+        with pytest.raises(d.DeslocError) as e:
+            eng.rel_change(0, then)
+        assert e.value.status == d.DESLOC_E_DEVICE_WAIT
+        d.desloc_testing_set_wait_limit(eng.ctx, -1)
+        assert np.allclose(eng.rel_change(0, then), 1.0, rtol=1e-5)
+    d.desloc_testing_set_wait_limit(eng.ctx, 0)
+    eng.step_normclip(1, 1e-3, gv, 1.0)
+    with pytest.raises(d.DeslocError) as e:
+        eng.grad_norms()
+    assert e.value.status == d.DESLOC_E_DEVICE_WAIT
+    d.desloc_testing_set_wait_limit(eng.ctx, -1)
+    eng.step_normclip(2, 1e-3, gv, 1.0)
+    assert np.array_equal(eng.grad_norms()[0], norms[0])
+    eng.close()

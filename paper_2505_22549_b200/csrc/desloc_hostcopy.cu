@@ -137,8 +137,11 @@ cudaError_t launch_host_copy(const HostRuns &runs, cudaStream_t stream) {
 
 cudaError_t launch_host_gather(const HostGather &a, cudaStream_t stream) {
     const long long warps = (a.last - a.first) * a.M, blocks = (warps + COPY_THREADS / 32 - 1) / (COPY_THREADS / 32);
-    host_gather_kernel<<<static_cast<unsigned>(blocks < GATHER_BLOCKS ? blocks : GATHER_BLOCKS), COPY_THREADS, 0, stream>>>(a);
-    return cudaGetLastError();
+    cudaLaunchConfig_t lc{};
+    lc.gridDim = dim3(static_cast<unsigned>(blocks < GATHER_BLOCKS ? blocks : GATHER_BLOCKS));
+    lc.blockDim = dim3(COPY_THREADS);
+    lc.stream = stream;
+    return cudaLaunchKernelEx(&lc, host_gather_kernel, a);   // (its own error: an older one of the thread is not this launch's)
 }
 
 }  // namespace desloc

@@ -80,6 +80,13 @@ def test_read_outs_wait_for_the_state_of_the_wait_flag(tmp_path):
     _run_check(tmp_path, "readout_check")
 
 
+def test_a_gather_launch_reports_its_own_error(d, tmp_path):
+    """Against a runtime in which an earlier call of the thread has failed: a launch between two groups of step_host() that succeeds is
+    not taken for one that did not."""
+    from paper_2505_22549_b200 import build
+    _run_check(tmp_path, "gather_launch_check", os.path.join(build.OBJ, "desloc_hostcopy.o"))
+
+
 def test_sync_mask_matches_oracle_schedule(d):
     for opt, oid in (("adam", oracle.ADAM), ("adopt", oracle.ADOPT), ("sgdm", oracle.SGDM)):
         for K in [(4, 8, 16), (1, 1, 1), (16, 64, 256), (0, 0, 0), (3, 0, 7), (256, 768, 1536)]:

@@ -212,8 +212,19 @@ constexpr int LANES_THREADS = 128;
 __host__ __device__ constexpr int lanes_groups(int mt) { return mt <= 4 ? mt : 8; }
 __host__ __device__ constexpr int lanes_part_elems(int mt) { return LANES_THREADS / 32 * 4 * (32 / lanes_groups(mt)); }
 
+// Blocks per SM that the compiler has to leave room for, where it would take a step of registers more without a need (34 to 44 instead of 32 or
+// 40, nothing spilled without them): a kernel of many blocks lives on those in flight.  Four workers, SGDM, x and u averaged, bf16 gradients,
+// 1 to 5 million coordinates: 16 blocks 0.84 to 0.95 of the time with 12, one of three arrays 0.94; Adam, five to eight workers, and ADOPT behind the
+// average, 0.5 to 1.5 million: 12 blocks 0.81 to 0.97 of 10.  (The others are faster with the registers: SGDM of two workers behind the
+// average 1.1 of the time with 16 blocks, Adam of five to seven that averages all arrays up to 1.16 with 12.)
+__host__ __device__ constexpr int lanes_min_blocks(int opt, int mask, int mt, bool post) {
+    if (opt == OPT_SGDM) return post ? (mt == 2 ? 10 : 16) : mt == 2 || mt == 3 ? 12 : 16;
+    if (opt == OPT_ADOPT) return post && mt >= 5 && mt < 8 ? 12 : 10;
+    return !post && mt >= 5 && (mt == 8 ? mask == 5 : mask == 1 || mask == 3) ? 12 : 10;
+}
+
 template <int OPT, int MASK, int MT, typename GT, bool POST>
-__global__ void __launch_bounds__(LANES_THREADS, 10) desloc_lanes_kernel(const __grid_constant__ StepArgs a) {
+__global__ void __launch_bounds__(LANES_THREADS, lanes_min_blocks(OPT, MASK, MT, POST)) desloc_lanes_kernel(const __grid_constant__ StepArgs a) {
     constexpr int G = lanes_groups(MT), LW = 32 / G;   // lanes of a worker
     begin_and_let_next_begin();
     const unsigned c = item_chunk(a, blockIdx.x);

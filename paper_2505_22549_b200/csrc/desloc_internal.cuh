@@ -377,10 +377,10 @@ inline int64_t lanes_most(int mt) {
 // 1.5 million 0.67 to 0.79, 2.2 million 0.9 to 0.97; 12 and 14 2.2 million 0.7 to 0.8, 3.2 million 0.87 to 0.98; 16 3.2 million 0.87, 4.6 million 1.0;
 // 20 and 24 3.2 million 0.67, 4.2 million 0.7, 5.6 million 0.9 (up to 1.2); 32 5.6 million 0.78, 10 million 0.9; 64 7 million 0.7, 10 million 0.98; 128 and
 // 256 up to ten million 0.03 to 0.82 (15: 0.7 to 1.2).  SGDM, which has the least to load, by itself: nine and ten 1.8 million 0.8, 2.4 million 1.13; 12 and
-// 14 2.4 million 0.72 to 1.28; 16 2.4 million 0.73, 3.2 million 1.09; 20 and 24 4.2 million 0.94, 5.6 million 1.03; 32 5.6 million 0.72, 10 million 1.03.
+// 14 2.3 to 2.5 million 0.6 to 0.95 (12 x 196 K 11.2 us, tiles 18.6), three lists of large aligned tensors 1.04; 16 2.4 million 0.73, 3.2 million 1.09; 20 and 24 4.2 million 0.94, 5.6 million 1.03; 32 5.6 million 0.72, 10 million 1.03.
 // Steps that moved with the count by coordinates, 900 points: nine and ten workers 0.8 of the time, 12 and 14 0.8, 16 0.72; 1 in 50 more than 5 % slower.
 inline int64_t crowd_most(int opt, int mt) {
-    if (opt == OPT_SGDM) return mt < 12 ? 1590000 : mt < 16 ? 2300000 : mt == 16 ? 2500000 : mt <= 24 ? 4000000 : mt <= 32 ? 5500000 : mt <= 64 ? 8000000 : 10000000;
+    if (opt == OPT_SGDM) return mt < 12 ? 1590000 : mt <= 16 ? 2500000 : mt <= 24 ? 4000000 : mt <= 32 ? 5500000 : mt <= 64 ? 8000000 : 10000000;
     return mt < 12 ? 2100000 : mt < 16 ? 3100000 : mt == 16 ? 4200000 : mt <= 24 ? 4500000 : mt <= 32 ? 8000000 : 10000000;
 }
 

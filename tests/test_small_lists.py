@@ -42,3 +42,10 @@ def test_sparse_lists_stay_with_the_tiles(M, numel, opt, kernel):
 ])
 def test_lists_are_counted_by_coordinates(M, numel, kernel):
     assert plan(M, numel, "adam", 7)[0] == kernel
+
+
+@pytest.mark.parametrize("M", [12, 13, 14, 15, 16])
+def test_momentum_of_twelve_to_sixteen_workers(M):
+    """Up to 2.5 million coordinates, where the tiles and the runtime-M kernel take up to 1.66 times as long."""
+    assert plan(M, [2_496_000 // M], "sgdm", 3)[0] == plan(M, [2_330_000 // M], "sgdm", 1)[0] == "crowd"
+    assert plan(M, [2_504_000 // M + 1], "sgdm", 3)[0] != "crowd"

@@ -82,6 +82,7 @@ struct WorkerRes {
     desloc::Chunk *d_chunks = nullptr;   // tiles of the step kernels
     int64_t nchunks = 0;
     desloc::ChunkSet set;                // all of them
+    bool full_round = false;             // a plan for them asks how the gradients lie (full_round_of_three)
     long long *d_tstart = nullptr;       // [num_tensors + 1] first tile of every tensor
     std::vector<int64_t> heads;          // [num_tensors] elements of the short first chunk
     std::vector<HostGroup> groups;
@@ -208,6 +209,7 @@ cudaError_t make_worker_res(WorkerRes &r, const desloc_config &cfg, int M, const
     // (a partial sum per chunk, or per block of a chunk where averaging steps run in desloc_crowd_kernel)
     desloc_config as = cfg;
     as.M = M;
+    r.full_round = desloc::full_round_of_three(as, r.set);
     const desloc::LaunchPlan crowd = desloc::plan_launch(as, DESLOC_SYNC_X, r.set, true, false, desloc::GradLayout::FIT);
     const int64_t row = crowd.kernel == desloc::Kernel::CROWD ? nchunks * crowd.parts : nchunks;
     static_assert(sizeof(int) == sizeof(float), "the number of parts lies behind the sums");
@@ -314,7 +316,7 @@ int stage_grads(desloc_ctx *ctx, const void *const *grads, cudaStream_t stream, 
     cudaError_t e = cudaMemcpyAsync(s.dev, s.host, bytes, cudaMemcpyHostToDevice, stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e);
     std::memcpy(ctx->last_grads.data(), grads, bytes);
-    ctx->last_layout = desloc::grad_layout(ctx->cfg, grads, ctx->res.heads.data());
+    ctx->last_layout = desloc::grad_layout(ctx->cfg, grads, ctx->res.heads.data(), ctx->res.full_round);
     ctx->cur_slot = ctx->next_slot;
     ctx->next_slot = (ctx->next_slot + 1) % kSlots;
     ctx->last_stream = stream;
@@ -466,7 +468,7 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
         }
 
         const desloc::GradLayout layout =
-            inline_g ? desloc::grad_layout(c, grads, ctx->res.heads.data()) : ctx->last_layout;
+            inline_g ? desloc::grad_layout(c, grads, ctx->res.heads.data(), ctx->res.full_round) : ctx->last_layout;
         const bool lanes_ok = ctx->staging_mode < 0 && ctx->max_blocks == 0;
         const desloc::LaunchPlan plan = desloc::plan_launch(c, mask, ctx->res.set, diag, max_norm > 0.f, layout, lanes_ok);
         if (!plan.fn) {

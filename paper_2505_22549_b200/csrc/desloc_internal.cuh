@@ -343,12 +343,13 @@ inline bool generic_fills_rounds_better(const desloc_config &c, uint32_t mask, l
 // the parameters have gradients that it cannot take, most of these (bf16) 8-byte aligned -- OFF -- or less -- NARROW.
 // fp32 gradients are FIT or OFF.  heads: elements of the short first chunks; grads: [M][num_tensors].
 enum class GradLayout { FIT, OFF, NARROW };
-inline GradLayout grad_layout(const desloc_config &c, const void *const *grads, const int64_t *heads) {
+// asked: a smaller problem's plan asks, too.
+inline GradLayout grad_layout(const desloc_config &c, const void *const *grads, const int64_t *heads, bool asked) {
     const bool bf16 = c.grad_dtype == DESLOC_BF16;
     int64_t total = 0, off = 0, narrow = 0;
     // (no plan for fewer elements than this asks: the look at 1088 pointers takes 6 us)
     for (int32_t k = 0; k < c.num_tensors; ++k) total += c.numel[k];
-    if (total * c.M < (1 << 21)) return GradLayout::FIT;
+    if (total * c.M < (1 << 21) && !asked) return GradLayout::FIT;
     for (int32_t k = 0; k < c.num_tensors; ++k) {
         const uintptr_t head = static_cast<uintptr_t>(heads[k]) * (bf16 ? 2 : 4);
         uintptr_t bits = 0;
@@ -371,6 +372,18 @@ inline GradLayout grad_layout(const desloc_config &c, const void *const *grads, 
 // to 1.35: a single round of blocks with three tiles each, exactly filled).
 inline int64_t lanes_most(int mt) {
     return mt == 1 ? 16000000 : mt == 2 ? 5000000 : mt == 3 ? 1700000 : mt == 4 ? 7000000 : mt == 8 ? 3800000 : 2000000;
+}
+
+// One round of tile blocks that each update three tiles, at least nineteen in twenty of them full, five workers, Adam or ADOPT, fp32 gradients that
+// fit: where all arrays are averaged, and before the update, the tiles take 0.81 to 1.03 of the lanes' time (once 1.14) from 1.6 million on, 0.9 on
+// average (5 x 350 K 10.8 us, 13.1).  (Smaller ones were not compared.  Not taken: one or two arrays 0.85 to 1.18, 1.0 on average; six workers 0.9 to
+// 1.26, 1.02; SGDM 1.2, averages behind the update 1.5, gradients off the state's layout 1.7.)
+inline bool full_round_of_three(const desloc_config &c, const ChunkSet &chunks) {
+    if (c.M != 5 || c.opt == DESLOC_SGDM || c.grad_dtype == DESLOC_BF16 || (c.flags & DESLOC_FLAG_POST_AVERAGE) ||
+        chunks.total * c.M <= 1600000 || chunks.total * c.M > lanes_most(c.M)) return false;
+    const int64_t tile = tile_elems(c.opt, c.M, false), tiles = (chunks.length + tile - 1) / tile, parts = parts_for(chunks.n, chunks.length, c.opt, c.M, false);
+    const int64_t blocks = chunks.n * parts;
+    return blocks <= static_cast<int64_t>(NUM_SMS) * step_min_blocks(c.opt, c.M, false) && (tiles + parts - 1) / parts == 3 && 20 * chunks.total >= 57 * blocks * tile;
 }
 
 // The same of averaging steps of more than eight workers that run in desloc_crowd_kernel.  Measured, as above: nine and ten workers
@@ -422,7 +435,8 @@ inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, const Chunk
         const bool sgdm = c.opt == OPT_SGDM, sparse = p.parts > 1 && 20 * chunks.total < (sgdm ? 9 : 5) * p.grid * p.part_elems;
         // Blocks for more than twice as many coordinates as the line allows, of lists of thousands of tensors: tiles, too.
         const bool crowded = p.grid * p.part_elems * c.M > 2 * lanes_most(mt);
-        if (!crowded && !(local && sparse && nchunks * c.M > (sgdm ? 2 : 4) * LANES_WAVE)) {
+        const bool tiles_full = kmask == 7 && layout == GradLayout::FIT && full_round_of_three(c, chunks);
+        if (!crowded && !tiles_full && !(local && sparse && nchunks * c.M > (sgdm ? 2 : 4) * LANES_WAVE)) {
             p.kernel = Kernel::LANES;
             p.fn = lookup_lanes_kernel(c.opt, post, bf16, mt, static_cast<int>(kmask));
             p.threads = LANES_THREADS;

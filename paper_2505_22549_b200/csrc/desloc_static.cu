@@ -99,7 +99,7 @@ extern "C" DESLOC_API int desloc_step_static(const desloc_config *cfg, float *co
     const int64_t nchunks = set.n;
     if (nchunks > kMaxChunks) return DESLOC_E_TOO_LARGE;
     const uint32_t mask = desloc::mask_at(cfg, t);
-    const desloc::LaunchPlan plan = desloc::plan_launch(*cfg, mask, set, false, false, desloc::grad_layout(*cfg, grads, g_heads));
+    const desloc::LaunchPlan plan = desloc::plan_launch(*cfg, mask, set, false, false, desloc::grad_layout(*cfg, grads, g_heads, desloc::full_round_of_three(*cfg, set)));
     if (!plan.fn) return DESLOC_E_INVALID;
 
     int dev_before = -1;

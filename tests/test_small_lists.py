@@ -49,3 +49,16 @@ def test_momentum_of_twelve_to_sixteen_workers(M):
     """Up to 2.5 million coordinates, where the tiles and the runtime-M kernel take up to 1.66 times as long."""
     assert plan(M, [2_496_000 // M], "sgdm", 3)[0] == plan(M, [2_330_000 // M], "sgdm", 1)[0] == "crowd"
     assert plan(M, [2_504_000 // M + 1], "sgdm", 3)[0] != "crowd"
+
+
+@pytest.mark.parametrize("M,n,opt,gd,flags,mask,kernel", [
+    (5, 360_000, "adam", "f32", 0, 7, "tiles"), (5, 399_000, "adopt", "f32", 1, 7, "tiles"), (5, 360_000, "adam", "f32", 0, 3, "lanes"),
+    (5, 310_000, "adam", "f32", 0, 7, "lanes"),                                                             # 1.55 million
+    (5, 360_000, "sgdm", "f32", 0, 3, "lanes"), (5, 360_000, "adam", "f32", 2, 7, "lanes"),                 # (averaging behind the update)
+    (5, 360_000, "adam", "bf16", 0, 7, "lanes"), (6, 310_000, "adam", "f32", 0, 7, "lanes"), (4, 500_000, "adam", "f32", 0, 7, "lanes"),
+])
+def test_a_full_round_of_three_tiles_is_left_to_them(M, n, opt, gd, flags, mask, kernel):
+    of = lambda numel, layout: B.desloc_testing_kernel_of(B.make_config(M, numel, opt, gd, flags=flags), mask, 0, layout)[0]
+    assert of([n], 0) == kernel
+    assert of([n], 1) == "lanes"                   # gradients off the state's layout
+    assert of([n // 1000] * 1000, 0) == "lanes"    # as many coordinates in tensors that leave tiles half empty

@@ -248,6 +248,12 @@ relchange_finalize_kernel(float *partial, long long n, long long stride, int M, 
 constexpr int SMALL_THREADS = 512, SMALL_BLOCKS = 8, SMALL_PIECE = 1024, SMALL_PIECES = REDUCE_CHUNK_ELEMS / SMALL_PIECE;
 constexpr int SMALL_WARPS = SMALL_BLOCKS * SMALL_THREADS / 32;
 constexpr int64_t SMALL_BYTES = 4 << 20;   // of all workers
+// Workers whose clusters are all resident at once (two blocks per SM with fp32 gradients, three with bf16), and the chunks from which on more of them
+// come in one launch, too: clusters come in waves then, which cost what the two stages pay for some 40 chunks per worker.  Norm-clipped steps in a
+// graph, one launch and two stages: 64 workers in 3 and 8 tensors 8.3 us and 7.3, 11.4 and 7.7; 128 x 2 K parameters 15.0 and 9.6, 256 x 1 K in 4
+// 28.2 and 16.2; but 64 x 29 K in 100 tensors 21.9 and 27.9, 128 x 100 in 100 14.5 and 20.1, 256 in 47 and 56 1.0 to 1.16 in favour of one.
+constexpr int SMALL_MANY_CHUNKS = 40;
+constexpr int small_workers(bool bf16) { return (bf16 ? 3 : 2) * 148 / SMALL_BLOCKS; }
 
 __device__ __forceinline__ uint32_t first_block_addr(const void *shared) {
     uint32_t r;
@@ -403,7 +409,8 @@ cudaError_t launch_grad_norms(const Chunk *chunks, long long nchunks, int64_t el
                               float *scales, int *err, int wait_limit, cudaStream_t stream, int *launches) {
     // A piece, half a chunk or a chunk for each warp of a cluster.  Beyond 4 MB in all the two stages read no slower (16 workers x 129 K parameters,
     // fp32, in 33 and 65 tensors, in a graph: 19.1 and 18.9 us in two stages, 20.0 and 20.2 in one; 2 bytes each 16.8 and 15.3, 15.7 and 14.1).
-    if (elems <= SMALL_WARPS * SMALL_PIECE && nchunks <= SMALL_WARPS && elems * M * (bf16 ? 2 : 4) <= SMALL_BYTES) {
+    if ((M <= small_workers(bf16) || nchunks >= SMALL_MANY_CHUNKS) && elems <= SMALL_WARPS * SMALL_PIECE && nchunks <= SMALL_WARPS &&
+        elems * M * (bf16 ? 2 : 4) <= SMALL_BYTES) {
         *launches = 1;
         return launch(bf16 ? small_norms_kernel<RED_BF16> : small_norms_kernel<RED_F32>, M * SMALL_BLOCKS, SMALL_THREADS, 0, stream, chunks,
                       nchunks, g, nt, max_norm, norms, scales);

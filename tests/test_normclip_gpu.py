@@ -197,3 +197,22 @@ def test_sums_of_small_problems(gd, numel, align, shift):
         assert np.allclose(n, want, rtol=bound, atol=0)
         assert np.allclose(s, np.minimum(1.0, 0.5 / want), rtol=bound, atol=0)
     eng.close()
+
+
+@pytest.mark.parametrize("gd,M,numel,launches", [
+    ("f32", 37, (33,) * 39, 1), ("f32", 38, (33,) * 39, 2), ("f32", 38, (33,) * 40, 1), ("bf16", 55, (700, 1031), 1),
+    ("bf16", 56, (700, 1031), 2), ("bf16", 256, (17,) * 40, 1), ("f32", 256, (1031,), 2),
+])
+def test_small_norms_of_many_workers(gd, M, numel, launches):
+    """One launch where the clusters of all workers are resident at once (eight blocks each), or the chunks are many."""
+    import paper_2505_22549_b200 as d
+    w = di.Workload("many_sums", "sgdm", M, numel, gd, "normal1", lr=1e-2, K=(0, 0, 0), seed=6)
+    st = State(w, torch.device("cuda:0"))
+    eng = make_engine(d, w, st)
+    st.fill_grads(0)
+    g = st.to_numpy(st.g)[:, _valid(st)].astype(np.float64)
+    before = eng.launches()
+    eng.step_normclip(0, 1e-2, st.views(st.g), 0.5)
+    assert eng.launches() - before == launches + 1
+    assert np.allclose(eng.grad_norms()[0], np.sqrt((g * g).sum(axis=1)), rtol=4.5e-6, atol=0)
+    eng.close()

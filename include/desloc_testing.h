@@ -42,12 +42,15 @@ DESLOC_API int desloc_testing_set_wait_limit(desloc_ctx *ctx, int32_t polls);
 
 /*
  * Which kernel a step with this sync mask runs over nchunks chunks (0: all) of a context created from cfg whose x starts on
- * 2 KB boundaries, without diagnostics: 0 = tiles, 1 = runtime-M, 2 = replicas in the lanes of a warp, 3 = a block of all
+ * 2 KB boundaries, with diagnostics if diag is not 0: 0 = tiles, 1 = runtime-M, 2 = replicas in the lanes of a warp, 3 = a block of all
  * replicas.  layout: how the gradients lie towards 16-byte pieces -- 0 = they fit, 1 = they do not, 2 = nor do bf16 ones
  * towards 8-byte pieces.  blocks, if not NULL: how many thread blocks.
  * Host-only.  Negative desloc_status on bad input.
  */
-DESLOC_API int32_t desloc_testing_kernel_of(const desloc_config *cfg, uint32_t mask, int64_t nchunks, int32_t layout, int64_t *blocks);
+DESLOC_API int32_t desloc_testing_kernel_of(const desloc_config *cfg, uint32_t mask, int64_t nchunks, int32_t layout, int32_t diag, int64_t *blocks);
+
+/* Groups of pieces that desloc_step_host() has had brought by a kernel, not by copies, in this context so far. */
+DESLOC_API int64_t desloc_testing_gathers(const desloc_ctx *ctx);
 
 #ifdef __cplusplus
 }

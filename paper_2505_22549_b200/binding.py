@@ -110,8 +110,10 @@ _lib.desloc_testing_set_max_blocks.argtypes = [_P, ctypes.c_int64]
 _lib.desloc_testing_set_staging.restype = ctypes.c_int
 _lib.desloc_testing_set_staging.argtypes = [_P, ctypes.c_int32]
 _lib.desloc_testing_kernel_of.restype = ctypes.c_int32
-_lib.desloc_testing_kernel_of.argtypes = [ctypes.POINTER(DeslocConfig), ctypes.c_uint32, ctypes.c_int64, ctypes.c_int32,
+_lib.desloc_testing_kernel_of.argtypes = [ctypes.POINTER(DeslocConfig), ctypes.c_uint32, ctypes.c_int64, ctypes.c_int32, ctypes.c_int32,
                                            ctypes.POINTER(ctypes.c_int64)]
+_lib.desloc_testing_gathers.restype = ctypes.c_int64
+_lib.desloc_testing_gathers.argtypes = [_P]
 _lib.desloc_testing_set_wait_limit.restype = ctypes.c_int
 _lib.desloc_testing_set_wait_limit.argtypes = [_P, ctypes.c_int32]
 _lib.desloc_plan_chunks.restype = ctypes.c_int64
@@ -331,13 +333,18 @@ def desloc_testing_set_staging(ctx: int, mode: int) -> None:
         raise DeslocError(rc, "desloc_testing_set_staging")
 
 
-def desloc_testing_kernel_of(cfg: DeslocConfig, mask: int, nchunks: int = 0, layout: int = 0):
+def desloc_testing_kernel_of(cfg: DeslocConfig, mask: int, nchunks: int = 0, layout: int = 0, diag: bool = False):
     """Test hook (include/desloc_testing.h): (kernel, thread blocks) of a step of so many chunks (0: all)."""
     blocks = ctypes.c_int64()
-    n = int(_lib.desloc_testing_kernel_of(ctypes.byref(cfg), mask, int(nchunks), layout, ctypes.byref(blocks)))
+    n = int(_lib.desloc_testing_kernel_of(ctypes.byref(cfg), mask, int(nchunks), layout, int(diag), ctypes.byref(blocks)))
     if n < 0:
         raise DeslocError(n, "desloc_testing_kernel_of")
     return ("tiles", "runtime_m", "lanes", "crowd")[n], blocks.value
+
+
+def desloc_testing_gathers(ctx: int) -> int:
+    """Test hook (include/desloc_testing.h): groups of host gradients brought by a kernel so far."""
+    return int(_lib.desloc_testing_gathers(ctx))
 
 
 def desloc_testing_set_wait_limit(ctx: int, polls: int) -> None:

@@ -260,6 +260,7 @@ struct desloc_ctx {
     cudaStream_t last_stream = nullptr;
     int64_t counters[4] = {0, 0, 0, 0};
     int64_t launches = 0;
+    int64_t gathers = 0;         // groups of host gradients that a kernel has brought (not in `launches`)
     int last_cuda_error = 0;
     bool diag_valid = false;        // a diagnostics step has run since the workers last changed
     int64_t max_blocks = 0;         // test hook: cap on the grid (0 = one block per work item)
@@ -537,6 +538,7 @@ int run_step(desloc_ctx *ctx, uint32_t mask, float lr_t, float clip_bound_t,
                                           c.grad_dtype == DESLOC_BF16 ? 2 : 4};
                     e = stage_host_table(ctx, host_grads, &hg.src);
                     if (e == cudaSuccess) e = desloc::launch_host_gather(hg, ctx->copy_stream);   // (in the copies' place, and not counted either)
+                    if (e == cudaSuccess) ctx->gathers += 1;
                 } else {
                     for_pieces(ctx, grp, host_grads, grads, [&](const char *hp, char *dp, size_t bytes) {
                         e = cudaMemcpyAsync(dp, hp, bytes, cudaMemcpyHostToDevice, ctx->copy_stream);
@@ -958,15 +960,17 @@ int desloc_testing_set_wait_limit(desloc_ctx *ctx, int32_t polls) {
     return DESLOC_OK;
 }
 
-int32_t desloc_testing_kernel_of(const desloc_config *cfg, uint32_t mask, int64_t nchunks, int32_t layout, int64_t *blocks) {
+int32_t desloc_testing_kernel_of(const desloc_config *cfg, uint32_t mask, int64_t nchunks, int32_t layout, int32_t diag, int64_t *blocks) {
     if (!cfg || !cfg->numel) return DESLOC_E_NULL;
     if (validate_config(cfg) != DESLOC_OK || (mask & ~7u) || nchunks < 0 || layout < 0 || layout > 2) return DESLOC_E_INVALID;
     desloc::ChunkSet set = desloc::chunk_set(cfg->numel, cfg->num_tensors, desloc::chunk_elems_for(*cfg, cfg->M));
     if (nchunks > 0) set.n = nchunks;
-    const desloc::LaunchPlan p = desloc::plan_launch(*cfg, mask, set, false, false, static_cast<desloc::GradLayout>(layout));
+    const desloc::LaunchPlan p = desloc::plan_launch(*cfg, mask, set, diag != 0, false, static_cast<desloc::GradLayout>(layout));
     if (blocks) *blocks = p.grid * p.grid_y;
     return p.fn ? static_cast<int32_t>(p.kernel) : DESLOC_E_INVALID;
 }
+
+int64_t desloc_testing_gathers(const desloc_ctx *ctx) { return ctx ? ctx->gathers : 0; }
 
 int desloc_last_cuda_error(const desloc_ctx *ctx) { return ctx ? ctx->last_cuda_error : 0; }
 

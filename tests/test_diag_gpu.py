@@ -162,12 +162,14 @@ def test_more_than_eight_workers_in_either_kernel(M, opt, gd, post, align):
     piece = 64 if M < 12 else 32 if M <= 32 else 16
     numel = (1, 3, piece - 1, piece, 2 * piece + 1, 516, 1031, 2049)
     w = di.Workload("diag", opt, M, numel, gd, "normal1", beta2=0.99, eps=1e-2, lr=1e-2, weight_decay=0.05, clip_rho=1.5,
-                    adopt_norm_clip=(opt == "adopt"), K=(1, 2, 2), seed=M)
+                    adopt_norm_clip=(opt == "adopt"), K=(2, 3, 4), seed=M)
+    cfg = d.make_config(M, numel, opt, gd, flags=(2 if post else 0) | (opt == "adopt"))
+    assert [d.desloc_testing_kernel_of(cfg, mask, diag=True)[0] for mask in (0, 1, 2, 3)] == ["tiles"] + ["crowd"] * 3
     dev = torch.device("cuda:0")
     a, b = (State(w, dev, align=align, v_init=0.25) for _ in range(2))
     ea, eb = make_engine(d, w, a, post), make_engine(d, w, b, post)
     d.desloc_testing_set_staging(eb.ctx, 0)
-    for t in range(3):
+    for t in range(5):       # everything averaged, nothing, x, u, x and v
         a.fill_grads(t)
         for m in range(M):
             b.g[m].copy_(a.g[m])

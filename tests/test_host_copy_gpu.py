@@ -72,8 +72,10 @@ def test_many_pieces_arrive_group_by_group(gd, shift_h, shift_d, M, numel, separ
         host = [[pin(n) for n in numel] for _ in range(M)] if separate else [[f[o + 1:o + 1 + n] for o, n in zip(st.offs, numel)] for f in flat]
         for g in st.g:
             g.fill_(7.0)
+        before = d.desloc_testing_gathers(eng.ctx)
         eng.step_host(t, 1e-2, host, st.views(st.g))
         torch.cuda.synchronize()
+        assert (d.desloc_testing_gathers(eng.ctx) > before) == pinned
         for m in range(M):
             for x, y in zip(host[m], st.views(st.g)[m]):
                 assert torch.equal(x, y.cpu())

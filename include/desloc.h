@@ -185,7 +185,8 @@ DESLOC_API int desloc_step_masked(desloc_ctx *ctx, uint32_t mask, float lr_t, fl
  * appendix gives the bound on the gradient's L2 norm, 1.0, in its rho column); Algorithms 1-3
  * only have the coordinate-wise clip.  Costs one more read of the gradients: two reduction
  * launches (per-chunk partial sums in fp32, per-worker totals in fp64, fixed order, no
- * atomics), or one for up to 131072 parameters in few tensors, ahead of the step kernel, all enqueued on `stream` without host synchronisation.
+ * atomics), or one where the gradients are small (up to 131072 parameters in 128 chunks of 4096 and 4 MB over all workers; beyond 37 workers, 55 with
+ * bf16 gradients, only from 40 chunks on), ahead of the step kernel, all enqueued on `stream` without host synchronisation.
  * max_norm must be > 0 and finite.  Other arguments as desloc_step().
  */
 DESLOC_API int desloc_step_normclip(desloc_ctx *ctx, int64_t t, float lr_t, float clip_bound_t,
@@ -210,7 +211,7 @@ DESLOC_API int desloc_get_grad_norms(desloc_ctx *ctx, float *norms_out, float *s
  * -- the gradient, parameter and update norms the paper tracks (gradient norms after the
  * workers are doubled, Section 6, RQ3; update and parameter norms of the billion-scale runs,
  * additional-results appendix).  The step kernel already has all three on chip, so the
- * sums of squares are formed there, one partial per (kind, worker, chunk): no extra pass over
+ * sums of squares are formed there, one partial per (kind, worker, chunk) or part of a chunk: no extra pass over
  * memory, and the step computes exactly what desloc_step() computes.
  *   max_norm : > 0 puts norm-based clipping in front as desloc_step_normclip() does; 0 = off.
  * Other arguments as desloc_step().  Not available with desloc_step_host().
@@ -224,10 +225,11 @@ DESLOC_API int desloc_step_diag(desloc_ctx *ctx, int64_t t, float lr_t, float cl
  *   per_tensor_out : host, [3][M][num_tensors] floats, entry (kind * M + m) * num_tensors + k,
  *                    or NULL;
  *   total_out      : host, [3][M] floats, the norm over the whole tensor list, or NULL.
- * Per-chunk partials are fp32; they are added per tensor, and the tensors per worker, in fp64
+ * Partials, of a chunk or a part of one, are fp32; they are added per tensor, and the tensors per worker, in fp64
  * in a fixed order (no atomics: the same buffers and inputs give the same bits; where the chunks
- * of a tensor begin follows the alignment of worker 0's x, see desloc_plan_chunks_at()).  One small launch on `stream`; the
- * call waits for `stream`.  DESLOC_E_INVALID if no diagnostics step has run since
+ * of a tensor begin follows the alignment of worker 0's x, see desloc_plan_chunks_at()).  "Latest" is the step that ran last on the
+ * device, a replayed graph's included (none yet, only captured ones: zeros).  One small launch on `stream`; the call waits for the result: what was on the stream before is complete
+ * then.  DESLOC_E_DEVICE_WAIT if a wait in front ran out.  DESLOC_E_INVALID if no diagnostics step has been made since
  * the context was created or its workers were changed.
  */
 DESLOC_API int desloc_get_diag_norms(desloc_ctx *ctx, float *per_tensor_out, float *total_out,

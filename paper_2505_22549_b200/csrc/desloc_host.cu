@@ -83,7 +83,7 @@ struct WorkerRes {
     int64_t nchunks = 0;
     desloc::ChunkSet set;                // all of them
     bool full_round = false;             // a plan for them asks how the gradients lie (full_round_of_three)
-    long long *d_tstart = nullptr;       // [num_tensors + 1] first tile of every tensor
+    long long *d_tstart = nullptr;       // [num_tensors + 1] first tile of every tensor, and a word for d_diag_parts
     std::vector<int64_t> heads;          // [num_tensors] elements of the short first chunk
     std::vector<HostGroup> groups;
     void **d_tables = nullptr;  // [3][nptr] x, u, v
@@ -96,7 +96,7 @@ struct WorkerRes {
     void **d_snap = nullptr;
     Slot host_slots[2];          // tables of addresses in host memory (desloc_step_host), staged on the copy stream
     // Diagnostics step: [3][M][row] sums of squares, of a chunk each or, in desloc_crowd_kernel, of a part of one.  How many a chunk
-    // has is written beside them by the step that leaves them: the host does not see when a captured step runs.
+    // has is written by the step that leaves them (behind d_tstart): the host does not see when a captured step runs.
     float *d_diag = nullptr;
     int *d_diag_parts = nullptr;
     // Results the host waits for go to its memory straight from the kernels, without a copy: [3][M][num_tensors] per-tensor norms,
@@ -175,7 +175,7 @@ cudaError_t make_worker_res(WorkerRes &r, const desloc_config &cfg, int M, const
     const int64_t nchunks = r.set.n;
     std::vector<desloc::Chunk> chunks(static_cast<size_t>(nchunks));
     desloc::fill_chunks(numel, num_tensors, chunk_elems, chunks.data(), heads.data());
-    std::vector<long long> tstart(static_cast<size_t>(num_tensors) + 1, 0);
+    std::vector<long long> tstart(static_cast<size_t>(num_tensors) + 2, 0);   // (the last one: *d_diag_parts, 0 before any step)
     for (int32_t k = 0; k < num_tensors; ++k)
         tstart[k + 1] = tstart[k] + desloc::chunks_of(numel[k], chunk_elems, heads[k]);
     plan_host_groups(r.groups, chunks, numel, total);
@@ -188,6 +188,7 @@ cudaError_t make_worker_res(WorkerRes &r, const desloc_config &cfg, int M, const
     if (e0 == cudaSuccess)
         e0 = cudaMemcpy(r.d_tstart, tstart.data(), tstart.size() * sizeof(long long), cudaMemcpyHostToDevice);
     if (e0 != cudaSuccess) return e0;
+    r.d_diag_parts = reinterpret_cast<int *>(r.d_tstart + num_tensors + 1);
 
     const int64_t nptr = static_cast<int64_t>(M) * num_tensors;
     std::vector<void *> tables(static_cast<size_t>(3 * nptr), nullptr);
@@ -212,12 +213,7 @@ cudaError_t make_worker_res(WorkerRes &r, const desloc_config &cfg, int M, const
     r.full_round = desloc::full_round_of_three(as, r.set);
     const desloc::LaunchPlan crowd = desloc::plan_launch(as, DESLOC_SYNC_X, r.set, true, false, desloc::GradLayout::FIT);
     const int64_t row = crowd.kernel == desloc::Kernel::CROWD ? nchunks * crowd.parts : nchunks;
-    static_assert(sizeof(int) == sizeof(float), "the number of parts lies behind the sums");
-    if (e == cudaSuccess) e = cudaMalloc(&r.d_diag, (ndiag * static_cast<size_t>(row) + 1) * sizeof(float));
-    if (e == cudaSuccess) {
-        r.d_diag_parts = reinterpret_cast<int *>(r.d_diag + ndiag * static_cast<size_t>(row));
-        e = cudaMemset(r.d_diag_parts, 0, sizeof(int));
-    }
+    if (e == cudaSuccess) e = cudaMalloc(&r.d_diag, ndiag * static_cast<size_t>(row) * sizeof(float));
     if (e == cudaSuccess)
         e = cudaHostAlloc(reinterpret_cast<void **>(&r.h_out), (ndiag * (num_tensors + 1) + M + 2) * sizeof(float),
                           cudaHostAllocMapped);
@@ -232,8 +228,6 @@ cudaError_t make_worker_res(WorkerRes &r, const desloc_config &cfg, int M, const
         s.dev = r.d_slots + i * room;
         e = cudaEventCreateWithFlags(&s.done, cudaEventDisableTiming);
     }
-    // (memsets are asynchronous, and the caller's stream need not wait for this one)
-    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
     return e;
 }
 
@@ -400,8 +394,8 @@ cudaError_t prepare_once(desloc_ctx *ctx, const desloc::LaunchPlan &plan) {
     return e;
 }
 
-// max_norm > 0: norm-based clipping first (two reduction launches), then the step.
-// diag: the step kernel also accumulates the per-chunk sums of squares of g, x_{t+1} and d_t.
+// max_norm > 0: norm-based clipping first (a reduction launch or two, see launch_grad_norms()), then the step.
+// diag: the step kernel also leaves sums of squares of g, x_{t+1} and d_t, per chunk or part of one.
 // host_grads != nullptr: the gradients are first brought from host memory into `grads` (device): by a kernel on `stream`
 // where host_runs_of() allows it, else tensor group by tensor group on the context's copy stream, each group's
 // kernel starting as soon as its copies have landed.

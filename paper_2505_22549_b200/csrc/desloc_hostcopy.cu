@@ -1,7 +1,7 @@
 // Gradients from pinned host memory to the device by kernels that read it: small problems in one launch, lists of many pieces group by group.
 //
-// Bound: PCIe.  A copy by the copy engine costs 6 us beside its bytes, one per worker and contiguous piece at best, and the
-// step waits for it through two events on two streams.  Here one kernel in the step's own stream reads the host's
+// Bound: PCIe.  A copy by the copy engine costs 4.3 us beside its bytes where others are behind it, 6 us by itself, one per worker and contiguous
+// piece at best, and the step waits for it through two events on two streams.  Here one kernel in the step's own stream reads the host's
 // memory directly, every byte requested at once, and the step kernel may begin behind it without a gap.
 // Measured on B200, the whole call of step_host (before, copies): two workers x 4096 parameters, fp32, 17.1 us (24.9); eight x 20 K 19.2
 // (50.2), x 100 K 69.2 (100.1); four x 189 K in 21 tensors, bf16, 36.0 (69.1), eight x 260 K 91.0 (123.5).  47 GB/s; large
@@ -9,7 +9,9 @@
 // of 4 MB: 85.2 us against 86.8).
 //
 // Lists whose tensors do not follow one another on both sides: a copy by the engine costs 4.3 us beside its bytes at 55.1 GB/s (752 of 237 KB:
-// 8.5 us each, 27.8 GB/s; on two to four streams the same), kernels read 51.0 GB/s whatever the pieces, with 16 blocks as with 600.
+// 8.5 us each, 27.8 GB/s; on two to four streams the same), kernels read 51.0 GB/s, with 16 blocks as with 600, where the two sides lie alike
+// within 16 bytes.  Else a lane brings less at a time: calls of 25 MB in pieces of 32 KB to 1 MB, SGDM step and all, 42 to 49 GB/s alike, 36 to 41
+// off by 4 or 8 bytes, 35 to 38 off by 2; by copies 7 (32 KB), 17 (128 KB), 18 to 32 (512 KB, 1 MB).
 #include "desloc_hostcopy.cuh"
 
 #include <cuda.h>

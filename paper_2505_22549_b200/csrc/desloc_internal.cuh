@@ -282,8 +282,8 @@ struct LaunchPlan {
     bool overlap = true;  // may begin while the kernel in front of it still runs (not the runtime-M kernel)
 };
 
-// Steps with norm diagnostics (small problems without them run in desloc_lanes_kernel and desloc_crowd_kernel): launches
-// of at most this many blocks of single-tile chunks (two per SM of a B200: one wave)
+// Steps with norm diagnostics (small problems without them, and averaging ones of more than eight workers with them, run in
+// desloc_lanes_kernel and desloc_crowd_kernel): launches of at most this many blocks of single-tile chunks (two per SM of a B200: one wave)
 // skip the staging.  Measured on 4096 parameters and two workers: 3.08 us per step in a
 // CUDA graph of 16 steps against 3.34 us staged.
 constexpr long long DIRECT_GRID = 2 * NUM_SMS;
@@ -368,8 +368,8 @@ inline GradLayout grad_layout(const desloc_config &c, const void *const *grads, 
 // 1.02 to 1.03; two workers 3 million 0.95, 4.6 million 1.02; four 5 to 7 million 0.98, 10 million 1.0; eight 3 to 5 million 0.8 to 0.9
 // (from 4.2 million on, behind one another from Python, 1.05 to 1.13), 10 million 1.07; three, and five to seven, of which lanes are idle, 1.5 million 0.7 to 0.9, 2.2 million 0.8 to 1.05, 5 million 1.02 to 1.06.
 // Counted by chunks times their length, as they were before, lists of many tensors left these kernels at half the size.  Averaging steps that
-// moved, 1400 other points, arrays cold and not: five to seven workers 0.86 of the time, eight 0.88; one in 50 is more than 5 % slower (up
-// to 1.35: a single round of blocks with three tiles each, exactly filled).
+// moved, 1600 random lists at the lines against the tiles: four workers 0.98 of the time (up to 1.07), five to seven 0.7 (five: see
+// full_round_of_three), eight 0.85 (3 in 100 lists above 1.04, up to 1.1: a single round of tile blocks, exactly filled).
 inline int64_t lanes_most(int mt) {
     return mt == 1 ? 16000000 : mt == 2 ? 5000000 : mt == 3 ? 1700000 : mt == 4 ? 7000000 : mt == 8 ? 3800000 : 2000000;
 }
@@ -391,7 +391,8 @@ inline bool full_round_of_three(const desloc_config &c, const ChunkSet &chunks) 
 // 20 and 24 3.2 million 0.67, 4.2 million 0.7, 5.6 million 0.9 (up to 1.2); 32 5.6 million 0.78, 10 million 0.9; 64 7 million 0.7, 10 million 0.98; 128 and
 // 256 up to ten million 0.03 to 0.82 (15: 0.7 to 1.2).  SGDM, which has the least to load, by itself: nine and ten 1.8 million 0.8, 2.4 million 1.13; 12 and
 // 14 2.3 to 2.5 million 0.6 to 0.95 (12 x 196 K 11.2 us, tiles 18.6), three lists of large aligned tensors 1.04; 16 2.4 million 0.73, 3.2 million 1.09; 20 and 24 4.2 million 0.94, 5.6 million 1.03; 32 5.6 million 0.72, 10 million 1.03.
-// Steps that moved with the count by coordinates, 900 points: nine and ten workers 0.8 of the time, 12 and 14 0.8, 16 0.72; 1 in 50 more than 5 % slower.
+// Steps that moved with the count by coordinates, 900 random lists: nine and ten workers 0.7 of the time, 12 and 14 0.82, 16 0.78; 2 in 100 above 1.04, up to
+// 1.19 (all arrays averaged, a single round of tile blocks, exactly filled; half of the lists that fill one so take 0.8, by how the workers' tensors lie).
 inline int64_t crowd_most(int opt, int mt) {
     if (opt == OPT_SGDM) return mt < 12 ? 1590000 : mt <= 16 ? 2500000 : mt <= 24 ? 4000000 : mt <= 32 ? 5500000 : mt <= 64 ? 8000000 : 10000000;
     return mt < 12 ? 2100000 : mt < 16 ? 3100000 : mt == 16 ? 4200000 : mt <= 24 ? 4500000 : mt <= 32 ? 8000000 : 10000000;
@@ -418,7 +419,7 @@ inline LaunchPlan plan_launch(const desloc_config &c, uint32_t mask, const Chunk
     const bool post = (c.flags & DESLOC_FLAG_POST_AVERAGE) != 0;
     const bool bf16 = c.grad_dtype == DESLOC_BF16;
     const bool local = kmask == 0;
-    // More than eight workers: tiles of all replicas up to sixteen, the runtime-M kernel beyond, for the
+    // More than eight workers, beyond crowd_most(): tiles of all replicas up to sixteen, the runtime-M kernel beyond, for the
     // post-average ordering and for the norm diagnostics.  All-sync steps of sixteen workers (Adam, bf16
     // gradients): 6.52 TB/s in tiles, 6.29 in the runtime-M kernel; nine workers 6.2 and 5.89.
     const int mt = local ? 1 : c.M;

@@ -139,7 +139,7 @@ class DesLoc:
 
     def diag_norms(self):
         """(per_tensor [3][M][num_tensors], total [3][M]) of the latest step_diag; kind 0 =
-        gradient as read, 1 = new parameters, 2 = update d_t.  Synchronises the current stream."""
+        gradient as read, 1 = new parameters, 2 = update d_t.  Waits for the results: what was on the current stream is done."""
         r = _native.diag_norms(self.ctx, self.M, len(self.numel), self._index)
         if isinstance(r, int):
             self._raise(r, "desloc_get_diag_norms")
@@ -151,7 +151,7 @@ class DesLoc:
         return B.desloc_get_grad_norms(self.ctx, self.M, stream)
 
     def rel_change(self, array: int, then: Sequence[Sequence[torch.Tensor]]):
-        """Per-worker ||s - then|| / ||then|| against a snapshot (lists like x); synchronises."""
+        """Per-worker ||s - then|| / ||then|| against a snapshot (lists like x); waits like diag_norms()."""
         r = _native.rel_change(self.ctx, array, self._fill(self._table2, then, B.DESLOC_F32, 0, _SNAP_MISFIT),
                                self._index, self.M)
         if not isinstance(r, list):

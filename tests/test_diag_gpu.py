@@ -215,3 +215,24 @@ def test_norms_are_those_of_the_step_that_ran_last(M):
     torch.cuda.synchronize()
     assert np.array_equal(a.to_numpy(a.x), b.to_numpy(b.x))
     ea.close(); eb.close()
+
+
+@pytest.mark.parametrize("M", [2, 12])
+def test_a_captured_step_that_has_not_run_has_no_norms(M):
+    import paper_2505_22549_b200 as d
+    w = di.Workload("unrun", "sgdm", M, (3000, 17), "f32", "normal1", lr=1e-2, K=(2, 2, 2), seed=M)
+    st = State(w, torch.device("cuda:0"))
+    eng = make_engine(d, w, st)
+    st.fill_grads(0)
+    side, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        with torch.cuda.graph(graph, stream=side):
+            eng.step_diag(0, 1e-2, st.views(st.g))
+        per, total = eng.diag_norms()
+        assert not np.any(per) and not np.any(total)
+        graph.replay()
+        assert np.all(np.asarray(eng.diag_norms()[1]) > 0)
+    torch.cuda.synchronize()
+    del graph
+    eng.close()

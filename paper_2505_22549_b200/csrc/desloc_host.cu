@@ -100,7 +100,7 @@ struct WorkerRes {
     float *d_diag = nullptr;
     int *d_diag_parts = nullptr;
     // Results the host waits for go to its memory straight from the kernels, without a copy: [3][M][num_tensors] per-tensor norms,
-    // [3][M] totals; [M] relative changes; a word behind either for the state of the wait flag.
+    // [3][M] totals; [M] relative changes; behind either a word that releases them.
     float *h_out = nullptr;      // mapped pinned memory, and
     float *d_out = nullptr;      // the same as the kernels address it
 };
@@ -747,10 +747,10 @@ int desloc_get_diag_norms(desloc_ctx *ctx, float *per_tensor_out, float *total_o
     float *const out = ctx->res.h_out;
     desloc::expect_results(out, per + rows + 1);
     e = desloc::launch_diag_norms(ctx->res.d_diag, ctx->res.nchunks, ctx->res.d_diag_parts, ctx->res.d_tstart, c.num_tensors, c.M,
-                                  ctx->res.d_out, ctx->res.d_out + per, ctx->d_err, ctx->res.d_out + per + rows, st);
+                                  ctx->res.d_out, ctx->res.d_out + per, ctx->res.d_out + per + rows, st);
     if (e == cudaSuccess) ctx->launches += 1;
     if (e == cudaSuccess) e = desloc::wait_for_results(out, per + rows + 1, [st] { return cudaStreamSynchronize(st); });
-    const bool valid = e == cudaSuccess && out[per + rows] == 0.f;
+    const bool valid = e == cudaSuccess && !wait_ran_out(ctx);
     if (valid) {
         if (per_tensor_out) std::memcpy(per_tensor_out, out, per * sizeof(float));
         if (total_out) std::memcpy(total_out, out + per, rows * sizeof(float));
@@ -841,7 +841,7 @@ int desloc_rel_change(desloc_ctx *ctx, int32_t array, const float *const *then, 
             ctx->res.d_partial, ctx->res.d_out + at, ctx->res.d_out + at + M, ctx->d_err, ctx->wait_limit, st);
     if (e == cudaSuccess) ctx->launches += 2;
     if (e == cudaSuccess) e = desloc::wait_for_results(change, M + 1, [st] { return cudaStreamSynchronize(st); });
-    const bool valid = e == cudaSuccess && change[M] == 0.f;
+    const bool valid = e == cudaSuccess && !wait_ran_out(ctx);
     if (valid) std::memcpy(out, change, M * sizeof(float));
     if (dev_before != ctx->device) cudaSetDevice(dev_before);
     if (e != cudaSuccess) return cuda_fail(ctx, e);

@@ -198,13 +198,12 @@ __device__ __forceinline__ void finish_norm(double ss, float max_norm, float *no
     *scale = (max_norm > 0.f && nrm > static_cast<double>(max_norm)) ? static_cast<float>(static_cast<double>(max_norm) / nrm) : 1.f;
 }
 
-// The last word of a read-out: has a bounded wait of a kernel in front run out?  Its flag lies in the host's memory: a block of its own, the first,
-// looks there and writes the word while the others add up (behind the sums of one of them: 2 us more).
-__device__ __forceinline__ void hand_over_flag(const int *err, float *word) {
+// The last word of a read-out: behind it, all that is complete for this kernel's wait is complete for the host that sees the word -- the flag of
+// a bounded wait that ran out, too, which an earlier kernel has stored there.  By a block of its own, the first, while the others add up.
+__device__ __forceinline__ void release_results(float *word) {
     if (threadIdx.x != 0) return;
-    const int flag = *reinterpret_cast<const volatile int *>(err);
-    __threadfence_system();   // what is complete for this thread is complete for the host that sees the word
-    *reinterpret_cast<volatile float *>(word) = flag != 0 ? 1.f : 0.f;
+    __threadfence_system();
+    *reinterpret_cast<volatile float *>(word) = 1.f;
 }
 
 constexpr int FINAL_THREADS = 512;
@@ -223,11 +222,11 @@ norm_finalize_kernel(float *partial, long long n, long long stride, float max_no
 }
 
 __global__ void __launch_bounds__(FINAL_THREADS)
-relchange_finalize_kernel(float *partial, long long n, long long stride, int M, float *out, const int *err, float *ran_out) {
+relchange_finalize_kernel(float *partial, long long n, long long stride, int M, float *out, float *released) {
     __shared__ double sh[FINAL_THREADS / 32];
     begin_and_let_next_begin();
     wait_for_earlier_kernels();
-    if (blockIdx.x == 0) return hand_over_flag(err, ran_out);
+    if (blockIdx.x == 0) return release_results(released);
     const int m = blockIdx.x - 1;
     float *row = partial + m * stride, *row2 = partial + (static_cast<long long>(M) + m) * stride;
     pad_row(row, n, stride);
@@ -356,11 +355,11 @@ constexpr int DIAG_THREADS = 256;
 
 __global__ void __launch_bounds__(DIAG_THREADS)
 diag_norms_kernel(const float *partial, long long nchunks, const int *parts_of, const long long *tstart, int nt, int rows, float *norms,
-                  float *totals, const int *err, float *ran_out) {
+                  float *totals, float *released) {
     __shared__ double sh[DIAG_THREADS / 32];
     begin_and_let_next_begin();
     wait_for_earlier_kernels();
-    if (blockIdx.x == 0) return hand_over_flag(err, ran_out);
+    if (blockIdx.x == 0) return release_results(released);
     const int parts = *parts_of, block = static_cast<int>(blockIdx.x) - 1;
     const long long stride = nchunks * parts;
     const bool whole = block < rows;
@@ -425,23 +424,23 @@ cudaError_t launch_grad_norms(const Chunk *chunks, long long nchunks, int64_t el
 }
 
 cudaError_t launch_rel_change(const Chunk *chunks, long long nchunks, const float *const *now,
-                              const float *const *then, int nt, int M, float *partial, float *out, float *ran_out,
+                              const float *const *then, int nt, int M, float *partial, float *out, float *released,
                               int *err, int wait_limit, cudaStream_t stream) {
     long long items, stride;
     const cudaError_t e = launch_sumsq<RED_CHANGE>(
         chunks, nchunks, reinterpret_cast<const void *const *>(now), reinterpret_cast<const void *const *>(then), nt, M,
         partial, &items, &stride, err, wait_limit, stream);
     if (e != cudaSuccess) return e;
-    return launch(relchange_finalize_kernel, M + 1, FINAL_THREADS, 0, stream, partial, items, stride, M, out, err, ran_out);
+    return launch(relchange_finalize_kernel, M + 1, FINAL_THREADS, 0, stream, partial, items, stride, M, out, released);
 }
 
 cudaError_t launch_diag_norms(const float *partial, long long nchunks, const int *parts, const long long *tstart,
-                              int nt, int M, float *per_tensor, float *totals, const int *err, float *ran_out,
+                              int nt, int M, float *per_tensor, float *totals, float *released,
                               cudaStream_t stream) {
     const int rows = DIAG_KINDS * M;
     const long long blocks = 1 + rows + static_cast<long long>(rows) * nt;
     return launch(diag_norms_kernel, grid_for(blocks), DIAG_THREADS, 0, stream, partial, nchunks, parts, tstart, nt, rows,
-                  per_tensor, totals, err, ran_out);
+                  per_tensor, totals, released);
 }
 
 cudaError_t launch_mean_fill(const Chunk *chunks, long long nchunks, const float *const *src,

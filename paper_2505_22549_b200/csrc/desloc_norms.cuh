@@ -17,16 +17,17 @@ cudaError_t launch_grad_norms(const Chunk *chunks, long long nchunks, int64_t el
                               float *scales, int *err, int wait_limit, cudaStream_t stream, int *launches);
 
 // partial: scratch of at least 2 * M * reduce_row(nchunks) floats; out[m] = ||now - then|| / ||then||
-// (out may be host memory that the device can write to).  *ran_out = 1 if *err is set behind that, else 0, written last.  Two launches.
+// (out may be host memory that the device can write to).  *released is written with a release at system
+// scope, behind all that is in front in the stream.  Two launches.
 cudaError_t launch_rel_change(const Chunk *chunks, long long nchunks, const float *const *now,
-                              const float *const *then, int nt, int M, float *partial, float *out, float *ran_out,
+                              const float *const *then, int nt, int M, float *partial, float *out, float *released,
                               int *err, int wait_limit, cudaStream_t stream);
 
 // Norms of a diagnostics step: partial [DIAG_KINDS][M][nchunks * *parts] sums of squares of the parts of a chunk,
 // tstart [nt + 1] first chunk of every tensor; writes per_tensor [DIAG_KINDS][M][nt] and totals
-// [DIAG_KINDS][M] (floats; may be host memory that the device can write to), and *ran_out as above.  One launch.
+// [DIAG_KINDS][M] (floats; may be host memory that the device can write to), and *released as above.  One launch.
 cudaError_t launch_diag_norms(const float *partial, long long nchunks, const int *parts, const long long *tstart,
-                              int nt, int M, float *per_tensor, float *totals, const int *err, float *ran_out,
+                              int nt, int M, float *per_tensor, float *totals, float *released,
                               cudaStream_t stream);
 
 // Every element of the m_dst destination replicas := mean over the m_src source replicas.

@@ -75,8 +75,8 @@ def _run_check(tmp_path, name, *objects):
     assert r.returncode == 0 and name + ": ok" in r.stdout, r.stdout + r.stderr
 
 
-def test_read_outs_wait_for_the_state_of_the_wait_flag(tmp_path):
-    """Results that are there before the word that says whether they are complete are not handed out."""
+def test_read_outs_wait_for_the_word_that_releases_them(tmp_path):
+    """Results that are there before what an earlier kernel has stored beside them, its wait flag, are not handed out."""
     _run_check(tmp_path, "readout_check")
 
 
